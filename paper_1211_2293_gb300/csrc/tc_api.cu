@@ -67,6 +67,8 @@ struct tc_ctx {
     int64_t* idx_dev = nullptr;
     int64_t cap_idx = 0;
     double* dir_out = nullptr;
+    double* dir_part = nullptr;  // per-slice partial sums of a direct sum
+    int64_t cap_dir_part = 0;
     // per-node scratch
     uint32_t *pre_level = nullptr, *pre_first = nullptr, *iota = nullptr, *bfs_of_pre = nullptr, *lvl_alt = nullptr;
     NodeTables nt{};
@@ -1287,9 +1289,15 @@ int tc_direct(tc_ctx* c, const int64_t* idx, int64_t ns, float eps, float G, dou
         TC_GROW(c, c->dir_out, 4 * ns);
         c->cap_idx = ns;
     }
+    const int64_t part = 4 * ns * direct_slices(c->n, ns);
+    if (part > c->cap_dir_part) {
+        c->cap_dir_part = 0;
+        TC_GROW(c, c->dir_part, part);
+        c->cap_dir_part = part;
+    }
     TC_CUDA(c, cudaMemcpyAsync(c->idx_dev, hidx.data(), ns * sizeof(int64_t), cudaMemcpyHostToDevice, c->stream));
-    launch_direct(c->pos, c->mass, c->sys_of, c->sysp, c->idx_dev, ns, eps * eps, G, c->dir_out, c->dir_out + 3 * ns,
-                  c->stream);
+    launch_direct(c->pos, c->mass, c->sys_of, c->sysp, c->idx_dev, c->n, ns, eps * eps, G, c->dir_part, c->dir_out,
+                  c->dir_out + 3 * ns, c->stream);
     TC_CUDA(c, cudaGetLastError());
     TC_CUDA(c, cudaMemcpyAsync(acc, c->dir_out, 3 * ns * sizeof(double), cudaMemcpyDefault, c->stream));
     if (pot) TC_CUDA(c, cudaMemcpyAsync(pot, c->dir_out + 3 * ns, ns * sizeof(double), cudaMemcpyDefault, c->stream));

@@ -1,0 +1,60 @@
+// tc_f32x2.cuh -- Blackwell's paired FP32 instructions and the SFU rsqrt.
+//
+// add/sub/mul/fma .f32x2 work on a 64-bit register holding two floats, each
+// half rounded as the scalar instruction rounds it.
+#pragma once
+#include <cuda_runtime.h>
+
+namespace tc {
+
+namespace {
+
+typedef unsigned long long f2;
+
+__device__ __forceinline__ f2 f2pack(float a, float b)
+{
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void f2unpack(f2 r, float& a, float& b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
+}
+__device__ __forceinline__ f2 f2sub(f2 a, f2 b)
+{
+    f2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 f2mul(f2 a, f2 b)
+{
+    f2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 f2fma(f2 a, f2 b, f2 c)
+{
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ float f2sum(f2 a)
+{
+    float x, y;
+    f2unpack(a, x, y);
+    return x + y;
+}
+
+// 1/sqrt(x) on the SFU, flushing subnormals (x >= eps^2 > 0 is normal here),
+// so no range fix-up surrounds the approximation
+__device__ __forceinline__ float rsqrt_sfu(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+}  // namespace
+
+}  // namespace tc

@@ -320,9 +320,10 @@ void launch_kick_drift(float* pos, float* vel, const float* acc, int64_t n, floa
 void launch_kick(float* vel, const float* acc, int64_t n, float hkick, const Info* info, cudaStream_t s);
 void launch_diag(const float* pos, const float* vel, const float* mass, const float* pot,
                  int64_t n, Info* info, cudaStream_t s);
+int direct_slices(int64_t n, int64_t ns);  // slices of launch_direct's scratch (each 4 ns doubles)
 void launch_direct(const float* pos, const float* mass, const uint32_t* sys_of, const SysParams* sysp,
-                   const int64_t* idx, int64_t ns, float eps2, float G, double* acc, double* pot,
-                   cudaStream_t s);
+                   const int64_t* idx, int64_t n, int64_t ns, float eps2, float G, double* part, double* acc,
+                   double* pot, cudaStream_t s);
 
 // fast multipole method (tc_fmm.cu).  Level starts: lstart[l] is the first
 // breadth-first index of level l, lstart[l] = M past the deepest level

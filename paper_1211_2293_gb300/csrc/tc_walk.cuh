@@ -39,6 +39,7 @@
 // (compensated accumulation); the plain mode uses absolute float centres of
 // mass and plain accumulation.
 #pragma once
+#include "tc_f32x2.cuh"
 #include "tc_internal.cuh"
 #include "tc_mma.cuh"
 
@@ -50,48 +51,11 @@ namespace {
 // flush may pad one entry, so a tile of TILE entries needs TILE + 34 slots
 __host__ __device__ constexpr int tile_cap(int tile) { return tile + 34; }
 
-// ---------------------------------------------------------------- packed FP32
-// Blackwell's paired FP32 instructions (add/sub/mul/fma .f32x2) work on a
-// 64-bit register holding two floats.  A list tile is stored pair-interleaved
-// -- {x_j, x_j+1}, {y_j, y_j+1}, {z_j, z_j+1}, {m_j, m_j+1} per pair of
-// entries -- so one pair of 16-byte shared loads yields two sources already
-// packed, and every FP32 operation of the force loop serves two sources.
-typedef unsigned long long f2;
-
-__device__ __forceinline__ f2 f2pack(float a, float b)
-{
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void f2unpack(f2 r, float& a, float& b)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
-}
-__device__ __forceinline__ f2 f2sub(f2 a, f2 b)
-{
-    f2 d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 f2mul(f2 a, f2 b)
-{
-    f2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 f2fma(f2 a, f2 b, f2 c)
-{
-    f2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ float f2sum(f2 a)
-{
-    float x, y;
-    f2unpack(a, x, y);
-    return x + y;
-}
+// A list tile is stored pair-interleaved -- {x_j, x_j+1}, {y_j, y_j+1},
+// {z_j, z_j+1}, {m_j, m_j+1} per pair of entries -- so one pair of 16-byte
+// shared loads yields two sources packed for the paired FP32 instructions
+// (tc_f32x2.cuh), and every FP32 operation of the force loop serves two
+// sources.
 
 // entry k of a pair-interleaved tile
 __device__ __forceinline__ void put_entry(float* tile, int k, float4 q)
@@ -174,15 +138,6 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& c, float x)
     float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z));
     s = t;
     c = __fadd_rn(c, e);
-}
-
-// 1/sqrt(x) on the SFU, flushing subnormals (x >= eps^2 > 0 is normal here),
-// so no range fix-up surrounds the approximation
-__device__ __forceinline__ float rsqrt_sfu(float x)
-{
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
 }
 
 // The force loop: npairs pairs of sources against the lane's B bodies.
