@@ -53,7 +53,8 @@ typedef struct tc_ctx tc_ctx;
  *             coordinates and plain accumulation
  *   want_pot  1: also compute the potential (tc_get_acc's pot, tc_diag's PE)
  *   verify    1: record per-group list lengths and hashes (tc_get_lists)
- *   stack     walk stack entries per warp (shared memory), 64..8192
+ *   stack     walk stack entries per walking warp (shared memory), 64..8192;
+ *             an entry is a node, in the split walk an opened cell
  *   blocks_per_sm  0 = as many as fit, else a cap
  *   quad      1: also reduce the cells' second moments about the centre of
  *             mass (FP32, within (leaf_max + 128) 2^-25 M s^2; the learned
@@ -72,24 +73,25 @@ typedef struct tc_ctx tc_ctx;
  *   quadrupole 1: every accepted cell adds its quadrupole term to its
  *             monopole (second-order expansion of the softened potential
  *             about the centre of mass; needs precise = 1, quad = 1)
- *   classes   1: with gmax 64 or 128 the walk runs one launch per group
- *             size class (the largest on the calling stream, the others
- *             beside it on a stream of the context's, joined back before the
- *             call returns its work to the stream): a group of at most 32 bodies is
- *             summed one body per lane, one of at most 64 two per lane, a
- *             larger one four (the default); 0: one launch, gmax / 32
- *             bodies per lane for every group.  Lists and forces are the
- *             same in both.
+ *   classes   1: with gmax 64 or 128 the walks on one warp per group run one
+ *             launch per group size class (the largest on the calling
+ *             stream, the others beside it on a stream of the context's,
+ *             joined back before the call returns its work to the stream): a
+ *             group of at most 32 bodies is summed one body per lane, one of
+ *             at most 64 two per lane, a larger one four (the default); 0:
+ *             one launch, gmax / 32 bodies per lane for every group.  Lists
+ *             and forces are the same in both.  The split walk lays every
+ *             group out over its lanes by its own size in one launch.
  *   split     1: the monopole walks (learned = 0, quadrupole = 0) run with
  *             the tree walk and the force loop on different warps: a
  *             producer warp walks and fills a ring of list tiles in shared
- *             memory, a consumer warp sums them (the default); the learned
- *             walk stays on one warp per group with the network evaluated
- *             inside the walk.  2: the learned walk also splits, its band
- *             cells recorded by the producers and the network run on all of
- *             them after the walk.  0: every warp walks and sums its own
- *             groups.  Same lists; the sums take the tiles in another order
- *             (rounding-level differences). */
+ *             memory, a consumer warp (several in small systems) sums them
+ *             (the default); the learned walk stays on one warp per group
+ *             with the network evaluated inside the walk.  2: the learned
+ *             walk also splits, its band cells recorded by the producers and
+ *             the network run on all of them after the walk.  0: every warp
+ *             walks and sums its own groups.  Same lists; the sums take the
+ *             entries in another order (rounding-level differences). */
 typedef struct {
     int32_t gmax;
     int32_t warps;

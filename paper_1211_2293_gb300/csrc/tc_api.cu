@@ -82,10 +82,11 @@ struct tc_ctx {
     bool walk_ready = false;
     int walk_grid = 0;
     size_t walk_smem = 0;
-    // groups split by size (walks of up to 64 / 128 bodies): class k goes to
-    // the kernel with 2^k bodies per lane
-    int32_t* glists = nullptr;   // 3 x cap_n group indices
-    int32_t* glist_n = nullptr;  // 3 counts, then the split's scratch
+    // size classes (walks of one warp per group): class k, of up to 32 << k
+    // bodies, goes to the kernel with 2^k bodies per lane
+    int32_t* gorder = nullptr;  // the groups in the order they are walked
+    int32_t* gseg = nullptr;    // 4 range ends of its size classes, then the ordering's scratch
+    bool gorder_ready = false;  // the order is that of the current groups
     int walk_ncls = 0;
     int depth_hint = -1;  // tree depth of the last build the host saw (-1: none)
     int64_t depth_hint_n = -1;  // its body count
@@ -318,8 +319,8 @@ int ensure_bodies(tc_ctx* c, int64_t n)
     TC_GROW(c, c->nbody, cap);
     TC_GROW(c, c->hash, cap);
     TC_GROW(c, c->totals, 4);
-    TC_GROW(c, c->glists, 3 * cap);
-    TC_GROW(c, c->glist_n, 3 + (int64_t)group_split_scratch());
+    TC_GROW(c, c->gorder, cap);
+    TC_GROW(c, c->gseg, 4 + (int64_t)group_order_scratch());
     c->cap_n = cap;
     c->cap_m = 0;  // node tables are sized with the first build at this capacity
     return TC_OK;
@@ -538,12 +539,30 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
     launch_group_marks(c->cap_m, c->info, c->nt, c->cfg.gmax, n, c->gflag, c->gref_at, s);
     scan_u32(c->gflag, c->gscan, n, &c->totals[1], c->sb.blocksum, s);
     launch_group_table(c->gflag, c->gscan, c->gref_at, n, &c->totals[1], c->gfirst, c->gref, c->info, s);
-    if (c->cfg.gmax > 32) launch_group_split(c->gfirst, c->info, c->cap_n, c->glists, c->glist_n, c->glist_n + 3, s);
+    c->gorder_ready = false;
     TC_CUDA(c, cudaGetLastError());
     phase_end(c, 0, t0, s);
     c->built = true;
     c->have_forces = false;
     return TC_OK;
+}
+
+// Consumer warps per producer of the split walk.  With many groups one: a
+// list takes about as long to walk as to sum.  With few, the walk waits for
+// its longest list (packed siblings whose box spans a dense octant list most
+// of a small system), which then several consumers sum together: seven while
+// every group finds a team of eight warps at once (two per SM), three up to a
+// few rounds of the half-size teams (Plummer spheres, theta 0.6, walk in us
+// with 1 / 3 / 7 consumers: 2000 bodies 58 / 39 / 38, 16000 347 / 205 / 224,
+// 50000 130 / 124 / 177, 70000 132 / 156 / 238).  A rule on n and gmax only
+// (a group holds about 0.7 gmax bodies), so a captured step and a direct
+// call sum alike.
+int walk_consumers(int64_t n, int gmax, int num_sms)
+{
+    const double groups = (double)n / (0.7 * gmax);
+    if (groups <= 2.0 * num_sms) return 7;
+    if (groups <= 8.0 * num_sms) return 3;
+    return 1;
 }
 
 int prepare_forces(tc_ctx* c)
@@ -558,11 +577,14 @@ int prepare_forces(tc_ctx* c)
     wc.tile = c->cfg.tile;
     wc.learned = c->cfg.learned && c->have_mlp;
     wc.quadw = c->cfg.quadrupole;
-    wc.classes = c->cfg.gmax > 32 ? c->cfg.classes : 0;
     // split 1: producer/consumer walks for the monopole walks, the learned
     // walk keeps the network inside the one-warp walk; 2: the learned walk
     // too, the network then evaluated after the walk
     wc.split = (!wc.quadw && (c->cfg.split == 2 || (c->cfg.split == 1 && !wc.learned))) ? 1 : 0;
+    // one launch per size class: one warp per group only (the split walk
+    // lays each group out over its lanes by its own size)
+    wc.classes = (c->cfg.gmax > 32 && !wc.split) ? c->cfg.classes : 0;
+    wc.consumers = wc.split ? walk_consumers(c->n, c->cfg.gmax, c->num_sms) : 0;
     int64_t st = c->cfg.stack;
     if (c->cap_m < st) st = c->cap_m < 32 ? 32 : c->cap_m;  // a stack of M entries cannot overflow
     st = (st + 3) & ~(int64_t)3;                            // keeps every warp's tiles 16-byte aligned
@@ -650,6 +672,14 @@ int run_forces(tc_ctx* c, float theta, float eps, float G, cudaStream_t s)
         cudaMemsetAsync(c->band_n, 0, sizeof(unsigned long long), s);
         cudaMemsetAsync(c->gcorr, 0, 3 * c->band_gcap * sizeof(float), s);
     }
+    // groups ordered by layout where a size-class launch walks a range of
+    // them, or where the split walk has many of them
+    const bool ordered = c->walk_ncls > 0 || (c->walk_cfg.split && c->walk_cfg.consumers == 1);
+    if (ordered) {
+        if (!c->gorder_ready) launch_group_order(c->gfirst, c->info, c->gorder, c->gseg, c->gseg + 4, s);
+        c->gorder_ready = true;
+        a.glist = c->gorder;
+    }
     if (c->walk_ncls == 0) {
         e = launch_walk(a, c->walk_cfg, c->walk_grid, c->walk_smem, s);
     } else {
@@ -664,8 +694,7 @@ int run_forces(tc_ctx* c, float theta, float eps, float G, cudaStream_t s)
         TC_CUDA(c, cudaEventRecord(c->ev_fork, s));
         TC_CUDA(c, cudaStreamWaitEvent(c->side_stream, c->ev_fork, 0));
         for (int k = c->walk_ncls - 1; k >= 0 && e == cudaSuccess; k--) {
-            a.glist = c->glists + (int64_t)k * c->cap_n;
-            a.glist_n = c->glist_n + k;
+            a.gseg = c->gseg + (2 - k);
             a.work_slot = k;
             e = launch_walk(a, c->walk_cls[k], c->walk_cls_grid[k], c->walk_cls_smem[k],
                             k == c->walk_ncls - 1 ? s : c->side_stream, false);
@@ -712,11 +741,11 @@ int step_eager(tc_ctx* c, float dt)
 std::string graph_key(tc_ctx* c, float dt)
 {
     char b[512];
-    snprintf(b, sizeof(b), "%lld/%lld/%d/%d/%a/%a/%a/%a/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%a/%d/%d", (long long)c->n,
+    snprintf(b, sizeof(b), "%lld/%lld/%d/%d/%a/%a/%a/%a/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%a/%d/%d/%d", (long long)c->n,
              (long long)c->cap_m, c->nsys, c->leaf_max, (double)dt, (double)c->theta, (double)c->eps, (double)c->Gc,
              c->cfg.gmax, c->cfg.warps, c->cfg.precise, c->cfg.want_pot, c->cfg.verify, c->cfg.stack,
              c->cfg.blocks_per_sm, c->cfg.quad, c->cfg.tile, c->cfg.learned && c->have_mlp, (double)c->mlp_band,
-             c->cfg.quadrupole, c->cfg.classes);
+             c->cfg.quadrupole, c->cfg.classes, c->cfg.split);
     return b;
 }
 
@@ -764,6 +793,7 @@ int step_graph(tc_ctx* c, float dt)
         c->gkey = key;
     }
     cudaEvent_t t0 = phase_begin(c, c->stream, 0);
+    c->gorder_ready = false;  // the graph rebuilds the groups
     TC_CUDA(c, cudaGraphLaunch(c->gexec, c->stream));
     count_launches((int)c->graph_kernels);
     phase_end(c, 0, t0, c->stream);  // (timing mode: kick + drift + rebuild)

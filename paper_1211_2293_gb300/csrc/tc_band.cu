@@ -30,6 +30,7 @@
 // CTA frees its tensor memory when both have stopped.  k_band_apply adds each
 // group's sum to the accelerations of its bodies.
 #include "tc_walk.cuh"
+#include "tc_walk_ws.cuh"
 
 namespace tc {
 

@@ -760,20 +760,25 @@ __global__ void k_group_table(const uint32_t* __restrict__ gflag, const uint32_t
     gref[g] = gref_at[s];
 }
 
-// Groups split by size for the walk, so that a group of at most 32 bodies is
-// summed one body per lane and one of at most 64 two per lane: class 0
-// holds at most 32 bodies, class 1 at most 64, class 2 more.  Block b of
-// kSplitBlocks takes the b-th contiguous range of the group table; a first
-// pass counts each range's groups per class, a second gives every group its
-// place (the counts of the ranges before it, then warp ballots within the
-// range), keeping the group order within each class.
+// The groups ordered by the layout the walk gives them (group_class), the
+// largest first and in tree order within a class: the warps of an SM then
+// sum with the same loop at the same time (the loops of all layouts together
+// do not fit its instruction cache: the 2^20 cube's walk waited 2.6 cycles
+// per issued instruction for fetches with the groups in tree order), and a
+// walk that launches one kernel per class finds its groups in one range.
+// Block b of kSplitBlocks takes the b-th contiguous range of the group
+// table; a first pass counts each range's groups per class, a second gives
+// every group its place (the classes before its own, the ranges before its
+// own, then warp ballots within the range).
 constexpr int kSplitBlocks = 256;
 constexpr int kSplitThreads = 256;
 
-__device__ __forceinline__ int size_class(const int32_t* __restrict__ gfirst, int64_t g)
+__device__ __forceinline__ int group_class(const int32_t* __restrict__ gfirst, int64_t g)
 {
-    const int cnt = gfirst[g + 1] - gfirst[g];
-    return cnt <= 32 ? 0 : (cnt <= 64 ? 1 : 2);
+    const int n = gfirst[g + 1] - gfirst[g];
+    if (n > 64) return n > 96 ? 0 : 1;
+    if (n > 32) return n > 48 ? 2 : (n > 40 ? 3 : 4);
+    return n > 16 ? 5 : 6;
 }
 
 __device__ __forceinline__ void split_range(const Info* info, int64_t& lo, int64_t& hi)
@@ -791,85 +796,99 @@ __device__ __forceinline__ int warp_sum_i(int v)
     return v;
 }
 
-__global__ void __launch_bounds__(kSplitThreads) k_split_count(const int32_t* __restrict__ gfirst, const Info* info,
+__global__ void __launch_bounds__(kSplitThreads) k_order_count(const int32_t* __restrict__ gfirst, const Info* info,
                                                                int32_t* __restrict__ bcount)
 {
-    __shared__ int red[kSplitThreads / 32][3];
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    __shared__ int cnt[kGroupClasses];
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid < kGroupClasses) cnt[tid] = 0;
+    __syncthreads();
     int64_t lo, hi;
     split_range(info, lo, hi);
-    int c[3] = {0, 0, 0};
-    for (int64_t g = lo + tid; g < hi; g += blockDim.x) {
-        const int k = size_class(gfirst, g);
-        c[0] += k == 0;
-        c[1] += k == 1;
-        c[2] += k == 2;
-    }
+    for (int64_t c0 = lo; c0 < hi; c0 += kSplitThreads) {
+        const int cls = c0 + tid < hi ? group_class(gfirst, c0 + tid) : -1;
 #pragma unroll
-    for (int k = 0; k < 3; k++) {
-        const int v = warp_sum_i(c[k]);
-        if (lane == 0) red[w][k] = v;
+        for (int k = 0; k < kGroupClasses; k++) {
+            const unsigned m = __ballot_sync(0xffffffffu, cls == k);
+            if (lane == 0 && m) atomicAdd(&cnt[k], __popc(m));
+        }
     }
     __syncthreads();
-    if (tid < 3) {
-        int t = 0;
-        for (int ww = 0; ww < kSplitThreads / 32; ww++) t += red[ww][tid];
-        bcount[3 * blockIdx.x + tid] = t;
-    }
+    if (tid < kGroupClasses) bcount[kGroupClasses * blockIdx.x + tid] = cnt[tid];
 }
 
-__global__ void __launch_bounds__(kSplitThreads) k_split_scatter(const int32_t* __restrict__ gfirst, const Info* info,
-                                                                 const int32_t* __restrict__ bcount, int64_t cap_g,
-                                                                 int32_t* __restrict__ lists,
-                                                                 int32_t* __restrict__ counts)
+__global__ void __launch_bounds__(kSplitThreads) k_order_scatter(const int32_t* __restrict__ gfirst, const Info* info,
+                                                                 const int32_t* __restrict__ bcount,
+                                                                 int32_t* __restrict__ order, int32_t* __restrict__ seg)
 {
-    constexpr int W = kSplitThreads / 32;
-    __shared__ int red[W][6];
-    __shared__ int wcnt[W][3];
-    __shared__ int base[3];
+    constexpr int W = kSplitThreads / 32, NC = kGroupClasses;
+    __shared__ int red[W][2 * NC];
+    __shared__ int wcnt[W][NC];
+    __shared__ int base[NC];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    // this range's offsets (the ranges before it) and the class totals
-    int v[6] = {0, 0, 0, 0, 0, 0};
+    // groups of each class in the ranges before this one, and in all
+    int v[2 * NC];
+#pragma unroll
+    for (int k = 0; k < 2 * NC; k++) v[k] = 0;
     for (int j = tid; j < (int)gridDim.x; j += blockDim.x) {
 #pragma unroll
-        for (int k = 0; k < 3; k++) {
-            const int x = bcount[3 * j + k];
+        for (int k = 0; k < NC; k++) {
+            const int x = bcount[NC * j + k];
             if (j < (int)blockIdx.x) v[k] += x;
-            v[3 + k] += x;
+            v[NC + k] += x;
         }
     }
 #pragma unroll
-    for (int k = 0; k < 6; k++) {
+    for (int k = 0; k < 2 * NC; k++) {
         const int s = warp_sum_i(v[k]);
         if (lane == 0) red[w][k] = s;
     }
     __syncthreads();
-    if (tid < 6) {
-        int t = 0;
-        for (int ww = 0; ww < W; ww++) t += red[ww][tid];
-        if (tid < 3) base[tid] = t;
-        else if (blockIdx.x == 0) counts[tid - 3] = t;
+    if (tid < NC) {
+        int mine = 0;
+        for (int ww = 0; ww < W; ww++) mine += red[ww][tid];
+        int start = 0;
+        for (int k = 0; k < tid; k++)
+            for (int ww = 0; ww < W; ww++) start += red[ww][NC + k];
+        base[tid] = start + mine;
+        if (blockIdx.x == 0) {
+            // the ranges of groups of more than 64 (classes 0, 1), 33 to 64
+            // (2 to 4) and up to 32 bodies
+            if (tid == 0) seg[0] = 0;
+            if (tid == 2) seg[1] = start;
+            if (tid == 5) seg[2] = start;
+            if (tid == NC - 1) {
+                int all = start;
+                for (int ww = 0; ww < W; ww++) all += red[ww][NC + tid];
+                seg[3] = all;
+            }
+        }
     }
     int64_t lo, hi;
     split_range(info, lo, hi);
     const unsigned lt = (1u << lane) - 1u;
     for (int64_t c0 = lo; c0 < hi; c0 += kSplitThreads) {
         const int64_t g = c0 + tid;
-        const int cls = g < hi ? size_class(gfirst, g) : -1;
-        unsigned m[3];
+        const int cls = g < hi ? group_class(gfirst, g) : -1;
+        int rank = 0;
+        unsigned m[NC];
 #pragma unroll
-        for (int k = 0; k < 3; k++) m[k] = __ballot_sync(0xffffffffu, cls == k);
+        for (int k = 0; k < NC; k++) {
+            m[k] = __ballot_sync(0xffffffffu, cls == k);
+            if (cls == k) rank = __popc(m[k] & lt);
+        }
         __syncthreads();  // base is set; the previous chunk's readers of wcnt and base are done
         if (lane == 0)
-            for (int k = 0; k < 3; k++) wcnt[w][k] = __popc(m[k]);
+#pragma unroll
+            for (int k = 0; k < NC; k++) wcnt[w][k] = __popc(m[k]);
         __syncthreads();
         if (cls >= 0) {
-            int off = base[cls] + __popc(m[cls] & lt);
+            int off = base[cls] + rank;
             for (int ww = 0; ww < w; ww++) off += wcnt[ww][cls];
-            lists[cls * cap_g + off] = (int32_t)g;
+            order[off] = (int32_t)g;
         }
         __syncthreads();
-        if (tid < 3) {
+        if (tid < NC) {
             int t = 0;
             for (int ww = 0; ww < W; ww++) t += wcnt[ww][tid];
             base[tid] += t;
@@ -992,13 +1011,13 @@ void launch_moments(const float4* body, int64_t cap_m, int depth, int depth_hint
     }
 }
 
-size_t group_split_scratch() { return (size_t)3 * kSplitBlocks; }
+size_t group_order_scratch() { return (size_t)kGroupClasses * kSplitBlocks; }
 
-void launch_group_split(const int32_t* gfirst, const Info* info, int64_t cap_g, int32_t* lists, int32_t* counts,
-                        int32_t* scratch, cudaStream_t s)
+void launch_group_order(const int32_t* gfirst, const Info* info, int32_t* order, int32_t* seg, int32_t* scratch,
+                        cudaStream_t s)
 {
-    k_split_count<<<kSplitBlocks, kSplitThreads, 0, s>>>(gfirst, info, scratch);
-    k_split_scatter<<<kSplitBlocks, kSplitThreads, 0, s>>>(gfirst, info, scratch, cap_g, lists, counts);
+    k_order_count<<<kSplitBlocks, kSplitThreads, 0, s>>>(gfirst, info, scratch);
+    k_order_scatter<<<kSplitBlocks, kSplitThreads, 0, s>>>(gfirst, info, scratch, order, seg);
     count_launches(2);
 }
 

@@ -171,12 +171,14 @@ void launch_moments(const float4* body, int64_t cap_m, int depth, int depth_hint
                     cudaStream_t s);
 void launch_group_marks(int64_t cap_m, const Info* info, const NodeTables nt, int gmax, int64_t n,
                         uint32_t* gflag, int32_t* gref_at, cudaStream_t s);
-// groups by size class, stable: lists[k * cap_g + i], counts[k], class 0
-// holding at most 32 bodies, class 1 at most 64, class 2 more; scratch holds
-// group_split_scratch() ints
-size_t group_split_scratch();
-void launch_group_split(const int32_t* gfirst, const Info* info, int64_t cap_g, int32_t* lists, int32_t* counts,
-                        int32_t* scratch, cudaStream_t s);
+// the groups by the walk's layout of their bodies (kGroupClasses of them),
+// the largest first, stable: order[0, G); seg[0..3] = the ranges of groups of
+// more than 64, 33 to 64 and up to 32 bodies in it; scratch holds
+// group_order_scratch() ints
+constexpr int kGroupClasses = 7;
+size_t group_order_scratch();
+void launch_group_order(const int32_t* gfirst, const Info* info, int32_t* order, int32_t* seg, int32_t* scratch,
+                        cudaStream_t s);
 void launch_group_table(const uint32_t* gflag, const uint32_t* gscan, const int32_t* gref_at,
                         int64_t n, const uint32_t* total, int32_t* gfirst, int32_t* gref, Info* info,
                         cudaStream_t s);
@@ -219,9 +221,10 @@ struct WalkArgs {
     int64_t list_cap;
     int64_t* list_n;
     int32_t list_group;
-    // group list (null: every group 0..G-1): walk glist[0, *glist_n) only
+    // the order in which groups are walked (null: 0..G-1); gseg (null: all of
+    // it): walk glist[gseg[0], gseg[1]) only
     const int32_t* glist;
-    const int32_t* glist_n;
+    const int32_t* gseg;
     int work_slot;  // this launch's work-queue counter, info->work[work_slot]
     // learned correction evaluated after the walk (split walk): the band
     // cells of every group recorded as (node, group) pairs in chunks of
@@ -247,7 +250,8 @@ struct WalkConfig {
     int learned;      // 1: learned far-field correction (precise mode, no potential)
     int quadw;        // 1: accepted cells add their quadrupole term (precise mode)
     int classes;      // 1: one launch per group size class (the smaller beside the largest); 0: one launch
-    int split;        // 1: monopole walks on producer/consumer warp pairs (k_walk_ws)
+    int split;        // 1: monopole walks on producer/consumer warps (k_walk_ws)
+    int consumers;    // split: consumer warps per producer (1, 3 or 7; as many as `warps` has room for)
 };
 // host-side preparation of the walk kernel's launch (attributes, occupancy);
 // call before a stream capture

@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(128, LEARNED ? kLearnedMinBlocks : (B >= 4 ? 3
     if (info->err & kErrCapacity) return;  // the build stopped: no tree to walk
     const bool list_mode = a.list_cells != nullptr;
     // list export walks one group: queue position 0 maps to list_group
-    const int64_t G = list_mode ? (int64_t)a.list_group + 1 : (a.glist ? (int64_t)*a.glist_n : info->G);
+    const int64_t G = list_mode ? (int64_t)a.list_group + 1 : (a.gseg ? (int64_t)(a.gseg[1] - a.gseg[0]) : info->G);
     const int g_shift = list_mode ? a.list_group : 0;
     const NodeTables nt = a.nt;
     MlpFrag* mlp = reinterpret_cast<MlpFrag*>(smem);
@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(128, LEARNED ? kLearnedMinBlocks : (B >= 4 ? 3
         if (lane == 0) g = (int)atomicAdd(&a.info->work[a.work_slot], 1u) + g_shift;
         g = __shfl_sync(0xffffffffu, g, 0);
         if (g >= G) break;
-        if (a.glist) g = __ldg(a.glist + g);  // this launch's size class
+        if (a.glist) g = __ldg(a.glist + (a.gseg ? __ldg(a.gseg) : 0) + g);  // this launch's size class
         const int gfirst = a.gfirst[g];
         const int gend = a.gfirst[g + 1];
         // the group's system: its root cube and its root node (roots are
@@ -811,14 +811,6 @@ __global__ void __launch_bounds__(128, LEARNED ? kLearnedMinBlocks : (B >= 4 ? 3
     }
 }
 
-}  // namespace
-}  // namespace tc
-
-#include "tc_walk_ws.cuh"
-
-namespace tc {
-namespace {
-
 template <int B, int TILE, bool PRECISE, bool POT, bool LEARNED, bool QUADW>
 cudaError_t prepare_t(const WalkConfig& c, int num_sms, int* grid, size_t* smem_out)
 {
@@ -864,17 +856,10 @@ cudaError_t dispatch_modes(const WalkConfig& c, Args... args)
     return F<B, TT, false, false, false, false>::run(args...);
 }
 
-// split = 1 runs the monopole walks (precise or plain, with or without the
-// potential) on k_walk_ws, producer and consumer warps apart; the learned
-// walk there records its band cells for k_band_eval instead of evaluating
-// the network inside the walk
 template <int B, int TILE, bool PRECISE, bool POT, bool LEARNED, bool QUADW>
 struct PrepareF {
     static cudaError_t run(const WalkConfig* c, int num_sms, int* grid, size_t* smem)
     {
-        if constexpr (!QUADW) {
-            if (c->split) return prepare_ws_t<B, TILE, PRECISE, POT, LEARNED>(*c, num_sms, grid, smem);
-        }
         return prepare_t<B, TILE, PRECISE, POT, LEARNED, QUADW>(*c, num_sms, grid, smem);
     }
 };
@@ -882,9 +867,6 @@ template <int B, int TILE, bool PRECISE, bool POT, bool LEARNED, bool QUADW>
 struct LaunchF {
     static cudaError_t run(const WalkArgs* a, const WalkConfig* c, int grid, size_t smem, cudaStream_t s)
     {
-        if constexpr (!QUADW) {
-            if (c->split) return launch_ws_t<B, TILE, PRECISE, POT, LEARNED>(*a, *c, grid, smem, s);
-        }
         return launch_t<B, TILE, PRECISE, POT, LEARNED, QUADW>(*a, *c, grid, smem, s);
     }
 };

@@ -1,23 +1,63 @@
 // tc_walk_ws.cuh -- the force phase with the tree walk and the force loop on
-// different warps (included by tc_walk.cuh after k_walk).
+// different warps (included by tc_walk_ws_unit.cu).
 //
 // k_walk gives each warp a whole group: it walks a step, sums a full list
-// tile, walks on.  Measured on a uniform cube of 2^20 bodies, its warps spend
-// 44 % of their time walking and the walk and the sums of the other warps of
-// an SM hardly overlap: the walk alone takes 0.45 ms, the whole kernel
-// 1.52 ms, while the force loop alone would need about 1.1 ms.
+// tile, walks on, and the walk of one warp hardly overlaps the sums of the
+// others.  Here a block holds teams of one producer warp and C consumer
+// warps.  The producer walks a group as k_walk does (opening test, ballots,
+// list compaction) but never sums: it fills list tiles in a ring of slots in
+// shared memory -- at any time one open tile of cells and one of bodies --
+// and hands a tile over when it is full or the group ends.  The consumers
+// hold the group's bodies and sum every tile they are handed (the
+// compensated paired-FP32 loop), then write the group's accelerations.
 //
-// Here a block holds P producer/consumer pairs.  The producer warp walks a
-// group exactly as k_walk does (opening test, ballots, list compaction into
-// pair-interleaved tiles) but never sums: it fills the slots of a ring in
-// shared memory, each slot carrying a cell part and a body part of up to
-// one tile each, and hands a slot over when either part is full or the group
-// ends.  The consumer warp holds the group's bodies in registers and sums
-// every slot it is handed (the same compensated paired-FP32 loop), then
-// writes the group's accelerations.  The ring has kWsSlots slots; one
-// mbarrier per slot tells the consumer a slot is full, one tells the
-// producer it is empty again.  Slots are filled and emptied in one order,
-// one slot open at a time, so the two never wait on each other in a cycle.
+// Bound.  Both kinds of warp share an SM partition's issue slots and
+// register-file ports; with two of each per partition the measured time is
+// the sum of the loop's cycles (29 per pair of sources and body, its rate
+// alone) and about 1.3 per producer instruction -- hiding latency (the next
+// step's nodes loaded ahead, three consumers for two producers, 24 warps of
+// 80 registers) changed nothing, fewer instructions and fewer empty lanes
+// did.  Walk of a 2^20 cube at theta 0.5 1.38 -> 1.22 ms, of a 2^22 Plummer
+// sphere at theta 0.62 5.64 -> 5.21 ms with the layouts, the ordering of the
+// groups by layout (launch_group_order) and the step below.
+//
+// The walk's step.  The stack holds opened cells.  A step tests the children
+// of eight of them, eight lanes to a cell, two cells to a lane; opened leaves
+// wait until 32 of them list their bodies together.  With single nodes on the
+// stack, scans that packed children and bodies were most of a step: 14.3
+// thousand instructions per group of the cube, now 10.2.
+//
+// Bodies over lanes.  A group holds 1 to gmax bodies, 45 of 64 on average.
+// With one or two bodies per lane a quarter of the loop's work went to lanes
+// without a body.  Instead a warp's lanes are cut into S slices of 32 / S
+// lanes; every slice holds all of the group's bodies, K per lane, and sums
+// every S-th quad of the list, so the work grows in steps of 32 K / S body
+// slots: (K, S) = (1, 2), (1, 1), (5, 4), (3, 2), (2, 1) take groups of up
+// to 16, 32, 40, 48, 64 bodies (three and four per lane up to 128).  Lanes
+// holding a body, over the groups of a 2^20 cube / Plummer sphere: 0.76 /
+// 0.78 -> 0.86 / 0.89.  The slices' compensated sums are added at the end of
+// the group by TwoSum.
+//
+// Consumers per team.  C = 1 fills the machine when there are many groups:
+// walking a list costs about as long as summing it.  With few groups the
+// longest list is what a walk waits for (a group of packed siblings whose
+// box spans a dense octant lists most of a small system), so the consumers
+// of a team share it: warp c takes every C-th round of each tile and the
+// C sums are added in order at the end.  walk_consumers (tc_api.cu) states
+// the rule.
+//
+// Tiles.  The four planes x, y, z, m of a tile are contiguous: 32 lanes
+// store 32 entries without bank conflicts (pair-interleaved entries of four
+// words met four-way conflicts) and a 16-byte load yields four sources as
+// two packed pairs.
+//
+// Order.  Tiles are handed over at positions 0, 1, 2, ...; position k uses
+// mbarriers full[k % kWsSlots] and empty[k % kWsSlots] and names its slot in
+// seq[k % kWsSlots].  The producer holds two slots, so at most kWsSlots - 2
+// positions are in flight; it takes slots in the order in which they were
+// handed over, after waiting for that position's empty barrier, so a
+// position's words are never rewritten before its consumers left it, and the
+// two sides never wait on each other in a cycle.
 //
 // Every wait is bounded (about a second of SM clock): a wait that runs out
 // raises kErrWorkLoop in the error word and its warp returns, so a fault in
@@ -28,31 +68,44 @@ namespace tc {
 
 namespace {
 
-constexpr int kWsSlots = 3;                      // ring depth per pair
+// tiles per team: two open, the others in flight
+__host__ __device__ constexpr int ws_slots(int tile) { return tile > 128 ? 5 : 6; }
 constexpr int kWsMaxPairs = 4;                   // pairs per block (block = 2 x pairs warps)
 constexpr long long kWsWaitCycles = 1ll << 31;   // about 1 s of SM clock
 
+// entries of a plane: a step adds at most 64 to a tile that was not full,
+// and the count is padded to a multiple of 16 (four slices of quads)
+__host__ __device__ constexpr int ws_cap(int tile) { return tile + 64; }
+
 // slot header (64 bytes at the front of a slot)
 struct WsHdr {
-    int32_t flags;  // kWsFirst | kWsLast | kWsDone | kWsAbort
-    int32_t cn;     // entries in the cell part
-    int32_t bn;     // entries in the body part
-    int32_t g;      // group
+    int32_t flags;  // kWs*
+    int32_t n;      // entries, padded to a multiple of 16 with massless ones
     int32_t gfirst, gend;
-    int32_t pad[2];
+    int32_t pad[4];
     double ref[3];  // centre of the group's reference cube (absolute, FP64)
     double pad2;
 };
 static_assert(sizeof(WsHdr) == 64, "slot header");
-enum : int32_t { kWsFirst = 1, kWsLast = 2, kWsDone = 4, kWsAbort = 8 };
+enum : int32_t { kWsFirst = 1, kWsLast = 2, kWsDone = 4, kWsAbort = 8, kWsBodies = 16 };
 
-__host__ __device__ constexpr size_t ws_slot_bytes(int tile) { return sizeof(WsHdr) + (size_t)2 * tile_cap(tile) * 16; }
-// one pair: 2 x kWsSlots mbarriers (padded to 64 bytes), the slots, the
-// producer's stack
-__host__ __device__ constexpr size_t ws_pair_bytes(int tile, int stack)
+// One team's shared memory: barriers and slot numbers (128 bytes), the ring,
+// the walk stack (first child and number of children of each opened cell),
+// the opened leaves, each consumer's body positions (absolute and
+// reference-relative) and, with C > 1, the consumers' sums (two groups in
+// turn).  nb: body slots of a group (64, or 128 for gmax 128).
+__host__ __device__ constexpr size_t ws_slot_bytes(int tile) { return sizeof(WsHdr) + (size_t)4 * ws_cap(tile) * 4; }
+__host__ __device__ constexpr size_t ws_pos_bytes(int nb) { return (size_t)6 * nb * 4; }
+__host__ __device__ constexpr size_t ws_comb_bytes(int C, int nb) { return C > 1 ? (size_t)2 * C * 8 * nb * 4 : 0; }
+constexpr int kWsLeaves = 96;  // opened leaves: up to 31 left over + 64 of a step
+__host__ __device__ constexpr size_t ws_team_bytes(int tile, int stack, int C, int nb)
 {
-    return 64 + kWsSlots * ws_slot_bytes(tile) + (size_t)stack * 4;
+    return 128 + ws_slots(tile) * ws_slot_bytes(tile) + (size_t)stack * 4 + ((stack + 15) & ~15) + kWsLeaves * 8 +
+           32 * 4 + C * ws_pos_bytes(nb) + ws_comb_bytes(C, nb);
 }
+static_assert(2 * 8 * ws_slots(64) + 8 + 4 * ws_slots(64) <= 128 && 2 * 8 * ws_slots(256) + 8 + 4 * ws_slots(256) <= 128,
+              "a team's barriers and slot numbers");
+__host__ __device__ constexpr int ws_body_slots(int gmax) { return gmax > 64 ? 128 : 64; }
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -61,18 +114,18 @@ __device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count)
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(b)), "r"(count) : "memory");
 }
 
-// every lane of the warp arrives (the barriers count 32 arrivals), each
-// releasing its own writes to the slot
+// one lane of a warp arrives, after a __syncwarp that orders the other
+// lanes' accesses before it
 __device__ __forceinline__ void mbar_arrive(uint64_t* b)
 {
     asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}" ::"r"(smem_addr(b)) : "memory");
 }
 
-// the opened leaves' bodies reach a slot by cp.async (put_entry_async);
-// before its arrival on the slot's full barrier every producer lane makes the
-// barrier track its copies (cp.async.mbarrier.arrive without .noinc: the
-// pending count rises now and falls when the lane's copies have landed), so
-// the phase completes only once the bodies are in the tile
+// the opened leaves' bodies reach a slot by cp.async; before the producer's
+// arrival on the full barrier every lane makes the barrier track its copies
+// (cp.async.mbarrier.arrive without .noinc: the pending count rises now and
+// falls when the lane's copies have landed), so the phase completes only
+// once the bodies are in the tile
 __device__ __forceinline__ void mbar_track_copies(uint64_t* b)
 {
     asm volatile("cp.async.mbarrier.arrive.shared::cta.b64 [%0];" ::"r"(smem_addr(b)) : "memory");
@@ -102,71 +155,304 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity)
     return __all_sync(0xffffffffu, ok);
 }
 
+// what the warps of a team share
+struct WsTeam {
+    uint64_t *full, *empty, *comb_full;
+    int32_t* seq;
+    unsigned char* slots;
+    int slot_bytes;
+    __device__ __forceinline__ WsHdr* hdr(int slot) const { return reinterpret_cast<WsHdr*>(slots + slot * slot_bytes); }
+    __device__ __forceinline__ float* tile(int slot) const
+    {
+        return reinterpret_cast<float*>(slots + slot * slot_bytes + sizeof(WsHdr));
+    }
+};
+
+// One group on one consumer warp (number c of C): positions from the warp's
+// shared-memory copy, K bodies per lane, S slices.  Starts at position k
+// (whose full barrier has been waited for) and returns the position after
+// the group's last tile, or -1 when a wait ran out.
+template <int K, int S, int TILE, bool PRECISE, bool POT>
+__device__ __forceinline__ int consume_group(const WsTeam& t, int k, int c, int C, const float* __restrict__ pos, int nb,
+                                             float* comb, int comb_phase, int gfirst, int ng, const WalkArgs& a)
+{
+    constexpr int L = 32 / S;                      // lanes of a slice
+    constexpr int CAP = ws_cap(TILE);
+    constexpr int kWsSlots = ws_slots(TILE);
+    constexpr int kUnroll = K >= 3 ? 1 : (K == 2 ? 2 : 4);  // about eight pairs of sources and bodies in flight
+    constexpr int kFold = (TILE + 32) / 2;                // pairs summed between two compensations
+    const int lane = threadIdx.x & 31;
+    const int sl = lane / L, j = lane % L;
+    const f2 E2 = f2pack(a.eps2, a.eps2);
+    f2 ax[K], ay[K], az[K], ph[K];
+    float sx[K], sy[K], sz[K], sp[K], cx[K], cy[K], cz[K], cp[K];
+#pragma unroll
+    for (int b = 0; b < K; b++) {
+        ax[b] = ay[b] = az[b] = ph[b] = 0ull;
+        sx[b] = sy[b] = sz[b] = sp[b] = cx[b] = cy[b] = cz[b] = cp[b] = 0.f;
+    }
+    auto fold = [&]() {
+#pragma unroll
+        for (int b = 0; b < K; b++) {
+            two_sum_acc(sx[b], cx[b], f2sum(ax[b]));
+            two_sum_acc(sy[b], cy[b], f2sum(ay[b]));
+            two_sum_acc(sz[b], cz[b], f2sum(az[b]));
+            if (POT) two_sum_acc(sp[b], cp[b], f2sum(ph[b]));
+            ax[b] = ay[b] = az[b] = ph[b] = 0ull;
+        }
+    };
+    int pairs = 0;
+    int flags;
+    for (;;) {
+        const int slot = t.seq[k % kWsSlots];
+        const WsHdr* h = t.hdr(slot);
+        flags = h->flags;
+        const int rounds = (h->n >> 2) / S;        // n is a multiple of 4 S
+        const int mine = rounds > c ? (rounds - c + C - 1) / C : 0;
+        if (mine > 0) {
+            if (PRECISE) {
+                if (pairs + 2 * mine > kFold && pairs > 0) {
+                    fold();
+                    pairs = 0;
+                }
+                pairs += 2 * mine;
+            }
+            // cells are relative to the group's reference cube in the
+            // precise mode, bodies absolute
+            const float* q = pos + ((PRECISE && !(flags & kWsBodies)) ? 3 * nb : 0) + j;
+            f2 X[K], Y[K], Z[K];
+#pragma unroll
+            for (int b = 0; b < K; b++) {
+                const float x = q[b * L], y = q[nb + b * L], z = q[2 * nb + b * L];
+                X[b] = f2pack(x, x);
+                Y[b] = f2pack(y, y);
+                Z[b] = f2pack(z, z);
+            }
+            const float* p = t.tile(slot) + 4 * (sl + S * c);
+#pragma unroll(kUnroll)
+            for (int r = 0; r < mine; r++, p += 4 * S * C) {
+                const ulonglong2 xx = *reinterpret_cast<const ulonglong2*>(p);
+                const ulonglong2 yy = *reinterpret_cast<const ulonglong2*>(p + CAP);
+                const ulonglong2 zz = *reinterpret_cast<const ulonglong2*>(p + 2 * CAP);
+                const ulonglong2 mm = *reinterpret_cast<const ulonglong2*>(p + 3 * CAP);
+#pragma unroll
+                for (int hh = 0; hh < 2; hh++) {
+                    const f2 x2 = hh ? xx.y : xx.x, y2 = hh ? yy.y : yy.x, z2 = hh ? zz.y : zz.x, m2 = hh ? mm.y : mm.x;
+#pragma unroll
+                    for (int b = 0; b < K; b++) {
+                        const f2 dx = f2sub(x2, X[b]);
+                        const f2 dy = f2sub(y2, Y[b]);
+                        const f2 dz = f2sub(z2, Z[b]);
+                        const f2 r2 = f2fma(dz, dz, f2fma(dy, dy, f2fma(dx, dx, E2)));
+                        float r2a, r2b;
+                        f2unpack(r2, r2a, r2b);
+                        const f2 ri = f2pack(rsqrt_sfu(r2a), rsqrt_sfu(r2b));
+                        const f2 mri = f2mul(m2, ri);
+                        const f2 mri3 = f2mul(mri, f2mul(ri, ri));
+                        ax[b] = f2fma(dx, mri3, ax[b]);
+                        ay[b] = f2fma(dy, mri3, ay[b]);
+                        az[b] = f2fma(dz, mri3, az[b]);
+                        if (POT) ph[b] = f2sub(ph[b], mri);
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&t.empty[k % kWsSlots]);
+        k++;
+        if (flags & kWsLast) break;
+        if (!mbar_wait(&t.full[k % kWsSlots], (k / kWsSlots) & 1)) return -1;
+    }
+    fold();  // (plain mode: the plain sums, uncompensated so far)
+    // the slices' sums: both lanes of an exchange form the same sum
+#pragma unroll
+    for (int o = L; o < 32; o <<= 1) {
+#pragma unroll
+        for (int b = 0; b < K; b++) {
+            auto join = [&](float& s, float& comp) {
+                const float s2 = __shfl_xor_sync(0xffffffffu, s, o), c2 = __shfl_xor_sync(0xffffffffu, comp, o);
+                comp = __fadd_rn(comp, c2);
+                two_sum_acc(s, comp, s2);
+            };
+            join(sx[b], cx[b]);
+            join(sy[b], cy[b]);
+            join(sz[b], cz[b]);
+            if (POT) join(sp[b], cp[b]);
+        }
+    }
+    if (C > 1) {
+        // every consumer leaves its sums; once all have, they are added in
+        // the consumers' order
+        float* mineC = comb + (size_t)c * 8 * nb;
+#pragma unroll
+        for (int b = 0; b < K; b++) {
+            const int i = j + b * L;
+            if (b % S == sl) {
+                mineC[0 * nb + i] = sx[b];
+                mineC[1 * nb + i] = cx[b];
+                mineC[2 * nb + i] = sy[b];
+                mineC[3 * nb + i] = cy[b];
+                mineC[4 * nb + i] = sz[b];
+                mineC[5 * nb + i] = cz[b];
+                if (POT) {
+                    mineC[6 * nb + i] = sp[b];
+                    mineC[7 * nb + i] = cp[b];
+                }
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(t.comb_full);
+        if (!mbar_wait(t.comb_full, comb_phase)) return -1;
+        if (flags & kWsAbort) return k;
+        constexpr int NV = POT ? 4 : 3;
+        for (int e = c * 32 + lane; e < NV * ng; e += C * 32) {
+            const int v = e / ng, i = e - v * ng;
+            float s = 0.f, comp = 0.f;
+            for (int cc = 0; cc < C; cc++) {
+                const float* o = comb + (size_t)cc * 8 * nb + (2 * v) * nb + i;
+                comp = __fadd_rn(comp, o[nb]);
+                two_sum_acc(s, comp, o[0]);
+            }
+            const int64_t o = a.perm[gfirst + i];
+            if (v < 3) a.acc[3 * o + v] = a.G * (s + comp);
+            else a.pot[o] = a.G * ((s + comp) + a.body[gfirst + i].w * rsqrtf(a.eps2));
+        }
+        return k;
+    }
+    if (flags & kWsAbort) return k;
+#pragma unroll
+    for (int b = 0; b < K; b++) {
+        const int i = j + b * L;
+        if (b % S != sl || i >= ng) continue;
+        const int64_t o = a.perm[gfirst + i];
+        a.acc[3 * o + 0] = a.G * (sx[b] + cx[b]);
+        a.acc[3 * o + 1] = a.G * (sy[b] + cy[b]);
+        a.acc[3 * o + 2] = a.G * (sz[b] + cz[b]);
+        // (the potential drops the body's own term, -m_i / eps, summed with the list)
+        if (POT) a.pot[o] = a.G * ((sp[b] + cp[b]) + a.body[gfirst + i].w * rsqrtf(a.eps2));
+    }
+    return k;
+}
+
+// inclusive warp prefix sum, two instructions a step
+__device__ __forceinline__ unsigned ws_incl_scan(unsigned x)
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+        asm volatile(
+            "{\n .reg .pred p;\n .reg .b32 t;\n shfl.sync.up.b32 t|p, %0, %1, 0, -1;\n @p add.u32 %0, %0, t;\n}"
+            : "+r"(x)
+            : "r"(o));
+    return x;
+}
+
 // LEARNED: the producer also records the group's band cells (accepted, two
 // bodies or more, s >= band d) for the network, which runs after the walk
 // (k_band_eval) as (node, group) pairs, and each group's record (box centre
 // and frame)
-template <int B, int TILE, bool PRECISE, bool POT, bool LEARNED>
-__global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, B >= 4 ? 1 : 2) k_walk_ws(WalkArgs a, int stack_cap)
+template <int TILE, bool PRECISE, bool POT, bool LEARNED>
+__global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a, int stack_cap, int C, int nb)
 {
     constexpr int kTile = TILE;
+    constexpr int CAP = ws_cap(TILE);
+    constexpr int kWsSlots = ws_slots(TILE);
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    const int pairs = blockDim.x >> 6;
-    const bool producer = warp < pairs;
-    const int q = producer ? warp : warp - pairs;  // the pair
-    unsigned char* base = smem + (size_t)q * ws_pair_bytes(TILE, stack_cap);
-    uint64_t* full = reinterpret_cast<uint64_t*>(base);
-    uint64_t* empty = full + kWsSlots;
-    unsigned char* slots = base + 64;
-    uint32_t* stk = reinterpret_cast<uint32_t*>(slots + kWsSlots * ws_slot_bytes(TILE));
-    const uint32_t lt = (1u << lane) - 1u;
+    const int teams = (int)(blockDim.x >> 5) / (1 + C);
+    const bool producer = warp < teams;
+    const int team = producer ? warp : (warp - teams) / C;
+    const size_t team_bytes = ws_team_bytes(TILE, stack_cap, C, nb);
+    unsigned char* base = smem + (size_t)team * team_bytes;
+    WsTeam t;
+    t.full = reinterpret_cast<uint64_t*>(base);
+    t.empty = t.full + kWsSlots;
+    t.comb_full = t.empty + kWsSlots;
+    t.seq = reinterpret_cast<int32_t*>(t.comb_full + 1);
+    t.slots = base + 128;
+    t.slot_bytes = (int)ws_slot_bytes(TILE);
+    uint32_t* stk = reinterpret_cast<uint32_t*>(base + 128 + kWsSlots * ws_slot_bytes(TILE));
+    int2* leaves = reinterpret_cast<int2*>(stk + stack_cap);  // first body, bodies
+    int32_t* row = reinterpret_cast<int32_t*>(leaves + kWsLeaves);
+    uint8_t* stn = reinterpret_cast<uint8_t*>(row + 32);
+    unsigned char* after = stn + ((stack_cap + 15) & ~15);
 
     const Info* info = a.info;
     if (info->err & kErrCapacity) return;  // the build stopped: no tree to walk (uniform: no barrier used yet)
-    if (threadIdx.x < pairs) {
+    if (producer && lane == 0) {
         for (int s = 0; s < kWsSlots; s++) {
-            mbar_init(reinterpret_cast<uint64_t*>(smem + (size_t)threadIdx.x * ws_pair_bytes(TILE, stack_cap)) + s,
-                      32);
-            mbar_init(reinterpret_cast<uint64_t*>(smem + (size_t)threadIdx.x * ws_pair_bytes(TILE, stack_cap)) +
-                          kWsSlots + s,
-                      32);
+            mbar_init(&t.full[s], 1);
+            mbar_init(&t.empty[s], C);
         }
+        mbar_init(t.comb_full, C);
     }
     __syncthreads();
-    auto slot_hdr = [&](int k) { return reinterpret_cast<WsHdr*>(slots + (size_t)(k % kWsSlots) * ws_slot_bytes(TILE)); };
-    auto slot_cells = [&](int k) {
-        return reinterpret_cast<float*>(slots + (size_t)(k % kWsSlots) * ws_slot_bytes(TILE) + sizeof(WsHdr));
-    };
-    auto slot_bodies = [&](int k) { return slot_cells(k) + 4 * tile_cap(TILE); };
 
     if (producer) {
         // ------------------------------------------------------------ producer
+        const uint32_t lt = (1u << lane) - 1u, le = lt | (1u << lane);
         const bool list_stats = a.hash != nullptr;
-        const int64_t G = a.glist ? (int64_t)*a.glist_n : info->G;
+        const int64_t G = info->G;
         const NodeTables nt = a.nt;
-        int k = 0;  // slots taken so far
+        int k = 0;              // positions handed over so far
+        int taken = 2;          // slots taken so far: two open ones
+        uint32_t handed = 0;    // slots of the last kWsSlots positions, the latest in the low nibble
+        int cs = 0, bs = 1;     // the open cell tile's and body tile's slots
+        float *ctile = t.tile(0), *btile = t.tile(1);
+        int cn = 0, bn = 0;     // their entries
+        int first = kWsFirst;   // the group's next position is its first
+        int gfirst = 0, gend = 0;
+        double gx = 0, gy = 0, gz = 0;
         bool alive = true;
-        // take slot k (wait until the consumer has emptied it)
-        auto take = [&]() -> bool {
-            if (!mbar_wait(&empty[k % kWsSlots], ((k / kWsSlots) & 1) ^ 1)) {
-                if (lane == 0) atomicOr(&a.info->err, kErrWorkLoop);
-                return false;
+        // hands a slot's tile of n entries over (flags: kind, last, ...) and
+        // takes the next free slot in its place (-1: a wait ran out)
+        auto hand_over = [&](int slot, int n, int flags) -> int {
+            float* tile = t.tile(slot);
+            const int n16 = (n + 15) & ~15;
+            if (n + lane < n16) {  // massless padding
+                tile[n + lane] = 0.f;
+                tile[CAP + n + lane] = 0.f;
+                tile[2 * CAP + n + lane] = 0.f;
+                tile[3 * CAP + n + lane] = 0.f;
             }
-            return true;
-        };
-        auto hand_over = [&](int flags, int cn, int bn) {
-            WsHdr* h = slot_hdr(k);
             if (lane == 0) {
-                h->flags |= flags;
-                h->cn = cn;
-                h->bn = bn;
+                WsHdr* h = t.hdr(slot);
+                h->flags = flags | first;
+                h->n = n16;
+                if (first) {
+                    h->gfirst = gfirst;
+                    h->gend = gend;
+                    h->ref[0] = gx;
+                    h->ref[1] = gy;
+                    h->ref[2] = gz;
+                }
+                t.seq[k % kWsSlots] = slot;
             }
+            first = 0;
+            if (flags & kWsBodies) mbar_track_copies(&t.full[k % kWsSlots]);
             __syncwarp();
-            mbar_track_copies(&full[k % kWsSlots]);
-            mbar_arrive(&full[k % kWsSlots]);
+            if (lane == 0) mbar_arrive(&t.full[k % kWsSlots]);
+            handed = (handed << 4) | (uint32_t)slot;
             k++;
+            const int take = taken++;
+            if (take < kWsSlots) return take;  // never used yet
+            const int pos = take - kWsSlots;   // the position whose slot is taken; k - 1 is the latest
+            if (!mbar_wait(&t.empty[pos % kWsSlots], (pos / kWsSlots) & 1)) {
+                if (lane == 0) atomicOr(&a.info->err, kErrWorkLoop);
+                alive = false;
+                return 0;
+            }
+            return (int)((handed >> (4 * (k - 1 - pos))) & 15u);
+        };
+        auto close_cells = [&](int flags) {
+            cs = hand_over(cs, cn, flags);
+            ctile = t.tile(cs);
+            cn = 0;
+        };
+        auto close_bodies = [&](int flags) {
+            bs = hand_over(bs, bn, flags | kWsBodies);
+            btile = t.tile(bs);
+            bn = 0;
         };
         // band cells: this warp's chunk of the record (cbase < 0: none yet)
         int64_t cbase = -1;
@@ -203,49 +489,38 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, B >= 4 ? 1 : 2) k_walk_w
                 cused += c;
             }
         };
-        auto open_slot = [&](int flags, int g) {
-            WsHdr* h = slot_hdr(k);
-            if (lane == 0) {
-                h->flags = flags;
-                h->g = g;
-            }
-        };
-        for (;;) {
+        while (alive) {
             int g = 0;
             if (lane == 0) g = (int)atomicAdd(&a.info->work[a.work_slot], 1u);
             g = __shfl_sync(0xffffffffu, g, 0);
             if (g >= G) {
-                if (take()) {
-                    open_slot(kWsDone, 0);
-                    hand_over(0, 0, 0);
-                }
+                first = 0;
+                close_cells(kWsDone);
                 // the unused tail of the chunk: no cell
                 if (LEARNED && cbase >= 0)
-                    for (int j = cused + lane; j < kBandChunk; j += 32) a.band[cbase + j] = make_int2(-1, 0);
+                    for (int i = cused + lane; i < kBandChunk; i += 32) a.band[cbase + i] = make_int2(-1, 0);
                 break;
             }
             if (a.glist) g = __ldg(a.glist + g);
-            const int gfirst = a.gfirst[g];
-            const int gend = a.gfirst[g + 1];
+            gfirst = a.gfirst[g];
+            gend = a.gfirst[g + 1];
+            first = kWsFirst;
             const uint32_t sysid = a.sys_of[gfirst];
             const SysParams& SP = a.sysp[sysid];
             const double ud = 0.5 * SP.h;
             const float uf = SP.uf;
             const float Lf = SP.Lf;
             const int4 rc = nt.c[a.gref[g]];
-            const double gx = SP.c0[0] + (double)rc.x * ud, gy = SP.c0[1] + (double)rc.y * ud,
-                         gz = SP.c0[2] + (double)rc.z * ud;
+            gx = SP.c0[0] + (double)rc.x * ud;
+            gy = SP.c0[1] + (double)rc.y * ud;
+            gz = SP.c0[2] + (double)rc.z * ud;
             // the group's bounding box
             float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-            for (int b = 0; b < B; b++) {
-                const int i = gfirst + lane + 32 * b;
-                if (i < gend) {
-                    const float4 qb = a.body[i];
-                    lo[0] = fminf(lo[0], qb.x); hi[0] = fmaxf(hi[0], qb.x);
-                    lo[1] = fminf(lo[1], qb.y); hi[1] = fmaxf(hi[1], qb.y);
-                    lo[2] = fminf(lo[2], qb.z); hi[2] = fmaxf(hi[2], qb.z);
-                }
+            for (int i = gfirst + lane; i < gend; i += 32) {
+                const float4 qb = a.body[i];
+                lo[0] = fminf(lo[0], qb.x); hi[0] = fmaxf(hi[0], qb.x);
+                lo[1] = fminf(lo[1], qb.y); hi[1] = fmaxf(hi[1], qb.y);
+                lo[2] = fminf(lo[2], qb.z); hi[2] = fmaxf(hi[2], qb.z);
             }
 #pragma unroll
             for (int kk = 0; kk < 3; kk++) {
@@ -262,10 +537,10 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, B >= 4 ? 1 : 2) k_walk_w
             if (lane < 6) {
                 const int ax = lane % 3;
                 const double gref = ax == 0 ? gx : (ax == 1 ? gy : gz);
-                const double t = (double)(lane < 3 ? lo[ax] : hi[ax]) - gref;
-                const double kf = floor(t / ud);
+                const double tt = (double)(lane < 3 ? lo[ax] : hi[ax]) - gref;
+                const double kf = floor(tt / ud);
                 kb = (int)kf;
-                fb = (float)(t - kf * ud);
+                fb = (float)(tt - kf * ud);
             }
             float klof[3], khif[3], flo[3], fhi[3];
             const float rcf[3] = {(float)rc.x, (float)rc.y, (float)rc.z};
@@ -286,153 +561,178 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, B >= 4 ? 1 : 2) k_walk_w
                 a.grec[2 * (int64_t)g + 1] =
                     make_float4(__int_as_float(rc.x), __int_as_float(rc.y), __int_as_float(rc.z), Lf);
             }
-            if (!take()) {
-                alive = false;
-                break;
-            }
-            open_slot(kWsFirst, g);
-            if (lane == 0) {
-                WsHdr* h = slot_hdr(k);
-                h->gfirst = gfirst;
-                h->gend = gend;
-                h->ref[0] = gx;
-                h->ref[1] = gy;
-                h->ref[2] = gz;
-            }
-            float* ctile = slot_cells(k);
-            float* btile = slot_bodies(k);
-            int cn = 0, bn = 0, Lc = 0, Lb = 0;
+            int Lc = 0, Lb = 0;
             unsigned long long hsh = 0;
             const bool fast_side = ((__float_as_int(Lf) >> 23) & 255) > kMaxLevel + 1;
             bool overflow = false;
-            int sp = 1;
-            if (lane == 0) stk[0] = sysid;  // the system's root: holds every body, always opened
-            __syncwarp();
-            while (sp > 0) {
-                const int np = min(sp, 32);
-                int v = -1;
-                if (lane < np) v = (int)stk[sp - np + lane];
-                sp -= np;
-                __syncwarp();
-                int4 nb = make_int4(0, 0, 0, 0);
-                bool acc = false, oleaf = false, oint = false;
-                float4 src = make_float4(0.f, 0.f, 0.f, 0.f);
-                float band_e2 = 0.f;
-                if (v >= 0) {
-                    nb = __ldg(&nt.b[v]);
-                    const float4 na = __ldg(&nt.a[v]);
-                    const int4 cc = __ldg(&nt.c[v]);
-                    const int nch = nb.w >> 8;
-                    const bool overlap = (nb.x < gend) && (gfirst < nb.x + nb.y);
-                    if (!overlap) {
-                        const float D[3] = {(float)cc.x - rcf[0], (float)cc.y - rcf[1], (float)cc.z - rcf[2]};
-                        const float off[3] = {na.x, na.y, na.z};
-                        float e2 = 0.f;
-#pragma unroll
-                        for (int kk = 0; kk < 3; kk++) {
-                            const float lo_c = fmaf(klof[kk] - D[kk], uf, flo[kk]);
-                            const float hi_c = fmaf(khif[kk] - D[kk], uf, fhi[kk]);
-                            const float e = fmaxf(fmaxf(lo_c - off[kk], off[kk] - hi_c), 0.f);
-                            e2 = fmaf(e, e, e2);
-                        }
-                        const float sz = pow2_down(Lf, nb.w & 255, fast_side);
-                        acc = (sz * sz) < a.theta2 * e2;
-                        band_e2 = e2;
-                        if (acc) {
-                            if (PRECISE) {
-                                src = make_float4(fmaf(D[0], uf, off[0]), fmaf(D[1], uf, off[1]),
-                                                  fmaf(D[2], uf, off[2]), na.w);
-                            } else {
-                                src = nt.d[v];
-                            }
-                        }
+            int sp = 0;  // opened cells whose children are to be tested
+            int ln = 0;  // opened leaves whose bodies are not listed yet
+            {
+                // the system's root: holds every body, always opened
+                const int4 rb = nt.b[sysid];
+                if ((rb.w >> 8) != 0) {
+                    if (lane == 0) {
+                        stk[0] = (uint32_t)rb.z;
+                        stn[0] = (uint8_t)(rb.w >> 8);
                     }
-                    if (!acc) {
-                        oleaf = (nch == 0);
-                        oint = (nch != 0);
+                    sp = 1;
+                } else {
+                    if (lane == 0) {
+                        leaves[0] = make_int2(rb.x, rb.y);
+                        if (list_stats) hsh = mix64(2ull * sysid + 2ull);
+                    }
+                    ln = 1;
+                }
+            }
+            __syncwarp();
+            // the bodies of the last m <= 32 opened leaves -> the body tile,
+            // 32 at a time: row[r] turns a body's offset among them into its
+            // index, r found by counting the leaves that start at or before it
+            auto list_leaves = [&](int m) {
+                int2 lf = make_int2(0, 0);
+                if (lane < m) lf = leaves[ln - m + lane];
+                ln -= m;
+                const int incl = (int)ws_incl_scan((unsigned)lf.y);
+                const int excl = incl - lf.y;
+                const int T = __shfl_sync(0xffffffffu, incl, 31);
+                Lb += T;
+                row[lane] = lf.x - excl;
+                __syncwarp();
+                const int32_t* r = row - 1;
+                for (int o = 0; o < T; o += 32) {
+                    const unsigned st = (unsigned)(excl - o);
+                    const unsigned starts = __reduce_or_sync(0xffffffffu, lane < m && st < 32u ? 1u << st : 0u);
+                    if (o + lane < T) {
+                        const float* src4 = reinterpret_cast<const float*>(&a.body[r[__popc(starts & le)] + o + lane]);
+                        float* q = btile + bn + lane;
+                        cp_async4(q, src4);
+                        cp_async4(q + CAP, src4 + 1);
+                        cp_async4(q + 2 * CAP, src4 + 2);
+                        cp_async4(q + 3 * CAP, src4 + 3);
+                    }
+                    r += __popc(starts);
+                    bn += min(32, T - o);
+                    if (bn >= kTile) {
+                        close_bodies(0);
+                        if (!alive) break;
                     }
                 }
-                // opened internal nodes push their children
-                const int npush = oint ? (nb.w >> 8) : 0;
-                int tot;
-                const int excl = warp_excl_small(npush, lt, tot);
-                if (sp + tot > stack_cap) {
+                __syncwarp();
+            };
+            const int slot8 = lane >> 3, child8 = lane & 7;
+            while (sp > 0) {
+                // A step tests the children of the up to eight topmost
+                // opened cells, eight lanes to a cell and two cells to a
+                // lane: cells have 7 to 8 children on average, so a fixed
+                // place for each beats scans that pack them, a cell's
+                // records are read as whole lines, and the two tests of a
+                // lane are independent.
+                const int np = min(sp, 8);
+                sp -= np;
+                int v[2];
+                int4 nbd[2];
+                float4 src[2];
+                float band_e2[2];
+                bool acc[2], oleaf[2], oint[2];
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    const int e = slot8 + 4 * u;
+                    const bool have = e < np && child8 < (int)stn[sp + min(e, np - 1)];
+                    v[u] = have ? (int)stk[sp + e] + child8 : (int)sysid;  // (the other lanes read a root's records)
+                    nbd[u] = __ldg(&nt.b[v[u]]);
+                    const float4 na = __ldg(&nt.a[v[u]]);
+                    const int4 cc = __ldg(&nt.c[v[u]]);
+                    const bool overlap = (nbd[u].x < gend) && (gfirst < nbd[u].x + nbd[u].y);
+                    const float D[3] = {(float)cc.x - rcf[0], (float)cc.y - rcf[1], (float)cc.z - rcf[2]};
+                    const float off[3] = {na.x, na.y, na.z};
+                    float e2 = 0.f;
+#pragma unroll
+                    for (int kk = 0; kk < 3; kk++) {
+                        const float lo_c = fmaf(klof[kk] - D[kk], uf, flo[kk]);
+                        const float hi_c = fmaf(khif[kk] - D[kk], uf, fhi[kk]);
+                        const float ee = fmaxf(fmaxf(lo_c - off[kk], off[kk] - hi_c), 0.f);
+                        e2 = fmaf(ee, ee, e2);
+                    }
+                    const float sz = pow2_down(Lf, nbd[u].w & 255, fast_side);
+                    acc[u] = have && !overlap && (sz * sz) < a.theta2 * e2;
+                    band_e2[u] = e2;
+                    if (PRECISE) {
+                        src[u] = make_float4(fmaf(D[0], uf, off[0]), fmaf(D[1], uf, off[1]), fmaf(D[2], uf, off[2]), na.w);
+                    } else {
+                        src[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (acc[u]) src[u] = nt.d[v[u]];
+                    }
+                    const bool open = have && !acc[u];
+                    oint[u] = open && (nbd[u].w >> 8) != 0;
+                    oleaf[u] = open && (nbd[u].w >> 8) == 0;
+                }
+                const unsigned om0 = __ballot_sync(0xffffffffu, oint[0]), om1 = __ballot_sync(0xffffffffu, oint[1]);
+                const unsigned lm0 = __ballot_sync(0xffffffffu, oleaf[0]), lm1 = __ballot_sync(0xffffffffu, oleaf[1]);
+                const unsigned am0 = __ballot_sync(0xffffffffu, acc[0]), am1 = __ballot_sync(0xffffffffu, acc[1]);
+                // (the ballots also order the lanes' reads of the stack before the pushes)
+                const int no0 = __popc(om0), no1 = __popc(om1);
+                if (sp + no0 + no1 > stack_cap) {
                     overflow = true;
                     break;
                 }
-                for (int c = 0; c < npush; c++) stk[sp + excl + c] = (uint32_t)(nb.z + c);
-                sp += tot;
-                // accepted cells -> the slot's cell part
-                const unsigned am = __ballot_sync(0xffffffffu, acc);
-                if (acc) {
-                    put_entry(ctile, cn + __popc(am & lt), src);
-                    if (list_stats) hsh += mix64(2ull * (unsigned)v + 1ull);
-                }
-                cn += __popc(am);
-                Lc += __popc(am);
-                if (LEARNED) {
-                    bool band = false;
-                    if (acc && nb.y >= 2) {
-                        const float sz = pow2_down(Lf, nb.w & 255, fast_side);
-                        band = sz * sz >= a.band2 * band_e2;
-                    }
-                    band_append(band, v, g);
-                }
-                // opened leaves -> the slot's body part, 32 bodies at a time
-                const unsigned lm = __ballot_sync(0xffffffffu, oleaf);
-                if (lm) {
-                    if (list_stats && oleaf) hsh += mix64(2ull * (unsigned)v + 2ull);
-                    const int cnt = oleaf ? nb.y : 0;
-                    const int incl_c = warp_incl_scan_i(cnt);
-                    const int excl_c = incl_c - cnt;
-                    const int T = __shfl_sync(0xffffffffu, incl_c, 31);
-                    Lb += T;
-                    for (int o = 0; o < T; o += 32) {
-                        const int t = min(o + lane, T - 1);
-                        int pos = 0;
+                const int nl0 = __popc(lm0), na0 = __popc(am0);
 #pragma unroll
-                        for (int step = 16; step; step >>= 1) {
-                            const int e = __shfl_sync(0xffffffffu, excl_c, pos + step);
-                            if (e <= t) pos += step;
-                        }
-                        const int f = __shfl_sync(0xffffffffu, nb.x, pos);
-                        const int e0 = __shfl_sync(0xffffffffu, excl_c, pos);
-                        if (o + lane < T) put_entry_async(btile, bn + lane, &a.body[f + (t - e0)]);
-                        bn += min(32, T - o);
-                        if (bn >= kTile) {
-                            hand_over(0, cn, bn);
-                            if (!take()) {
-                                alive = false;
-                                break;
-                            }
-                            open_slot(0, g);
-                            ctile = slot_cells(k);
-                            btile = slot_bodies(k);
-                            cn = bn = 0;
-                        }
+                for (int u = 0; u < 2; u++) {
+                    if (oint[u]) {
+                        const int q = sp + (u ? no0 + __popc(om1 & lt) : __popc(om0 & lt));
+                        stk[q] = (uint32_t)nbd[u].z;
+                        stn[q] = (uint8_t)(nbd[u].w >> 8);
                     }
-                    if (!alive) break;
+                    if (oleaf[u]) {
+                        leaves[ln + (u ? nl0 + __popc(lm1 & lt) : __popc(lm0 & lt))] = make_int2(nbd[u].x, nbd[u].y);
+                        if (list_stats) hsh += mix64(2ull * (unsigned)v[u] + 2ull);
+                    }
+                    if (acc[u]) {
+                        float* q = ctile + cn + (u ? na0 + __popc(am1 & lt) : __popc(am0 & lt));
+                        q[0] = src[u].x;
+                        q[CAP] = src[u].y;
+                        q[2 * CAP] = src[u].z;
+                        q[3 * CAP] = src[u].w;
+                        if (list_stats) hsh += mix64(2ull * (unsigned)v[u] + 1ull);
+                    }
+                }
+                sp += no0 + no1;
+                ln += nl0 + __popc(lm1);
+                const int nacc = na0 + __popc(am1);
+                cn += nacc;
+                Lc += nacc;
+                if (LEARNED) {
+#pragma unroll
+                    for (int u = 0; u < 2; u++) {
+                        bool band = false;
+                        if (acc[u] && nbd[u].y >= 2) {
+                            const float sz = pow2_down(Lf, nbd[u].w & 255, fast_side);
+                            band = sz * sz >= a.band2 * band_e2[u];
+                        }
+                        band_append(band, v[u], g);
+                    }
                 }
                 __syncwarp();
                 if (cn >= kTile) {
-                    hand_over(0, cn, bn);
-                    if (!take()) {
-                        alive = false;
-                        break;
-                    }
-                    open_slot(0, g);
-                    ctile = slot_cells(k);
-                    btile = slot_bodies(k);
-                    cn = bn = 0;
+                    close_cells(0);
+                    if (!alive) break;
                 }
+                while (ln >= 32 && alive) list_leaves(32);
+                if (!alive) break;
             }
+            if (alive && !overflow && ln > 0) list_leaves(ln);
             if (!alive) break;
             if (overflow) {
                 if (lane == 0) atomicOr(&a.info->err, kErrStack);
-                hand_over(kWsLast | kWsAbort, 0, 0);
+                cp_async_wait_all();  // copies into the dropped tile
+                __syncwarp();
+                cn = bn = 0;
+                close_bodies(kWsLast | kWsAbort);
                 continue;
             }
-            hand_over(kWsLast, cn, bn);
+            if (cn > 0) close_cells(0);
+            if (!alive) break;
+            close_bodies(kWsLast);
             if (list_stats) {
 #pragma unroll
                 for (int o = 16; o; o >>= 1) hsh += __shfl_xor_sync(0xffffffffu, hsh, o);
@@ -448,96 +748,93 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, B >= 4 ? 1 : 2) k_walk_w
             }
             __syncwarp();
         }
-        (void)alive;
         cp_async_wait_all();  // (a warp that gave up may still have copies in flight)
         return;
     }
 
     // ---------------------------------------------------------------- consumer
-    constexpr int kUnroll = B >= 4 ? 4 : 8;
-    const f2 E2 = f2pack(a.eps2, a.eps2);
-    f2 XA[B], YA[B], ZA[B], XR[B], YR[B], ZR[B];
-    float mi[B];
-    bool act[B];
-#pragma unroll
-    for (int b = 0; b < B; b++) {
-        XA[b] = YA[b] = ZA[b] = XR[b] = YR[b] = ZR[b] = 0ull;
-        mi[b] = 0.f;
-        act[b] = false;
-    }
-    int gfirst = 0;
-    Accum<B, PRECISE, POT, kUnroll> fsum;
-    fsum.init();
-    for (int k = 0;; k++) {
-        if (!mbar_wait(&full[k % kWsSlots], (k / kWsSlots) & 1)) {
+    const int c = (warp - teams) % C;
+    float* pos = reinterpret_cast<float*>(after + (size_t)c * ws_pos_bytes(nb));
+    float* comb = reinterpret_cast<float*>(after + (size_t)C * ws_pos_bytes(nb));
+    int groups = 0;
+    for (int k = 0;;) {
+        bool ok = mbar_wait(&t.full[k % kWsSlots], (k / kWsSlots) & 1);
+        if (ok) {
+            const WsHdr* h = t.hdr(t.seq[k % kWsSlots]);
+            if (h->flags & kWsDone) return;
+            const int gfirst = h->gfirst, ng = h->gend - h->gfirst;
+            const double gx = h->ref[0], gy = h->ref[1], gz = h->ref[2];
+            // positions of every body slot (slots past the group repeat its
+            // first body; their sums are dropped)
+            const int slots = ng <= 32 ? 32 : (ng <= 64 ? 64 : nb);
+            __syncwarp();
+            for (int i = lane; i < slots; i += 32) {
+                const float4 q = a.body[gfirst + (i < ng ? i : 0)];
+                pos[i] = q.x;
+                pos[nb + i] = q.y;
+                pos[2 * nb + i] = q.z;
+                pos[3 * nb + i] = (float)((double)q.x - gx);
+                pos[4 * nb + i] = (float)((double)q.y - gy);
+                pos[5 * nb + i] = (float)((double)q.z - gz);
+            }
+            __syncwarp();
+            float* cb = comb + (groups & 1) * (size_t)C * 8 * nb;
+            const int cph = groups & 1;
+            groups++;
+#define TC_WS_GROUP(K, S) consume_group<K, S, TILE, PRECISE, POT>(t, k, c, C, pos, nb, cb, cph, gfirst, ng, a)
+            if (ng <= 16) k = TC_WS_GROUP(1, 2);
+            else if (ng <= 32) k = TC_WS_GROUP(1, 1);
+            else if (ng <= 40) k = TC_WS_GROUP(5, 4);
+            else if (ng <= 48) k = TC_WS_GROUP(3, 2);
+            else if (ng <= 64) k = TC_WS_GROUP(2, 1);
+            else if (ng <= 96) k = TC_WS_GROUP(3, 1);
+            else k = TC_WS_GROUP(4, 1);
+#undef TC_WS_GROUP
+            ok = k >= 0;
+        }
+        if (!ok) {
             if (lane == 0) atomicOr(&a.info->err, kErrWorkLoop);
             return;
-        }
-        const WsHdr* h = slot_hdr(k);
-        const int flags = h->flags;
-        if (flags & kWsDone) return;
-        const int cn = h->cn, bn = h->bn;
-        if (flags & kWsFirst) {
-            gfirst = h->gfirst;
-            const int gend = h->gend;
-            const double gx = h->ref[0], gy = h->ref[1], gz = h->ref[2];
-#pragma unroll
-            for (int b = 0; b < B; b++) {
-                const int i = gfirst + lane + 32 * b;
-                act[b] = i < gend;
-                const float4 qb = a.body[act[b] ? i : gfirst];
-                XA[b] = f2pack(qb.x, qb.x);
-                YA[b] = f2pack(qb.y, qb.y);
-                ZA[b] = f2pack(qb.z, qb.z);
-                mi[b] = qb.w;
-                if (PRECISE) {
-                    const float rx = (float)((double)qb.x - gx), ry = (float)((double)qb.y - gy),
-                                rz = (float)((double)qb.z - gz);
-                    XR[b] = f2pack(rx, rx);
-                    YR[b] = f2pack(ry, ry);
-                    ZR[b] = f2pack(rz, rz);
-                }
-            }
-            fsum.init();
-        }
-        float* ct = slot_cells(k);
-        float* bt = slot_bodies(k);
-        if (PRECISE) fsum.flush(ct, cn, XR, YR, ZR, E2);
-        else fsum.flush(ct, cn, XA, YA, ZA, E2);
-        fsum.flush(bt, bn, XA, YA, ZA, E2);
-        __syncwarp();
-        mbar_arrive(&empty[k % kWsSlots]);
-        if ((flags & kWsLast) && !(flags & kWsAbort)) {
-#pragma unroll
-            for (int b = 0; b < B; b++) {
-                if (!act[b]) continue;
-                const int i = gfirst + lane + 32 * b;
-                const int64_t o = a.perm[i];
-                float sx_, sy_, sz_, sp_, kx, ky, kz, kp;
-                fsum.result(b, sx_, sy_, sz_, sp_);
-                fsum.comp(b, kx, ky, kz, kp);
-                a.acc[3 * o + 0] = a.G * (sx_ + kx);
-                a.acc[3 * o + 1] = a.G * (sy_ + ky);
-                a.acc[3 * o + 2] = a.G * (sz_ + kz);
-                if (POT) {
-                    const float self = mi[b] * rsqrtf(a.eps2);
-                    a.pot[o] = a.G * ((sp_ + kp) + self);
-                }
-            }
         }
     }
 }
 
-template <int B, int TILE, bool PRECISE, bool POT, bool LEARNED>
+// a launch's team, block and shared memory
+struct WsShape {
+    int C, threads, nb, stack;
+    size_t smem;
+};
+constexpr size_t kWsSmemMax = 227 * 1024;
+
+__host__ __forceinline__ WsShape ws_shape(const WalkConfig& c, int tile)
+{
+    WsShape w;
+    const int pairs = c.warps < 1 ? 1 : (c.warps > kWsMaxPairs ? kWsMaxPairs : c.warps);
+    w.C = c.consumers < 1 ? 1 : c.consumers;
+    while (w.C > 1 && (1 + w.C) > 2 * pairs) w.C = (w.C - 1) / 2;  // 7 -> 3 -> 1
+    const int teams = 2 * pairs / (1 + w.C);
+    w.threads = teams * (1 + w.C) * 32;
+    w.nb = ws_body_slots(c.gmax);
+    // a stack that leaves no room for the ring is cut (an entry stands for
+    // all the children of a cell, so it holds several times as many nodes
+    // as one entry per node)
+    w.stack = (c.stack + 3) & ~3;
+    while (w.stack > 64 && ws_team_bytes(tile, w.stack, w.C, w.nb) * teams > kWsSmemMax) w.stack -= 16;
+    w.smem = ws_team_bytes(tile, w.stack, w.C, w.nb) * teams;
+    return w;
+}
+
+template <int TILE, bool PRECISE, bool POT, bool LEARNED>
 cudaError_t prepare_ws_t(const WalkConfig& c, int num_sms, int* grid, size_t* smem_out)
 {
-    const int pairs = c.warps < 1 ? 1 : (c.warps > kWsMaxPairs ? kWsMaxPairs : c.warps);
-    const size_t smem = ws_pair_bytes(TILE, c.stack) * pairs;
-    auto kern = k_walk_ws<B, TILE, PRECISE, POT, LEARNED>;
+    const WsShape w = ws_shape(c, TILE);
+    const int threads = w.threads;
+    const size_t smem = w.smem;
+    auto kern = k_walk_ws<TILE, PRECISE, POT, LEARNED>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, pairs * 64, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     if (c.blocks_per_sm > 0 && c.blocks_per_sm < per_sm) per_sm = c.blocks_per_sm;
@@ -546,15 +843,15 @@ cudaError_t prepare_ws_t(const WalkConfig& c, int num_sms, int* grid, size_t* sm
     return cudaSuccess;
 }
 
-template <int B, int TILE, bool PRECISE, bool POT, bool LEARNED>
+template <int TILE, bool PRECISE, bool POT, bool LEARNED>
 cudaError_t launch_ws_t(const WalkArgs& a, const WalkConfig& c, int grid, size_t smem, cudaStream_t s)
 {
-    // the split walk has no list export, training pairs or quadrupole
-    // terms (those run on k_walk); its learned walk records band cells
-    if (a.list_cells || a.pair_body) return cudaErrorInvalidValue;
+    // the split walk has no list export, training pairs, size classes or
+    // quadrupole terms (those run on k_walk); its learned walk records band cells
+    if (a.list_cells || a.pair_body || a.gseg) return cudaErrorInvalidValue;
     if (LEARNED && (!a.band || !a.band_n || !a.grec)) return cudaErrorInvalidValue;
-    const int pairs = c.warps < 1 ? 1 : (c.warps > kWsMaxPairs ? kWsMaxPairs : c.warps);
-    k_walk_ws<B, TILE, PRECISE, POT, LEARNED><<<grid, pairs * 64, smem, s>>>(a, c.stack);
+    const WsShape w = ws_shape(c, TILE);
+    k_walk_ws<TILE, PRECISE, POT, LEARNED><<<grid, w.threads, smem, s>>>(a, w.stack, w.C, w.nb);
     count_launches(1);
     return cudaGetLastError();
 }

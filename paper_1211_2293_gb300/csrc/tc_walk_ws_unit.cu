@@ -1,0 +1,41 @@
+// tc_walk_ws_unit.cu -- the walk on producer and consumer warps for list
+// tiles of TC_WALK_TILE entries, every mode.  The build compiles this file
+// once per tile in {64, 128, 256}, defining the macro.
+#include "tc_walk.cuh"
+#include "tc_walk_ws.cuh"
+
+#if !defined(TC_WALK_TILE)
+#error "compile with -DTC_WALK_TILE=<64|128|256>"
+#endif
+
+#define TC_PASTE2(a, b) a##b
+#define TC_UNIT_NAME(stem, t) TC_PASTE2(stem, t)
+
+namespace tc {
+
+// precise or plain, with or without the potential; the learned walk (precise,
+// no potential) records its band cells for k_band_eval
+cudaError_t TC_UNIT_NAME(prepare_walk_ws_t, TC_WALK_TILE)(const WalkConfig& c, int num_sms, int* grid, size_t* smem)
+{
+    const bool p = c.precise != 0, pot = c.want_pot != 0;
+    if (c.quadw || (c.learned && (!p || pot))) return cudaErrorInvalidValue;
+    if (c.learned) return prepare_ws_t<TC_WALK_TILE, true, false, true>(c, num_sms, grid, smem);
+    if (p && pot) return prepare_ws_t<TC_WALK_TILE, true, true, false>(c, num_sms, grid, smem);
+    if (p) return prepare_ws_t<TC_WALK_TILE, true, false, false>(c, num_sms, grid, smem);
+    if (pot) return prepare_ws_t<TC_WALK_TILE, false, true, false>(c, num_sms, grid, smem);
+    return prepare_ws_t<TC_WALK_TILE, false, false, false>(c, num_sms, grid, smem);
+}
+
+cudaError_t TC_UNIT_NAME(launch_walk_ws_t, TC_WALK_TILE)(const WalkArgs& a, const WalkConfig& c, int grid, size_t smem,
+                                                         cudaStream_t s)
+{
+    const bool p = c.precise != 0, pot = c.want_pot != 0;
+    if (c.quadw || (c.learned && (!p || pot))) return cudaErrorInvalidValue;
+    if (c.learned) return launch_ws_t<TC_WALK_TILE, true, false, true>(a, c, grid, smem, s);
+    if (p && pot) return launch_ws_t<TC_WALK_TILE, true, true, false>(a, c, grid, smem, s);
+    if (p) return launch_ws_t<TC_WALK_TILE, true, false, false>(a, c, grid, smem, s);
+    if (pot) return launch_ws_t<TC_WALK_TILE, false, true, false>(a, c, grid, smem, s);
+    return launch_ws_t<TC_WALK_TILE, false, false, false>(a, c, grid, smem, s);
+}
+
+}  // namespace tc
