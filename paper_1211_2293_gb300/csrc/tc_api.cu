@@ -58,23 +58,20 @@ struct tc_ctx {
     float4* body = nullptr;
     SortBufs sb{};
     int8_t *w = nullptr, *delta = nullptr, *top = nullptr;
-    uint32_t *nstart = nullptr, *prepos = nullptr;
-    uint32_t *gflag = nullptr, *gscan = nullptr;
+    uint32_t* lcnt = nullptr;    // nodes per level and block of bodies, then their places
+    uint32_t* lstart = nullptr;  // first node of each level
+    unsigned long long* scan = nullptr;  // the build's look-back words
     int32_t *gref_at = nullptr, *gfirst = nullptr, *gref = nullptr;
     int32_t *ncell = nullptr, *nbody = nullptr;
     unsigned long long* hash = nullptr;
-    uint32_t* totals = nullptr;  // [0] nodes, [1] groups
     int64_t* idx_dev = nullptr;
     int64_t cap_idx = 0;
     double* dir_out = nullptr;
     double* dir_part = nullptr;  // per-slice partial sums of a direct sum
     int64_t cap_dir_part = 0;
-    // per-node scratch
-    uint32_t *pre_level = nullptr, *pre_first = nullptr, *iota = nullptr, *bfs_of_pre = nullptr, *lvl_alt = nullptr;
     NodeTables nt{};
     Info* info = nullptr;
     Info* info_h = nullptr;  // pinned mirror
-    int64_t cap_m_h = 0;     // source of the device copy of cap_m
     size_t allocated = 0;
     std::unordered_map<void*, size_t> sizes;
 
@@ -301,24 +298,21 @@ int ensure_bodies(tc_ctx* c, int64_t n)
     TC_GROW(c, c->sb.status, (int64_t)kSortMaxPasses * radix_tiles(cap) * 256);
     TC_GROW(c, c->sb.tiles, kSortMaxPasses);
     c->sb.err = &c->info->err;
-    TC_GROW(c, c->sb.blocksum, scan_blocksum_size(cap));
     TC_GROW(c, c->sb.runs, cap / 32 + 16);  // runs of more than 32 items
     c->sb.run_cap = cap / 32 + 16;
     TC_GROW(c, c->sb.nruns, 1);
     TC_GROW(c, c->w, cap);
     TC_GROW(c, c->delta, cap);
     TC_GROW(c, c->top, cap);
-    TC_GROW(c, c->nstart, cap);
-    TC_GROW(c, c->prepos, cap);
-    TC_GROW(c, c->gflag, cap);
-    TC_GROW(c, c->gscan, cap);
+    TC_GROW(c, c->lcnt, level_counts_size(cap));
+    TC_GROW(c, c->lstart, kMaxLevel + 2);
+    TC_GROW(c, c->scan, build_scan_words(cap));
     TC_GROW(c, c->gref_at, cap);
     TC_GROW(c, c->gfirst, cap + 1);
     TC_GROW(c, c->gref, cap);
     TC_GROW(c, c->ncell, cap);
     TC_GROW(c, c->nbody, cap);
     TC_GROW(c, c->hash, cap);
-    TC_GROW(c, c->totals, 4);
     TC_GROW(c, c->gorder, cap);
     TC_GROW(c, c->gseg, 4 + (int64_t)group_order_scratch());
     c->cap_n = cap;
@@ -344,11 +338,6 @@ int ensure_nodes(tc_ctx* c, int64_t M)
 {
     if (M <= c->cap_m) return TC_OK;
     const int64_t cap = M + M / 2 + 1024;  // headroom for the rebuilds of later steps
-    TC_GROW(c, c->pre_level, cap);
-    TC_GROW(c, c->pre_first, cap);
-    TC_GROW(c, c->iota, cap);
-    TC_GROW(c, c->bfs_of_pre, cap);
-    TC_GROW(c, c->lvl_alt, cap);
     TC_GROW(c, c->nt.a, cap);
     TC_GROW(c, c->nt.b, cap);
     TC_GROW(c, c->nt.c, cap);
@@ -358,10 +347,9 @@ int ensure_nodes(tc_ctx* c, int64_t M)
     TC_GROW(c, c->nt.mass64, cap);
     TC_GROW(c, c->nt.dsum, 2 * cap);
     TC_GROW(c, c->nt.com64, 3 * cap);
-    // the level sort reuses the body sort's value ping-pong buffer and status words
-    if (cap > c->cap_n) TC_GROW(c, c->sb.vals_alt, cap);
-    if (radix_tiles(cap) > (int64_t)kSortMaxPasses * radix_tiles(c->cap_n))
-        TC_GROW(c, c->sb.status, radix_tiles(cap) * 256);
+    TC_GROW(c, c->nt.parent, cap);
+    TC_GROW(c, c->nt.fam, cap);
+    TC_GROW(c, c->nt.pend, cap);
     c->cap_m = cap;
     c->walk_ready = false;  // the stack bound may follow the capacity
     return TC_OK;
@@ -495,50 +483,34 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
                    synced ? kSortRunMaxSynced : kSortRunMax);
     launch_gather(c->pos, c->mass, c->perm, n, c->body, s);
     TC_CUDA(c, cudaMemsetAsync(&c->info->depth, 0, sizeof(int32_t), s));
-    launch_node_counts(c->keys, c->sys_of, n, c->leaf_max, c->w, c->delta, c->top, c->nstart, &c->info->depth, s);
-    scan_u32(c->nstart, c->prepos, n, &c->totals[0], c->sb.blocksum, s);
+    TC_CUDA(c, cudaMemsetAsync(c->scan, 0, build_scan_words(n) * sizeof(unsigned long long), s));
+    launch_node_levels(c->keys, c->sys_of, n, c->leaf_max, c->w, c->delta, c->top, c->gref_at, c->lcnt, c->scan,
+                       synced ? -1 : c->cap_m, c->info, s);
     int depth = -1;
     if (synced) {
+        // one round trip: the error word, the number of nodes and the depth
         TC_CUDA(c, cudaGetLastError());
-        if (low_bit > 0) {
+        TC_CUDA(c, cudaMemcpyAsync(c->info_h, c->info, sizeof(Info), cudaMemcpyDeviceToHost, s));
+        TC_CUDA(c, cudaStreamSynchronize(s));
+        if (low_bit > 0 && (c->info_h->err & kErrSortRun)) {
             // a run too long for the completion: build again, sorting every digit
-            TC_CUDA(c, cudaStreamSynchronize(s));
-            int32_t err = 0;
-            TC_CUDA(c, cudaMemcpy(&err, &c->info->err, sizeof(err), cudaMemcpyDeviceToHost));
-            if (err & kErrSortRun) {
-                TC_CUDA(c, cudaMemsetAsync(&c->info->err, 0, sizeof(int32_t), s));
-                phase_end(c, 0, t0, s);
-                return build_tree(c, true, s, true);
-            }
+            TC_CUDA(c, cudaMemsetAsync(&c->info->err, 0, sizeof(int32_t), s));
+            phase_end(c, 0, t0, s);
+            return build_tree(c, true, s, true);
         }
-        int r = check_device(c);  // synchronises; reports invalid input
+        if (c->info_h->err) return check_device(c);  // invalid input; clears the word
+        if (c->info_h->M < 1) return fail(c, TC_EDEVICE, "empty node table");
+        int r = ensure_nodes(c, c->info_h->M);
         if (r) return r;
-        uint32_t M32 = 0;
-        TC_CUDA(c, cudaMemcpy(&M32, &c->totals[0], sizeof(uint32_t), cudaMemcpyDeviceToHost));
-        if (M32 < 1) return fail(c, TC_EDEVICE, "empty node table");
-        r = ensure_nodes(c, M32);
-        if (r) return r;
-        c->M = M32;
-        c->cap_m_h = c->cap_m;
-        TC_CUDA(c, cudaMemcpyAsync(&c->info->cap_m, &c->cap_m_h, sizeof(int64_t), cudaMemcpyHostToDevice, s));
+        c->M = c->info_h->M;
         depth = c->info_h->depth;
         c->depth_hint = depth;
         c->depth_hint_n = n;
     }
-    launch_check_capacity(&c->totals[0], c->info, s);
-    launch_emit_preorder(c->delta, c->nstart, c->prepos, n, c->info, c->pre_level, c->pre_first, c->iota, s);
-    // breadth-first order: stable sort of the pre-order nodes by level
-    SortBufs lb = c->sb;
-    radix_sort_u32(c->pre_level, c->iota, c->cap_m, &c->info->M, 8, lb, c->lvl_alt, s);
-    launch_inverse_perm(c->iota, c->cap_m, c->info, c->bfs_of_pre, s);
-    launch_node_finalize(c->keys, c->top, c->sys_of, c->sysp, n, c->pre_level, c->iota, c->pre_first, c->bfs_of_pre,
-                         c->cap_m, c->info, c->nt, s);
-    // after the level sort, ghist[l] is the first breadth-first index of level l
-    launch_moments(c->body, c->cap_m, depth, c->depth_hint, c->sb.ghist, c->sys_of, c->sysp, c->info, c->nt, c->cfg.quad != 0, s);
-    launch_sys_mass(c->sysp, c->nsys, c->nt, c->info, s);
-    launch_group_marks(c->cap_m, c->info, c->nt, c->cfg.gmax, n, c->gflag, c->gref_at, s);
-    scan_u32(c->gflag, c->gscan, n, &c->totals[1], c->sb.blocksum, s);
-    launch_group_table(c->gflag, c->gscan, c->gref_at, n, &c->totals[1], c->gfirst, c->gref, c->info, s);
+    launch_emit_nodes(c->keys, c->delta, c->top, c->sys_of, n, c->lcnt, c->info, c->lstart, c->nt, s);
+    launch_moments(c->body, c->delta, n, c->nsys, c->cap_m, depth, c->depth_hint, c->lstart, c->sysp, c->info, c->nt,
+                   c->cfg.quad != 0, s);
+    launch_groups(c->cap_m, c->info, c->nt, c->cfg.gmax, n, c->gref_at, c->scan, c->gfirst, c->gref, s);
     c->gorder_ready = false;
     TC_CUDA(c, cudaGetLastError());
     phase_end(c, 0, t0, s);
@@ -1641,7 +1613,6 @@ int tc_mlp_pairs(tc_ctx* c, float theta, float eps, float band, float prob, uint
         TC_GROW(c, c->pair_sb.ghist, kSortMaxPasses * 256);
         TC_GROW(c, c->pair_sb.status, (int64_t)kSortMaxPasses * radix_tiles(cap) * 256);
         TC_GROW(c, c->pair_sb.tiles, kSortMaxPasses);
-        TC_GROW(c, c->pair_sb.blocksum, scan_blocksum_size(cap));
         c->pair_sb.err = &c->info->err;
         c->pair_sort_cap = cap;
     }

@@ -13,16 +13,19 @@
 //   2. k_keys      63-bit Morton keys (exact FP64 quantisation)
 //   3. radix sort  stable sort by (system, key, index)    [tc_sort.cu]
 //   4. k_gather    bodies in Morton order as float4 (x, y, z, m)
-//   5. k_window / k_node_counts
+//   5. k_window / k_node_levels, k_scan_levels
 //                  which cubes of the recursive subdivision start at each
-//                  sorted body (a sliding-window test, below)
-//   6. scan + k_emit_preorder      node table in pre-order
-//   7. one stable radix pass by level  -> breadth-first order
-//   8. k_node_finalize  counts, children, integer centres
-//   9. k_leaf_moments, then k_level_moments level by level from the deepest
-//                  mass / centre of mass (float-pair sums, FP64-class, stored
-//                  in FP64) / second moments (FP32), bottom-up
-//  10. k_group_marks + scan + k_group_table   body groups for the walk
+//                  sorted body (a sliding-window test, below), how many of
+//                  each level per block of bodies, and their scan: the
+//                  nodes' places in breadth-first order
+//   6. k_emit_nodes  the node records: first body, first child, parent,
+//                  integer centre
+//   7. k_leaf_nodes  children and counts; mass / centre of mass (float-pair
+//                  sums, FP64-class, stored in FP64) / second moments (FP32)
+//                  of the leaves; the internal cells bottom-up in the same
+//                  launch (small trees) or by k_level_moments level by level
+//                  from the deepest
+//   8. k_group_marks + k_group_table   body groups for the walk
 //
 // Which cubes exist.  Let cd(a, b) be the number of leading octal digits two
 // keys share.  The level-l run of equal l-digit prefixes that contains sorted
@@ -33,10 +36,10 @@
 // more than leaf_max bodies (and the parent is above level 21).  So the cubes
 // whose first body is s are the levels l with
 //     delta_s < l <= min(W_s + 1, 21),   delta_s = cd(key_{s-1}, key_s)
-// (delta_0 = -1), and the deepest of them is a leaf.  Pre-order of the tree
-// is the order of (first body, level), so one scan over the per-body counts
-// places every node.
+// (delta_0 = -1), and the deepest of them is a leaf.  Breadth-first order of
+// the tree is the order of (level, first body).
 #include "tc_internal.cuh"
+#include "tc_lookback.cuh"
 
 // With several systems, cd() of two bodies of different systems is taken as
 // -1 (no common cube), so delta_s = -1 at the first body of every system and
@@ -253,6 +256,48 @@ __global__ void k_gather(const float* __restrict__ pos, const float* __restrict_
 }
 
 // ------------------------------------------------------------------ nodes
+// Blocks of kNodeBlock sorted bodies count and place the nodes that start at
+// their bodies.  Breadth-first order is (level, first body), so the exclusive
+// scan of the blocks' counts, laid out level by level, is the place of each
+// block's first node of each level: no pre-order table and no sort by level
+// lie between the counts and the node table.
+constexpr int kNodeBlock = 1024;
+constexpr int kLevels = kMaxLevel + 1;
+constexpr int kTileWindow = 256;
+
+// per level, the block's nodes (levels d < l <= t of every body) -> cnt[l][block]
+__device__ __forceinline__ void count_levels(int d, int t, uint32_t* __restrict__ cnt)
+{
+    __shared__ uint32_t wc[kNodeBlock / 32][kLevels];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t mine = 0;
+#pragma unroll
+    for (int l = 0; l < kLevels; l++) {
+        const unsigned m = __ballot_sync(0xffffffffu, d < l && l <= t);
+        if (lane == l) mine = __popc(m);
+    }
+    if (lane < kLevels) wc[w][lane] = mine;
+    __syncthreads();
+    if (threadIdx.x < kLevels) {
+        uint32_t c = 0;
+        for (int k = 0; k < kNodeBlock / 32; k++) c += wc[k][threadIdx.x];
+        cnt[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = c;
+    }
+}
+
+// the deepest level of the forest: a block maximum, then one atomic a block
+__device__ __forceinline__ void block_depth(int t, int32_t* depth)
+{
+    __shared__ int wmax[kNodeBlock / 32];
+    t = __reduce_max_sync(0xffffffffu, t);
+    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = t;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        t = __reduce_max_sync(0xffffffffu, wmax[threadIdx.x]);
+        if (threadIdx.x == 0) atomicMax(depth, t);
+    }
+}
+
 __global__ void k_window(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ sys_of, int64_t n,
                          int leaf_max, int8_t* __restrict__ w)
 {
@@ -263,66 +308,58 @@ __global__ void k_window(const uint64_t* __restrict__ keys, const uint32_t* __re
                : (int8_t)-1;
 }
 
-__global__ void k_node_counts(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ sys_of,
-                              const int8_t* __restrict__ w, int64_t n, int leaf_max, int8_t* __restrict__ delta,
-                              int8_t* __restrict__ top, uint32_t* __restrict__ nstart, int32_t* __restrict__ depth)
+// leaf_max > kTileWindow: the window digits come from k_window
+__global__ void __launch_bounds__(kNodeBlock) k_node_levels(const uint64_t* __restrict__ keys,
+                                                            const uint32_t* __restrict__ sys_of,
+                                                            const int8_t* __restrict__ w, int64_t n, int leaf_max,
+                                                            int8_t* __restrict__ delta, int8_t* __restrict__ top,
+                                                            int32_t* __restrict__ gref_at, uint32_t* __restrict__ cnt,
+                                                            int32_t* __restrict__ depth)
 {
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int t = 0;
+    const int64_t s = (int64_t)blockIdx.x * kNodeBlock + threadIdx.x;
+    int t = -1, d = 0;
     if (s < n) {
-        const int d = (s == 0 || sys_of[s] != sys_of[s - 1]) ? -1 : common_digits(keys[s - 1], keys[s]);
+        d = (s == 0 || sys_of[s] != sys_of[s - 1]) ? -1 : common_digits(keys[s - 1], keys[s]);
         int W = -1;
         const int64_t j0 = s - leaf_max < 0 ? 0 : s - leaf_max;
         for (int64_t j = j0; j <= s; j++) W = max(W, (int)w[j]);
         t = min(W + 1, kMaxLevel);
         delta[s] = (int8_t)d;
         top[s] = (int8_t)t;
-        nstart[s] = (uint32_t)max(0, t - d);
+        gref_at[s] = 0;
     }
-    // deepest level of the forest: a block maximum, then one atomic per
-    // block (blocks of 256)
-    __shared__ int wmax[8];
-#pragma unroll
-    for (int o = 16; o; o >>= 1) t = max(t, __shfl_xor_sync(0xffffffffu, t, o));
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = t;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 1; k < (int)(blockDim.x >> 5); k++) t = max(t, wmax[k]);
-        atomicMax(depth, t);
-    }
+    block_depth(t, depth);
+    count_levels(d, t, cnt);
 }
 
-// The same two steps in one kernel for leaf_max <= kTileWindow: a block of
-// kCountThreads sorted bodies stages the keys and systems of
-// [b0 - leaf_max, b0 + kCountThreads + leaf_max) in shared memory, forms the
-// window digits cd(key_j, key_j+leaf_max) of [b0 - leaf_max, b0 + kCountThreads)
-// there, and takes each body's window maximum from them.
-constexpr int kCountThreads = 256;
-constexpr int kTileWindow = 256;
-
-__global__ void __launch_bounds__(kCountThreads) k_node_counts_tiled(const uint64_t* __restrict__ keys,
-                                                                     const uint32_t* __restrict__ sys_of, int64_t n,
-                                                                     int leaf_max, int8_t* __restrict__ delta,
-                                                                     int8_t* __restrict__ top,
-                                                                     uint32_t* __restrict__ nstart,
-                                                                     int32_t* __restrict__ depth)
+// The same in one kernel for leaf_max <= kTileWindow: a block stages the keys
+// and systems of [b0 - leaf_max, b0 + kNodeBlock + leaf_max) in shared memory,
+// forms the window digits cd(key_j, key_j+leaf_max) there, and takes each
+// body's window maximum from them.
+__global__ void __launch_bounds__(kNodeBlock) k_node_levels_tiled(const uint64_t* __restrict__ keys,
+                                                                  const uint32_t* __restrict__ sys_of, int64_t n,
+                                                                  int leaf_max, int8_t* __restrict__ delta,
+                                                                  int8_t* __restrict__ top,
+                                                                  int32_t* __restrict__ gref_at,
+                                                                  uint32_t* __restrict__ cnt,
+                                                                  int32_t* __restrict__ depth)
 {
-    __shared__ uint64_t sk[kCountThreads + 2 * kTileWindow];
-    __shared__ uint32_t ss[kCountThreads + 2 * kTileWindow];
-    __shared__ int8_t sw[kCountThreads + kTileWindow];
-    const int64_t b0 = (int64_t)blockIdx.x * kCountThreads;
+    __shared__ uint64_t sk[kNodeBlock + 2 * kTileWindow];
+    __shared__ uint32_t ss[kNodeBlock + 2 * kTileWindow];
+    __shared__ int8_t sw[kNodeBlock + kTileWindow];
+    const int64_t b0 = (int64_t)blockIdx.x * kNodeBlock;
     const int64_t base = b0 - leaf_max;  // smem index 0 holds body base
-    const int nk = kCountThreads + 2 * leaf_max;
-    for (int i = threadIdx.x; i < nk; i += kCountThreads) {
+    const int nk = kNodeBlock + 2 * leaf_max;
+    for (int i = threadIdx.x; i < nk; i += kNodeBlock) {
         const int64_t j = base + i;
         const bool in = j >= 0 && j < n;
         sk[i] = in ? keys[j] : 0ull;
         ss[i] = in ? sys_of[j] : 0xffffffffu;
     }
     __syncthreads();
-    // window digits of bodies base .. b0 + kCountThreads - 1
-    const int nw = kCountThreads + leaf_max;
-    for (int i = threadIdx.x; i < nw; i += kCountThreads) {
+    // window digits of bodies base .. b0 + kNodeBlock - 1
+    const int nw = kNodeBlock + leaf_max;
+    for (int i = threadIdx.x; i < nw; i += kNodeBlock) {
         const int64_t j = base + i;
         int8_t v = -1;
         if (j >= 0 && j + leaf_max < n && ss[i] == ss[i + leaf_max]) v = (int8_t)common_digits(sk[i], sk[i + leaf_max]);
@@ -330,108 +367,180 @@ __global__ void __launch_bounds__(kCountThreads) k_node_counts_tiled(const uint6
     }
     __syncthreads();
     const int64_t s = b0 + threadIdx.x;
-    int t = 0;
+    int t = -1, d = 0;
     if (s < n) {
         const int i = threadIdx.x + leaf_max;  // smem index of body s
-        const int d = (s == 0 || ss[i] != ss[i - 1]) ? -1 : common_digits(sk[i - 1], sk[i]);
+        d = (s == 0 || ss[i] != ss[i - 1]) ? -1 : common_digits(sk[i - 1], sk[i]);
         int W = -1;
         const int i0 = s - leaf_max < 0 ? (int)(leaf_max - s) : 0;  // window clipped at body 0
         for (int k = i0; k <= leaf_max; k++) W = max(W, (int)sw[threadIdx.x + k]);
         t = min(W + 1, kMaxLevel);
         delta[s] = (int8_t)d;
         top[s] = (int8_t)t;
-        nstart[s] = (uint32_t)max(0, t - d);
+        gref_at[s] = 0;
     }
-    // deepest level: a block maximum, then one atomic per block (one per
-    // warp made the atomics on the single word the kernel's bottleneck)
-    __shared__ int wmax[kCountThreads / 32];
+    block_depth(t, depth);
+    count_levels(d, t, cnt);
+}
+
+// Exclusive scan of the counts in place, one pass; the total is the number of
+// nodes.  A look-back that gave up raises kErrCapacity too, so nothing is
+// placed by offsets that are not known.
+constexpr int kScanThreads = 256;
+constexpr int kScanItems = 16;
+constexpr int kScanTile = kScanThreads * kScanItems;
+
+__device__ __forceinline__ uint32_t warp_incl(uint32_t x)
+{
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int o = 16; o; o >>= 1) t = max(t, __shfl_xor_sync(0xffffffffu, t, o));
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = t;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    return x;
+}
+
+// the block's exclusive scan of one value per thread (kScanThreads of them),
+// plus the sum of the tiles before this one; *total: this prefix + the tile
+__device__ __forceinline__ uint32_t scan_tile(uint32_t x, int64_t tile, unsigned long long* st, uint32_t* total,
+                                              bool* ok)
+{
+    __shared__ uint32_t wsum[kScanThreads / 32];
+    __shared__ uint32_t pre_sh;
+    __shared__ bool ok_sh;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint32_t incl = warp_incl(x);
+    if (lane == 31) wsum[w] = incl;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 1; k < kCountThreads / 32; k++) t = max(t, wmax[k]);
-        atomicMax(depth, t);
+    uint32_t before = 0, all = 0;
+#pragma unroll
+    for (int k = 0; k < kScanThreads / 32; k++) {
+        if (k < w) before += wsum[k];
+        all += wsum[k];
     }
-}
-
-__global__ void k_check_capacity(const uint32_t* __restrict__ m_total, Info* info)
-{
-    const int64_t M = *m_total;
-    info->M = M;
-    if (M > info->cap_m) atomicOr(&info->err, kErrCapacity);
-}
-
-__global__ void k_emit_preorder(const int8_t* __restrict__ delta, const uint32_t* __restrict__ nstart,
-                                const uint32_t* __restrict__ prepos, int64_t n, const Info* info,
-                                uint32_t* __restrict__ pre_level, uint32_t* __restrict__ pre_first,
-                                uint32_t* __restrict__ iota)
-{
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n || capacity_failed(info)) return;
-    const uint32_t c = nstart[s], p = prepos[s];
-    const int l0 = delta[s] + 1;
-    for (uint32_t k = 0; k < c; k++) {
-        pre_level[p + k] = (uint32_t)(l0 + (int)k);
-        pre_first[p + k] = (uint32_t)s;
-        iota[p + k] = p + k;
-    }
-}
-
-__global__ void k_inverse_perm(const uint32_t* __restrict__ perm, const Info* info, uint32_t* __restrict__ inv)
-{
-    if (capacity_failed(info)) return;
-    const int64_t M = info->M;
-    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < M; b += (int64_t)gridDim.x * blockDim.x)
-        inv[perm[b]] = (uint32_t)b;
-}
-
-// first index e in [lo, hi) with (keys[e] >> sh) > pfx, or hi
-__device__ __forceinline__ int64_t run_end(const uint64_t* __restrict__ keys, int64_t lo, int64_t hi,
-                                           int sh, uint64_t pfx)
-{
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if ((keys[mid] >> sh) > pfx) hi = mid;
-        else lo = mid + 1;
-    }
-    return lo;
-}
-
-__global__ void k_node_finalize(const uint64_t* __restrict__ keys, const int8_t* __restrict__ top,
-                                const uint32_t* __restrict__ sys_of, const SysParams* __restrict__ sysp,
-                                const uint32_t* __restrict__ bfs_level, const uint32_t* __restrict__ bfs_pre,
-                                const uint32_t* __restrict__ pre_first, const uint32_t* __restrict__ bfs_of_pre,
-                                const Info* info, NodeTables nt)
-{
-    if (capacity_failed(info)) return;
-    const int64_t M = info->M;
-    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < M; b += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t p = bfs_pre[b];
-        const int l = (int)bfs_level[b];
-        const int64_t s = pre_first[p];
-        const uint32_t sy = sys_of[s];
-        const int64_t send = sysp[sy].end;
-        const int sh = 3 * (kMaxLevel - l);
-        const uint64_t pfx = (l == 0) ? 0ull : (keys[s] >> sh);
-        const int64_t e = (l == 0) ? send : run_end(keys, s + 1, send, sh, pfx);
-        int nch = 0;
-        int32_t cf = -1;
-        if (l < (int)top[s]) {
-            cf = (int32_t)bfs_of_pre[p + 1];
-            const int shc = sh - 3;
-            int64_t c = s;
-            while (c < e) {
-                const uint64_t cp = keys[c] >> shc;
-                c = run_end(keys, c + 1, e, shc, cp);
-                nch++;
-            }
+    if (w == 0) {
+        bool good;
+        const uint32_t pre = tile_prefix(st, tile, all, &good);
+        if (lane == 0) {
+            pre_sh = pre;
+            ok_sh = good;
         }
-        nt.b[b] = make_int4((int)s, (int)(e - s), cf, l | (nch << 8));
-        const uint32_t ix = compact3(pfx >> 2), iy = compact3(pfx >> 1), iz = compact3(pfx);
-        const int c1 = 1 << (kMaxLevel - l);
-        nt.c[b] = make_int4((int)(2 * ix + 1) * c1, (int)(2 * iy + 1) * c1, (int)(2 * iz + 1) * c1, (int)sy);
     }
+    __syncthreads();
+    *total = pre_sh + all;
+    *ok = ok_sh;
+    return pre_sh + before + incl - x;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_levels(uint32_t* __restrict__ cnt, int64_t ncnt,
+                                                              unsigned long long* st, uint32_t* counter, int64_t cap_m,
+                                                              Info* info)
+{
+    __shared__ int tile_sh;
+    if (threadIdx.x == 0) tile_sh = (int)atomicAdd(counter, 1u);
+    __syncthreads();
+    const int64_t tile = tile_sh, t0 = tile * kScanTile + (int64_t)threadIdx.x * kScanItems;
+    uint32_t v[kScanItems], sum = 0;
+#pragma unroll
+    for (int i = 0; i < kScanItems; i++) {
+        v[i] = t0 + i < ncnt ? cnt[t0 + i] : 0u;
+        sum += v[i];
+    }
+    uint32_t total;
+    bool ok;
+    uint32_t e = scan_tile(sum, tile, st, &total, &ok);
+#pragma unroll
+    for (int i = 0; i < kScanItems; i++) {
+        if (t0 + i < ncnt) cnt[t0 + i] = e;
+        e += v[i];
+    }
+    if (threadIdx.x == 0) {
+        if (!ok) atomicOr(&info->err, kErrWorkLoop | kErrCapacity);
+        if (tile == gridDim.x - 1) {
+            info->M = total;
+            if (cap_m >= 0 && (int64_t)total > cap_m) atomicOr(&info->err, kErrCapacity);
+        }
+    }
+}
+
+// The node records of every body of a block: (s, l) for delta < l <= top, at
+// place offs[l][block] + its rank among the block's starts of level l.  Its
+// first child is (s, l + 1); its parent the last node of level l - 1 that
+// starts at or before s.  fam = 1 marks a node that follows a sibling (the
+// topmost one starting at its body), so the children of a cell are its first
+// child and the marked nodes right after it.  Counts follow bottom-up.
+__global__ void __launch_bounds__(kNodeBlock) k_emit_nodes(const uint64_t* __restrict__ keys,
+                                                           const int8_t* __restrict__ delta,
+                                                           const int8_t* __restrict__ top,
+                                                           const uint32_t* __restrict__ sys_of, int64_t n,
+                                                           const uint32_t* __restrict__ offs, const Info* info,
+                                                           uint32_t* __restrict__ lstart, NodeTables nt)
+{
+    if (capacity_failed(info)) return;
+    __shared__ uint32_t wc[kNodeBlock / 32][kLevels];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u, le = lt | (1u << lane);
+    const int64_t s = (int64_t)blockIdx.x * kNodeBlock + threadIdx.x;
+    const int d = s < n ? delta[s] : 0, t = s < n ? top[s] : -1;
+    if (blockIdx.x == 0 && threadIdx.x <= kLevels)  // the first node of each level
+        lstart[threadIdx.x] = threadIdx.x < kLevels ? offs[(int64_t)threadIdx.x * gridDim.x] : (uint32_t)info->M;
+    uint32_t mine = 0;
+#pragma unroll
+    for (int l = 0; l < kLevels; l++) {
+        const unsigned m = __ballot_sync(0xffffffffu, d < l && l <= t);
+        if (lane == l) mine = __popc(m);
+    }
+    if (lane < kLevels) wc[w][lane] = mine;
+    __syncthreads();
+    if (threadIdx.x < kLevels) {
+        uint32_t run = offs[(int64_t)threadIdx.x * gridDim.x + blockIdx.x];
+        for (int k = 0; k < kNodeBlock / 32; k++) {
+            const uint32_t c = wc[k][threadIdx.x];
+            wc[k][threadIdx.x] = run;
+            run += c;
+        }
+    }
+    __syncthreads();
+    const int lhi = __reduce_max_sync(0xffffffffu, t);  // no level of the warp above it
+    const int llo = __reduce_min_sync(0xffffffffu, t >= 0 ? d : kMaxLevel) + 1;
+    if (lhi < llo) return;
+    const uint64_t key = s < n ? keys[s] : 0ull;
+    const uint32_t sy = s < n ? sys_of[s] : 0u;
+    uint32_t before = llo > 0 ? wc[w][llo - 1] : 0u;  // nodes of the level above up to body s
+    bool had = false;
+    uint32_t pos = 0;
+    int32_t par = -1;
+    for (int l = llo; l <= lhi + 1; l++) {
+        const bool here = l < kLevels && d < l && l <= t;
+        const unsigned m = __ballot_sync(0xffffffffu, here);
+        const uint32_t base = l < kLevels ? wc[w][l] : 0u;
+        const uint32_t p = base + __popc(m & lt);
+        if (had) {  // node (s, l - 1), whose first child is (s, l) if that exists
+            const int lv = l - 1, sh = 3 * (kMaxLevel - lv);
+            const uint64_t pfx = lv == 0 ? 0ull : (key >> sh);
+            const int c1 = 1 << (kMaxLevel - lv);
+            nt.b[pos] = make_int4((int)s, 0, here ? (int32_t)p : -1, lv);
+            nt.c[pos] = make_int4((int)(2 * compact3(pfx >> 2) + 1) * c1, (int)(2 * compact3(pfx >> 1) + 1) * c1,
+                                  (int)(2 * compact3(pfx) + 1) * c1, (int)sy);
+            nt.fam[pos] = lv == d + 1;
+            nt.parent[pos] = par;
+            nt.pend[pos] = 0u;
+        }
+        par = l > 0 ? (int32_t)before - 1 : -1;
+        before = base + __popc(m & le);
+        pos = p;
+        had = here;
+    }
+}
+
+// children of the cell whose first child is cf: cf and the marked nodes after it
+__device__ __forceinline__ int family(const uint8_t* __restrict__ fam, int64_t cf, int64_t M)
+{
+    unsigned marks = 0;
+#pragma unroll
+    for (int k = 1; k < 8; k++) marks |= (cf + k < M && fam[cf + k]) ? 1u << (k - 1) : 0u;
+    return __ffs(~marks);  // 1 + the run of marks
 }
 
 // ------------------------------------------------------------------ moments
@@ -442,9 +551,15 @@ __global__ void k_node_finalize(const uint64_t* __restrict__ keys, const int8_t*
 // they summed in FP64.  Leaves sum their bodies;
 // an internal cell combines its children: M = sum M_c,
 // com = sum M_c com_c / M, Q = sum Q_c + M_c dc dc^T with dc = com_c - com.
-// Leaves are done in one launch; internal cells level by level from the
-// deepest, one thread per cell of the level (cells of a level are contiguous
-// in breadth-first order), so every lane of a warp has a cell to do.
+// Leaves are done in one launch.  Internal cells follow level by level from
+// the deepest, one thread per cell of the level (cells of a level are
+// contiguous in breadth-first order), so every lane of a warp has a cell to
+// do; in small trees, where each of those launches is a few microseconds of
+// latency, the thread that completes a cell's last child computes the cell
+// in the leaves' launch (k_leaf_nodes): a build of 4096 / 100003 / 300000
+// bodies takes 174 / 204 / 238 us so, 187 / 220 / 247 with a launch per
+// level, but 370 against 366 us at 10^6 and 990 against 852 at 2^22, where
+// the fences of every climb cost more.
 __device__ __forceinline__ void cube_centre(const SysParams& P, int4 c, double* C)
 {
     const double u = 0.5 * P.h;
@@ -501,7 +616,7 @@ __device__ __forceinline__ void pair_quotient(const float (&Sh)[3], const float 
 // comf / Mf: the float roundings of com and M when the caller has
 // them (the same values, without the FP64 pipe's conversions)
 template <bool QUAD>
-__device__ void store_node(NodeTables& nt, int64_t v, double M, const double* com, const float* Q, const double* C,
+__device__ void store_node(const NodeTables& nt, int64_t v, double M, const double* com, const float* Q, const double* C,
                            const float* comf = nullptr, float Mf = 0.f)
 {
     nt.mass64[v] = M;
@@ -525,15 +640,103 @@ __device__ void store_node(NodeTables& nt, int64_t v, double M, const double* co
 // against C split into C_hi = fl(C) and C_lo = fl(C - C_hi): (x - C_hi) -
 // C_lo, within 2 FP32 roundings of x - C (the first subtraction is exact
 // unless |C| < 2 s, where its rounding is one of a number below 2 s).
-template <bool QUAD>
-__global__ void k_leaf_moments(const float4* __restrict__ body, const SysParams* __restrict__ sysp,
-                               const Info* info, NodeTables nt)
+// loads of what another thread of the same launch may have written (CG): past
+// the first-level cache, which other SMs' writes do not reach
+template <bool CG, typename T>
+__device__ __forceinline__ T ld(const T* p)
+{
+    return CG ? __ldcg(p) : *p;
+}
+
+// one internal cell v from its nch children: mass and
+// the sum of m x as float pairs, the children's pairs added by two_sum_acc
+// (each addition errs by at most about 2^-47 of the magnitudes added, so a
+// body's term collects at most depth x 2^-47 of relative error on its way
+// to the root: 1.5e-13 at depth 21), the centre of mass as their float-pair
+// quotient, both stored in FP64 too; second moments in FP32 by the parallel-axis rule
+// from the children's, Q_v = sum_c Q_c + m_c d_c d_c^T, d_c = com_c - com_v
+// formed in FP32 from the stored offsets of the centres of mass from their
+// cube centres, d_c = (a_c - a_v) + (k_c - k_v) u (k the integer cube
+// centres in units u = h/2, their difference exact).  The loads of all
+// children are issued before the first sum: in turn they were most of a
+// level's time.
+template <bool QUAD, bool CG>
+__device__ __forceinline__ void level_node(int64_t v, int4 pb, int nch, SysParams* __restrict__ sysp,
+                                           const NodeTables& nt)
+{
+    float4 h[8], lo[8];
+#pragma unroll
+    for (int k = 0; k < 8; k++)
+        if (k < nch) {
+            h[k] = ld<CG>(&nt.dsum[2 * ((int64_t)pb.z + k)]);
+            lo[k] = ld<CG>(&nt.dsum[2 * ((int64_t)pb.z + k) + 1]);
+        }
+    const int4 last = ld<CG>(&nt.b[pb.z + nch - 1]);
+    const int4 cc = nt.c[v];
+    SysParams& P = sysp[cc.w];
+    float mh = 0.f, ml = 0.f, Sh[3] = {0.f, 0.f, 0.f}, Sl[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 8; k++)
+        if (k < nch) {
+            two_sum_acc(mh, ml, h[k].x, lo[k].x);
+            two_sum_acc(Sh[0], Sl[0], h[k].y, lo[k].y);
+            two_sum_acc(Sh[1], Sl[1], h[k].z, lo[k].z);
+            two_sum_acc(Sh[2], Sl[2], h[k].w, lo[k].w);
+        }
+    const double m = widen(mh) + widen(ml);
+    double com[3];
+    float comf[3];
+    pair_quotient(Sh, Sl, mh, ml, com, comf);
+    nt.b[v] = make_int4(pb.x, last.x + last.y - pb.x, pb.z, (pb.w & 255) | (nch << 8));
+    nt.dsum[2 * v] = make_float4(mh, Sh[0], Sh[1], Sh[2]);
+    nt.dsum[2 * v + 1] = make_float4(ml, Sl[0], Sl[1], Sl[2]);
+    double C[3];
+    cube_centre(P, cc, C);
+    float Q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const float av[3] = {(float)(com[0] - C[0]), (float)(com[1] - C[1]), (float)(com[2] - C[2])};
+    const float uf = P.uf;
+    for (int k = 0; QUAD && k < nch; k++) {
+        const int64_t c = pb.z + k;
+        const float4 ac = ld<CG>(&nt.a[c]);
+        const int4 kc = nt.c[c];
+        const float mc = ac.w;
+        const float d[3] = {fmaf((float)(kc.x - cc.x), uf, ac.x - av[0]), fmaf((float)(kc.y - cc.y), uf, ac.y - av[1]),
+                            fmaf((float)(kc.z - cc.z), uf, ac.z - av[2])};
+        const float* qc = nt.quad + 6 * c;
+        Q[0] += fmaf(mc * d[0], d[0], ld<CG>(qc));
+        Q[1] += fmaf(mc * d[0], d[1], ld<CG>(qc + 1));
+        Q[2] += fmaf(mc * d[0], d[2], ld<CG>(qc + 2));
+        Q[3] += fmaf(mc * d[1], d[1], ld<CG>(qc + 3));
+        Q[4] += fmaf(mc * d[1], d[2], ld<CG>(qc + 4));
+        Q[5] += fmaf(mc * d[2], d[2], ld<CG>(qc + 5));
+    }
+    store_node<QUAD>(nt, v, m, com, Q, C, comf, mh + ml);
+    if ((pb.w & 255) == 0) P.msys = (float)m;  // a system's root
+}
+
+// Per node: a leaf's body count (its run of bodies) and moments; an internal
+// cell's number of children.  CLIMB: the thread that completes a cell's last
+// child computes the cell and goes on to its parent, so no launch per level
+// follows.
+template <bool QUAD, bool CLIMB>
+__global__ void k_leaf_nodes(const float4* __restrict__ body, const int8_t* __restrict__ delta, int64_t n,
+                             SysParams* __restrict__ sysp, const Info* info, NodeTables nt)
 {
     if (capacity_failed(info)) return;
     const int64_t M = info->M;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < M; v += (int64_t)gridDim.x * blockDim.x) {
-        const int4 b = nt.b[v];
-        if ((b.w >> 8) != 0) continue;  // internal
+        int4 b = nt.b[v];
+        const int l = b.w & 255;
+        if (b.z >= 0) {  // internal
+            if (!CLIMB) nt.b[v].w = l | (family(nt.fam, b.z, M) << 8);
+            continue;
+        }
+        // the leaf's run: bodies sharing l digits with their predecessor
+        int64_t e = (int64_t)b.x + 1;
+        while (e < n && delta[e] >= l) e++;
+        b.y = (int)(e - b.x);
+        b.w = l;
+        nt.b[v] = b;
         const int4 c = nt.c[v];
         double C[3];
         cube_centre(sysp[c.w], c, C);
@@ -560,8 +763,8 @@ __global__ void k_leaf_moments(const float4* __restrict__ body, const SysParams*
 #pragma unroll
             for (int a = 0; a < 3; a++) {
                 const float p = q.w * xs[a];
-                const float e = fmaf(q.w, xs[a], -p);  // q.w x = p + e exactly
-                two_sum_acc(Sh[a], Sl[a], p, e);
+                const float err = fmaf(q.w, xs[a], -p);  // q.w x = p + err exactly
+                two_sum_acc(Sh[a], Sl[a], p, err);
             }
             if (QUAD) {
                 const float dx = (q.x - Chi[0]) - Clo[0], dy = (q.y - Chi[1]) - Clo[1], dz = (q.z - Chi[2]) - Clo[2];
@@ -590,101 +793,60 @@ __global__ void k_leaf_moments(const float4* __restrict__ body, const SysParams*
             Q[5] = fmaf(-mf * ez, ez, QC[5]);
         }
         store_node<QUAD>(nt, v, m, com, Q, C, comf, mh + ml);
+        if (l == 0) sysp[c.w].msys = (float)m;  // a system's root
         nt.dsum[2 * v] = make_float4(mh, Sh[0], Sh[1], Sh[2]);
         nt.dsum[2 * v + 1] = make_float4(ml, Sl[0], Sl[1], Sl[2]);
+        if (CLIMB) {
+            for (int64_t u = v;;) {
+                const int32_t p = nt.parent[u];
+                if (p < 0) break;
+                const int4 pb = nt.b[p];  // (x, z and the level: written before this launch)
+                const int nch = family(nt.fam, pb.z, M);
+                __threadfence();  // this child's record before its arrival
+                if (atomicAdd(&nt.pend[p], 1u) + 1u < (uint32_t)nch) break;
+                __threadfence();  // the other children's arrivals before their records
+                level_node<QUAD, true>(p, pb, nch, sysp, nt);
+                u = p;
+            }
+        }
     }
-}
-
-// one internal cell v from its children (a leaf returns at once): mass and
-// the sum of m x as float pairs, the children's pairs added by two_sum_acc
-// (each addition errs by at most about 2^-47 of the magnitudes added, so a
-// body's term collects at most depth x 2^-47 of relative error on its way
-// to the root: 1.5e-13 at depth 21), the centre of mass as their float-pair
-// quotient, both stored in FP64 too; second moments in FP32 by the parallel-axis rule
-// from the children's, Q_v = sum_c Q_c + m_c d_c d_c^T, d_c = com_c - com_v
-// formed in FP32 from the stored offsets of the centres of mass from their
-// cube centres, d_c = (a_c - a_v) + (k_c - k_v) u (k the integer cube
-// centres in units u = h/2, their difference exact)
-template <bool QUAD>
-__device__ __forceinline__ void level_node(int64_t v, const SysParams* __restrict__ sysp, NodeTables& nt)
-{
-    const int4 pb = nt.b[v];
-    const int nch = pb.w >> 8;
-    if (nch == 0) return;  // leaf: done by k_leaf_moments
-    float mh = 0.f, ml = 0.f, Sh[3] = {0.f, 0.f, 0.f}, Sl[3] = {0.f, 0.f, 0.f};
-    for (int k = 0; k < nch; k++) {
-        const int64_t c = pb.z + k;
-        const float4 h = nt.dsum[2 * c], l = nt.dsum[2 * c + 1];
-        two_sum_acc(mh, ml, h.x, l.x);
-        two_sum_acc(Sh[0], Sl[0], h.y, l.y);
-        two_sum_acc(Sh[1], Sl[1], h.z, l.z);
-        two_sum_acc(Sh[2], Sl[2], h.w, l.w);
-    }
-    const double m = widen(mh) + widen(ml);
-    double com[3];
-    float comf[3];
-    pair_quotient(Sh, Sl, mh, ml, com, comf);
-    nt.dsum[2 * v] = make_float4(mh, Sh[0], Sh[1], Sh[2]);
-    nt.dsum[2 * v + 1] = make_float4(ml, Sl[0], Sl[1], Sl[2]);
-    const int4 cc = nt.c[v];
-    double C[3];
-    cube_centre(sysp[cc.w], cc, C);
-    float Q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const float av[3] = {(float)(com[0] - C[0]), (float)(com[1] - C[1]), (float)(com[2] - C[2])};
-    const float uf = sysp[cc.w].uf;
-    for (int k = 0; QUAD && k < nch; k++) {
-        const int64_t c = pb.z + k;
-        const float4 ac = nt.a[c];
-        const int4 kc = nt.c[c];
-        const float mc = ac.w;
-        const float d[3] = {fmaf((float)(kc.x - cc.x), uf, ac.x - av[0]), fmaf((float)(kc.y - cc.y), uf, ac.y - av[1]),
-                            fmaf((float)(kc.z - cc.z), uf, ac.z - av[2])};
-        const float* qc = nt.quad + 6 * c;
-        Q[0] += fmaf(mc * d[0], d[0], qc[0]);
-        Q[1] += fmaf(mc * d[0], d[1], qc[1]);
-        Q[2] += fmaf(mc * d[0], d[2], qc[2]);
-        Q[3] += fmaf(mc * d[1], d[1], qc[3]);
-        Q[4] += fmaf(mc * d[1], d[2], qc[4]);
-        Q[5] += fmaf(mc * d[2], d[2], qc[5]);
-    }
-    store_node<QUAD>(nt, v, m, com, Q, C, comf, mh + ml);
 }
 
 // internal cells of level `lev`: [level_start[lev], level_start[lev + 1])
 template <bool QUAD>
-__global__ void k_level_moments(int lev, const uint32_t* __restrict__ level_start,
-                                const SysParams* __restrict__ sysp, const Info* info, NodeTables nt)
+__global__ void k_level_moments(int lev, const uint32_t* __restrict__ level_start, SysParams* __restrict__ sysp,
+                                const Info* info, NodeTables nt)
 {
     if (capacity_failed(info)) return;
     const int64_t start = level_start[lev];
     const int64_t end = level_start[lev + 1];
     for (int64_t v = start + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < end;
-         v += (int64_t)gridDim.x * blockDim.x)
-        level_node<QUAD>(v, sysp, nt);
-}
-
-// every level from the deepest possible down to lev_lo, in one block: the
-// cells past the depth a captured step expects (normally none)
-template <bool QUAD>
-__global__ void __launch_bounds__(256) k_level_moments_deep(int lev_lo, const uint32_t* __restrict__ level_start,
-                                                             const SysParams* __restrict__ sysp, const Info* info,
-                                                             NodeTables nt)
-{
-    if (capacity_failed(info)) return;
-    for (int lev = kMaxLevel - 1; lev >= lev_lo; lev--) {
-        const int64_t start = level_start[lev];
-        const int64_t end = level_start[lev + 1];
-        for (int64_t v = start + threadIdx.x; v < end; v += blockDim.x) level_node<QUAD>(v, sysp, nt);
-        __syncthreads();
+         v += (int64_t)gridDim.x * blockDim.x) {
+        const int4 pb = nt.b[v];
+        if (pb.z >= 0) level_node<QUAD, false>(v, pb, pb.w >> 8, sysp, nt);
     }
 }
 
-// total mass of each system: its root's mass
-__global__ void k_sys_mass(SysParams* __restrict__ sysp, int nsys, const NodeTables nt, const Info* info)
+// levels lev_hi - 1 down to lev_lo in one block: those past the depth a
+// captured step expects (normally none), and the topmost, which hold few
+// cells
+template <bool QUAD>
+__global__ void __launch_bounds__(512) k_level_moments_block(int lev_hi, int lev_lo,
+                                                             const uint32_t* __restrict__ level_start,
+                                                             SysParams* __restrict__ sysp, const Info* info,
+                                                             NodeTables nt)
 {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsys || capacity_failed(info)) return;
-    sysp[s].msys = (float)nt.mass64[s];
+    if (capacity_failed(info)) return;
+    for (int lev = lev_hi - 1; lev >= lev_lo; lev--) {
+        const int64_t start = level_start[lev];
+        const int64_t end = level_start[lev + 1];
+        for (int64_t v = start + threadIdx.x; v < end; v += blockDim.x) {
+            const int4 pb = nt.b[v];
+            if (pb.z >= 0) level_node<QUAD, true>(v, pb, pb.w >> 8, sysp, nt);
+        }
+        __threadfence_block();
+        __syncthreads();
+    }
 }
 
 // ------------------------------------------------------------------ groups
@@ -696,8 +858,8 @@ __global__ void k_sys_mass(SysParams* __restrict__ sysp, int nsys, const NodeTab
 // thread).  A root holding at most gmax is one group.  Each group records a
 // reference cube (itself, the leaf it was cut from, or the common parent of
 // the packed children); the walk measures positions from that cube's centre.
-__global__ void k_group_marks(const Info* info, const NodeTables nt, int gmax, uint32_t* __restrict__ gflag,
-                              int32_t* __restrict__ gref_at)
+// gref_at[s] = the reference cube + 1 of the group that starts at body s (0: none)
+__global__ void k_group_marks(const Info* info, const NodeTables nt, int gmax, int32_t* __restrict__ gref_at)
 {
     if (capacity_failed(info)) return;
     const int64_t M = info->M;
@@ -705,59 +867,74 @@ __global__ void k_group_marks(const Info* info, const NodeTables nt, int gmax, u
         const int4 b = nt.b[v];
         const int nch = b.w >> 8;
         if (b.y <= gmax) {
-            if ((b.w & 255) == 0) {  // a root
-                gflag[b.x] = 1;
-                gref_at[b.x] = (int32_t)v;
-            }
+            if ((b.w & 255) == 0) gref_at[b.x] = (int32_t)v + 1;  // a root
             continue;
         }
         if (nch == 0) {
-            for (int s = 0; s < b.y; s += gmax) {
-                gflag[b.x + s] = 1;
-                gref_at[b.x + s] = (int32_t)v;
-            }
+            for (int s = 0; s < b.y; s += gmax) gref_at[b.x + s] = (int32_t)v + 1;
             continue;
         }
+        int2 kid[8];  // first body and bodies of each child, loaded together
+#pragma unroll
+        for (int k = 0; k < 8; k++)
+            if (k < nch) kid[k] = *reinterpret_cast<const int2*>(&nt.b[b.z + k]);
         int run_first = -1, run_count = 0, run_len = 0, run_only = -1;
-        for (int k = 0; k < nch; k++) {
-            const int c = b.z + k;
-            const int4 cb = nt.b[c];
-            if (cb.y > gmax || run_count + cb.y > gmax) {
-                if (run_len > 0) {
-                    gflag[run_first] = 1;
-                    gref_at[run_first] = run_len == 1 ? run_only : (int32_t)v;
-                }
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            if (k >= nch) break;
+            if (kid[k].y > gmax || run_count + kid[k].y > gmax) {
+                if (run_len > 0) gref_at[run_first] = (run_len == 1 ? run_only : (int32_t)v) + 1;
                 run_len = 0;
                 run_count = 0;
             }
-            if (cb.y > gmax) continue;
+            if (kid[k].y > gmax) continue;
             if (run_len == 0) {
-                run_first = cb.x;
-                run_only = c;
+                run_first = kid[k].x;
+                run_only = b.z + k;
             }
-            run_count += cb.y;
+            run_count += kid[k].y;
             run_len++;
         }
-        if (run_len > 0) {
-            gflag[run_first] = 1;
-            gref_at[run_first] = run_len == 1 ? run_only : (int32_t)v;
-        }
+        if (run_len > 0) gref_at[run_first] = (run_len == 1 ? run_only : (int32_t)v) + 1;
     }
 }
 
-__global__ void k_group_table(const uint32_t* __restrict__ gflag, const uint32_t* __restrict__ gscan,
-                              const int32_t* __restrict__ gref_at, int64_t n, const uint32_t* __restrict__ total,
-                              int32_t* __restrict__ gfirst, int32_t* __restrict__ gref, Info* info)
+// the marked bodies in order -> the group table, one pass
+__global__ void __launch_bounds__(kScanThreads) k_group_table(const int32_t* __restrict__ gref_at, int64_t n,
+                                                              unsigned long long* st, uint32_t* counter,
+                                                              int32_t* __restrict__ gfirst, int32_t* __restrict__ gref,
+                                                              Info* info)
 {
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s == 0) {
-        gfirst[*total] = (int32_t)n;
-        info->G = *total;
+    __shared__ int tile_sh;
+    __shared__ int32_t mark[kScanTile];
+    if (threadIdx.x == 0) tile_sh = (int)atomicAdd(counter, 1u);
+    __syncthreads();
+    const int64_t tile = tile_sh, t0 = tile * kScanTile;
+#pragma unroll
+    for (int i = 0; i < kScanItems; i++) {
+        const int p = i * kScanThreads + threadIdx.x;
+        mark[p] = t0 + p < n ? gref_at[t0 + p] : 0;
     }
-    if (s >= n || !gflag[s]) return;
-    const uint32_t g = gscan[s];
-    gfirst[g] = (int32_t)s;
-    gref[g] = gref_at[s];
+    __syncthreads();
+    uint32_t has = 0;  // which of the thread's kScanItems consecutive bodies start a group
+#pragma unroll
+    for (int i = 0; i < kScanItems; i++) has |= mark[threadIdx.x * kScanItems + i] ? 1u << i : 0u;
+    uint32_t total;
+    bool ok;
+    uint32_t g = scan_tile(__popc(has), tile, st, &total, &ok);
+    if (!ok) {
+        if (threadIdx.x == 0) atomicOr(&info->err, kErrWorkLoop | kErrCapacity);
+        return;
+    }
+    for (; has; has &= has - 1, g++) {
+        const int i = threadIdx.x * kScanItems + __ffs(has) - 1;
+        gfirst[g] = (int32_t)(t0 + i);
+        gref[g] = mark[i] - 1;
+    }
+    if (tile == gridDim.x - 1 && threadIdx.x == 0) {
+        gfirst[total] = (int32_t)n;
+        info->G = total;
+    }
 }
 
 // The groups ordered by the layout the walk gives them (group_class), the
@@ -938,77 +1115,93 @@ void launch_gather(const float* pos, const float* mass, const uint32_t* perm, in
     count_launches(1);
 }
 
-void launch_node_counts(const uint64_t* keys, const uint32_t* sys_of, int64_t n, int leaf_max, int8_t* w,
-                        int8_t* delta, int8_t* top, uint32_t* nstart, int32_t* depth, cudaStream_t s)
+int64_t level_counts_size(int64_t n) { return (int64_t)kLevels * ((n + kNodeBlock - 1) / kNodeBlock); }
+
+// words of the two single-pass scans' look-back: the levels' counts, then the
+// groups' marks, then two tile counters (all zeroed by the caller)
+namespace {
+int64_t scan_tiles(int64_t n) { return (n + kScanTile - 1) / kScanTile; }
+}  // namespace
+int64_t build_scan_words(int64_t n) { return scan_tiles(level_counts_size(n)) + scan_tiles(n) + 1; }
+
+void launch_node_levels(const uint64_t* keys, const uint32_t* sys_of, int64_t n, int leaf_max, int8_t* w,
+                        int8_t* delta, int8_t* top, int32_t* gref_at, uint32_t* cnt, unsigned long long* scan,
+                        int64_t cap_m, Info* info, cudaStream_t s)
 {
+    const unsigned nb = nblk(n, kNodeBlock);
     if (leaf_max <= kTileWindow) {
-        k_node_counts_tiled<<<nblk(n, kCountThreads), kCountThreads, 0, s>>>(keys, sys_of, n, leaf_max, delta, top,
-                                                                            nstart, depth);
+        k_node_levels_tiled<<<nb, kNodeBlock, 0, s>>>(keys, sys_of, n, leaf_max, delta, top, gref_at, cnt, &info->depth);
+        count_launches(1);
+    } else {
+        k_window<<<nblk(n, 256), 256, 0, s>>>(keys, sys_of, n, leaf_max, w);
+        k_node_levels<<<nb, kNodeBlock, 0, s>>>(keys, sys_of, w, n, leaf_max, delta, top, gref_at, cnt, &info->depth);
+        count_launches(2);
+    }
+    const int64_t nc = level_counts_size(n);
+    uint32_t* counters = reinterpret_cast<uint32_t*>(scan + build_scan_words(n) - 1);
+    k_scan_levels<<<(unsigned)scan_tiles(nc), kScanThreads, 0, s>>>(cnt, nc, scan, counters, cap_m, info);
+    count_launches(1);
+}
+
+void launch_emit_nodes(const uint64_t* keys, const int8_t* delta, const int8_t* top, const uint32_t* sys_of, int64_t n,
+                       const uint32_t* offs, const Info* info, uint32_t* lstart, NodeTables nt, cudaStream_t s)
+{
+    k_emit_nodes<<<nblk(n, kNodeBlock), kNodeBlock, 0, s>>>(keys, delta, top, sys_of, n, offs, info, lstart, nt);
+    count_launches(1);
+}
+
+void launch_moments(const float4* body, const int8_t* delta, int64_t n, int nsys, int64_t cap_m, int depth,
+                    int depth_hint, const uint32_t* level_start, SysParams* sysp, const Info* info, NodeTables nt,
+                    bool quad, cudaStream_t s)
+{
+    const unsigned g = gsgrid(cap_m, 128);
+    const bool climb = n <= kClimbBodies;
+    if (climb) {
+        if (quad) k_leaf_nodes<true, true><<<g, 128, 0, s>>>(body, delta, n, sysp, info, nt);
+        else k_leaf_nodes<false, true><<<g, 128, 0, s>>>(body, delta, n, sysp, info, nt);
         count_launches(1);
         return;
     }
-    k_window<<<nblk(n, 256), 256, 0, s>>>(keys, sys_of, n, leaf_max, w);
-    k_node_counts<<<nblk(n, 256), 256, 0, s>>>(keys, sys_of, w, n, leaf_max, delta, top, nstart, depth);
-    count_launches(2);
-}
-
-void launch_check_capacity(const uint32_t* m_total, Info* info, cudaStream_t s)
-{
-    k_check_capacity<<<1, 1, 0, s>>>(m_total, info);
-    count_launches(1);
-}
-
-void launch_emit_preorder(const int8_t* delta, const uint32_t* nstart, const uint32_t* prepos, int64_t n,
-                          const Info* info, uint32_t* pre_level, uint32_t* pre_first, uint32_t* iota, cudaStream_t s)
-{
-    k_emit_preorder<<<nblk(n, 256), 256, 0, s>>>(delta, nstart, prepos, n, info, pre_level, pre_first, iota);
-    count_launches(1);
-}
-
-void launch_inverse_perm(const uint32_t* perm, int64_t cap_m, const Info* info, uint32_t* inv, cudaStream_t s)
-{
-    k_inverse_perm<<<gsgrid(cap_m, 256), 256, 0, s>>>(perm, info, inv);
-    count_launches(1);
-}
-
-void launch_node_finalize(const uint64_t* keys, const int8_t* top, const uint32_t* sys_of, const SysParams* sysp,
-                          int64_t n, const uint32_t* bfs_level, const uint32_t* bfs_pre, const uint32_t* pre_first,
-                          const uint32_t* bfs_of_pre, int64_t cap_m, const Info* info, NodeTables nt, cudaStream_t s)
-{
-    (void)n;
-    k_node_finalize<<<gsgrid(cap_m, 128), 128, 0, s>>>(keys, top, sys_of, sysp, bfs_level, bfs_pre, pre_first,
-                                                       bfs_of_pre, info, nt);
-    count_launches(1);
-}
-
-void launch_moments(const float4* body, int64_t cap_m, int depth, int depth_hint, const uint32_t* level_start,
-                    const uint32_t* sys_of, const SysParams* sysp, const Info* info, NodeTables nt, bool quad,
-                    cudaStream_t s)
-{
-    (void)sys_of;
-    const unsigned g = gsgrid(cap_m, 128);
-    if (quad) k_leaf_moments<true><<<g, 128, 0, s>>>(body, sysp, info, nt);
-    else k_leaf_moments<false><<<g, 128, 0, s>>>(body, sysp, info, nt);
+    if (quad) k_leaf_nodes<true, false><<<g, 128, 0, s>>>(body, delta, n, sysp, info, nt);
+    else k_leaf_nodes<false, false><<<g, 128, 0, s>>>(body, delta, n, sysp, info, nt);
     count_launches(1);
     // the level launches take a small grid (4 blocks per SM): most levels
     // hold few internal cells, the launches past the tree's depth none, and a
     // large grid costs more to start than they work
     const unsigned glim = 4u * (unsigned)sm_count();
     const unsigned gl = g < glim ? g : glim;
+    auto block = [&](int hi, int lo) {
+        if (quad) k_level_moments_block<true><<<1, 512, 0, s>>>(hi, lo, level_start, sysp, info, nt);
+        else k_level_moments_block<false><<<1, 512, 0, s>>>(hi, lo, level_start, sysp, info, nt);
+        count_launches(1);
+    };
     int top = depth < 0 ? kMaxLevel : depth;
     if (depth < 0 && depth_hint >= 0 && depth_hint + 3 < kMaxLevel) {
         // depth unknown on the host (a captured step): the levels from the
         // expected depth + 3 down get a launch each, any deeper ones one block
         top = depth_hint + 3;
-        if (quad) k_level_moments_deep<true><<<1, 256, 0, s>>>(top, level_start, sysp, info, nt);
-        else k_level_moments_deep<false><<<1, 256, 0, s>>>(top, level_start, sysp, info, nt);
-        count_launches(1);
+        block(kMaxLevel, top);
     }
-    for (int lev = top - 1; lev >= 0; lev--) {
+    // the topmost levels, of at most 2048 cells each, share a block too
+    int few = 0;
+    while (few < top && ((int64_t)nsys << (3 * few)) <= 2048) few++;
+    if (few < 2) few = 0;
+    for (int lev = top - 1; lev >= few; lev--) {
         if (quad) k_level_moments<true><<<gl, 128, 0, s>>>(lev, level_start, sysp, info, nt);
         else k_level_moments<false><<<gl, 128, 0, s>>>(lev, level_start, sysp, info, nt);
         count_launches(1);
     }
+    if (few) block(few, 0);
+}
+
+void launch_groups(int64_t cap_m, Info* info, const NodeTables nt, int gmax, int64_t n, int32_t* gref_at,
+                   unsigned long long* scan, int32_t* gfirst, int32_t* gref, cudaStream_t s)
+{
+    k_group_marks<<<gsgrid(cap_m, 128), 128, 0, s>>>(info, nt, gmax, gref_at);
+    uint32_t* counters = reinterpret_cast<uint32_t*>(scan + build_scan_words(n) - 1);
+    k_group_table<<<(unsigned)scan_tiles(n), kScanThreads, 0, s>>>(
+        gref_at, n, scan + scan_tiles(level_counts_size(n)), counters + 1, gfirst, gref, info);
+    count_launches(2);
 }
 
 size_t group_order_scratch() { return (size_t)kGroupClasses * kSplitBlocks; }
@@ -1019,27 +1212,6 @@ void launch_group_order(const int32_t* gfirst, const Info* info, int32_t* order,
     k_order_count<<<kSplitBlocks, kSplitThreads, 0, s>>>(gfirst, info, scratch);
     k_order_scatter<<<kSplitBlocks, kSplitThreads, 0, s>>>(gfirst, info, scratch, order, seg);
     count_launches(2);
-}
-
-void launch_sys_mass(SysParams* sysp, int nsys, const NodeTables nt, const Info* info, cudaStream_t s)
-{
-    k_sys_mass<<<nblk(nsys, 128), 128, 0, s>>>(sysp, nsys, nt, info);
-    count_launches(1);
-}
-
-void launch_group_marks(int64_t cap_m, const Info* info, const NodeTables nt, int gmax, int64_t n, uint32_t* gflag,
-                        int32_t* gref_at, cudaStream_t s)
-{
-    cudaMemsetAsync(gflag, 0, n * sizeof(uint32_t), s);
-    k_group_marks<<<gsgrid(cap_m, 128), 128, 0, s>>>(info, nt, gmax, gflag, gref_at);
-    count_launches(1);
-}
-
-void launch_group_table(const uint32_t* gflag, const uint32_t* gscan, const int32_t* gref_at, int64_t n,
-                        const uint32_t* total, int32_t* gfirst, int32_t* gref, Info* info, cudaStream_t s)
-{
-    k_group_table<<<nblk(n, 256), 256, 0, s>>>(gflag, gscan, gref_at, n, total, gfirst, gref, info);
-    count_launches(1);
 }
 
 }  // namespace tc

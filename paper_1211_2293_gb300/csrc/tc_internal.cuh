@@ -53,7 +53,6 @@ struct Info {
     int32_t depth;     // deepest level of the forest
     int64_t M;         // number of nodes
     int64_t G;         // number of groups
-    int64_t cap_m;     // node table capacity (for the device-side check)
     uint32_t work[4];  // walk work-queue counters, one per launch of a force phase
     unsigned long long interactions;  // body-source interactions of the last walk
     unsigned long long cells;         // body-cell interactions (group size x accepted cells)
@@ -78,6 +77,9 @@ struct NodeTables {
     double* mass64;  // the bottom-up reduction's results in FP64
     double* com64;   // 3 per node
     float4* dsum;    // 2 per node: the bottom-up sums {m, m x} as float pairs, hi parts then lo parts
+    int32_t* parent; // -1 for a root
+    uint8_t* fam;    // 1: the node follows a sibling (its predecessor in the table)
+    uint32_t* pend;  // children of an internal cell that are done (bottom-up in one launch)
 };
 
 // scratch of the radix sort / scans
@@ -88,7 +90,6 @@ struct SortBufs {
     unsigned long long* status;      // look-back words, passes x tiles x 256
     uint32_t* tiles;                 // tile counters, one per pass
     int32_t* err;                    // device error word (bounded look-back)
-    uint32_t* blocksum;              // scan partials
     // a sort of the keys' top bits only: the starts of runs of equal top bits
     // longer than the per-thread completion takes (capacity run_cap), their count
     int64_t* runs = nullptr;
@@ -108,12 +109,6 @@ int sm_count();
 // records the reason of a failure outside any context (tc_last_error(NULL))
 void set_thread_error(const char* msg);
 
-// exclusive scan of n uint32 values into out (out may alias in), total to
-// *total_dev (device pointer, nullable)
-void scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* total_dev,
-              uint32_t* blocksum, cudaStream_t s);
-int64_t scan_blocksum_size(int64_t n);
-
 // Stable LSD radix sort of (key, val) by bits [0, nbits) of key, then (if
 // sys_bits > 0) by the system of each value's body, sys_of[val], so the
 // result is ordered by (system, key).  Afterwards b.ghist[p * 256 + d] is
@@ -129,10 +124,6 @@ void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int nbits, const 
                     int sys_bits, SortBufs& b, cudaStream_t s, int low_bit = 0, int64_t run_max = kSortRunMax);
 constexpr int64_t kSortRunMaxSynced = 1024;  // a synchronised build re-sorts every digit past this
 constexpr int kSortMarginLevels = 2;  // levels below the last synchronised depth a step's sort orders
-// The same for 32-bit keys when the item count is only known on the device:
-// n_cap bounds it, *n_dev (device) holds it.
-void radix_sort_u32(uint32_t* keys, uint32_t* vals, int64_t n_cap, const int64_t* n_dev, int nbits,
-                    SortBufs& b, uint32_t* keys_alt32, cudaStream_t s);
 int64_t radix_tiles(int64_t n);  // tiles of one pass (status words: 256 per tile per pass)
 // self-test of the radix pass's bounded look-back (see tc_sort.cu)
 cudaError_t sort_wait_selftest(uint64_t* keys, uint32_t* vals, uint64_t* kout, uint32_t* vout,
@@ -149,28 +140,33 @@ void launch_keys(const float* pos, const float* mass, int64_t n, const uint32_t*
                  uint64_t* keys, uint32_t* idx, int32_t* err, cudaStream_t s);
 void launch_gather(const float* pos, const float* mass, const uint32_t* perm, int64_t n,
                    float4* body, cudaStream_t s);
-void launch_node_counts(const uint64_t* keys, const uint32_t* sys_of, int64_t n, int leaf_max, int8_t* w,
-                        int8_t* delta, int8_t* top, uint32_t* nstart, int32_t* depth, cudaStream_t s);
-void launch_check_capacity(const uint32_t* m_total, Info* info, cudaStream_t s);
-void launch_emit_preorder(const int8_t* delta, const uint32_t* nstart, const uint32_t* prepos,
-                          int64_t n, const Info* info, uint32_t* pre_level, uint32_t* pre_first,
-                          uint32_t* iota, cudaStream_t s);
-void launch_node_finalize(const uint64_t* keys, const int8_t* top, const uint32_t* sys_of,
-                          const SysParams* sysp, int64_t n, const uint32_t* bfs_level, const uint32_t* bfs_pre,
-                          const uint32_t* pre_first, const uint32_t* bfs_of_pre, int64_t cap_m, const Info* info,
-                          NodeTables nt, cudaStream_t s);
-void launch_inverse_perm(const uint32_t* perm, int64_t cap_m, const Info* info, uint32_t* inv, cudaStream_t s);
-// moments: leaves, then internal levels depth-1 .. 0 (depth < 0: the depth
-// is known on the device only; with depth_hint >= 0, the depth of an earlier
-// build, levels depth_hint+2 .. 0 get a launch each and any deeper ones one
-// block, else all 21 levels get a launch); each level reads its range on the
-// device: level_start[l] is the first node of level l (the level sort's
-// digit offsets; level_start[l+1] ends it)
-void launch_moments(const float4* body, int64_t cap_m, int depth, int depth_hint, const uint32_t* level_start,
-                    const uint32_t* sys_of, const SysParams* sysp, const Info* info, NodeTables nt, bool quad,
-                    cudaStream_t s);
-void launch_group_marks(int64_t cap_m, const Info* info, const NodeTables nt, int gmax, int64_t n,
-                        uint32_t* gflag, int32_t* gref_at, cudaStream_t s);
+// The levels of the cubes that start at each sorted body (delta < l <= top),
+// their number per level and block of bodies, and the exclusive scan of those
+// (level by level, so the nodes' breadth-first places); zeroes gref_at;
+// info->M = nodes, kErrCapacity where cap_m >= 0 and M exceeds it.  cnt:
+// level_counts_size(n) words; scan: build_scan_words(n) words, zeroed.
+int64_t level_counts_size(int64_t n);
+int64_t build_scan_words(int64_t n);
+void launch_node_levels(const uint64_t* keys, const uint32_t* sys_of, int64_t n, int leaf_max, int8_t* w,
+                        int8_t* delta, int8_t* top, int32_t* gref_at, uint32_t* cnt, unsigned long long* scan,
+                        int64_t cap_m, Info* info, cudaStream_t s);
+// the node records at those places (counts and children follow with the
+// moments) and lstart[0..22], the first node of each level
+void launch_emit_nodes(const uint64_t* keys, const int8_t* delta, const int8_t* top, const uint32_t* sys_of, int64_t n,
+                       const uint32_t* offs, const Info* info, uint32_t* lstart, NodeTables nt, cudaStream_t s);
+// counts, children and moments: the leaves, then the internal cells, in the
+// same launch for up to kClimbBodies bodies, else level by level from
+// depth - 1 (depth < 0: the depth is known on the device only; with
+// depth_hint >= 0, the depth of an earlier build, levels depth_hint + 2 .. 0
+// get a launch each and any deeper ones one block, else all 21 levels get a
+// launch); each level reads its range on the device.  Also each system's mass.
+constexpr int64_t kClimbBodies = 1 << 19;  // (both ways timed: tc_build.cu, "moments")
+void launch_moments(const float4* body, const int8_t* delta, int64_t n, int nsys, int64_t cap_m, int depth,
+                    int depth_hint, const uint32_t* level_start, SysParams* sysp, const Info* info, NodeTables nt,
+                    bool quad, cudaStream_t s);
+// the body groups: gfirst[0..G], gref[0..G), info->G
+void launch_groups(int64_t cap_m, Info* info, const NodeTables nt, int gmax, int64_t n, int32_t* gref_at,
+                   unsigned long long* scan, int32_t* gfirst, int32_t* gref, cudaStream_t s);
 // the groups by the walk's layout of their bodies (kGroupClasses of them),
 // the largest first, stable: order[0, G); seg[0..3] = the ranges of groups of
 // more than 64, 33 to 64 and up to 32 bodies in it; scratch holds
@@ -179,10 +175,6 @@ constexpr int kGroupClasses = 7;
 size_t group_order_scratch();
 void launch_group_order(const int32_t* gfirst, const Info* info, int32_t* order, int32_t* seg, int32_t* scratch,
                         cudaStream_t s);
-void launch_group_table(const uint32_t* gflag, const uint32_t* gscan, const int32_t* gref_at,
-                        int64_t n, const uint32_t* total, int32_t* gfirst, int32_t* gref, Info* info,
-                        cudaStream_t s);
-
 // walk + force
 struct WalkArgs {
     const float4* body;        // Morton order (x, y, z, m)
@@ -299,7 +291,6 @@ void launch_pair_order(int32_t* pb, int32_t* pv, int64_t np, uint64_t* keys, uin
 void launch_pair_labels(const int32_t* pb, const int32_t* pv, int64_t np, const float4* body, const uint32_t* sys_of,
                         const SysParams* sysp, NodeTables nt, float eps, float G, float* feat, float* lab,
                         float* fac, cudaStream_t s);
-void launch_sys_mass(SysParams* sysp, int nsys, const NodeTables nt, const Info* info, cudaStream_t s);
 // training data on the device: FP64 sums of x, x^2, t^2 (and F^2) over the
 // pairs (kMlpSums doubles), the model's maps from them (and the factor-weight
 // scale), normalised rows and scaled targets, loss weights (mode 0: check

@@ -7,14 +7,11 @@
 #include <mutex>
 
 #include "tc_internal.cuh"
+#include "tc_lookback.cuh"
 
 namespace tc {
 
 namespace {
-
-constexpr int kScanThreads = 256;
-constexpr int kScanItems = 16;
-constexpr int kScanTile = kScanThreads * kScanItems;  // 4096
 
 constexpr int kMaxDevices = 64;
 constexpr int kSortThreads = 256;
@@ -55,90 +52,6 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t& total,
     return r;
 }
 
-__global__ void k_scan_reduce(const uint32_t* __restrict__ in, int64_t n, uint32_t* __restrict__ bsum)
-{
-    __shared__ uint32_t sm[33];
-    int64_t base = (int64_t)blockIdx.x * kScanTile;
-    uint32_t s = 0;
-#pragma unroll
-    for (int i = 0; i < kScanItems; i++) {
-        int64_t k = base + (int64_t)i * kScanThreads + threadIdx.x;
-        if (k < n) s += in[k];
-    }
-    uint32_t tot;
-    block_excl_scan<kScanThreads>(s, tot, sm);
-    if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
-}
-
-// single block: exclusive scan of nb partials, in place; total -> *total
-__global__ void k_scan_top(uint32_t* __restrict__ bsum, int64_t nb, uint32_t* __restrict__ total)
-{
-    __shared__ uint32_t sm[33];
-    uint32_t carry = 0;
-    for (int64_t c = 0; c < nb; c += 1024) {
-        int64_t k = c + threadIdx.x;
-        uint32_t v = k < nb ? bsum[k] : 0;
-        uint32_t tot;
-        uint32_t e = block_excl_scan<1024>(v, tot, sm);
-        if (k < nb) bsum[k] = carry + e;
-        carry += tot;
-    }
-    if (threadIdx.x == 0 && total) *total = carry;
-}
-
-// PREFIX: the block's offset is the sum of the raw partials of the blocks
-// before it (no k_scan_top; the last block writes the total) -- for up to
-// kScanFusedBlocks blocks, where that sum is cheaper than another launch
-constexpr int64_t kScanFusedBlocks = 256;
-
-template <bool PREFIX>
-__global__ void k_scan_down(const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t n,
-                            const uint32_t* __restrict__ bsum, uint32_t* __restrict__ total)
-{
-    __shared__ uint32_t sm[33];
-    uint32_t off = 0;
-    if (PREFIX) {
-        uint32_t t = 0;
-        for (int64_t j = threadIdx.x; j < (int64_t)blockIdx.x; j += kScanThreads) t += bsum[j];
-        block_excl_scan<kScanThreads>(t, off, sm);  // off = the block-wide sum
-    } else {
-        off = bsum[blockIdx.x];
-    }
-    // the tile through shared memory: coalesced loads and stores, each
-    // thread scanning kScanItems consecutive items (padded every 32 words,
-    // so the threads' strided reads hit distinct banks)
-    __shared__ uint32_t tile[kScanTile + kScanTile / 32];
-    auto pad = [](int p) { return p + (p >> 5); };
-    const int64_t t0 = (int64_t)blockIdx.x * kScanTile;
-#pragma unroll
-    for (int i = 0; i < kScanItems; i++) {
-        const int p = i * kScanThreads + threadIdx.x;
-        tile[pad(p)] = t0 + p < n ? in[t0 + p] : 0u;
-    }
-    __syncthreads();
-    uint32_t v[kScanItems];
-    uint32_t s = 0;
-#pragma unroll
-    for (int i = 0; i < kScanItems; i++) {
-        v[i] = tile[pad(threadIdx.x * kScanItems + i)];
-        s += v[i];
-    }
-    uint32_t tot;
-    uint32_t e = block_excl_scan<kScanThreads>(s, tot, sm) + off;
-    if (PREFIX && total && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total = off + tot;
-#pragma unroll
-    for (int i = 0; i < kScanItems; i++) {
-        tile[pad(threadIdx.x * kScanItems + i)] = e;
-        e += v[i];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < kScanItems; i++) {
-        const int p = i * kScanThreads + threadIdx.x;
-        if (t0 + p < n) out[t0 + p] = tile[pad(p)];
-    }
-}
-
 // ------------------------------------------------------------------ radix sort
 // Onesweep LSD radix sort (8-bit digits): one kernel computes the global
 // digit histograms of every pass, one kernel turns them into exclusive
@@ -150,10 +63,6 @@ __global__ void k_scan_down(const uint32_t* __restrict__ in, uint32_t* __restric
 // counter in launch order, so a tile only ever waits for tiles that have
 // already started and publish before they look back themselves.  Every wait
 // is bounded; a tile that gives up sets the error word and writes nothing.
-constexpr unsigned long long kFlagAgg = 1ull << 62;
-constexpr unsigned long long kFlagPrefix = 2ull << 62;
-constexpr unsigned kLookbackMaxPolls = 1u << 22;  // about a second of polling
-
 template <typename K>
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist_all(const K* __restrict__ keys, int64_t n_host,
                                                                 const int64_t* __restrict__ n_dev, int npass,
@@ -384,27 +293,6 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_onesweep(const K* __restric
 
 }  // namespace
 
-int64_t scan_blocksum_size(int64_t n) { return (n + kScanTile - 1) / kScanTile + 1; }
-
-void scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* total_dev, uint32_t* blocksum,
-              cudaStream_t s)
-{
-    if (n <= 0) {
-        if (total_dev) cudaMemsetAsync(total_dev, 0, sizeof(uint32_t), s);
-        return;
-    }
-    int64_t nb = (n + kScanTile - 1) / kScanTile;
-    k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, blocksum);
-    if (nb <= kScanFusedBlocks) {
-        k_scan_down<true><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, blocksum, total_dev);
-        count_launches(2);
-        return;
-    }
-    k_scan_top<<<1, 1024, 0, s>>>(blocksum, nb, total_dev);
-    k_scan_down<false><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, blocksum, nullptr);
-    count_launches(3);
-}
-
 // ---------------------------------------------------- per-run completion
 // After passes over bits [low_bit, 63) only, items with equal top bits (and
 // equal system) sit together in value order; each such run is put in
@@ -615,12 +503,6 @@ void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int nbits, const 
     if (low_bit < 0 || low_bit >= nbits || (low_bit > 0 && (!b.runs || !b.nruns))) low_bit = 0;
     if (run_max < 1 || run_max > kSortRunMax) run_max = kSortRunMax;
     radix_sort_impl<uint64_t>(keys, vals, n, nullptr, nbits, sys_of, sys_bits, b, b.keys_alt, s, low_bit, run_max);
-}
-
-void radix_sort_u32(uint32_t* keys, uint32_t* vals, int64_t n_cap, const int64_t* n_dev, int nbits, SortBufs& b,
-                    uint32_t* keys_alt32, cudaStream_t s)
-{
-    radix_sort_impl<uint32_t>(keys, vals, n_cap, n_dev, nbits, nullptr, 0, b, keys_alt32, s);
 }
 
 }  // namespace tc
