@@ -109,13 +109,16 @@ struct tc_ctx {
     float* mlp_part = nullptr;    // per-warp partial gradients of a training step
     int64_t mlp_part_cap = 0;
     float* mlp_loss = nullptr;
+    float* mlp_sched = nullptr;   // learning rate and Adam bias corrections of every step
+    int64_t mlp_sched_cap = 0;
+    uint32_t* mlp_bar = nullptr;  // the training kernel's grid barrier
     unsigned long long* mlp_evals = nullptr;
     float* mlp_x = nullptr;       // scratch: features / normalised rows / outputs
     float* mlp_t = nullptr;
     float* mlp_w = nullptr;       // per-pair loss weights / label factors
     int32_t* mlp_idx = nullptr;
     float* mlp_raw = nullptr;     // scratch: raw features as given (n x 13)
-    double* mlp_sums = nullptr;   // FP64 sums of the training data (kMlpSums)
+    double* mlp_sums = nullptr;   // FP64 sums of the training data, per block
     float* mlp_wscale = nullptr;  // n / sum F^2 (factor weights)
     int32_t* mlp_bad = nullptr;   // a given loss weight was negative or not finite
     // learned correction evaluated after the split walk: the band-cell
@@ -1368,7 +1371,7 @@ int mlp_alloc(tc_ctx* c)
     TC_GROW(c, c->mlp_grad, kMlpNParamHost);
     TC_GROW(c, c->mlp_loss, 4);
     TC_GROW(c, c->mlp_evals, 1);
-    TC_GROW(c, c->mlp_sums, kMlpSums);
+    TC_GROW(c, c->mlp_sums, kMlpSums * kMlpSumBlocks);
     TC_GROW(c, c->mlp_wscale, 1);
     TC_GROW(c, c->mlp_bad, 1);
     TC_CUDA(c, cudaMemsetAsync(c->mlp_evals, 0, sizeof(*c->mlp_evals), c->stream));
@@ -1500,11 +1503,10 @@ int tc_mlp_loss_grad(tc_ctx* c, const float* X, const float* T, const float* W, 
     const float* wdev = nullptr;
     if ((r = mlp_weights(c, W, 0, n, &wdev))) return r;
     TC_CUDA(c, cudaMemsetAsync(c->mlp_loss, 0, sizeof(float), c->stream));
-    int64_t blocks = (n + 63) / 64;
-    if (blocks > 2 * c->num_sms) blocks = 2 * c->num_sms;
-    if ((r = mlp_part(c, (int)blocks))) return r;
+    const int blocks = mlp_train_blocks((int)n, 2 * c->num_sms);
+    if ((r = mlp_part(c, blocks))) return r;
     cudaError_t e = launch_mlp_train(c->mlp_x, c->mlp_t, wdev, c->mlp_idx, (int)n, c->mlp_dev, c->mlp_grad,
-                                     c->mlp_loss, c->mlp_part, (int)blocks, c->stream);
+                                     c->mlp_loss, c->mlp_part, blocks, c->stream);
     if (e != cudaSuccess) return fail(c, TC_ECUDA, "mlp training kernel: %s", cudaGetErrorString(e));
     if (grad) TC_CUDA(c, cudaMemcpyAsync(grad, c->mlp_grad, kMlpNParamHost * sizeof(float), cudaMemcpyDefault, c->stream));
     if (loss) TC_CUDA(c, cudaMemcpyAsync(loss, c->mlp_loss, sizeof(float), cudaMemcpyDefault, c->stream));
@@ -1530,9 +1532,8 @@ int tc_mlp_train(tc_ctx* c, const float* X, const float* T, const float* W, int3
     TC_CUDA(c, cudaMemcpyAsync(c->mlp_raw, X, n * 13 * sizeof(float), cudaMemcpyDefault, c->stream));
     TC_CUDA(c, cudaMemcpyAsync(c->mlp_t, T, n * 3 * sizeof(float), cudaMemcpyDefault, c->stream));
     if (W) TC_CUDA(c, cudaMemcpyAsync(c->mlp_w, W, n * sizeof(float), cudaMemcpyDefault, c->stream));
-    launch_mlp_sums(c->mlp_raw, c->mlp_t, weight_mode == TC_MLP_FACTORS ? c->mlp_w : nullptr, n, c->mlp_sums,
-                    c->stream);
-    launch_mlp_maps(c->mlp_sums, n, c->mlp_maps, c->mlp_wscale, c->stream);
+    launch_mlp_maps(c->mlp_raw, c->mlp_t, weight_mode == TC_MLP_FACTORS ? c->mlp_w : nullptr, n, c->mlp_sums,
+                    c->mlp_maps, c->mlp_wscale, c->stream);
     launch_mlp_init(c->mlp_params, seed, c->stream);
     launch_mlp_pack(c->mlp_params, c->mlp_maps, c->mlp_dev, c->stream);
     launch_mlp_rows(c->mlp_raw, c->mlp_t, n, c->mlp_maps, c->mlp_x, c->mlp_t, c->stream);
@@ -1557,35 +1558,44 @@ int tc_mlp_train(tc_ctx* c, const float* X, const float* T, const float* W, int3
     }
     TC_CUDA(c, cudaMemsetAsync(c->mlp_m, 0, kMlpNParamHost * sizeof(float), c->stream));
     TC_CUDA(c, cudaMemsetAsync(c->mlp_v, 0, kMlpNParamHost * sizeof(float), c->stream));
-    int step = 0;
-    const int64_t total_steps = (int64_t)epochs * ((n + batch - 1) / batch);
+    // every step's learning rate (cosine decay over all steps) and Adam bias
+    // corrections
+    const int64_t steps = (n + batch - 1) / batch, total_steps = epochs * steps;
+    const int blocks = mlp_train_blocks((int)std::min<int64_t>(batch, n), 2 * c->num_sms);
+    if ((r = mlp_part(c, blocks))) return r;
+    if (3 * total_steps > c->mlp_sched_cap) {
+        c->mlp_sched_cap = 0;
+        TC_GROW(c, c->mlp_sched, 3 * total_steps);
+        c->mlp_sched_cap = 3 * total_steps;
+    }
+    if (!c->mlp_bar) TC_GROW(c, c->mlp_bar, 1);
+    {
+        std::vector<float> sched(3 * total_steps);
+        for (int64_t k = 0; k < total_steps; k++) {
+            sched[3 * k] = (float)(0.5 * lr * (1.0 + std::cos(3.141592653589793 * (double)k / (double)total_steps)));
+            mlp_adam_corrections((int)(k + 1), &sched[3 * k + 1], &sched[3 * k + 2]);
+        }
+        TC_COPY(c, c->mlp_sched, sched.data(), sched.size() * sizeof(float));
+    }
     uint64_t key = seed;
     for (int ep = 0; ep < epochs; ep++) {
         // a fresh seeded permutation of the pairs each pass (on the device)
         key = key * 6364136223846793005ull + 1442695040888963407ull;
         launch_mlp_shuffle(n, key, c->mlp_idx, c->stream);
         TC_CUDA(c, cudaMemsetAsync(c->mlp_loss, 0, sizeof(float), c->stream));
-        int nb = 0;
-        for (int64_t b0 = 0; b0 < n; b0 += batch) {
-            const int B = (int)std::min<int64_t>(batch, n - b0);
-            int64_t blocks = (B + 63) / 64;
-            if (blocks > 2 * c->num_sms) blocks = 2 * c->num_sms;
-            if ((r = mlp_part(c, (int)blocks))) return r;
-            cudaError_t e = launch_mlp_train(c->mlp_x, c->mlp_t, wdev, c->mlp_idx + b0, B, c->mlp_dev,
-                                             c->mlp_grad, c->mlp_loss, c->mlp_part, (int)blocks, c->stream);
-            if (e != cudaSuccess) return fail(c, TC_ECUDA, "mlp training kernel: %s", cudaGetErrorString(e));
-            // cosine decay of the learning rate over all steps
-            const float lr_t = (float)(0.5 * lr * (1.0 + std::cos(3.141592653589793 * step / (double)total_steps)));
-            launch_adam(c->mlp_params, c->mlp_m, c->mlp_v, c->mlp_grad, kMlpNParamHost, lr_t, ++step, c->stream);
-            launch_mlp_pack(c->mlp_params, c->mlp_maps, c->mlp_dev, c->stream);
-            nb++;
-        }
+        cudaError_t e = launch_mlp_epoch(c->mlp_x, c->mlp_t, wdev, c->mlp_idx, (int)n, batch, blocks,
+                                         c->mlp_dev, c->mlp_params, c->mlp_m, c->mlp_v,
+                                         c->mlp_sched + 3 * steps * ep, c->mlp_part, c->mlp_loss, c->mlp_bar,
+                                         &c->info->err, c->stream);
+        if (e != cudaSuccess) return fail(c, TC_ECUDA, "mlp training kernel: %s", cudaGetErrorString(e));
         if (losses) {
             float l = 0.f;
             TC_COPY(c, &l, c->mlp_loss, sizeof(float));
-            losses[ep] = l / (float)nb;
+            losses[ep] = l / (float)steps;
         }
     }
+    launch_mlp_pack(c->mlp_params, c->mlp_maps, c->mlp_dev, c->stream);
+    TC_CUDA(c, cudaGetLastError());
     return check_device(c);
 }
 

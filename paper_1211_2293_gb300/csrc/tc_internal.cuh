@@ -263,14 +263,22 @@ double launch_force_probe(int blocks, int reps, float* out, cudaStream_t s);
 size_t mlp_dev_size();
 size_t mlp_frag_size();  // the inference part at the front of a device model
 size_t mlp_train_smem();
-// training step on B rows: per-warp partial gradients in part (at least
-// mlp_train_part_floats(blocks) floats), added in warp order into grad (the
-// packed gradient, overwritten) and the loss added to *loss
+// loss and gradient on B rows: per-warp partial gradients in part (at least
+// mlp_train_part_floats(max_blocks) floats), added in warp order into grad
+// (the packed gradient, overwritten) and the loss added to *loss
 int64_t mlp_train_part_floats(int blocks);
+int mlp_train_blocks(int B, int max_blocks);  // blocks of a mini-batch of B rows
 cudaError_t launch_mlp_train(const float* X, const float* T, const float* W, const int32_t* idx, int B,
-                             const void* model, float* grad, float* loss, float* part, int blocks, cudaStream_t s);
+                             const void* model, float* grad, float* loss, float* part, int max_blocks, cudaStream_t s);
+// one pass over n rows in mini-batches of `batch`, a cooperative launch; sched
+// holds three floats per step: the learning rate and Adam's bias corrections
+// (mlp_adam_corrections).  The model's copies for inference and W1's k-major
+// one are not kept up (launch_mlp_pack does).
+cudaError_t launch_mlp_epoch(const float* X, const float* T, const float* W, const int32_t* idx, int n, int batch,
+                             int max_blocks, void* model, float* params, float* mom, float* vel, const float* sched,
+                             float* part, float* loss, uint32_t* bar, int32_t* err, cudaStream_t s);
+void mlp_adam_corrections(int t, float* c1, float* c2);
 void launch_mlp_pack(const float* params, const float* maps, void* model, cudaStream_t s);
-void launch_adam(float* p, float* m, float* v, const float* g, int n, float lr, int t, cudaStream_t s);
 void launch_mlp_infer(const float* X, int64_t n, const void* model, float* Y, cudaStream_t s);
 // the learned correction evaluated after a split walk: every recorded band
 // cell's row at its group's centre through the network on the tensor cores,
@@ -291,14 +299,16 @@ void launch_pair_order(int32_t* pb, int32_t* pv, int64_t np, uint64_t* keys, uin
 void launch_pair_labels(const int32_t* pb, const int32_t* pv, int64_t np, const float4* body, const uint32_t* sys_of,
                         const SysParams* sysp, NodeTables nt, float eps, float G, float* feat, float* lab,
                         float* fac, cudaStream_t s);
-// training data on the device: FP64 sums of x, x^2, t^2 (and F^2) over the
-// pairs (kMlpSums doubles), the model's maps from them (and the factor-weight
-// scale), normalised rows and scaled targets, loss weights (mode 0: check
-// the given ones, mode 1: F^2 n / sum F^2; *bad = 1 for a non-finite or
-// negative weight), fresh parameters, and a seeded permutation of [0, n)
+// training data on the device: the model's maps (and the factor-weight scale
+// n / sum F^2) from FP64 sums of x, x^2, t^2 (and F^2) over the pairs (part:
+// kMlpSumBlocks x kMlpSums doubles), normalised rows and scaled targets, loss
+// weights (mode 0: check the given ones, mode 1: F^2 n / sum F^2; *bad = 1
+// for a non-finite or negative weight), fresh parameters, and a seeded
+// permutation of [0, n)
 constexpr int kMlpSums = 13 + 13 + 3 + 1;
-void launch_mlp_sums(const float* X, const float* T, const float* F, int64_t n, double* sums, cudaStream_t s);
-void launch_mlp_maps(const double* sums, int64_t n, float* maps, float* wscale, cudaStream_t s);
+constexpr int kMlpSumBlocks = 608;
+void launch_mlp_maps(const float* X, const float* T, const float* F, int64_t n, double* part, float* maps,
+                     float* wscale, cudaStream_t s);
 void launch_mlp_rows(const float* X, const float* T, int64_t n, const float* maps, float* rows, float* tout,
                      cudaStream_t s);
 void launch_mlp_weights(float* w, int64_t n, int mode, const float* wscale, int32_t* bad, cudaStream_t s);

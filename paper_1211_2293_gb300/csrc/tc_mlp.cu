@@ -12,8 +12,8 @@
 //   dY = 2 w (Y - T) / B,  dW3 = H2^T dY,  dH2 = (dY W3^T) * [H2 > 0],
 //   dW2 = H1^T dH2,      dH1 = (dH2 W2^T) * [H1 > 0],   dW1 = X^T dH1,
 // biases by column sums; the transposed operands are staged in shared
-// memory.  Gradients are summed per block in shared memory, then added to
-// the global gradient; a separate kernel applies Adam.
+// memory and read with ldmatrix.  Every warp sums its tiles' gradient into a
+// partial of its own; the partials are added in warp order.
 #include <cuda_bf16.h>
 
 #include "tc_internal.cuh"
@@ -34,46 +34,48 @@ constexpr int kGW3 = kGB2 + kMlpHid;                      // [64][8]
 constexpr int kGB3 = kGW3 + kMlpHid * kMlpOutPad;         // [8]
 constexpr int kGPad = kGB3 + kMlpOutPad;
 
-// per-warp staging (BF16): X[16][16], H1[16][64], H2[16][64], dY[16][8],
-// dH2[16][64], dH1[16][64]
+// per-warp staging (BF16): X, H1, H2, dY, dH2, dH1 of a 16-row tile, row-major;
+// rows of 48, 144 and 16 bytes, so that the eight rows an ldmatrix reads lie
+// in distinct banks
+constexpr int kLdX = 24, kLdH = 72, kLdY = 8;
 constexpr int kStX = 0;
-constexpr int kStH1 = kStX + 16 * kMlpInPad;
-constexpr int kStH2 = kStH1 + 16 * kMlpHid;
-constexpr int kStDY = kStH2 + 16 * kMlpHid;
-constexpr int kStDH2 = kStDY + 16 * kMlpOutPad;
-constexpr int kStDH1 = kStDH2 + 16 * kMlpHid;
-constexpr int kStSize = kStDH1 + 16 * kMlpHid;
+constexpr int kStH1 = kStX + 16 * kLdX;
+constexpr int kStH2 = kStH1 + 16 * kLdH;
+constexpr int kStDY = kStH2 + 16 * kLdH;
+constexpr int kStDH2 = kStDY + 16 * kLdY;
+constexpr int kStDH1 = kStDH2 + 16 * kLdH;
+constexpr int kStSize = kStDH1 + 16 * kLdH;
 
 // store a C tile (16 x 8, column block nb) into a row-major BF16 matrix
 __device__ __forceinline__ void store_c(__nv_bfloat16* M, int ld, int nb, const float (&c)[4], int lane)
 {
     const int g = lane >> 2, q = lane & 3;
-    M[g * ld + nb * 8 + 2 * q] = __float2bfloat16_rn(c[0]);
-    M[g * ld + nb * 8 + 2 * q + 1] = __float2bfloat16_rn(c[1]);
-    M[(g + 8) * ld + nb * 8 + 2 * q] = __float2bfloat16_rn(c[2]);
-    M[(g + 8) * ld + nb * 8 + 2 * q + 1] = __float2bfloat16_rn(c[3]);
+    *reinterpret_cast<uint32_t*>(&M[g * ld + nb * 8 + 2 * q]) = pack_bf16(c[0], c[1]);
+    *reinterpret_cast<uint32_t*>(&M[(g + 8) * ld + nb * 8 + 2 * q]) = pack_bf16(c[2], c[3]);
 }
 
 // A fragment of the transpose of a row-major BF16 matrix S (S is k x m:
 // A[m][k] = S[k][m]), m-tile mt, one 16-deep k-step at k = 0
 __device__ __forceinline__ void load_at(uint32_t (&a)[4], const __nv_bfloat16* S, int ld, int mt, int lane)
 {
-    const int g = lane >> 2, q = lane & 3;
-    const int m0 = mt * 16 + g, k0 = 2 * q;
-    a[0] = pack_raw(S[k0 * ld + m0], S[(k0 + 1) * ld + m0]);
-    a[1] = pack_raw(S[k0 * ld + m0 + 8], S[(k0 + 1) * ld + m0 + 8]);
-    a[2] = pack_raw(S[(k0 + 8) * ld + m0], S[(k0 + 9) * ld + m0]);
-    a[3] = pack_raw(S[(k0 + 8) * ld + m0 + 8], S[(k0 + 9) * ld + m0 + 8]);
+    // matrices: (k 0-7, m 0-7), (k 0-7, m 8-15), (k 8-15, m 0-7), (k 8-15, m 8-15)
+    const int i = lane >> 3, r = lane & 7;
+    const uint32_t p = (uint32_t)__cvta_generic_to_shared(&S[(r + 8 * (i >> 1)) * ld + mt * 16 + 8 * (i & 1)]);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
+                 : "r"(p)
+                 : "memory");
 }
 
 // B fragment of a row-major BF16 matrix S (B[k][n] = S[k][n]), k-step 0,
 // column block nb
 __device__ __forceinline__ void load_bs(uint32_t (&b)[2], const __nv_bfloat16* S, int ld, int nb, int lane)
 {
-    const int g = lane >> 2, q = lane & 3;
-    const int n = nb * 8 + g, k = 2 * q;
-    b[0] = pack_raw(S[k * ld + n], S[(k + 1) * ld + n]);
-    b[1] = pack_raw(S[(k + 8) * ld + n], S[(k + 9) * ld + n]);
+    const uint32_t p = (uint32_t)__cvta_generic_to_shared(&S[(lane & 15) * ld + nb * 8]);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+                 : "=r"(b[0]), "=r"(b[1])
+                 : "r"(p)
+                 : "memory");
 }
 
 // B fragment of the transpose of a k-major weight W[n][k] (B[k][n] = W[n][k]
@@ -81,25 +83,33 @@ __device__ __forceinline__ void load_bs(uint32_t (&b)[2], const __nv_bfloat16* S
 __device__ __forceinline__ void load_bt(uint32_t (&b)[2], const __nv_bfloat16* W, int ldk, int ks, int nb, int lane)
 {
     const int g = lane >> 2, q = lane & 3;
-    const int n = nb * 8 + g, k = ks * 16 + 2 * q;
-    b[0] = pack_raw(W[n * ldk + k], W[n * ldk + k + 1]);
-    b[1] = pack_raw(W[n * ldk + k + 8], W[n * ldk + k + 9]);
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(&W[(nb * 8 + g) * ldk + ks * 16 + 2 * q]);
+    b[0] = w[0];
+    b[1] = w[4];
 }
 
-// G is the warp's own partial gradient: each element always belongs to the
-// same lane, so the sums are plain additions in the warp's order of tiles
-__device__ __forceinline__ void add_c(float* G, int ld, int mt, int nb, const float (&c)[4], int lane)
+// a C tile into the warp's own partial gradient G: each element belongs to
+// the same lane for every tile, so the sums are plain additions in the warp's
+// order of tiles (the first tile's are stored)
+__device__ __forceinline__ void add_c(float* G, int ld, int mt, int nb, const float (&c)[4], int lane, bool first)
 {
     const int g = lane >> 2, q = lane & 3;
-    const int r = mt * 16 + g, col = nb * 8 + 2 * q;
-    G[r * ld + col] += c[0];
-    G[r * ld + col + 1] += c[1];
-    G[(r + 8) * ld + col] += c[2];
-    G[(r + 8) * ld + col + 1] += c[3];
+    float2* p0 = reinterpret_cast<float2*>(&G[(mt * 16 + g) * ld + nb * 8 + 2 * q]);
+    float2* p1 = reinterpret_cast<float2*>(&G[(mt * 16 + g + 8) * ld + nb * 8 + 2 * q]);
+    float2 a = make_float2(c[0], c[1]), b = make_float2(c[2], c[3]);
+    if (!first) {
+        const float2 x = *p0, y = *p1;
+        a.x += x.x;
+        a.y += x.y;
+        b.x += y.x;
+        b.y += y.y;
+    }
+    *p0 = a;
+    *p1 = b;
 }
 
 // column sums of a C tile over its 16 rows into G[col]
-__device__ __forceinline__ void colsum_c(float* G, int nb, const float (&c)[4], int lane)
+__device__ __forceinline__ void colsum_c(float* G, int nb, const float (&c)[4], int lane, bool first)
 {
     float s0 = c[0] + c[2], s1 = c[1] + c[3];
 #pragma unroll
@@ -108,16 +118,220 @@ __device__ __forceinline__ void colsum_c(float* G, int nb, const float (&c)[4], 
         s1 += __shfl_xor_sync(0xffffffffu, s1, o);
     }
     if (lane < 4) {
-        G[nb * 8 + 2 * lane] += s0;
-        G[nb * 8 + 2 * lane + 1] += s1;
+        float2* p = reinterpret_cast<float2*>(&G[nb * 8 + 2 * lane]);
+        float2 v = make_float2(s0, s1);
+        if (!first) {
+            const float2 x = *p;
+            v.x += x.x;
+            v.y += x.y;
+        }
+        *p = v;
     }
+}
+
+// what a lane holds of a tile's rows before the network runs: row r0 = tile x
+// 16 + g and r0 + 8, features 2q, 2q + 1, 2q + 8, 2q + 9 of each, the targets
+// of its output columns 2q, 2q + 1 and the loss weights (rows past B: zero)
+struct TrainRows {
+    float a[8];
+    float t[4];
+    float w[2];
+    bool v[2];
+};
+
+__device__ __forceinline__ TrainRows train_rows(const float* __restrict__ X, const float* __restrict__ T,
+                                                const float* __restrict__ W, const int32_t* __restrict__ idx, int B,
+                                                int tile, int lane)
+{
+    TrainRows r;
+    const int g = lane >> 2, q = lane & 3;
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        const int row = tile * 16 + g + 8 * h;
+        r.v[h] = row < B;
+        const int64_t i = r.v[h] ? idx[row] : 0;
+        const float2 z = make_float2(0.f, 0.f);
+        const float2 lo = r.v[h] ? *reinterpret_cast<const float2*>(&X[i * kMlpInPad + 2 * q]) : z;
+        const float2 hi = r.v[h] ? *reinterpret_cast<const float2*>(&X[i * kMlpInPad + 2 * q + 8]) : z;
+        r.a[2 * h] = lo.x;
+        r.a[2 * h + 1] = lo.y;
+        r.a[4 + 2 * h] = hi.x;
+        r.a[4 + 2 * h + 1] = hi.y;
+        r.t[2 * h] = r.v[h] && 2 * q < kMlpOut ? T[i * kMlpOut + 2 * q] : 0.f;
+        r.t[2 * h + 1] = r.v[h] && 2 * q + 1 < kMlpOut ? T[i * kMlpOut + 2 * q + 1] : 0.f;
+        r.w[h] = W && r.v[h] ? W[i] : 1.f;
+    }
+    return r;
+}
+
+// Forward and backward of one 16-row tile on one warp; the gradient into gs
+// (the warp's partial, kGPad floats), the weighted squared errors onto lsum.
+__device__ __forceinline__ void train_tile(const MlpDev& m, const TrainRows& r, __nv_bfloat16* st, float* gs, bool first,
+                                           float inv_b, float& lsum, int lane)
+{
+    const int g = lane >> 2, q = lane & 3;
+    uint32_t x[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) x[k] = pack_bf16(r.a[2 * k], r.a[2 * k + 1]);
+    // X tile, row-major, for dW1 = X^T dH1
+    *reinterpret_cast<uint32_t*>(&st[kStX + g * kLdX + 2 * q]) = x[0];
+    *reinterpret_cast<uint32_t*>(&st[kStX + (g + 8) * kLdX + 2 * q]) = x[1];
+    *reinterpret_cast<uint32_t*>(&st[kStX + g * kLdX + 2 * q + 8]) = x[2];
+    *reinterpret_cast<uint32_t*>(&st[kStX + (g + 8) * kLdX + 2 * q + 8]) = x[3];
+    float h1[8][4], h2[8][4], y[4];
+    mlp16(m.frag, x, h1, h2, y, lane);
+    // dY = 2 w (Y - T) / B on the 3 used columns of valid rows
+    float dy[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int h = k >> 1;
+        if (r.v[h] && 2 * q + (k & 1) < kMlpOut) {
+            const float e = y[k] - r.t[k];
+            lsum += r.w[h] * e * e;
+            dy[k] = 2.f * r.w[h] * e * inv_b;
+        }
+    }
+#pragma unroll
+    for (int nb = 0; nb < 8; nb++) {
+        store_c(st + kStH1, kLdH, nb, h1[nb], lane);
+        store_c(st + kStH2, kLdH, nb, h2[nb], lane);
+    }
+    store_c(st + kStDY, kLdY, 0, dy, lane);
+    __syncwarp();
+    colsum_c(gs + kGB3, 0, dy, lane, first);
+    // dW3 = H2^T dY
+    uint32_t by[2];
+    load_bs(by, st + kStDY, kLdY, 0, lane);
+#pragma unroll
+    for (int mt = 0; mt < 4; mt++) {
+        uint32_t a[4];
+        load_at(a, st + kStH2, kLdH, mt, lane);
+        float c[4] = {0.f, 0.f, 0.f, 0.f};
+        mma_bf16(c, a, by);
+        add_c(gs + kGW3, kMlpOutPad, mt, 0, c, lane, first);
+    }
+    // dH2 = dY W3^T * [H2 > 0]; dY padded to a 16-deep k-step with zeros
+    float dh2[8][4];
+    {
+        const uint32_t a[4] = {pack_bf16(dy[0], dy[1]), pack_bf16(dy[2], dy[3]), 0u, 0u};
+#pragma unroll
+        for (int nb = 0; nb < 8; nb++) {
+            const uint32_t b[2] = {*reinterpret_cast<const uint32_t*>(&m.w3[(nb * 8 + g) * kMlpOutPad + 2 * q]), 0u};
+            dh2[nb][0] = dh2[nb][1] = dh2[nb][2] = dh2[nb][3] = 0.f;
+            mma_bf16(dh2[nb], a, b);
+#pragma unroll
+            for (int e = 0; e < 4; e++) dh2[nb][e] = h2[nb][e] > 0.f ? dh2[nb][e] : 0.f;
+            store_c(st + kStDH2, kLdH, nb, dh2[nb], lane);
+        }
+    }
+    __syncwarp();
+    // dH1 = dH2 W2^T * [H1 > 0]
+    float dh1[8][4];
+#pragma unroll
+    for (int nb = 0; nb < 8; nb++) dh1[nb][0] = dh1[nb][1] = dh1[nb][2] = dh1[nb][3] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < 4; ks++) {
+        uint32_t a[4];
+        c_to_a(a, dh2[2 * ks], dh2[2 * ks + 1]);
+#pragma unroll
+        for (int nb = 0; nb < 8; nb++) {
+            uint32_t b[2];
+            load_bt(b, m.w2, kMlpHid, ks, nb, lane);
+            mma_bf16(dh1[nb], a, b);
+        }
+    }
+#pragma unroll
+    for (int nb = 0; nb < 8; nb++) {
+#pragma unroll
+        for (int e = 0; e < 4; e++) dh1[nb][e] = h1[nb][e] > 0.f ? dh1[nb][e] : 0.f;
+        store_c(st + kStDH1, kLdH, nb, dh1[nb], lane);
+    }
+#pragma unroll
+    for (int nb = 0; nb < 8; nb++) {
+        colsum_c(gs + kGB2, nb, dh2[nb], lane, first);
+        colsum_c(gs + kGB1, nb, dh1[nb], lane, first);
+    }
+    // dW2 = H1^T dH2
+#pragma unroll
+    for (int nb = 0; nb < 8; nb++) {
+        uint32_t b[2];
+        load_bs(b, st + kStDH2, kLdH, nb, lane);
+#pragma unroll
+        for (int mt = 0; mt < 4; mt++) {
+            uint32_t a[4];
+            load_at(a, st + kStH1, kLdH, mt, lane);
+            float c[4] = {0.f, 0.f, 0.f, 0.f};
+            mma_bf16(c, a, b);
+            add_c(gs + kGW2, kMlpHid, mt, nb, c, lane, first);
+        }
+    }
+    __syncwarp();
+    // dW1 = X^T dH1
+    {
+        uint32_t a[4];
+        load_at(a, st + kStX, kLdX, 0, lane);
+#pragma unroll
+        for (int nb = 0; nb < 8; nb++) {
+            uint32_t b[2];
+            load_bs(b, st + kStDH1, kLdH, nb, lane);
+            float c[4] = {0.f, 0.f, 0.f, 0.f};
+            mma_bf16(c, a, b);
+            add_c(gs + kGW1, kMlpHid, 0, nb, c, lane, first);
+        }
+    }
+    __syncwarp();
+}
+
+// blocks of a mini-batch of B rows (one warp per 16 rows, at most max_blocks),
+// and the warps of them that have a tile
+__host__ __device__ __forceinline__ int train_blocks(int B, int max_blocks)
+{
+    const int b = (B + 16 * kTrainWarps - 1) / (16 * kTrainWarps);
+    return b < max_blocks ? b : max_blocks;
+}
+__device__ __forceinline__ int train_warps(int B, int blocks)
+{
+    const int t = (B + 15) / 16;
+    return t < blocks * kTrainWarps ? t : blocks * kTrainWarps;
+}
+
+// the tiles of a mini-batch on this warp; r: its first tile's rows
+__device__ __forceinline__ void train_warp(const MlpDev& m, TrainRows r, const float* __restrict__ X,
+                                           const float* __restrict__ T, const float* __restrict__ W,
+                                           const int32_t* __restrict__ idx, int B, int blocks, __nv_bfloat16* st,
+                                           float* __restrict__ part, float* __restrict__ lpart, int lane)
+{
+    const int gw = blockIdx.x * kTrainWarps + (threadIdx.x >> 5);
+    const int ntiles = (B + 15) / 16;
+    if (gw >= ntiles) return;
+    const float inv_b = 1.0f / (float)B;
+    float* gs = part + (int64_t)gw * kGPad;
+    float lsum = 0.f;
+    for (int tile = gw; tile < ntiles; tile += blocks * kTrainWarps) {
+        if (tile != gw) r = train_rows(X, T, W, idx, B, tile, lane);
+        train_tile(m, r, st, gs, tile == gw, inv_b, lsum, lane);
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+    if (lane == 0) lpart[gw] = lsum * inv_b;
+}
+
+__device__ __forceinline__ void load_model(MlpDev& m, const MlpDev* __restrict__ model)
+{
+    static_assert(sizeof(MlpDev) % 16 == 0, "the model is copied in 16-byte chunks");
+    for (int i = threadIdx.x; i < (int)(sizeof(MlpDev) / 16); i += blockDim.x)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(reinterpret_cast<uint4*>(&m) + i)),
+                     "l"(reinterpret_cast<const uint4*>(model) + i)
+                     : "memory");
+    asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // X: n x 16 normalised features (FP32, padding zero); T: n x 3 scaled
 // targets; W: n weights (nullable); idx: the batch's row indices (B of
 // them).  Every warp sums its tiles' gradient into its own partial (part,
-// kGPad floats per warp of the grid) and its loss into lpart; k_grad_reduce
-// adds the partials in warp order, so a training run repeats bit for bit.
+// kGPad floats per warp) and its loss into lpart; the partials are added in
+// warp order, so a training run repeats bit for bit.
 __global__ void __launch_bounds__(kTrainWarps * 32) k_mlp_train(const float* __restrict__ X,
                                                                  const float* __restrict__ T,
                                                                  const float* __restrict__ W,
@@ -127,180 +341,209 @@ __global__ void __launch_bounds__(kTrainWarps * 32) k_mlp_train(const float* __r
 {
     extern __shared__ __align__(16) unsigned char smem[];
     MlpDev& m = *reinterpret_cast<MlpDev*>(smem);
-    __nv_bfloat16* stage = reinterpret_cast<__nv_bfloat16*>(smem + sizeof(MlpDev));
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __nv_bfloat16* st = stage + w * kStSize;
-    float* gs = part + ((int64_t)blockIdx.x * kTrainWarps + w) * kGPad;  // this warp's partial
-    for (int i = threadIdx.x; i < (int)(sizeof(MlpDev) / 4); i += blockDim.x)
-        reinterpret_cast<uint32_t*>(&m)[i] = reinterpret_cast<const uint32_t*>(model)[i];
-    for (int i = lane; i < kGPad; i += 32) gs[i] = 0.f;
+    __nv_bfloat16* st = reinterpret_cast<__nv_bfloat16*>(smem + sizeof(MlpDev)) + (threadIdx.x >> 5) * kStSize;
+    const int lane = threadIdx.x & 31;
+    const TrainRows r = train_rows(X, T, W, idx, B, blockIdx.x * kTrainWarps + (threadIdx.x >> 5), lane);
+    load_model(m, model);
     __syncthreads();
-    const int g = lane >> 2, q = lane & 3;
-    const float inv_b = 1.0f / (float)B;
-    float lsum = 0.f;
-    const int ntiles = (B + 15) / 16;
-    for (int tile = blockIdx.x * kTrainWarps + w; tile < ntiles; tile += gridDim.x * kTrainWarps) {
-        // rows of this tile (a row past B is all zero and has zero gradient)
-        const int r0 = tile * 16 + g, r1 = r0 + 8;
-        const bool v0 = r0 < B, v1 = r1 < B;
-        const int64_t i0 = v0 ? idx[r0] : 0, i1 = v1 ? idx[r1] : 0;
-        uint32_t x[4];
-        {
-            float a0 = v0 ? X[i0 * kMlpInPad + 2 * q] : 0.f, a1 = v0 ? X[i0 * kMlpInPad + 2 * q + 1] : 0.f;
-            float a2 = v1 ? X[i1 * kMlpInPad + 2 * q] : 0.f, a3 = v1 ? X[i1 * kMlpInPad + 2 * q + 1] : 0.f;
-            float a4 = v0 ? X[i0 * kMlpInPad + 2 * q + 8] : 0.f, a5 = v0 ? X[i0 * kMlpInPad + 2 * q + 9] : 0.f;
-            float a6 = v1 ? X[i1 * kMlpInPad + 2 * q + 8] : 0.f, a7 = v1 ? X[i1 * kMlpInPad + 2 * q + 9] : 0.f;
-            x[0] = pack_bf16(a0, a1);
-            x[1] = pack_bf16(a2, a3);
-            x[2] = pack_bf16(a4, a5);
-            x[3] = pack_bf16(a6, a7);
-            // X tile, row-major, for dW1 = X^T dH1
-            st[kStX + g * 16 + 2 * q] = __float2bfloat16_rn(a0);
-            st[kStX + g * 16 + 2 * q + 1] = __float2bfloat16_rn(a1);
-            st[kStX + (g + 8) * 16 + 2 * q] = __float2bfloat16_rn(a2);
-            st[kStX + (g + 8) * 16 + 2 * q + 1] = __float2bfloat16_rn(a3);
-            st[kStX + g * 16 + 2 * q + 8] = __float2bfloat16_rn(a4);
-            st[kStX + g * 16 + 2 * q + 9] = __float2bfloat16_rn(a5);
-            st[kStX + (g + 8) * 16 + 2 * q + 8] = __float2bfloat16_rn(a6);
-            st[kStX + (g + 8) * 16 + 2 * q + 9] = __float2bfloat16_rn(a7);
-        }
-        float h1[8][4], h2[8][4], y[4];
-        mlp16(m, x, h1, h2, y, lane);
-        // dY = 2 w (Y - T) / B on the 3 used columns of valid rows
-        float dy[4] = {0.f, 0.f, 0.f, 0.f};
-        {
-            const int c0 = 2 * q, c1 = 2 * q + 1;
-            const float w0 = (W && v0) ? W[i0] : 1.f, w1 = (W && v1) ? W[i1] : 1.f;
-            if (v0 && c0 < 3) { const float e = y[0] - T[i0 * 3 + c0]; lsum += w0 * e * e; dy[0] = 2.f * w0 * e * inv_b; }
-            if (v0 && c1 < 3) { const float e = y[1] - T[i0 * 3 + c1]; lsum += w0 * e * e; dy[1] = 2.f * w0 * e * inv_b; }
-            if (v1 && c0 < 3) { const float e = y[2] - T[i1 * 3 + c0]; lsum += w1 * e * e; dy[2] = 2.f * w1 * e * inv_b; }
-            if (v1 && c1 < 3) { const float e = y[3] - T[i1 * 3 + c1]; lsum += w1 * e * e; dy[3] = 2.f * w1 * e * inv_b; }
-        }
-        for (int nb = 0; nb < 8; nb++) {
-            store_c(st + kStH1, kMlpHid, nb, h1[nb], lane);
-            store_c(st + kStH2, kMlpHid, nb, h2[nb], lane);
-        }
-        store_c(st + kStDY, kMlpOutPad, 0, dy, lane);
-        __syncwarp();
-        colsum_c(gs + kGB3, 0, dy, lane);
-        // dW3 = H2^T dY
-        for (int mt = 0; mt < 4; mt++) {
-            uint32_t a[4], b[2];
-            load_at(a, st + kStH2, kMlpHid, mt, lane);
-            load_bs(b, st + kStDY, kMlpOutPad, 0, lane);
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
-            mma_bf16(c, a, b);
-            add_c(gs + kGW3, kMlpOutPad, mt, 0, c, lane);
-        }
-        // dH2 = dY W3^T * [H2 > 0]; dY padded to a 16-deep k-step with zeros
-        float dh2[8][4];
-        {
-            uint32_t a[4];
-            a[0] = pack_bf16(dy[0], dy[1]);
-            a[1] = pack_bf16(dy[2], dy[3]);
-            a[2] = 0u;
-            a[3] = 0u;
-            for (int nb = 0; nb < 8; nb++) {
-                const int n = nb * 8 + g, k = 2 * q;
-                uint32_t b[2];
-                b[0] = pack_raw(m.w3[n * kMlpOutPad + k], m.w3[n * kMlpOutPad + k + 1]);
-                b[1] = 0u;
-                dh2[nb][0] = dh2[nb][1] = dh2[nb][2] = dh2[nb][3] = 0.f;
-                mma_bf16(dh2[nb], a, b);
-#pragma unroll
-                for (int e = 0; e < 4; e++) dh2[nb][e] = h2[nb][e] > 0.f ? dh2[nb][e] : 0.f;
-                store_c(st + kStDH2, kMlpHid, nb, dh2[nb], lane);
-                colsum_c(gs + kGB2, nb, dh2[nb], lane);
-            }
-        }
-        __syncwarp();
-        // dW2 = H1^T dH2
-        for (int mt = 0; mt < 4; mt++) {
-            uint32_t a[4];
-            load_at(a, st + kStH1, kMlpHid, mt, lane);
-            for (int nb = 0; nb < 8; nb++) {
-                uint32_t b[2];
-                load_bs(b, st + kStDH2, kMlpHid, nb, lane);
-                float c[4] = {0.f, 0.f, 0.f, 0.f};
-                mma_bf16(c, a, b);
-                add_c(gs + kGW2, kMlpHid, mt, nb, c, lane);
-            }
-        }
-        // dH1 = dH2 W2^T * [H1 > 0]
-        float dh1[8][4];
-        for (int nb = 0; nb < 8; nb++) dh1[nb][0] = dh1[nb][1] = dh1[nb][2] = dh1[nb][3] = 0.f;
-        for (int ks = 0; ks < 4; ks++) {
-            uint32_t a[4];
-            c_to_a(a, dh2[2 * ks], dh2[2 * ks + 1]);
-            for (int nb = 0; nb < 8; nb++) {
-                uint32_t b[2];
-                load_bt(b, m.w2, kMlpHid, ks, nb, lane);
-                mma_bf16(dh1[nb], a, b);
-            }
-        }
-        for (int nb = 0; nb < 8; nb++) {
-#pragma unroll
-            for (int e = 0; e < 4; e++) dh1[nb][e] = h1[nb][e] > 0.f ? dh1[nb][e] : 0.f;
-            store_c(st + kStDH1, kMlpHid, nb, dh1[nb], lane);
-            colsum_c(gs + kGB1, nb, dh1[nb], lane);
-        }
-        __syncwarp();
-        // dW1 = X^T dH1
-        {
-            uint32_t a[4];
-            load_at(a, st + kStX, kMlpInPad, 0, lane);
-            for (int nb = 0; nb < 8; nb++) {
-                uint32_t b[2];
-                load_bs(b, st + kStDH1, kMlpHid, nb, lane);
-                float c[4] = {0.f, 0.f, 0.f, 0.f};
-                mma_bf16(c, a, b);
-                add_c(gs + kGW1, kMlpHid, 0, nb, c, lane);
-            }
-        }
-        __syncwarp();
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-    if (lane == 0) lpart[(int64_t)blockIdx.x * kTrainWarps + w] = lsum * inv_b;
+    train_warp(m, r, X, T, W, idx, B, gridDim.x, st, part, lpart, lane);
 }
 
-// the partials of nw warps, added in one fixed order, into the packed
-// gradient (W1[13][64], b1, W2, b2, W3[64][3], b3) and the loss (element
-// kMlpNParam, added to *loss).  A block takes 32 elements; its 8 warps sum
-// the warps k = y, y + 8, ... in turn, and warp 0 adds the 8 sums in order.
+// Element e of the packed gradient (W1[13][64], b1, W2, b2, W3[64][3], b3;
+// e = kMlpNParam: the loss) from the nw partials: eight sums, of the warps
+// k = j, j + 8, ..., then the eight in turn -- one fixed order.
 constexpr int kReduceSlices = 8;
-__global__ void __launch_bounds__(32 * kReduceSlices) k_grad_reduce(const float* __restrict__ part,
-                                                                    const float* __restrict__ lpart, int nw,
-                                                                    float* __restrict__ grad, float* __restrict__ loss)
+constexpr int kPB1 = kMlpIn * kMlpHid, kPW2 = kPB1 + kMlpHid, kPB2 = kPW2 + kMlpHid * kMlpHid;
+constexpr int kPW3 = kPB2 + kMlpHid, kPB3 = kPW3 + kMlpHid * kMlpOut;
+static_assert(kPB3 + kMlpOut == kMlpNParam, "packed gradient layout");
+
+// NT = 1, 2, 4 or 8 neighbouring lanes share an element; lane sub of them
+// takes the sums j = sub NT' .. and all return the element's sum
+template <int NT>
+__device__ __forceinline__ float reduce_element(const float* part, const float* lpart, int nw, int e, int sub)
 {
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int e = blockIdx.x * 32 + tx;
+    constexpr int NS = kReduceSlices / NT;
     // packed index -> the padded index of a warp's partial (stride kGPad),
     // or the loss partials (stride 1)
-    const float* src = nullptr;
+    const float* src = lpart;
     int64_t stride = kGPad;
-    constexpr int kB1 = kMlpIn * kMlpHid, kW2 = kB1 + kMlpHid, kB2 = kW2 + kMlpHid * kMlpHid;
-    constexpr int kW3 = kB2 + kMlpHid, kB3 = kW3 + kMlpHid * kMlpOut;
-    static_assert(kB3 + kMlpOut == kMlpNParam, "packed gradient layout");
-    if (e < kB1) src = part + kGW1 + e;
-    else if (e < kW2) src = part + kGB1 + (e - kB1);
-    else if (e < kB2) src = part + kGW2 + (e - kW2);
-    else if (e < kW3) src = part + kGB2 + (e - kB2);
-    else if (e < kB3) src = part + kGW3 + ((e - kW3) / kMlpOut) * kMlpOutPad + ((e - kW3) % kMlpOut);
-    else if (e < kMlpNParam) src = part + kGB3 + (e - kB3);
-    else if (e == kMlpNParam) { src = lpart; stride = 1; }
-    float s = 0.f;
-    if (src)
-        for (int k = ty; k < nw; k += kReduceSlices) s += src[(int64_t)k * stride];
-    __shared__ float red[kReduceSlices][33];
-    red[ty][tx] = s;
-    __syncthreads();
-    if (ty == 0 && src) {
-        float t = red[0][tx];
+    if (e < kPB1) src = part + kGW1 + e;
+    else if (e < kPW2) src = part + kGB1 + (e - kPB1);
+    else if (e < kPB2) src = part + kGW2 + (e - kPW2);
+    else if (e < kPW3) src = part + kGB2 + (e - kPB2);
+    else if (e < kPB3) src = part + kGW3 + ((e - kPW3) / kMlpOut) * kMlpOutPad + ((e - kPW3) % kMlpOut);
+    else if (e < kMlpNParam) src = part + kGB3 + (e - kPB3);
+    else stride = 1;
+    float s[NS];
 #pragma unroll
-        for (int j = 1; j < kReduceSlices; j++) t += red[j][tx];
-        if (e < kMlpNParam) grad[e] = t;
-        else *loss += t;
+    for (int j = 0; j < NS; j++) s[j] = 0.f;
+#pragma unroll 8
+    for (int k = sub * NS; k < nw; k += kReduceSlices) {
+#pragma unroll
+        for (int j = 0; j < NS; j++)
+            if (k + j < nw) s[j] += __ldcg(src + (int64_t)(k + j) * stride);
+    }
+    float t = 0.f;
+#pragma unroll
+    for (int j = 0; j < kReduceSlices; j++) {
+        const float x = NT == 1 ? s[j % NS] : __shfl_sync(0xffffffffu, s[j % NS], j / NS, NT);
+        t = j == 0 ? x : t + x;
+    }
+    return t;
+}
+
+__global__ void __launch_bounds__(128) k_grad_reduce(const float* __restrict__ part, const float* __restrict__ lpart,
+                                                     int nw, float* __restrict__ grad, float* __restrict__ loss)
+{
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e > kMlpNParam) return;
+    const float t = reduce_element<1>(part, lpart, nw, e, 0);
+    if (e < kMlpNParam) grad[e] = t;
+    else *loss += t;
+}
+
+// Adam on one FP32 master parameter (the contractions written out, so that
+// the rounding does not depend on what is compiled around it)
+__device__ __forceinline__ void adam_update(float& p, float& mom, float& vel, float gi, float lr, float b1, float b2,
+                                            float eps, float c1, float c2)
+{
+    const float mi = fmaf(1.f - b1, gi, b1 * mom);
+    const float vi = fmaf((1.f - b2) * gi, gi, b2 * vel);
+    mom = mi;
+    vel = vi;
+    p -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+}
+
+// the parts of the device model that a training step reads, for parameter e:
+// its place in the forward fragments, and for W2 and W3 the k-major copy the
+// backward pass takes its transposes from
+__device__ __forceinline__ void put_parameter(MlpDev* m, int e, float p)
+{
+    const __nv_bfloat16 v = __float2bfloat16_rn(p);
+    auto frag = [](uint2* f, int k, int n) {  // 16-bit slot of W[k][n] in a 16 x 8 block's fragment, k < 16, n < 8
+        return reinterpret_cast<__nv_bfloat16*>(f + n * 4 + ((k & 7) >> 1)) + 2 * (k >> 3) + (k & 1);
+    };
+    if (e < kPB1) {
+        const int k = e / kMlpHid, n = e % kMlpHid;
+        *frag(m->frag.f1[n >> 3], k, n & 7) = v;
+    } else if (e < kPW2) {
+        const int n = e - kPB1;
+        reinterpret_cast<float*>(m->frag.b1)[n] = p;  // [column block][q] pairs: plain column order
+    } else if (e < kPB2) {
+        const int k = (e - kPW2) / kMlpHid, n = (e - kPW2) % kMlpHid;
+        *frag(m->frag.f2[k >> 4][n >> 3], k & 15, n & 7) = v;
+        m->w2[e - kPW2] = v;
+    } else if (e < kPW3) {
+        reinterpret_cast<float*>(m->frag.b2)[e - kPB2] = p;
+    } else if (e < kPB3) {
+        const int k = (e - kPW3) / kMlpOut, n = (e - kPW3) % kMlpOut;
+        *frag(m->frag.f3[k >> 4], k & 15, n) = v;
+        m->w3[k * kMlpOutPad + n] = v;
+    } else {
+        reinterpret_cast<float*>(m->frag.b3)[e - kPB3] = p;
+    }
+}
+
+// all blocks of a cooperative launch; a wait that runs out (about a second)
+// raises kErrWorkLoop and returns false in every thread of the block
+__device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target, int32_t* err)
+{
+    __shared__ bool ok_sh;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();  // (the block's writes, ordered before this thread by the barrier above)
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        bool ok = true;
+        const long long t0 = clock64();
+        for (;;) {
+            uint32_t v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if (v >= target) break;
+            if (clock64() - t0 > (1ll << 31)) {
+                ok = false;
+                atomicOr(err, kErrWorkLoop);
+                break;
+            }
+        }
+        ok_sh = ok;
+    }
+    __syncthreads();
+    const bool ok = ok_sh;
+    __syncthreads();
+    return ok;
+}
+
+constexpr int kUpdateLanes = 2;
+
+// One pass over the pairs in mini-batches, one cooperative launch.  A step
+// used to be four dependent launches (gradient, reduction, Adam, packing) of
+// a few blocks each, 43 us of latency for 1024 rows, 15 us now; the blocks
+// meet at two grid barriers a step: after the gradient (a warp per 16 rows),
+// and after the update, where two lanes per parameter (1 / 2 / 4 lanes: 21 /
+// 15 / 17 us a step) add the partials in their order and one of them keeps
+// the master parameter and its Adam moments in registers through the pass
+// and writes the BF16 copies the next step reads.  The next step's rows are
+// loaded before the barriers.  Same operations in the same order as the
+// single kernels: the same network bit for bit.
+__global__ void __launch_bounds__(kTrainWarps * 32) k_mlp_epoch(const float* __restrict__ X, const float* __restrict__ T,
+                                                                 const float* __restrict__ W,
+                                                                 const int32_t* __restrict__ idx, int n, int batch,
+                                                                 int max_blocks, MlpDev* model, float* params,
+                                                                 float* mom, float* vel,
+                                                                 const float* __restrict__ sched, float b1, float b2,
+                                                                 float eps, float* part, float* lpart, float* loss,
+                                                                 uint32_t* bar, int32_t* err)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    MlpDev& m = *reinterpret_cast<MlpDev*>(smem);
+    __nv_bfloat16* st = reinterpret_cast<__nv_bfloat16*>(smem + sizeof(MlpDev)) + (threadIdx.x >> 5) * kStSize;
+    const int lane = threadIdx.x & 31;
+    const int gw = blockIdx.x * kTrainWarps + (threadIdx.x >> 5);
+    // kUpdateLanes neighbouring lanes to a parameter; the last parameter's
+    // follow is the loss, and lanes past it repeat it
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, sub = t % kUpdateLanes;
+    const int e = min(t / kUpdateLanes, kMlpNParam);
+    const bool own = sub == 0 && t / kUpdateLanes <= kMlpNParam;
+    const bool any = (t & ~31) / kUpdateLanes <= kMlpNParam;  // the warp holds an element
+    float pe = 0.f, me = 0.f, ve = 0.f;
+    if (e < kMlpNParam) {
+        pe = params[e];
+        me = mom[e];
+        ve = vel[e];
+    } else if (e == kMlpNParam) {
+        pe = *loss;
+    }
+    uint32_t target = 0;
+    TrainRows r = train_rows(X, T, W, idx, min(batch, n), gw, lane);
+    for (int b0 = 0, step = 0; b0 < n; b0 += batch, step++) {
+        const int B = min(batch, n - b0), blocks = train_blocks(B, max_blocks);
+        if (blockIdx.x < blocks) {
+            load_model(m, model);
+            __syncthreads();
+            train_warp(m, r, X, T, W, idx + b0, B, blocks, st, part, lpart, lane);
+        }
+        if (b0 + batch < n) r = train_rows(X, T, W, idx + b0 + batch, min(batch, n - b0 - batch), gw, lane);
+        target += gridDim.x;
+        if (!grid_barrier(bar, target, err)) return;
+        if (any) {
+            const float g = reduce_element<kUpdateLanes>(part, lpart, train_warps(B, blocks), e, sub);
+            if (!own) {
+            } else if (e < kMlpNParam) {
+                adam_update(pe, me, ve, g, sched[3 * step], b1, b2, eps, sched[3 * step + 1], sched[3 * step + 2]);
+                put_parameter(model, e, pe);
+            } else {
+                pe += g;
+            }
+        }
+        target += gridDim.x;
+        if (!grid_barrier(bar, target, err)) return;
+    }
+    if (own && e < kMlpNParam) {
+        params[e] = pe;
+        mom[e] = me;
+        vel[e] = ve;
+    } else if (own) {
+        *loss = pe;
     }
 }
 
@@ -362,20 +605,6 @@ __global__ void k_mlp_pack(const float* __restrict__ p, const float* __restrict_
         f.xscale[i] = i < kMlpIn ? maps[kMlpIn + i] : 0.f;
         f.xoff[i] = i < kMlpIn ? -maps[i] * maps[kMlpIn + i] : 0.f;
     }
-}
-
-// Adam on the FP32 master parameters
-__global__ void k_adam(float* __restrict__ p, float* __restrict__ mom, float* __restrict__ vel,
-                       const float* __restrict__ g, int n, float lr, float b1, float b2, float eps, float c1, float c2)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * mom[i] + (1.f - b1) * gi;
-    const float vi = b2 * vel[i] + (1.f - b2) * gi * gi;
-    mom[i] = mi;
-    vel[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
 // batch inference: Y (n x 3) = network(X) * yscale, X normalised n x 16 --
@@ -501,43 +730,67 @@ __global__ void k_node_features(const Info* info, const SysParams* __restrict__ 
 }
 
 // ---------------------------------------------------------------- training data
-// Sums over the n training pairs, in FP64: column c of blockIdx.y takes
-//   c < 13: x_c,  13 <= c < 26: x_(c-13)^2,  26 <= c < 29: t_(c-26)^2,
-//   c = 29: F^2 (the pairs' label factors; F null: skipped)
-__global__ void k_mlp_sums(const float* __restrict__ X, const float* __restrict__ T, const float* __restrict__ F,
-                           int64_t n, double* __restrict__ sums)
+// Sums over the n training pairs, in FP64: x_c (13), x_c^2 (13), t_c^2 (3)
+// and F^2 of the label factors (F null: skipped).  Every block takes every
+// gridDim-th run of rows and leaves its sums in part[block]; k_mlp_maps adds
+// the blocks in order, so the maps (and the training that follows) repeat
+// bit for bit.  (One block per column read each row thirty times over: 373 us
+// for 2^18 pairs, a quarter of the pass.)
+constexpr int kSumThreads = 128;
+__global__ void __launch_bounds__(kSumThreads) k_mlp_sums(const float* __restrict__ X, const float* __restrict__ T,
+                                                          const float* __restrict__ F, int64_t n,
+                                                          double* __restrict__ part)
 {
-    const int c = blockIdx.y;
-    if (c == kMlpSums - 1 && !F) return;
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        double v;
-        if (c < kMlpIn) v = X[i * kMlpIn + c];
-        else if (c < 2 * kMlpIn) { v = X[i * kMlpIn + c - kMlpIn]; v *= v; }
-        else if (c < 2 * kMlpIn + kMlpOut) { v = T[i * kMlpOut + c - 2 * kMlpIn]; v *= v; }
-        else { v = F[i]; v *= v; }
-        s += v;
+    double s[kMlpSums];
+#pragma unroll
+    for (int c = 0; c < kMlpSums; c++) s[c] = 0.0;
+    for (int64_t i = (int64_t)blockIdx.x * kSumThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kSumThreads) {
+        float x[kMlpIn], t[kMlpOut];
+#pragma unroll
+        for (int c = 0; c < kMlpIn; c++) x[c] = X[i * kMlpIn + c];
+#pragma unroll
+        for (int c = 0; c < kMlpOut; c++) t[c] = T[i * kMlpOut + c];
+        const double f = F ? (double)F[i] : 0.0;
+#pragma unroll
+        for (int c = 0; c < kMlpIn; c++) {
+            const double v = x[c];
+            s[c] += v;
+            s[kMlpIn + c] += v * v;
+        }
+#pragma unroll
+        for (int c = 0; c < kMlpOut; c++) s[2 * kMlpIn + c] += (double)t[c] * (double)t[c];
+        s[kMlpSums - 1] += f * f;
     }
-    __shared__ double red[32];
+    __shared__ double red[kSumThreads / 32][kMlpSums];
 #pragma unroll
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    for (int c = 0; c < kMlpSums; c++) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][c] = s[c];
+    }
     __syncthreads();
-    if (threadIdx.x < 32) {
-        s = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-#pragma unroll
-        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) atomicAdd(&sums[c], s);
+    if (threadIdx.x < kMlpSums) {
+        double v = red[0][threadIdx.x];
+        for (int w = 1; w < kSumThreads / 32; w++) v += red[w][threadIdx.x];
+        part[(int64_t)blockIdx.x * kMlpSums + threadIdx.x] = v;
     }
 }
 
 // the model's maps from the sums: feature means and inverse standard
 // deviations (0 for a constant feature), output RMS (1 for an all-zero
 // output); and the factor-weight scale n / sum F^2
-__global__ void k_mlp_maps(const double* __restrict__ sums, int64_t n, float* __restrict__ maps,
+__global__ void k_mlp_maps(const double* __restrict__ part, int nblocks, int64_t n, float* __restrict__ maps,
                            float* __restrict__ wscale)
 {
+    __shared__ double sums[kMlpSums];
     const int k = threadIdx.x;
+    if (k < kMlpSums) {
+        double v = 0.0;
+#pragma unroll 16
+        for (int b = 0; b < nblocks; b++) v += part[(int64_t)b * kMlpSums + k];
+        sums[k] = v;
+    }
+    __syncwarp();
     const double inv_n = 1.0 / (double)n;
     if (k < kMlpIn) {
         const double mean = sums[k] * inv_n;
@@ -639,33 +892,58 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 }  // namespace
 
 size_t mlp_train_smem() { return sizeof(MlpDev) + (size_t)kTrainWarps * kStSize * 2; }
+int mlp_train_blocks(int B, int max_blocks) { return train_blocks(B, max_blocks); }
 int64_t mlp_train_part_floats(int blocks) { return (int64_t)blocks * kTrainWarps * (kGPad + 1); }
 
 cudaError_t launch_mlp_train(const float* X, const float* T, const float* W, const int32_t* idx, int B,
-                             const void* model, float* grad, float* loss, float* part, int blocks, cudaStream_t s)
+                             const void* model, float* grad, float* loss, float* part, int max_blocks, cudaStream_t s)
 {
     const size_t smem = mlp_train_smem();
     cudaError_t e = cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int nw = blocks * kTrainWarps;
-    float* lpart = part + (int64_t)nw * kGPad;
+    const int blocks = train_blocks(B, max_blocks);
+    const int ntiles = (B + 15) / 16, nw = ntiles < blocks * kTrainWarps ? ntiles : blocks * kTrainWarps;
+    float* lpart = part + (int64_t)blocks * kTrainWarps * kGPad;
     k_mlp_train<<<blocks, kTrainWarps * 32, smem, s>>>(X, T, W, idx, B, (const MlpDev*)model, part, lpart);
-    k_grad_reduce<<<(kMlpNParam + 1 + 31) / 32, 32 * kReduceSlices, 0, s>>>(part, lpart, nw, grad, loss);
+    k_grad_reduce<<<(kMlpNParam + 1 + 127) / 128, 128, 0, s>>>(part, lpart, nw, grad, loss);
     count_launches(2);
     return cudaGetLastError();
+}
+
+cudaError_t launch_mlp_epoch(const float* X, const float* T, const float* W, const int32_t* idx, int n, int batch,
+                             int max_blocks, void* model, float* params, float* mom, float* vel, const float* sched,
+                             float* part, float* loss, uint32_t* bar, int32_t* err, cudaStream_t s)
+{
+    const size_t smem = mlp_train_smem();
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_epoch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(bar, 0, sizeof(uint32_t), s);
+    if (e != cudaSuccess) return e;
+    // a thread per parameter (and one for the loss), a warp per tile
+    const int threads = kTrainWarps * 32;
+    int grid = ((kMlpNParam + 1) * kUpdateLanes + threads - 1) / threads;
+    const int blocks = train_blocks(batch < n ? batch : n, max_blocks);
+    if (blocks > grid) grid = blocks;
+    float* lpart = part + (int64_t)max_blocks * kTrainWarps * kGPad;
+    MlpDev* mdl = (MlpDev*)model;
+    float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+    void* args[] = {&X, &T, &W, &idx, &n, &batch, &max_blocks, &mdl, &params, &mom, &vel, &sched,
+                    &b1, &b2, &eps, &part, &lpart, &loss, &bar, &err};
+    e = cudaLaunchCooperativeKernel((const void*)k_mlp_epoch, dim3(grid), dim3(threads), args, smem, s);
+    count_launches(1);
+    return e;
+}
+
+void mlp_adam_corrections(int t, float* c1, float* c2)
+{
+    const float b1 = 0.9f, b2 = 0.999f;
+    *c1 = 1.f - powf(b1, (float)t);
+    *c2 = 1.f - powf(b2, (float)t);
 }
 
 void launch_mlp_pack(const float* params, const float* maps, void* model, cudaStream_t s)
 {
     k_mlp_pack<<<1, 256, 0, s>>>(params, maps, (MlpDev*)model);
-    count_launches(1);
-}
-
-void launch_adam(float* p, float* m, float* v, const float* g, int n, float lr, int t, cudaStream_t s)
-{
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = 1.f - powf(b1, (float)t), c2 = 1.f - powf(b2, (float)t);
-    k_adam<<<nblk(n, 256), 256, 0, s>>>(p, m, v, g, n, lr, b1, b2, 1e-8f, c1, c2);
     count_launches(1);
 }
 
@@ -718,19 +996,19 @@ void launch_pair_labels(const int32_t* pb, const int32_t* pv, int64_t np, const 
     count_launches(1);
 }
 
-void launch_mlp_sums(const float* X, const float* T, const float* F, int64_t n, double* sums, cudaStream_t s)
+int mlp_sum_blocks(int64_t n)
 {
-    // one block per column: each sum is taken in one fixed order, so the
-    // maps (and the training that follows) repeat bit for bit
-    cudaMemsetAsync(sums, 0, kMlpSums * sizeof(double), s);
-    k_mlp_sums<<<dim3(1, kMlpSums), 1024, 0, s>>>(X, T, F, n, sums);
-    count_launches(1);
+    const int64_t b = (n + kSumThreads - 1) / kSumThreads;
+    return (int)(b < kMlpSumBlocks ? b : kMlpSumBlocks);
 }
 
-void launch_mlp_maps(const double* sums, int64_t n, float* maps, float* wscale, cudaStream_t s)
+void launch_mlp_maps(const float* X, const float* T, const float* F, int64_t n, double* part, float* maps,
+                     float* wscale, cudaStream_t s)
 {
-    k_mlp_maps<<<1, 32, 0, s>>>(sums, n, maps, wscale);
-    count_launches(1);
+    const int nb = mlp_sum_blocks(n);
+    k_mlp_sums<<<nb, kSumThreads, 0, s>>>(X, T, F, n, part);
+    k_mlp_maps<<<1, 32, 0, s>>>(part, nb, n, maps, wscale);
+    count_launches(2);
 }
 
 void launch_mlp_rows(const float* X, const float* T, int64_t n, const float* maps, float* rows, float* tout,

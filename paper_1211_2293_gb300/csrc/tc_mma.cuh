@@ -38,9 +38,10 @@ struct MlpFrag {
     float yscale[kMlpOutPad]; // network output x yscale = label
 };
 
-// Device copy of a model: the inference part, then the k-major weights
-// ([in][out], padded) the training kernel reads its transposes from.
-struct MlpDev {
+// Device copy of a model: the fragments, then the k-major weights ([in][out],
+// padded) the backward pass reads its transposes from (W1 and the biases for
+// completeness).
+struct __align__(16) MlpDev {
     MlpFrag frag;
     __nv_bfloat16 w1[kMlpInPad * kMlpHid];
     __nv_bfloat16 w2[kMlpHid * kMlpHid];
@@ -86,16 +87,6 @@ __device__ __forceinline__ void mma_frag(float (&c)[4], const uint32_t (&a)[4], 
 {
     const uint32_t b[2] = {w.x, w.y};
     mma_bf16(c, a, b);
-}
-
-// B fragment of a k-major BF16 matrix W[k][n] (row stride ld), k-step ks,
-// column block nb
-__device__ __forceinline__ void load_b(uint32_t (&b)[2], const __nv_bfloat16* W, int ld, int ks, int nb, int lane)
-{
-    const int g = lane >> 2, q = lane & 3;
-    const int n = nb * 8 + g, k = ks * 16 + 2 * q;
-    b[0] = pack_raw(W[(k) * ld + n], W[(k + 1) * ld + n]);
-    b[1] = pack_raw(W[(k + 8) * ld + n], W[(k + 9) * ld + n]);
 }
 
 // A fragment from C tiles (FP32) of column blocks 2ks and 2ks+1
@@ -161,59 +152,38 @@ __device__ __forceinline__ void mlp16_infer(const MlpFrag& m, const uint32_t (&x
     }
 }
 
-// The MLP on 16 rows for training, from the k-major weights: returns the
-// hidden activations too (h1, h2 as C tiles after ReLU).
-__device__ __forceinline__ void mlp16(const MlpDev& m, const uint32_t (&x)[4], float (&h1)[8][4], float (&h2)[8][4],
+// The MLP on 16 rows for training: returns the hidden activations too (h1,
+// h2 as C tiles after ReLU).
+__device__ __forceinline__ void mlp16(const MlpFrag& m, const uint32_t (&x)[4], float (&h1)[8][4], float (&h2)[8][4],
                                       float (&y)[4], int lane)
 {
     const int q = lane & 3;
 #pragma unroll
     for (int nb = 0; nb < 8; nb++) {
-        const float bb0 = m.b1[nb * 8 + 2 * q], bb1 = m.b1[nb * 8 + 2 * q + 1];
-        h1[nb][0] = bb0;
-        h1[nb][1] = bb1;
-        h1[nb][2] = bb0;
-        h1[nb][3] = bb1;
-        uint32_t b[2];
-        load_b(b, m.w1, kMlpHid, 0, nb, lane);
-        mma_bf16(h1[nb], x, b);
+        bias_init(h1[nb], m.b1[nb][q]);
+        mma_frag(h1[nb], x, m.f1[nb][lane]);
 #pragma unroll
         for (int e = 0; e < 4; e++) h1[nb][e] = fmaxf(h1[nb][e], 0.f);
     }
 #pragma unroll
-    for (int nb = 0; nb < 8; nb++) {
-        const float bb0 = m.b2[nb * 8 + 2 * q], bb1 = m.b2[nb * 8 + 2 * q + 1];
-        h2[nb][0] = bb0;
-        h2[nb][1] = bb1;
-        h2[nb][2] = bb0;
-        h2[nb][3] = bb1;
-    }
+    for (int nb = 0; nb < 8; nb++) bias_init(h2[nb], m.b2[nb][q]);
 #pragma unroll
     for (int ks = 0; ks < 4; ks++) {
         uint32_t a[4];
         c_to_a(a, h1[2 * ks], h1[2 * ks + 1]);
 #pragma unroll
-        for (int nb = 0; nb < 8; nb++) {
-            uint32_t b[2];
-            load_b(b, m.w2, kMlpHid, ks, nb, lane);
-            mma_bf16(h2[nb], a, b);
-        }
+        for (int nb = 0; nb < 8; nb++) mma_frag(h2[nb], a, m.f2[ks][nb][lane]);
     }
 #pragma unroll
     for (int nb = 0; nb < 8; nb++)
 #pragma unroll
         for (int e = 0; e < 4; e++) h2[nb][e] = fmaxf(h2[nb][e], 0.f);
-    y[0] = m.b3[2 * q];
-    y[1] = m.b3[2 * q + 1];
-    y[2] = y[0];
-    y[3] = y[1];
+    bias_init(y, m.b3[q]);
 #pragma unroll
     for (int ks = 0; ks < 4; ks++) {
         uint32_t a[4];
         c_to_a(a, h2[2 * ks], h2[2 * ks + 1]);
-        uint32_t b[2];
-        load_b(b, m.w3, kMlpOutPad, ks, 0, lane);
-        mma_bf16(y, a, b);
+        mma_frag(y, a, m.f3[ks][lane]);
     }
 }
 
