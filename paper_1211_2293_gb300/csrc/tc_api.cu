@@ -60,7 +60,8 @@ struct tc_ctx {
     int8_t *w = nullptr, *delta = nullptr, *top = nullptr;
     uint32_t* lcnt = nullptr;    // nodes per level and block of bodies, then their places
     uint32_t* lstart = nullptr;  // first node of each level
-    unsigned long long* scan = nullptr;  // the build's look-back words
+    uint4* zero = nullptr;               // scratch that a build starts from zero (zero_words)
+    unsigned long long* scan = nullptr;  // in it: the scans' look-back words
     int32_t *gref_at = nullptr, *gfirst = nullptr, *gref = nullptr;
     int32_t *ncell = nullptr, *nbody = nullptr;
     unsigned long long* hash = nullptr;
@@ -282,6 +283,12 @@ int grow(tc_ctx* c, T** p, int64_t count)
         if (r_) return r_;                \
     } while (0)
 
+// 64-bit words of a build's zeroed scratch
+int64_t zero_words(int64_t n, int64_t status)
+{
+    return kSortMaxPasses * 128 + 8 + build_scan_words(n) + status;
+}
+
 int ensure_bodies(tc_ctx* c, int64_t n)
 {
     if (n <= c->cap_n) return TC_OK;
@@ -297,19 +304,15 @@ int ensure_bodies(tc_ctx* c, int64_t n)
     TC_GROW(c, c->body, cap);
     TC_GROW(c, c->sb.keys_alt, cap);
     TC_GROW(c, c->sb.vals_alt, cap);
-    TC_GROW(c, c->sb.ghist, kSortMaxPasses * 256);
-    TC_GROW(c, c->sb.status, (int64_t)kSortMaxPasses * radix_tiles(cap) * 256);
-    TC_GROW(c, c->sb.tiles, kSortMaxPasses);
+    // what a build starts from zero, in one piece: digit counts, tile
+    // counters, the scans' look-back words, the sort's
+    TC_GROW(c, c->zero, 2 * zero_words(cap, radix_status_words(cap)) / 4 + 4);
     c->sb.err = &c->info->err;
-    TC_GROW(c, c->sb.runs, cap / 32 + 16);  // runs of more than 32 items
-    c->sb.run_cap = cap / 32 + 16;
-    TC_GROW(c, c->sb.nruns, 1);
     TC_GROW(c, c->w, cap);
     TC_GROW(c, c->delta, cap);
     TC_GROW(c, c->top, cap);
     TC_GROW(c, c->lcnt, level_counts_size(cap));
     TC_GROW(c, c->lstart, kMaxLevel + 2);
-    TC_GROW(c, c->scan, build_scan_words(cap));
     TC_GROW(c, c->gref_at, cap);
     TC_GROW(c, c->gfirst, cap + 1);
     TC_GROW(c, c->gref, cap);
@@ -441,9 +444,11 @@ int sys_bits(int nsys)
 int setup_systems(tc_ctx* c, const int64_t* off, int nsys)
 {
     std::vector<int4> ch;
+    const int64_t chunk = off[nsys] <= (1 << 19) ? kBboxChunkSmall : kBboxChunk;
     for (int s = 0; s < nsys; s++)
-        for (int64_t a = off[s]; a < off[s + 1]; a += kBboxChunk)
-            ch.push_back(make_int4(s, (int)a, (int)std::min(off[s + 1], a + (int64_t)kBboxChunk), 0));
+        for (int64_t a = off[s]; a < off[s + 1]; a += chunk)
+            ch.push_back(make_int4(s, (int)a, (int)std::min(off[s + 1], a + chunk),
+                                   (int)((off[s + 1] - off[s] + chunk - 1) / chunk)));
     int r = ensure_systems(c, nsys, (int)ch.size());
     if (r) return r;
     c->off_h.assign(off, off + nsys + 1);
@@ -466,9 +471,6 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
 {
     const int64_t n = c->n;
     cudaEvent_t t0 = phase_begin(c, s, 0);
-    if (synced) TC_CUDA(c, cudaMemsetAsync(&c->info->err, 0, sizeof(int32_t), s));
-    launch_bbox(c->pos, c->chunks, c->nchunks, c->sysp, c->nsys, &c->info->err, s);
-    launch_keys(c->pos, c->mass, n, c->sys_of, c->sysp, c->keys, c->perm, &c->info->err, s);
     // The passes sort only the key digits of the levels down to the last
     // synchronised build's depth + kSortMarginLevels; runs of equal top
     // digits, a leaf's bodies as long as the tree is no deeper than that,
@@ -482,11 +484,37 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
         const int levels = std::min(kMaxLevel, c->depth_hint + kSortMarginLevels);
         low_bit = 63 - 3 * levels;
     }
-    radix_sort_u64(c->keys, c->perm, n, 63, c->sys_of, c->nsys > 1 ? sys_bits(c->nsys) : 0, c->sb, s, low_bit,
-                   synced ? kSortRunMaxSynced : kSortRunMax);
-    launch_gather(c->pos, c->mass, c->perm, n, c->body, s);
-    TC_CUDA(c, cudaMemsetAsync(&c->info->depth, 0, sizeof(int32_t), s));
-    TC_CUDA(c, cudaMemsetAsync(c->scan, 0, build_scan_words(n) * sizeof(unsigned long long), s));
+    SortPlan plan = SortPlan::make(63, low_bit, c->nsys > 1 ? sys_bits(c->nsys) : 0);
+    if (n < 2) {
+        plan.npass = 0;
+        low_bit = 0;
+    }
+    // the zeroed scratch
+    const bool one_block = n >= 2 && n <= kBlockSortMax;
+    const int64_t status = one_block ? 0 : radix_status_words(n, plan.npass);
+    c->sb.ghist = reinterpret_cast<uint32_t*>(c->zero);
+    c->sb.tiles = c->sb.ghist + kSortMaxPasses * 256;
+    c->scan = reinterpret_cast<unsigned long long*>(c->sb.tiles + 16);
+    c->sb.status = c->scan + build_scan_words(n);
+    launch_build_init(c->zero, (zero_words(n, status) + 1) / 2, c->sysp, c->nsys, c->info, synced, s);
+    launch_bbox(c->pos, c->chunks, c->nchunks, c->sysp, &c->info->err, s);
+    // the keys go where the passes (and the completion) end in keys / perm
+    const int moves = one_block ? 1 : plan.npass + (low_bit > 0 ? 1 : 0);
+    uint64_t *ka = moves % 2 ? c->sb.keys_alt : c->keys, *kb = moves % 2 ? c->keys : c->sb.keys_alt;
+    uint32_t *va = moves % 2 ? c->sb.vals_alt : c->perm, *vb = moves % 2 ? c->perm : c->sb.vals_alt;
+    launch_keys(c->pos, c->mass, n, c->sys_of, c->sysp, ka, va, plan, one_block ? nullptr : c->sb.ghist, &c->info->err,
+                s);
+    const int64_t run_max = synced ? kSortRunMaxSynced : kSortRunMax;
+    if (one_block) {
+        launch_sort_block(ka, va, kb, vb, n, plan, c->sys_of, c->pos, c->mass, c->body, run_max, &c->info->err, s);
+    } else {
+        launch_sort_passes(ka, va, kb, vb, n, plan, c->sys_of, c->sb, s);
+        if (low_bit > 0)
+            launch_sort_runs(c->sb.keys_alt, c->sb.vals_alt, c->keys, c->perm, n, low_bit, c->nsys > 1 ? c->sys_of : nullptr,
+                             c->pos, c->mass, c->body, run_max, &c->info->err, s);
+        else
+            launch_gather(c->pos, c->mass, c->perm, n, c->body, s);
+    }
     launch_node_levels(c->keys, c->sys_of, n, c->leaf_max, c->w, c->delta, c->top, c->gref_at, c->lcnt, c->scan,
                        synced ? -1 : c->cap_m, c->info, s);
     int depth = -1;
@@ -1621,7 +1649,7 @@ int tc_mlp_pairs(tc_ctx* c, float theta, float eps, float band, float prob, uint
         TC_GROW(c, c->pair_sb.keys_alt, cap);
         TC_GROW(c, c->pair_sb.vals_alt, cap);
         TC_GROW(c, c->pair_sb.ghist, kSortMaxPasses * 256);
-        TC_GROW(c, c->pair_sb.status, (int64_t)kSortMaxPasses * radix_tiles(cap) * 256);
+        TC_GROW(c, c->pair_sb.status, radix_status_words(cap));
         TC_GROW(c, c->pair_sb.tiles, kSortMaxPasses);
         c->pair_sb.err = &c->info->err;
         c->pair_sort_cap = cap;

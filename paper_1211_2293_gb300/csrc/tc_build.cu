@@ -8,11 +8,13 @@
 // difference in the first digit of two keys.
 //
 // Pipeline (all on one stream):
-//   1. k_bbox, k_sys_cube  per-system bounding box -> power-of-two root cube
-//                  on a 2^21 grid (FP64)
-//   2. k_keys      63-bit Morton keys (exact FP64 quantisation)
+//   1. k_build_init, k_bbox  scratch zeroed; per-system bounding box ->
+//                  power-of-two root cube on a 2^21 grid (FP64)
+//   2. k_keys      63-bit Morton keys (exact quantisation) and the sort's
+//                  digit counts
 //   3. radix sort  stable sort by (system, key, index)    [tc_sort.cu]
-//   4. k_gather    bodies in Morton order as float4 (x, y, z, m)
+//   4. the bodies in Morton order as float4 (x, y, z, m): k_gather, or with
+//                  the sort's completion
 //   5. k_window / k_node_levels, k_scan_levels
 //                  which cubes of the recursive subdivision start at each
 //                  sorted body (a sliding-window test, below), how many of
@@ -128,17 +130,63 @@ __device__ __forceinline__ float warp_max(float x)
     return x;
 }
 
-__global__ void k_bbox_init(SysParams* __restrict__ sysp, int nsys)
+__global__ void k_build_init(uint4* __restrict__ zero, int64_t nzero, SysParams* __restrict__ sysp, int nsys, Info* info,
+                             int reset_err)
 {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsys) return;
-    for (int a = 0; a < 3; a++) {
-        sysp[s].bb[a] = f2o(INFINITY);
-        sysp[s].bb[3 + a] = f2o(-INFINITY);
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = t; i < nzero; i += stride) zero[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int64_t s = t; s < nsys; s += stride) {
+        for (int a = 0; a < 3; a++) {
+            sysp[s].bb[a] = f2o(INFINITY);
+            sysp[s].bb[3 + a] = f2o(-INFINITY);
+        }
+        sysp[s].done = 0;
+    }
+    if (t == 0) {
+        info->depth = 0;
+        if (reset_err) info->err = 0;
     }
 }
 
-// one block per chunk (system, start, end) of at most kBboxChunk bodies
+// Root cube of each system: side L = smallest power of two with
+// L >= extent * (1 + 2^-20), grid step h = L / 2^21, corner c0 = floor(min/h) h.
+__device__ void sys_cube(SysParams& P)
+{
+    double dlo[3], dhi[3];
+    for (int a = 0; a < 3; a++) {
+        dlo[a] = (double)o2f(__ldcg(&P.bb[a]));
+        dhi[a] = (double)o2f(__ldcg(&P.bb[3 + a]));
+    }
+    double extent = 0.0;
+    for (int a = 0; a < 3; a++) {
+        const double e = dhi[a] - dlo[a];
+        if (e > extent) extent = e;
+    }
+    const double target = extent * (1.0 + 0x1p-20);
+    double L = 1.0;  // all bodies coincide (or a non-finite input): unit cube
+    if (target > 0.0 && target < INFINITY) {
+        int e;
+        const double m = frexp(target, &e);
+        L = (m == 0.5) ? target : ldexp(1.0, e);
+    }
+    const double h = L / 2097152.0;
+    int eh;
+    frexp(h, &eh);        // h = 2^(eh - 1)
+    P.qexp = 1 - eh;      // 1/h = 2^qexp
+    for (int a = 0; a < 3; a++) {
+        double K0 = floor(dlo[a] / h);
+        if (!(K0 == K0) || K0 > 9e15 || K0 < -9e15) K0 = 0.0;  // non-finite input: keys are reported, not used
+        P.c0[a] = K0 * h;
+        P.qoff[a] = (long long)K0;
+    }
+    P.L = L;
+    P.h = h;
+    P.Lf = (float)L;
+    P.uf = (float)(h * 0.5);
+}
+
+// one block per chunk (system, start, end, chunks of the system); the block
+// that completes a system's last chunk forms its root cube
 __global__ void __launch_bounds__(kBboxThreads) k_bbox(const float* __restrict__ pos, const int4* __restrict__ chunks,
                                                        SysParams* __restrict__ sysp, int32_t* __restrict__ err)
 {
@@ -172,47 +220,13 @@ __global__ void __launch_bounds__(kBboxThreads) k_bbox(const float* __restrict__
         for (int k = 0; k < kBboxThreads / 32; k++) r = a < 3 ? fminf(r, sm[a][k]) : fmaxf(r, sm[a][k]);
         if (a < 3) atomicMin(&sysp[ch.x].bb[a], f2o(r));
         else atomicMax(&sysp[ch.x].bb[a], f2o(r));
+        __threadfence();  // before this chunk counts as done
+        __syncwarp(0x3fu);
+        if (a == 0 && atomicAdd(&sysp[ch.x].done, 1) == ch.w - 1) {
+            __threadfence();
+            sys_cube(sysp[ch.x]);
+        }
     }
-}
-
-// Root cube of each system: side L = smallest power of two with
-// L >= extent * (1 + 2^-20), grid step h = L / 2^21, corner c0 = floor(min/h) h.
-__global__ void k_sys_cube(SysParams* __restrict__ sysp, int nsys)
-{
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsys) return;
-    SysParams& P = sysp[s];
-    double dlo[3], dhi[3];
-    for (int a = 0; a < 3; a++) {
-        dlo[a] = (double)o2f(P.bb[a]);
-        dhi[a] = (double)o2f(P.bb[3 + a]);
-    }
-    double extent = 0.0;
-    for (int a = 0; a < 3; a++) {
-        const double e = dhi[a] - dlo[a];
-        if (e > extent) extent = e;
-    }
-    const double target = extent * (1.0 + 0x1p-20);
-    double L = 1.0;  // all bodies coincide (or a non-finite input): unit cube
-    if (target > 0.0 && target < INFINITY) {
-        int e;
-        const double m = frexp(target, &e);
-        L = (m == 0.5) ? target : ldexp(1.0, e);
-    }
-    const double h = L / 2097152.0;
-    int eh;
-    frexp(h, &eh);        // h = 2^(eh - 1)
-    P.qexp = 1 - eh;      // 1/h = 2^qexp
-    for (int a = 0; a < 3; a++) {
-        double K0 = floor(dlo[a] / h);
-        if (!(K0 == K0) || K0 > 9e15 || K0 < -9e15) K0 = 0.0;  // non-finite input: keys are reported, not used
-        P.c0[a] = K0 * h;
-        P.qoff[a] = (long long)K0;
-    }
-    P.L = L;
-    P.h = h;
-    P.Lf = (float)L;
-    P.uf = (float)(h * 0.5);
 }
 
 // ------------------------------------------------------------------ keys
@@ -229,21 +243,65 @@ __device__ __forceinline__ uint64_t quantise(float x, int k, long long K0)
     return (uint64_t)q;
 }
 
-__global__ void k_keys(const float* __restrict__ pos, const float* __restrict__ mass, int64_t n,
-                       const uint32_t* __restrict__ sys_of, const SysParams* __restrict__ sysp,
-                       uint64_t* __restrict__ keys, uint32_t* __restrict__ idx, int32_t* err)
+constexpr int kKeyRounds = 4;  // bodies of a thread whose loads are in flight together
+
+// also (ghist not null) the digit counts of the sort's passes, per block in
+// shared memory
+__global__ void __launch_bounds__(256) k_keys(const float* __restrict__ pos, const float* __restrict__ mass, int64_t n,
+                                              const uint32_t* __restrict__ sys_of, const SysParams* __restrict__ sysp,
+                                              uint64_t* __restrict__ keys, uint32_t* __restrict__ idx, SortPlan plan,
+                                              uint32_t* __restrict__ ghist, int32_t* err)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const SysParams& P = sysp[sys_of[i]];
-    const int k = P.qexp;
-    const uint64_t qx = quantise(pos[3 * i], k, P.qoff[0]);
-    const uint64_t qy = quantise(pos[3 * i + 1], k, P.qoff[1]);
-    const uint64_t qz = quantise(pos[3 * i + 2], k, P.qoff[2]);
-    keys[i] = (spread3(qx) << 2) | (spread3(qy) << 1) | spread3(qz);
-    idx[i] = (uint32_t)i;
-    const float m = mass[i];
-    if (!(isfinite(m) && m > 0.0f)) atomicOr(err, kErrNonFinite);
+    __shared__ uint32_t h[kSortMaxPasses][256];
+    const int npass = ghist ? plan.npass : 0;
+    for (int p = 0; p < npass; p++) h[p][threadIdx.x] = 0u;
+    __syncthreads();
+    bool bad = false;
+    for (int64_t i0 = (int64_t)blockIdx.x * (256 * kKeyRounds); i0 < n; i0 += (int64_t)gridDim.x * (256 * kKeyRounds)) {
+        float x[kKeyRounds][3], m[kKeyRounds];
+        uint32_t sy[kKeyRounds];
+#pragma unroll
+        for (int r = 0; r < kKeyRounds; r++) {
+            const int64_t i = min(i0 + r * 256 + threadIdx.x, n - 1);
+            sy[r] = sys_of[i];
+            x[r][0] = pos[3 * i];
+            x[r][1] = pos[3 * i + 1];
+            x[r][2] = pos[3 * i + 2];
+            m[r] = mass[i];
+        }
+#pragma unroll
+        for (int r = 0; r < kKeyRounds; r++) {
+            const int64_t i = i0 + r * 256 + threadIdx.x;
+            const int64_t left = n - (i - (threadIdx.x & 31));  // bodies from the warp's first on
+            const unsigned act = left >= 32 ? 0xffffffffu : (left > 0 ? (1u << left) - 1u : 0u);
+            if (i >= n) continue;
+            const SysParams& P = sysp[sy[r]];
+            const int k = P.qexp;
+            const uint64_t qx = quantise(x[r][0], k, P.qoff[0]);
+            const uint64_t qy = quantise(x[r][1], k, P.qoff[1]);
+            const uint64_t qz = quantise(x[r][2], k, P.qoff[2]);
+            const uint64_t key = (spread3(qx) << 2) | (spread3(qy) << 1) | spread3(qz);
+            keys[i] = key;
+            idx[i] = (uint32_t)i;
+            bad |= !(isfinite(m[r]) && m[r] > 0.0f);
+            for (int p = 0; p < npass; p++) {
+                const SortDigit dg = plan.digit(p);
+                const uint32_t d = dg.of(key, sy[r]);
+                if (dg.sys) {  // shared by most of a warp: one add for its equal digits
+                    const unsigned same = __match_any_sync(act, d);
+                    if ((same & ((1u << (threadIdx.x & 31)) - 1u)) == 0u) atomicAdd(&h[p][d], (uint32_t)__popc(same));
+                } else {
+                    atomicAdd(&h[p][d], 1u);
+                }
+            }
+        }
+    }
+    if (bad) atomicOr(err, kErrNonFinite);
+    __syncthreads();
+    for (int p = 0; p < npass; p++) {
+        const uint32_t c = h[p][threadIdx.x];
+        if (c) atomicAdd(&ghist[p * 256 + threadIdx.x], c);
+    }
 }
 
 __global__ void k_gather(const float* __restrict__ pos, const float* __restrict__ mass,
@@ -261,40 +319,66 @@ __global__ void k_gather(const float* __restrict__ pos, const float* __restrict_
 // scan of the blocks' counts, laid out level by level, is the place of each
 // block's first node of each level: no pre-order table and no sort by level
 // lie between the counts and the node table.
-constexpr int kNodeBlock = 1024;
+// A thread takes kNodeRounds bodies, so that a block's chain of barriers and
+// loads is shared by four times as many bodies as with one each (59 -> 40 and
+// 94 -> 47 us for the two kernels at 2^22).
+constexpr int kNodeThreads = 256, kNodeRounds = 4;
+constexpr int kNodeBlock = kNodeThreads * kNodeRounds;
+constexpr int kNodeSets = kNodeBlock / 32;  // runs of 32 consecutive bodies, set r * 8 + warp
 constexpr int kLevels = kMaxLevel + 1;
 constexpr int kTileWindow = 256;
 
-// per level, the block's nodes (levels d < l <= t of every body) -> cnt[l][block]
-__device__ __forceinline__ void count_levels(int d, int t, uint32_t* __restrict__ cnt)
+__device__ __forceinline__ uint32_t warp_incl(uint32_t x)
 {
-    __shared__ uint32_t wc[kNodeBlock / 32][kLevels];
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    return x;
+}
+
+// the starts per level of a set of 32 bodies (levels d < l <= t of each): lane l
+// holds level l's
+__device__ __forceinline__ uint32_t set_levels(int d, int t)
+{
+    uint32_t mine = 0;
+    const int hi = __reduce_max_sync(0xffffffffu, t);  // the set's levels
+    for (int l = __reduce_min_sync(0xffffffffu, t > d ? d : kMaxLevel) + 1; l <= hi; l++) {
+        const unsigned m = __ballot_sync(0xffffffffu, d < l && l <= t);
+        if ((int)(threadIdx.x & 31) == l) mine = __popc(m);
+    }
+    return mine;
+}
+
+// per level, the block's nodes -> cnt[l][block]; the deepest level of the
+// forest (a block maximum, then one atomic a block)
+__device__ __forceinline__ void count_levels(const int (&d)[kNodeRounds], const int (&t)[kNodeRounds],
+                                             uint32_t* __restrict__ cnt, int32_t* depth)
+{
+    __shared__ uint32_t wc[kNodeThreads / 32][kLevels];
+    __shared__ int wmax[kNodeThreads / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     uint32_t mine = 0;
+    int hi = -1;
 #pragma unroll
-    for (int l = 0; l < kLevels; l++) {
-        const unsigned m = __ballot_sync(0xffffffffu, d < l && l <= t);
-        if (lane == l) mine = __popc(m);
+    for (int r = 0; r < kNodeRounds; r++) {
+        mine += set_levels(d[r], t[r]);
+        hi = max(hi, t[r]);
     }
+    hi = __reduce_max_sync(0xffffffffu, hi);
     if (lane < kLevels) wc[w][lane] = mine;
+    if (lane == 31) wmax[w] = hi;
     __syncthreads();
     if (threadIdx.x < kLevels) {
         uint32_t c = 0;
-        for (int k = 0; k < kNodeBlock / 32; k++) c += wc[k][threadIdx.x];
+#pragma unroll
+        for (int k = 0; k < kNodeThreads / 32; k++) c += wc[k][threadIdx.x];
         cnt[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = c;
-    }
-}
-
-// the deepest level of the forest: a block maximum, then one atomic a block
-__device__ __forceinline__ void block_depth(int t, int32_t* depth)
-{
-    __shared__ int wmax[kNodeBlock / 32];
-    t = __reduce_max_sync(0xffffffffu, t);
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = t;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        t = __reduce_max_sync(0xffffffffu, wmax[threadIdx.x]);
-        if (threadIdx.x == 0) atomicMax(depth, t);
+    } else if (threadIdx.x == 32) {
+        for (int k = 0; k < kNodeThreads / 32; k++) hi = max(hi, wmax[k]);
+        atomicMax(depth, hi);
     }
 }
 
@@ -309,40 +393,44 @@ __global__ void k_window(const uint64_t* __restrict__ keys, const uint32_t* __re
 }
 
 // leaf_max > kTileWindow: the window digits come from k_window
-__global__ void __launch_bounds__(kNodeBlock) k_node_levels(const uint64_t* __restrict__ keys,
-                                                            const uint32_t* __restrict__ sys_of,
-                                                            const int8_t* __restrict__ w, int64_t n, int leaf_max,
-                                                            int8_t* __restrict__ delta, int8_t* __restrict__ top,
-                                                            int32_t* __restrict__ gref_at, uint32_t* __restrict__ cnt,
-                                                            int32_t* __restrict__ depth)
+__global__ void __launch_bounds__(kNodeThreads) k_node_levels(const uint64_t* __restrict__ keys,
+                                                              const uint32_t* __restrict__ sys_of,
+                                                              const int8_t* __restrict__ w, int64_t n, int leaf_max,
+                                                              int8_t* __restrict__ delta, int8_t* __restrict__ top,
+                                                              int32_t* __restrict__ gref_at, uint32_t* __restrict__ cnt,
+                                                              int32_t* __restrict__ depth)
 {
-    const int64_t s = (int64_t)blockIdx.x * kNodeBlock + threadIdx.x;
-    int t = -1, d = 0;
-    if (s < n) {
-        d = (s == 0 || sys_of[s] != sys_of[s - 1]) ? -1 : common_digits(keys[s - 1], keys[s]);
-        int W = -1;
-        const int64_t j0 = s - leaf_max < 0 ? 0 : s - leaf_max;
-        for (int64_t j = j0; j <= s; j++) W = max(W, (int)w[j]);
-        t = min(W + 1, kMaxLevel);
-        delta[s] = (int8_t)d;
-        top[s] = (int8_t)t;
-        gref_at[s] = 0;
+    int d[kNodeRounds], t[kNodeRounds];
+#pragma unroll
+    for (int r = 0; r < kNodeRounds; r++) {
+        const int64_t s = (int64_t)blockIdx.x * kNodeBlock + r * kNodeThreads + threadIdx.x;
+        t[r] = -1;
+        d[r] = 0;
+        if (s < n) {
+            d[r] = (s == 0 || sys_of[s] != sys_of[s - 1]) ? -1 : common_digits(keys[s - 1], keys[s]);
+            int W = -1;
+            const int64_t j0 = s - leaf_max < 0 ? 0 : s - leaf_max;
+            for (int64_t j = j0; j <= s; j++) W = max(W, (int)w[j]);
+            t[r] = min(W + 1, kMaxLevel);
+            delta[s] = (int8_t)d[r];
+            top[s] = (int8_t)t[r];
+            gref_at[s] = 0;
+        }
     }
-    block_depth(t, depth);
-    count_levels(d, t, cnt);
+    count_levels(d, t, cnt, depth);
 }
 
 // The same in one kernel for leaf_max <= kTileWindow: a block stages the keys
 // and systems of [b0 - leaf_max, b0 + kNodeBlock + leaf_max) in shared memory,
 // forms the window digits cd(key_j, key_j+leaf_max) there, and takes each
 // body's window maximum from them.
-__global__ void __launch_bounds__(kNodeBlock) k_node_levels_tiled(const uint64_t* __restrict__ keys,
-                                                                  const uint32_t* __restrict__ sys_of, int64_t n,
-                                                                  int leaf_max, int8_t* __restrict__ delta,
-                                                                  int8_t* __restrict__ top,
-                                                                  int32_t* __restrict__ gref_at,
-                                                                  uint32_t* __restrict__ cnt,
-                                                                  int32_t* __restrict__ depth)
+__global__ void __launch_bounds__(kNodeThreads) k_node_levels_tiled(const uint64_t* __restrict__ keys,
+                                                                    const uint32_t* __restrict__ sys_of, int64_t n,
+                                                                    int leaf_max, int8_t* __restrict__ delta,
+                                                                    int8_t* __restrict__ top,
+                                                                    int32_t* __restrict__ gref_at,
+                                                                    uint32_t* __restrict__ cnt,
+                                                                    int32_t* __restrict__ depth)
 {
     __shared__ uint64_t sk[kNodeBlock + 2 * kTileWindow];
     __shared__ uint32_t ss[kNodeBlock + 2 * kTileWindow];
@@ -350,7 +438,8 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_levels_tiled(const uint64_t
     const int64_t b0 = (int64_t)blockIdx.x * kNodeBlock;
     const int64_t base = b0 - leaf_max;  // smem index 0 holds body base
     const int nk = kNodeBlock + 2 * leaf_max;
-    for (int i = threadIdx.x; i < nk; i += kNodeBlock) {
+#pragma unroll 6
+    for (int i = threadIdx.x; i < nk; i += kNodeThreads) {
         const int64_t j = base + i;
         const bool in = j >= 0 && j < n;
         sk[i] = in ? keys[j] : 0ull;
@@ -359,28 +448,33 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_levels_tiled(const uint64_t
     __syncthreads();
     // window digits of bodies base .. b0 + kNodeBlock - 1
     const int nw = kNodeBlock + leaf_max;
-    for (int i = threadIdx.x; i < nw; i += kNodeBlock) {
+    for (int i = threadIdx.x; i < nw; i += kNodeThreads) {
         const int64_t j = base + i;
         int8_t v = -1;
         if (j >= 0 && j + leaf_max < n && ss[i] == ss[i + leaf_max]) v = (int8_t)common_digits(sk[i], sk[i + leaf_max]);
         sw[i] = v;
     }
     __syncthreads();
-    const int64_t s = b0 + threadIdx.x;
-    int t = -1, d = 0;
-    if (s < n) {
-        const int i = threadIdx.x + leaf_max;  // smem index of body s
-        d = (s == 0 || ss[i] != ss[i - 1]) ? -1 : common_digits(sk[i - 1], sk[i]);
-        int W = -1;
-        const int i0 = s - leaf_max < 0 ? (int)(leaf_max - s) : 0;  // window clipped at body 0
-        for (int k = i0; k <= leaf_max; k++) W = max(W, (int)sw[threadIdx.x + k]);
-        t = min(W + 1, kMaxLevel);
-        delta[s] = (int8_t)d;
-        top[s] = (int8_t)t;
-        gref_at[s] = 0;
+    int d[kNodeRounds], t[kNodeRounds];
+#pragma unroll
+    for (int r = 0; r < kNodeRounds; r++) {
+        const int at = r * kNodeThreads + threadIdx.x;
+        const int64_t s = b0 + at;
+        t[r] = -1;
+        d[r] = 0;
+        if (s < n) {
+            const int i = at + leaf_max;  // smem index of body s
+            d[r] = (s == 0 || ss[i] != ss[i - 1]) ? -1 : common_digits(sk[i - 1], sk[i]);
+            int W = -1;
+            const int i0 = s - leaf_max < 0 ? (int)(leaf_max - s) : 0;  // window clipped at body 0
+            for (int k = i0; k <= leaf_max; k++) W = max(W, (int)sw[at + k]);
+            t[r] = min(W + 1, kMaxLevel);
+            delta[s] = (int8_t)d[r];
+            top[s] = (int8_t)t[r];
+            gref_at[s] = 0;
+        }
     }
-    block_depth(t, depth);
-    count_levels(d, t, cnt);
+    count_levels(d, t, cnt, depth);
 }
 
 // Exclusive scan of the counts in place, one pass; the total is the number of
@@ -389,17 +483,6 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_levels_tiled(const uint64_t
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 16;
 constexpr int kScanTile = kScanThreads * kScanItems;
-
-__device__ __forceinline__ uint32_t warp_incl(uint32_t x)
-{
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    return x;
-}
 
 // the block's exclusive scan of one value per thread (kScanThreads of them),
 // plus the sum of the tiles before this one; *total: this prefix + the tile
@@ -470,68 +553,106 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_levels(uint32_t* __restri
 // starts at or before s.  fam = 1 marks a node that follows a sibling (the
 // topmost one starting at its body), so the children of a cell are its first
 // child and the marked nodes right after it.  Counts follow bottom-up.
-__global__ void __launch_bounds__(kNodeBlock) k_emit_nodes(const uint64_t* __restrict__ keys,
-                                                           const int8_t* __restrict__ delta,
-                                                           const int8_t* __restrict__ top,
-                                                           const uint32_t* __restrict__ sys_of, int64_t n,
-                                                           const uint32_t* __restrict__ offs, const Info* info,
-                                                           uint32_t* __restrict__ lstart, NodeTables nt)
+__global__ void __launch_bounds__(kNodeThreads) k_emit_nodes(const uint64_t* __restrict__ keys,
+                                                             const int8_t* __restrict__ delta,
+                                                             const int8_t* __restrict__ top,
+                                                             const uint32_t* __restrict__ sys_of, int64_t n,
+                                                             const uint32_t* __restrict__ offs, const Info* info,
+                                                             uint32_t* __restrict__ lstart, NodeTables nt)
 {
     if (capacity_failed(info)) return;
-    __shared__ uint32_t wc[kNodeBlock / 32][kLevels];
+    __shared__ uint32_t wc[kNodeSets][kLevels];
+    __shared__ uint4 list[kNodeThreads / 32][64];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u, le = lt | (1u << lane);
-    const int64_t s = (int64_t)blockIdx.x * kNodeBlock + threadIdx.x;
-    const int d = s < n ? delta[s] : 0, t = s < n ? top[s] : -1;
+    const int64_t b0 = (int64_t)blockIdx.x * kNodeBlock;
+    int d[kNodeRounds], t[kNodeRounds];
+    uint64_t key[kNodeRounds];
+    uint32_t sy[kNodeRounds];
+#pragma unroll
+    for (int r = 0; r < kNodeRounds; r++) {
+        const int64_t s = b0 + r * kNodeThreads + threadIdx.x;
+        d[r] = s < n ? delta[s] : 0;
+        t[r] = s < n ? top[s] : -1;
+        key[r] = s < n ? keys[s] : 0ull;
+        sy[r] = s < n ? sys_of[s] : 0u;
+    }
     if (blockIdx.x == 0 && threadIdx.x <= kLevels)  // the first node of each level
         lstart[threadIdx.x] = threadIdx.x < kLevels ? offs[(int64_t)threadIdx.x * gridDim.x] : (uint32_t)info->M;
-    uint32_t mine = 0;
 #pragma unroll
-    for (int l = 0; l < kLevels; l++) {
-        const unsigned m = __ballot_sync(0xffffffffu, d < l && l <= t);
-        if (lane == l) mine = __popc(m);
+    for (int r = 0; r < kNodeRounds; r++) {
+        const uint32_t mine = set_levels(d[r], t[r]);
+        if (lane < kLevels) wc[r * (kNodeThreads / 32) + w][lane] = mine;
     }
-    if (lane < kLevels) wc[w][lane] = mine;
     __syncthreads();
-    if (threadIdx.x < kLevels) {
-        uint32_t run = offs[(int64_t)threadIdx.x * gridDim.x + blockIdx.x];
-        for (int k = 0; k < kNodeBlock / 32; k++) {
-            const uint32_t c = wc[k][threadIdx.x];
-            wc[k][threadIdx.x] = run;
-            run += c;
+    // a warp per level: the sets' counts -> the place of each set's first node
+    for (int l = w; l < kLevels; l += kNodeThreads / 32) {
+        static_assert(kNodeSets == 32, "a lane per set");
+        const uint32_t c = wc[lane][l];
+        wc[lane][l] = offs[(int64_t)l * gridDim.x + blockIdx.x] + warp_incl(c) - c;
+    }
+    __syncthreads();
+    // the warp's nodes pass through a list, so that 32 lanes write 32 records
+    // (a set has about a dozen, spread over its levels)
+    int cnt = 0;
+    auto flush = [&](int m) {  // the last m <= 32 nodes of the list
+        uint4 q = make_uint4(0u, 0u, 0u, 0u);
+        if (lane < m) q = list[w][cnt - m + lane];
+        cnt -= m;
+        const int from = q.x & 31, lv = (q.x >> 5) & 31, r = (q.x >> 11) & (kNodeRounds - 1);
+        uint64_t k = 0ull;
+        uint32_t ky = 0u;
+#pragma unroll
+        for (int u = 0; u < kNodeRounds; u++) {
+            const uint64_t ku = __shfl_sync(0xffffffffu, key[u], from);
+            const uint32_t su = __shfl_sync(0xffffffffu, sy[u], from);
+            if (u == r) {
+                k = ku;
+                ky = su;
+            }
         }
-    }
-    __syncthreads();
-    const int lhi = __reduce_max_sync(0xffffffffu, t);  // no level of the warp above it
-    const int llo = __reduce_min_sync(0xffffffffu, t >= 0 ? d : kMaxLevel) + 1;
-    if (lhi < llo) return;
-    const uint64_t key = s < n ? keys[s] : 0ull;
-    const uint32_t sy = s < n ? sys_of[s] : 0u;
-    uint32_t before = llo > 0 ? wc[w][llo - 1] : 0u;  // nodes of the level above up to body s
-    bool had = false;
-    uint32_t pos = 0;
-    int32_t par = -1;
-    for (int l = llo; l <= lhi + 1; l++) {
-        const bool here = l < kLevels && d < l && l <= t;
-        const unsigned m = __ballot_sync(0xffffffffu, here);
-        const uint32_t base = l < kLevels ? wc[w][l] : 0u;
-        const uint32_t p = base + __popc(m & lt);
-        if (had) {  // node (s, l - 1), whose first child is (s, l) if that exists
-            const int lv = l - 1, sh = 3 * (kMaxLevel - lv);
-            const uint64_t pfx = lv == 0 ? 0ull : (key >> sh);
+        __syncwarp();
+        if (lane < m) {
+            const uint32_t at = q.y;
+            const uint64_t pfx = lv == 0 ? 0ull : (k >> (3 * (kMaxLevel - lv)));
             const int c1 = 1 << (kMaxLevel - lv);
-            nt.b[pos] = make_int4((int)s, 0, here ? (int32_t)p : -1, lv);
-            nt.c[pos] = make_int4((int)(2 * compact3(pfx >> 2) + 1) * c1, (int)(2 * compact3(pfx >> 1) + 1) * c1,
-                                  (int)(2 * compact3(pfx) + 1) * c1, (int)sy);
-            nt.fam[pos] = lv == d + 1;
-            nt.parent[pos] = par;
-            nt.pend[pos] = 0u;
+            nt.b[at] = make_int4((int)b0 + r * kNodeThreads + w * 32 + from, 0, (int32_t)q.z, lv);
+            nt.c[at] = make_int4((int)(2 * compact3(pfx >> 2) + 1) * c1, (int)(2 * compact3(pfx >> 1) + 1) * c1,
+                                 (int)(2 * compact3(pfx) + 1) * c1, (int)ky);
+            nt.fam[at] = (uint8_t)((q.x >> 10) & 1u);
+            nt.parent[at] = (int32_t)q.w;
+            nt.pend[at] = 0u;
         }
-        par = l > 0 ? (int32_t)before - 1 : -1;
-        before = base + __popc(m & le);
-        pos = p;
-        had = here;
+    };
+#pragma unroll
+    for (int r = 0; r < kNodeRounds; r++) {
+        const uint32_t* place = wc[r * (kNodeThreads / 32) + w];
+        const int lhi = __reduce_max_sync(0xffffffffu, t[r]);  // the set's levels
+        const int llo = __reduce_min_sync(0xffffffffu, t[r] > d[r] ? d[r] : kMaxLevel) + 1;
+        if (lhi < llo) continue;
+        uint32_t before = llo > 0 ? place[llo - 1] : 0u;  // nodes of the level above up to body s
+        bool had = false;
+        uint32_t pos = 0;
+        int32_t par = -1;
+        for (int l = llo; l <= lhi + 1; l++) {
+            const bool here = l < kLevels && d[r] < l && l <= t[r];
+            const unsigned m = __ballot_sync(0xffffffffu, here), hm = __ballot_sync(0xffffffffu, had);
+            const uint32_t base = l < kLevels ? place[l] : 0u;
+            const uint32_t p = base + __popc(m & lt);
+            if (had)  // node (s, l - 1), whose first child is (s, l) if that exists
+                list[w][cnt + __popc(hm & lt)] =
+                    make_uint4((unsigned)lane | ((unsigned)(l - 1) << 5) | (l == d[r] + 2 ? 1024u : 0u) | ((unsigned)r << 11),
+                               pos, here ? p : 0xffffffffu, (uint32_t)par);
+            cnt += __popc(hm);
+            __syncwarp();
+            if (cnt >= 32) flush(32);
+            par = l > 0 ? (int32_t)before - 1 : -1;
+            before = base + __popc(m & le);
+            pos = p;
+            had = here;
+        }
     }
+    if (cnt > 0) flush(cnt);
 }
 
 // children of the cell whose first child is cf: cf and the marked nodes after it
@@ -797,16 +918,18 @@ __global__ void k_leaf_nodes(const float4* __restrict__ body, const int8_t* __re
         nt.dsum[2 * v] = make_float4(mh, Sh[0], Sh[1], Sh[2]);
         nt.dsum[2 * v + 1] = make_float4(ml, Sl[0], Sl[1], Sl[2]);
         if (CLIMB) {
-            for (int64_t u = v;;) {
-                const int32_t p = nt.parent[u];
+            for (int32_t p = nt.parent[v];;) {
                 if (p < 0) break;
                 const int4 pb = nt.b[p];  // (x, z and the level: written before this launch)
+                const int32_t up = nt.parent[p];
                 const int nch = family(nt.fam, pb.z, M);
-                __threadfence();  // this child's record before its arrival
-                if (atomicAdd(&nt.pend[p], 1u) + 1u < (uint32_t)nch) break;
-                __threadfence();  // the other children's arrivals before their records
+                // the arrival releases this child's record and, the last one,
+                // acquires the others'
+                uint32_t old;
+                asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(&nt.pend[p]) : "memory");
+                if (old + 1u < (uint32_t)nch) break;
                 level_node<QUAD, true>(p, pb, nch, sysp, nt);
-                u = p;
+                p = up;
             }
         }
     }
@@ -1092,19 +1215,26 @@ void launch_sys_ids(const int64_t* offsets, int nsys, int64_t n, uint32_t* sys_o
     count_launches(1);
 }
 
-void launch_bbox(const float* pos, const int4* chunks, int nchunks, SysParams* sysp, int nsys, int32_t* err,
-                 cudaStream_t s)
+void launch_build_init(uint4* zero, int64_t nzero, SysParams* sysp, int nsys, Info* info, bool reset_err,
+                       cudaStream_t s)
 {
-    k_bbox_init<<<nblk(nsys, 128), 128, 0, s>>>(sysp, nsys);
+    const int64_t m = nzero > nsys ? nzero : nsys;
+    k_build_init<<<gsgrid(m, 256), 256, 0, s>>>(zero, nzero, sysp, nsys, info, reset_err);
+    count_launches(1);
+}
+
+void launch_bbox(const float* pos, const int4* chunks, int nchunks, SysParams* sysp, int32_t* err, cudaStream_t s)
+{
     k_bbox<<<nchunks, kBboxThreads, 0, s>>>(pos, chunks, sysp, err);
-    k_sys_cube<<<nblk(nsys, 128), 128, 0, s>>>(sysp, nsys);
-    count_launches(3);
+    count_launches(1);
 }
 
 void launch_keys(const float* pos, const float* mass, int64_t n, const uint32_t* sys_of, const SysParams* sysp,
-                 uint64_t* keys, uint32_t* idx, int32_t* err, cudaStream_t s)
+                 uint64_t* keys, uint32_t* idx, const SortPlan& plan, uint32_t* ghist, int32_t* err, cudaStream_t s)
 {
-    k_keys<<<nblk(n, 256), 256, 0, s>>>(pos, mass, n, sys_of, sysp, keys, idx, err);
+    int64_t g = (n + 1023) / 1024;
+    if (g > 6 * sm_count()) g = 6 * sm_count();
+    k_keys<<<(unsigned)g, 256, 0, s>>>(pos, mass, n, sys_of, sysp, keys, idx, plan, ghist, err);
     count_launches(1);
 }
 
@@ -1130,11 +1260,11 @@ void launch_node_levels(const uint64_t* keys, const uint32_t* sys_of, int64_t n,
 {
     const unsigned nb = nblk(n, kNodeBlock);
     if (leaf_max <= kTileWindow) {
-        k_node_levels_tiled<<<nb, kNodeBlock, 0, s>>>(keys, sys_of, n, leaf_max, delta, top, gref_at, cnt, &info->depth);
+        k_node_levels_tiled<<<nb, kNodeThreads, 0, s>>>(keys, sys_of, n, leaf_max, delta, top, gref_at, cnt, &info->depth);
         count_launches(1);
     } else {
         k_window<<<nblk(n, 256), 256, 0, s>>>(keys, sys_of, n, leaf_max, w);
-        k_node_levels<<<nb, kNodeBlock, 0, s>>>(keys, sys_of, w, n, leaf_max, delta, top, gref_at, cnt, &info->depth);
+        k_node_levels<<<nb, kNodeThreads, 0, s>>>(keys, sys_of, w, n, leaf_max, delta, top, gref_at, cnt, &info->depth);
         count_launches(2);
     }
     const int64_t nc = level_counts_size(n);
@@ -1146,7 +1276,7 @@ void launch_node_levels(const uint64_t* keys, const uint32_t* sys_of, int64_t n,
 void launch_emit_nodes(const uint64_t* keys, const int8_t* delta, const int8_t* top, const uint32_t* sys_of, int64_t n,
                        const uint32_t* offs, const Info* info, uint32_t* lstart, NodeTables nt, cudaStream_t s)
 {
-    k_emit_nodes<<<nblk(n, kNodeBlock), kNodeBlock, 0, s>>>(keys, delta, top, sys_of, n, offs, info, lstart, nt);
+    k_emit_nodes<<<nblk(n, kNodeBlock), kNodeThreads, 0, s>>>(keys, delta, top, sys_of, n, offs, info, lstart, nt);
     count_launches(1);
 }
 

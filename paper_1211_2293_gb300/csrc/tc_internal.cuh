@@ -15,7 +15,8 @@ namespace tc {
 
 constexpr int kMaxLevel = 21;      // 21 bits per axis, 63-bit Morton keys
 constexpr int kLeafMaxLimit = 4096;
-constexpr int kBboxChunk = 4096;   // bodies per bounding-box block (never across systems)
+constexpr int kBboxChunk = 4096;   // bodies per bounding-box block (never across systems) ...
+constexpr int kBboxChunkSmall = 1024;  // ... of up to 2^19 bodies
 
 // error bits of the device error word
 enum : int32_t {
@@ -43,7 +44,7 @@ struct SysParams {
     int32_t end;
     int32_t bb[6];     // bounding box as order-preserving ints: lo xyz, hi xyz
     float msys;        // total mass (for the learned correction's features)
-    int32_t pad;
+    int32_t done;      // bounding-box chunks of the system that are done
 };
 
 // Per-context scalars kept in device memory (written by kernels, read by
@@ -82,21 +83,16 @@ struct NodeTables {
     uint32_t* pend;  // children of an internal cell that are done (bottom-up in one launch)
 };
 
-// scratch of the radix sort / scans
+// scratch of the radix sort
 struct SortBufs {
     uint64_t* keys_alt;
     uint32_t* vals_alt;
-    uint32_t* ghist;                 // passes x 256 digit counts -> exclusive offsets
+    uint32_t* ghist;                 // passes x 256 digit counts
     unsigned long long* status;      // look-back words, passes x tiles x 256
     uint32_t* tiles;                 // tile counters, one per pass
     int32_t* err;                    // device error word (bounded look-back)
-    // a sort of the keys' top bits only: the starts of runs of equal top bits
-    // longer than the per-thread completion takes (capacity run_cap), their count
-    int64_t* runs = nullptr;
-    unsigned long long* nruns = nullptr;
-    int64_t run_cap = 0;
 };
-constexpr int kSortMaxPasses = 10;   // 8 key passes + up to 2 system passes
+constexpr int kSortMaxPasses = 10;   // 63 key bits + up to 16 system bits
 
 // ---------------------------------------------------------------- launchers
 // all launches go on `s`; none synchronises.  Every launcher adds the number
@@ -109,35 +105,85 @@ int sm_count();
 // records the reason of a failure outside any context (tc_last_error(NULL))
 void set_thread_error(const char* msg);
 
-// Stable LSD radix sort of (key, val) by bits [0, nbits) of key, then (if
-// sys_bits > 0) by the system of each value's body, sys_of[val], so the
-// result is ordered by (system, key).  Afterwards b.ghist[p * 256 + d] is
-// the number of items whose pass-p digit is below d.
-// low_bit > 0 (needs b.runs): the passes sort bits [low_bit, nbits) only
-// (8-bit digits from low_bit up), then every run of items with equal top bits (and
-// system) is put in (key, val) order by a per-run completion, so the
-// result is the same as the full sort's whenever the values are distinct
-// (the bodies' indices); a run longer than run_max (at most kSortRunMax)
-// raises kErrSortRun and kErrCapacity instead.
+// One 8-bit digit of the sort's order: the bits of (system, key >> low_bit)
+// taken as one number, the system above the kb key bits.
+struct SortDigit {
+    int kshift;   // right shift of the key (past its bits for the topmost digits)
+    int sys;      // 1: the digit holds bits of the system
+    int sleft;    // left shift of the system (where key bits share the digit), else
+    int sright;   // right shift
+    __host__ __device__ uint32_t of(uint64_t key, uint32_t system) const
+    {
+        const uint32_t k = kshift < 64 ? (uint32_t)(key >> kshift) : 0u;
+        return (sys ? (k | ((system << sleft) >> sright)) : k) & 255u;
+    }
+};
+// The passes of a sort by the key bits [low_bit, nbits) and then sys_bits
+// bits of the system: as few digits as hold them together.
+struct SortPlan {
+    int npass, low_bit, kb, sys_bits;
+    static SortPlan make(int nbits, int low_bit, int sys_bits)
+    {
+        const int kb = nbits - low_bit;
+        return SortPlan{(kb + sys_bits + 7) / 8, low_bit, kb, sys_bits};
+    }
+    __host__ __device__ SortDigit digit(int p) const
+    {
+        SortDigit d;
+        d.kshift = 8 * p < kb ? low_bit + 8 * p : 64;
+        d.sys = sys_bits > 0 && 8 * p + 8 > kb;
+        d.sleft = d.sys && 8 * p < kb ? kb - 8 * p : 0;
+        d.sright = d.sys && 8 * p > kb ? 8 * p - kb : 0;
+        return d;
+    }
+};
+
+// The passes of a plan from (ka, va) to (kb, vb) and back, n >= 2 items; the
+// result lies in (ka, va) after an even number of passes.  b.ghist holds the
+// digit counts of every pass; b.tiles and radix_status_words(n, npass) words
+// of b.status are zero.
+void launch_sort_passes(uint64_t* ka, uint32_t* va, uint64_t* kb, uint32_t* vb, int64_t n, const SortPlan& plan,
+                        const uint32_t* sys_of, const SortBufs& b, cudaStream_t s);
+int64_t radix_status_words(int64_t n, int npass);
+int64_t radix_status_words(int64_t n);  // enough for any sort of up to n items
+// After passes over bits [low_bit, 63): every run of items with equal top
+// bits (and system; sys_of null: one system) in (key, val) order, which is
+// the full sort's order as the values are distinct (the bodies' indices),
+// and body[] in it.  A run longer than run_max (at most kSortRunMax) raises
+// kErrSortRun and kErrCapacity instead.
 constexpr int64_t kSortRunMax = 16384;
-void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int nbits, const uint32_t* sys_of,
-                    int sys_bits, SortBufs& b, cudaStream_t s, int low_bit = 0, int64_t run_max = kSortRunMax);
 constexpr int64_t kSortRunMaxSynced = 1024;  // a synchronised build re-sorts every digit past this
 constexpr int kSortMarginLevels = 2;  // levels below the last synchronised depth a step's sort orders
-int64_t radix_tiles(int64_t n);  // tiles of one pass (status words: 256 per tile per pass)
+void launch_sort_runs(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout, int64_t n,
+                      int low_bit, const uint32_t* sys_of, const float* pos, const float* mass, float4* body,
+                      int64_t run_max, int32_t* err, cudaStream_t s);
+// Up to kBlockSortMax items: the passes, the completion (low_bit > 0) and the
+// bodies in one launch of one block; no digit counts or scratch needed.
+constexpr int64_t kBlockSortMax = 4096;
+void launch_sort_block(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout, int64_t n,
+                       const SortPlan& plan, const uint32_t* sys_of, const float* pos, const float* mass, float4* body,
+                       int64_t run_max, int32_t* err, cudaStream_t s);
+// A whole sort of (key, val) by bits [0, nbits) of key, in place.
+void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int nbits, SortBufs& b, cudaStream_t s);
 // self-test of the radix pass's bounded look-back (see tc_sort.cu)
 cudaError_t sort_wait_selftest(uint64_t* keys, uint32_t* vals, uint64_t* kout, uint32_t* vout,
-                               unsigned long long* status, uint32_t* counter, uint32_t* goff, int32_t* err,
+                               unsigned long long* status, uint32_t* counter, uint32_t* hist, int32_t* err,
                                cudaStream_t s);
 int64_t sort_selftest_items();
 
 // build pieces
 void launch_sys_ids(const int64_t* offsets, int nsys, int64_t n, uint32_t* sys_of, SysParams* sysp,
                     cudaStream_t s);
-void launch_bbox(const float* pos, const int4* chunks, int nchunks, SysParams* sysp, int nsys, int32_t* err,
-                 cudaStream_t s);
+// start of a build: nzero 16-byte words of scratch zeroed, info->depth (and,
+// reset_err, info->err) too, the bounding boxes emptied
+void launch_build_init(uint4* zero, int64_t nzero, SysParams* sysp, int nsys, Info* info, bool reset_err,
+                       cudaStream_t s);
+// bounding boxes, and each system's root cube once its last chunk is done;
+// chunks: (system, start, end, chunks of the system)
+void launch_bbox(const float* pos, const int4* chunks, int nchunks, SysParams* sysp, int32_t* err, cudaStream_t s);
+// Morton keys, indices and (ghist not null) the digit counts of the plan's passes
 void launch_keys(const float* pos, const float* mass, int64_t n, const uint32_t* sys_of, const SysParams* sysp,
-                 uint64_t* keys, uint32_t* idx, int32_t* err, cudaStream_t s);
+                 uint64_t* keys, uint32_t* idx, const SortPlan& plan, uint32_t* ghist, int32_t* err, cudaStream_t s);
 void launch_gather(const float* pos, const float* mass, const uint32_t* perm, int64_t n,
                    float4* body, cudaStream_t s);
 // The levels of the cubes that start at each sorted body (delta < l <= top),

@@ -983,7 +983,7 @@ void launch_pair_order(int32_t* pb, int32_t* pv, int64_t np, uint64_t* keys, uin
     if (g > 8 * sm_count()) g = 8 * sm_count();
     k_pair_keys<<<(unsigned)(g < 1 ? 1 : g), 256, 0, s>>>(pb, pv, np, keys, vals);
     count_launches(1);
-    radix_sort_u64(keys, vals, np, 63, nullptr, 0, b, s);
+    radix_sort_u64(keys, vals, np, 63, b, s);
     k_pair_unkey<<<(unsigned)(g < 1 ? 1 : g), 256, 0, s>>>(keys, np, pb, pv);
     count_launches(1);
 }
