@@ -84,6 +84,9 @@ struct tc_ctx {
     // bodies, goes to the kernel with 2^k bodies per lane
     int32_t* gorder = nullptr;  // the groups in the order they are walked
     int32_t* gseg = nullptr;    // 4 range ends of its size classes, then the ordering's scratch
+    int32_t* part_done = nullptr;  // split walk: parts of each group done
+    float* part_sum = nullptr;
+    int64_t cap_part = 0;
     bool gorder_ready = false;  // the order is that of the current groups
     int walk_ncls = 0;
     int depth_hint = -1;  // tree depth of the last build the host saw (-1: none)
@@ -320,6 +323,7 @@ int ensure_bodies(tc_ctx* c, int64_t n)
     TC_GROW(c, c->nbody, cap);
     TC_GROW(c, c->hash, cap);
     TC_GROW(c, c->gorder, cap);
+    TC_GROW(c, c->part_done, cap);
     TC_GROW(c, c->gseg, 4 + (int64_t)group_order_scratch());
     c->cap_n = cap;
     c->cap_m = 0;  // node tables are sized with the first build at this capacity
@@ -369,6 +373,8 @@ int check_device(tc_ctx* c)
     int32_t e = c->info_h->err;
     if (e) {
         TC_CUDA(c, cudaMemsetAsync(&c->info->err, 0, sizeof(int32_t), c->stream));
+        // a walk whose wait gave up leaves its groups' counts
+        if (c->part_done) TC_CUDA(c, cudaMemsetAsync(c->part_done, 0, c->cap_n * sizeof(int32_t), c->stream));
         TC_CUDA(c, cudaStreamSynchronize(c->stream));
         if (e & kErrNonFinite)
             return fail(c, TC_EINVAL, "input holds a non-finite coordinate or a non-positive/non-finite mass");
@@ -541,7 +547,7 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
     launch_emit_nodes(c->keys, c->delta, c->top, c->sys_of, n, c->lcnt, c->info, c->lstart, c->nt, s);
     launch_moments(c->body, c->delta, n, c->nsys, c->cap_m, depth, c->depth_hint, c->lstart, c->sysp, c->info, c->nt,
                    c->cfg.quad != 0, s);
-    launch_groups(c->cap_m, c->info, c->nt, c->cfg.gmax, n, c->gref_at, c->scan, c->gfirst, c->gref, s);
+    launch_groups(c->cap_m, c->info, c->nt, c->cfg.gmax, n, c->gref_at, c->scan, c->gfirst, c->gref, c->part_done, s);
     c->gorder_ready = false;
     TC_CUDA(c, cudaGetLastError());
     phase_end(c, 0, t0, s);
@@ -550,22 +556,24 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
     return TC_OK;
 }
 
-// Consumer warps per producer of the split walk.  With many groups one: a
-// list takes about as long to walk as to sum.  With few, the walk waits for
-// its longest list (packed siblings whose box spans a dense octant list most
-// of a small system), which then several consumers sum together: seven while
-// every group finds a team of eight warps at once (two per SM), three up to a
-// few rounds of the half-size teams (Plummer spheres, theta 0.6, walk in us
-// with 1 / 3 / 7 consumers: 2000 bodies 58 / 39 / 38, 16000 347 / 205 / 224,
-// 50000 130 / 124 / 177, 70000 132 / 156 / 238).  A rule on n and gmax only
-// (a group holds about 0.7 gmax bodies), so a captured step and a direct
-// call sum alike.
-int walk_consumers(int64_t n, int gmax, int num_sms)
+// Parts per group of the split walk (log2): as many as 20 tasks per SM give
+// work to (eight teams run on one), at most eight.  Walk of Plummer spheres at
+// theta 0.5, us, with 1 / 2 / 4 / 8 / 16 parts: 1000 bodies 38 / 35 / 30 / 27
+// / 26, 4096 86 / 55 / 40 / 38 / 45, 10000 185 / 113 / 73 / 55 / 69, 16000 357
+// / 203 / 122 / 101 / 101, 30000 140 / 88 / 96 / 113, 50000 149 / 128 / 144,
+// 70000 159 / 169 / 182, 10^6 1751 / 1868 / 2126: with many groups the cells
+// that all parts walk and the shorter tiles are lost time.  A rule on n, the
+// systems and gmax only (a group holds about 0.7 gmax bodies), so a captured
+// step and a direct call sum alike.  A stack set below the default is kept as
+// the limit of whole walks.
+constexpr int kDefaultStack = 1024;
+int walk_parts(const tc_ctx* c)
 {
-    const double groups = (double)n / (0.7 * gmax);
-    if (groups <= 2.0 * num_sms) return 7;
-    if (groups <= 8.0 * num_sms) return 3;
-    return 1;
+    if (c->cfg.stack < kDefaultStack) return 0;
+    const double groups = std::max((double)c->n / (0.7 * c->cfg.gmax), (double)c->nsys);
+    int log2 = 0;
+    while (log2 < 3 && groups * (2 << log2) <= 20.0 * c->num_sms) log2++;
+    return log2;
 }
 
 int prepare_forces(tc_ctx* c)
@@ -587,7 +595,15 @@ int prepare_forces(tc_ctx* c)
     // one launch per size class: one warp per group only (the split walk
     // lays each group out over its lanes by its own size)
     wc.classes = (c->cfg.gmax > 32 && !wc.split) ? c->cfg.classes : 0;
-    wc.consumers = wc.split ? walk_consumers(c->n, c->cfg.gmax, c->num_sms) : 0;
+    wc.part_log2 = wc.split ? walk_parts(c) : 0;
+    if (wc.part_log2) {
+        const int64_t want = ((int64_t)8 << wc.part_log2) * c->n;
+        if (want > c->cap_part) {
+            TC_GROW(c, c->part_sum, want);
+            c->cap_part = want;
+            drop_graph(c);
+        }
+    }
     int64_t st = c->cfg.stack;
     if (c->cap_m < st) st = c->cap_m < 32 ? 32 : c->cap_m;  // a stack of M entries cannot overflow
     st = (st + 3) & ~(int64_t)3;                            // keeps every warp's tiles 16-byte aligned
@@ -676,12 +692,26 @@ int run_forces(tc_ctx* c, float theta, float eps, float G, cudaStream_t s)
         cudaMemsetAsync(c->gcorr, 0, 3 * c->band_gcap * sizeof(float), s);
     }
     // groups ordered by layout where a size-class launch walks a range of
-    // them, or where the split walk has many of them
-    const bool ordered = c->walk_ncls > 0 || (c->walk_cfg.split && c->walk_cfg.consumers == 1);
+    // them, or where the split walk has several for an SM (Plummer spheres of
+    // 4096 / 10000 / 16000 bodies, in tree order and ordered: 38 / 69 / 120 and
+    // 36 / 55 / 101 us, the ordering itself 5)
+    const bool ordered =
+        c->walk_ncls > 0 || (c->walk_cfg.split && (double)c->n / (0.7 * c->cfg.gmax) > (double)c->num_sms);
     if (ordered) {
         if (!c->gorder_ready) launch_group_order(c->gfirst, c->info, c->gorder, c->gseg, c->gseg + 4, s);
         c->gorder_ready = true;
         a.glist = c->gorder;
+    }
+    if (c->walk_cfg.part_log2) {
+        a.part_log2 = c->walk_cfg.part_log2;
+        a.part_sum = c->part_sum;
+        a.part_done = c->part_done;
+        a.part_stride = c->n;
+        if (c->cfg.verify) {  // the parts add to their group's records
+            TC_CUDA(c, cudaMemsetAsync(c->ncell, 0, c->n * sizeof(int32_t), s));
+            TC_CUDA(c, cudaMemsetAsync(c->nbody, 0, c->n * sizeof(int32_t), s));
+            TC_CUDA(c, cudaMemsetAsync(c->hash, 0, c->n * sizeof(unsigned long long), s));
+        }
     }
     if (c->walk_ncls == 0) {
         e = launch_walk(a, c->walk_cfg, c->walk_grid, c->walk_smem, s);
@@ -839,7 +869,7 @@ int tc_create(tc_ctx** out, void* stream)
     c->cfg.precise = 1;
     c->cfg.want_pot = 0;
     c->cfg.verify = 0;
-    c->cfg.stack = 1024;
+    c->cfg.stack = kDefaultStack;
     c->cfg.blocks_per_sm = 0;
     c->cfg.quad = 0;
     c->cfg.tile = 128;

@@ -1026,7 +1026,7 @@ __global__ void k_group_marks(const Info* info, const NodeTables nt, int gmax, i
 __global__ void __launch_bounds__(kScanThreads) k_group_table(const int32_t* __restrict__ gref_at, int64_t n,
                                                               unsigned long long* st, uint32_t* counter,
                                                               int32_t* __restrict__ gfirst, int32_t* __restrict__ gref,
-                                                              Info* info)
+                                                              int32_t* __restrict__ part_done, Info* info)
 {
     __shared__ int tile_sh;
     __shared__ int32_t mark[kScanTile];
@@ -1053,6 +1053,7 @@ __global__ void __launch_bounds__(kScanThreads) k_group_table(const int32_t* __r
         const int i = threadIdx.x * kScanItems + __ffs(has) - 1;
         gfirst[g] = (int32_t)(t0 + i);
         gref[g] = mark[i] - 1;
+        part_done[g] = 0;
     }
     if (tile == gridDim.x - 1 && threadIdx.x == 0) {
         gfirst[total] = (int32_t)n;
@@ -1325,12 +1326,12 @@ void launch_moments(const float4* body, const int8_t* delta, int64_t n, int nsys
 }
 
 void launch_groups(int64_t cap_m, Info* info, const NodeTables nt, int gmax, int64_t n, int32_t* gref_at,
-                   unsigned long long* scan, int32_t* gfirst, int32_t* gref, cudaStream_t s)
+                   unsigned long long* scan, int32_t* gfirst, int32_t* gref, int32_t* part_done, cudaStream_t s)
 {
     k_group_marks<<<gsgrid(cap_m, 128), 128, 0, s>>>(info, nt, gmax, gref_at);
     uint32_t* counters = reinterpret_cast<uint32_t*>(scan + build_scan_words(n) - 1);
     k_group_table<<<(unsigned)scan_tiles(n), kScanThreads, 0, s>>>(
-        gref_at, n, scan + scan_tiles(level_counts_size(n)), counters + 1, gfirst, gref, info);
+        gref_at, n, scan + scan_tiles(level_counts_size(n)), counters + 1, gfirst, gref, part_done, info);
     count_launches(2);
 }
 

@@ -212,7 +212,7 @@ void launch_moments(const float4* body, const int8_t* delta, int64_t n, int nsys
                     bool quad, cudaStream_t s);
 // the body groups: gfirst[0..G], gref[0..G), info->G
 void launch_groups(int64_t cap_m, Info* info, const NodeTables nt, int gmax, int64_t n, int32_t* gref_at,
-                   unsigned long long* scan, int32_t* gfirst, int32_t* gref, cudaStream_t s);
+                   unsigned long long* scan, int32_t* gfirst, int32_t* gref, int32_t* part_done, cudaStream_t s);
 // the groups by the walk's layout of their bodies (kGroupClasses of them),
 // the largest first, stable: order[0, G); seg[0..3] = the ranges of groups of
 // more than 64, 33 to 64 and up to 32 bodies in it; scratch holds
@@ -264,6 +264,13 @@ struct WalkArgs {
     const int32_t* glist;
     const int32_t* gseg;
     int work_slot;  // this launch's work-queue counter, info->work[work_slot]
+    // split walk: 2^part_log2 parts per group; a part's compensated sums in
+    // part_sum[((8 part) + 2 component (+ 1: compensation)) part_stride + body],
+    // the parts done so far in part_done[group] (zero before and after)
+    int part_log2;
+    float* part_sum;
+    int32_t* part_done;
+    int64_t part_stride;
     // learned correction evaluated after the walk (split walk): the band
     // cells of every group recorded as (node, group) pairs in chunks of
     // kBandChunk entries taken from *band_n (unused tails hold node -1), at
@@ -289,7 +296,7 @@ struct WalkConfig {
     int quadw;        // 1: accepted cells add their quadrupole term (precise mode)
     int classes;      // 1: one launch per group size class (the smaller beside the largest); 0: one launch
     int split;        // 1: monopole walks on producer/consumer warps (k_walk_ws)
-    int consumers;    // split: consumer warps per producer (1, 3 or 7; as many as `warps` has room for)
+    int part_log2;    // split: each group is walked in 2^part_log2 parts
 };
 // host-side preparation of the walk kernel's launch (attributes, occupancy);
 // call before a stream capture

@@ -38,13 +38,19 @@
 // 0.78 -> 0.86 / 0.89.  The slices' compensated sums are added at the end of
 // the group by TwoSum.
 //
-// Consumers per team.  C = 1 fills the machine when there are many groups:
-// walking a list costs about as long as summing it.  With few groups the
-// longest list is what a walk waits for (a group of packed siblings whose
-// box spans a dense octant lists most of a small system), so the consumers
-// of a team share it: warp c takes every C-th round of each tile and the
-// C sums are added in order at the end.  walk_consumers (tc_api.cu) states
-// the rule.
+// Parts of a group.  With few groups the longest list is what a walk waits
+// for (a group of packed siblings whose box spans a dense octant lists most
+// of a small system: 16000 bodies, 357 us on a team while the chip idles).
+// Then every group is walked in P parts, a task each.  All parts walk the
+// cells that hold more than a 64th of the system, and of what is below those
+// each takes every P-th cell, by its place (sharing out the stack after
+// some steps instead left one part the dense core that most of a Plummer
+// sphere's lists lie in: 317 us).  A part leaves its compensated
+// sums in memory; the one that ends last adds them in the parts' order, so
+// the sums don't depend on which it is.  Walk of Plummer spheres at theta
+// 0.5, us, with the consumers of a team sharing its list as before / with
+// parts: 4096 bodies 81 / 38, 10000 171 / 55, 16000 205 / 100, 50000 130 /
+// 128.  walk_parts (tc_api.cu) states the rule.
 //
 // Tiles.  The four planes x, y, z, m of a tile are contiguous: 32 lanes
 // store 32 entries without bank conflicts (pair-interleaved entries of four
@@ -82,7 +88,8 @@ struct WsHdr {
     int32_t flags;  // kWs*
     int32_t n;      // entries, padded to a multiple of 16 with massless ones
     int32_t gfirst, gend;
-    int32_t pad[4];
+    int32_t group, part;
+    int32_t pad[2];
     double ref[3];  // centre of the group's reference cube (absolute, FP64)
     double pad2;
 };
@@ -91,19 +98,19 @@ enum : int32_t { kWsFirst = 1, kWsLast = 2, kWsDone = 4, kWsAbort = 8, kWsBodies
 
 // One team's shared memory: barriers and slot numbers (128 bytes), the ring,
 // the walk stack (first child and number of children of each opened cell),
-// the opened leaves, each consumer's body positions (absolute and
-// reference-relative) and, with C > 1, the consumers' sums (two groups in
-// turn).  nb: body slots of a group (64, or 128 for gmax 128).
+// the opened leaves, the consumer's body positions (absolute and
+// reference-relative).  nb: body slots of a group (64, or 128 for gmax 128).
 __host__ __device__ constexpr size_t ws_slot_bytes(int tile) { return sizeof(WsHdr) + (size_t)4 * ws_cap(tile) * 4; }
 __host__ __device__ constexpr size_t ws_pos_bytes(int nb) { return (size_t)6 * nb * 4; }
-__host__ __device__ constexpr size_t ws_comb_bytes(int C, int nb) { return C > 1 ? (size_t)2 * C * 8 * nb * 4 : 0; }
+constexpr int kWsShared = 128;     // of a stack entry's number of children: all parts walk it
+constexpr int kWsSharedFrac = 64;  // cells of more than this fraction of a system (16 to 128 measure alike)
 constexpr int kWsLeaves = 96;  // opened leaves: up to 31 left over + 64 of a step
-__host__ __device__ constexpr size_t ws_team_bytes(int tile, int stack, int C, int nb)
+__host__ __device__ constexpr size_t ws_team_bytes(int tile, int stack, int nb)
 {
     return 128 + ws_slots(tile) * ws_slot_bytes(tile) + (size_t)stack * 4 + ((stack + 15) & ~15) + kWsLeaves * 8 +
-           32 * 4 + C * ws_pos_bytes(nb) + ws_comb_bytes(C, nb);
+           32 * 4 + ws_pos_bytes(nb);
 }
-static_assert(2 * 8 * ws_slots(64) + 8 + 4 * ws_slots(64) <= 128 && 2 * 8 * ws_slots(256) + 8 + 4 * ws_slots(256) <= 128,
+static_assert(2 * 8 * ws_slots(64) + 4 * ws_slots(64) <= 128 && 2 * 8 * ws_slots(256) + 4 * ws_slots(256) <= 128,
               "a team's barriers and slot numbers");
 __host__ __device__ constexpr int ws_body_slots(int gmax) { return gmax > 64 ? 128 : 64; }
 
@@ -157,7 +164,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity)
 
 // what the warps of a team share
 struct WsTeam {
-    uint64_t *full, *empty, *comb_full;
+    uint64_t *full, *empty;
     int32_t* seq;
     unsigned char* slots;
     int slot_bytes;
@@ -168,13 +175,13 @@ struct WsTeam {
     }
 };
 
-// One group on one consumer warp (number c of C): positions from the warp's
-// shared-memory copy, K bodies per lane, S slices.  Starts at position k
+// One group, or part `part` of one (part < 0: whole), on one consumer warp:
+// positions from the warp's shared-memory copy, K bodies per lane, S slices.  Starts at position k
 // (whose full barrier has been waited for) and returns the position after
 // the group's last tile, or -1 when a wait ran out.
 template <int K, int S, int TILE, bool PRECISE, bool POT>
-__device__ __forceinline__ int consume_group(const WsTeam& t, int k, int c, int C, const float* __restrict__ pos, int nb,
-                                             float* comb, int comb_phase, int gfirst, int ng, const WalkArgs& a)
+__device__ __forceinline__ int consume_group(const WsTeam& t, int k, const float* __restrict__ pos, int nb, int part,
+                                             int gfirst, int ng, const WalkArgs& a)
 {
     constexpr int L = 32 / S;                      // lanes of a slice
     constexpr int CAP = ws_cap(TILE);
@@ -208,14 +215,13 @@ __device__ __forceinline__ int consume_group(const WsTeam& t, int k, int c, int 
         const WsHdr* h = t.hdr(slot);
         flags = h->flags;
         const int rounds = (h->n >> 2) / S;        // n is a multiple of 4 S
-        const int mine = rounds > c ? (rounds - c + C - 1) / C : 0;
-        if (mine > 0) {
+        if (rounds > 0) {
             if (PRECISE) {
-                if (pairs + 2 * mine > kFold && pairs > 0) {
+                if (pairs + 2 * rounds > kFold && pairs > 0) {
                     fold();
                     pairs = 0;
                 }
-                pairs += 2 * mine;
+                pairs += 2 * rounds;
             }
             // cells are relative to the group's reference cube in the
             // precise mode, bodies absolute
@@ -228,9 +234,9 @@ __device__ __forceinline__ int consume_group(const WsTeam& t, int k, int c, int 
                 Y[b] = f2pack(y, y);
                 Z[b] = f2pack(z, z);
             }
-            const float* p = t.tile(slot) + 4 * (sl + S * c);
+            const float* p = t.tile(slot) + 4 * sl;
 #pragma unroll(kUnroll)
-            for (int r = 0; r < mine; r++, p += 4 * S * C) {
+            for (int r = 0; r < rounds; r++, p += 4 * S) {
                 const ulonglong2 xx = *reinterpret_cast<const ulonglong2*>(p);
                 const ulonglong2 yy = *reinterpret_cast<const ulonglong2*>(p + CAP);
                 const ulonglong2 zz = *reinterpret_cast<const ulonglong2*>(p + 2 * CAP);
@@ -280,42 +286,22 @@ __device__ __forceinline__ int consume_group(const WsTeam& t, int k, int c, int 
             if (POT) join(sp[b], cp[b]);
         }
     }
-    if (C > 1) {
-        // every consumer leaves its sums; once all have, they are added in
-        // the consumers' order
-        float* mineC = comb + (size_t)c * 8 * nb;
+    if (part >= 0) {
+        float* o = a.part_sum + (int64_t)part * 8 * a.part_stride + gfirst;
 #pragma unroll
         for (int b = 0; b < K; b++) {
             const int i = j + b * L;
-            if (b % S == sl) {
-                mineC[0 * nb + i] = sx[b];
-                mineC[1 * nb + i] = cx[b];
-                mineC[2 * nb + i] = sy[b];
-                mineC[3 * nb + i] = cy[b];
-                mineC[4 * nb + i] = sz[b];
-                mineC[5 * nb + i] = cz[b];
-                if (POT) {
-                    mineC[6 * nb + i] = sp[b];
-                    mineC[7 * nb + i] = cp[b];
-                }
+            if (b % S != sl || i >= ng) continue;
+            o[0 * a.part_stride + i] = sx[b];
+            o[1 * a.part_stride + i] = cx[b];
+            o[2 * a.part_stride + i] = sy[b];
+            o[3 * a.part_stride + i] = cy[b];
+            o[4 * a.part_stride + i] = sz[b];
+            o[5 * a.part_stride + i] = cz[b];
+            if (POT) {
+                o[6 * a.part_stride + i] = sp[b];
+                o[7 * a.part_stride + i] = cp[b];
             }
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(t.comb_full);
-        if (!mbar_wait(t.comb_full, comb_phase)) return -1;
-        if (flags & kWsAbort) return k;
-        constexpr int NV = POT ? 4 : 3;
-        for (int e = c * 32 + lane; e < NV * ng; e += C * 32) {
-            const int v = e / ng, i = e - v * ng;
-            float s = 0.f, comp = 0.f;
-            for (int cc = 0; cc < C; cc++) {
-                const float* o = comb + (size_t)cc * 8 * nb + (2 * v) * nb + i;
-                comp = __fadd_rn(comp, o[nb]);
-                two_sum_acc(s, comp, o[0]);
-            }
-            const int64_t o = a.perm[gfirst + i];
-            if (v < 3) a.acc[3 * o + v] = a.G * (s + comp);
-            else a.pot[o] = a.G * ((s + comp) + a.body[gfirst + i].w * rsqrtf(a.eps2));
         }
         return k;
     }
@@ -332,6 +318,42 @@ __device__ __forceinline__ int consume_group(const WsTeam& t, int k, int c, int 
         if (POT) a.pot[o] = a.G * ((sp[b] + cp[b]) + a.body[gfirst + i].w * rsqrtf(a.eps2));
     }
     return k;
+}
+
+// A part of group g has been summed (the sums are in memory): the warp of
+// the group's last part adds the parts' sums in their order.
+template <bool POT>
+__device__ __forceinline__ void add_parts(int g, int gfirst, int ng, const WalkArgs& a)
+{
+    const int lane = threadIdx.x & 31;
+    const int parts = 1 << a.part_log2;
+    __threadfence();  // each lane's sums before the count
+    __syncwarp();
+    int32_t done = 0;
+    if (lane == 0) done = atomicAdd(&a.part_done[g], 1);
+    done = __shfl_sync(0xffffffffu, done, 0);
+    if (done != parts - 1) return;
+    __threadfence();
+    if (lane == 0) a.part_done[g] = 0;  // for the next force phase on this tree
+    for (int i = lane; i < ng; i += 32) {
+        float s[POT ? 4 : 3], c[POT ? 4 : 3];
+#pragma unroll
+        for (int v = 0; v < (POT ? 4 : 3); v++) s[v] = c[v] = 0.f;
+        const float* o = a.part_sum + gfirst + i;
+        for (int p = 0; p < parts; p++, o += 8 * a.part_stride) {
+#pragma unroll
+            for (int v = 0; v < (POT ? 4 : 3); v++) {
+                c[v] = __fadd_rn(c[v], __ldcg(o + (2 * v + 1) * a.part_stride));
+                two_sum_acc(s[v], c[v], __ldcg(o + 2 * v * a.part_stride));
+            }
+        }
+        const int64_t b = a.perm[gfirst + i];
+        a.acc[3 * b + 0] = a.G * (s[0] + c[0]);
+        a.acc[3 * b + 1] = a.G * (s[1] + c[1]);
+        a.acc[3 * b + 2] = a.G * (s[2] + c[2]);
+        if (POT) a.pot[b] = a.G * ((s[POT ? 3 : 0] + c[POT ? 3 : 0]) + a.body[gfirst + i].w * rsqrtf(a.eps2));
+    }
+    __syncwarp();
 }
 
 // inclusive warp prefix sum, two instructions a step
@@ -351,7 +373,7 @@ __device__ __forceinline__ unsigned ws_incl_scan(unsigned x)
 // (k_band_eval) as (node, group) pairs, and each group's record (box centre
 // and frame)
 template <int TILE, bool PRECISE, bool POT, bool LEARNED>
-__global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a, int stack_cap, int C, int nb)
+__global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a, int stack_cap, int nb)
 {
     constexpr int kTile = TILE;
     constexpr int CAP = ws_cap(TILE);
@@ -359,32 +381,30 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    const int teams = (int)(blockDim.x >> 5) / (1 + C);
+    const int teams = (int)(blockDim.x >> 6);
     const bool producer = warp < teams;
-    const int team = producer ? warp : (warp - teams) / C;
-    const size_t team_bytes = ws_team_bytes(TILE, stack_cap, C, nb);
+    const int team = producer ? warp : warp - teams;
+    const size_t team_bytes = ws_team_bytes(TILE, stack_cap, nb);
     unsigned char* base = smem + (size_t)team * team_bytes;
     WsTeam t;
     t.full = reinterpret_cast<uint64_t*>(base);
     t.empty = t.full + kWsSlots;
-    t.comb_full = t.empty + kWsSlots;
-    t.seq = reinterpret_cast<int32_t*>(t.comb_full + 1);
+    t.seq = reinterpret_cast<int32_t*>(t.empty + kWsSlots);
     t.slots = base + 128;
     t.slot_bytes = (int)ws_slot_bytes(TILE);
     uint32_t* stk = reinterpret_cast<uint32_t*>(base + 128 + kWsSlots * ws_slot_bytes(TILE));
     int2* leaves = reinterpret_cast<int2*>(stk + stack_cap);  // first body, bodies
     int32_t* row = reinterpret_cast<int32_t*>(leaves + kWsLeaves);
     uint8_t* stn = reinterpret_cast<uint8_t*>(row + 32);
-    unsigned char* after = stn + ((stack_cap + 15) & ~15);
+    float* pos = reinterpret_cast<float*>(stn + ((stack_cap + 15) & ~15));
 
     const Info* info = a.info;
     if (info->err & kErrCapacity) return;  // the build stopped: no tree to walk (uniform: no barrier used yet)
     if (producer && lane == 0) {
         for (int s = 0; s < kWsSlots; s++) {
             mbar_init(&t.full[s], 1);
-            mbar_init(&t.empty[s], C);
+            mbar_init(&t.empty[s], 1);
         }
-        mbar_init(t.comb_full, C);
     }
     __syncthreads();
 
@@ -401,7 +421,9 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
         float *ctile = t.tile(0), *btile = t.tile(1);
         int cn = 0, bn = 0;     // their entries
         int first = kWsFirst;   // the group's next position is its first
-        int gfirst = 0, gend = 0;
+        int gfirst = 0, gend = 0, g = 0;
+        const int parts = 1 << a.part_log2;
+        int part = 0;
         double gx = 0, gy = 0, gz = 0;
         bool alive = true;
         // hands a slot's tile of n entries over (flags: kind, last, ...) and
@@ -422,6 +444,8 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                 if (first) {
                     h->gfirst = gfirst;
                     h->gend = gend;
+                    h->group = g;
+                    h->part = part;
                     h->ref[0] = gx;
                     h->ref[1] = gy;
                     h->ref[2] = gz;
@@ -490,9 +514,11 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
             }
         };
         while (alive) {
-            int g = 0;
-            if (lane == 0) g = (int)atomicAdd(&a.info->work[a.work_slot], 1u);
-            g = __shfl_sync(0xffffffffu, g, 0);
+            unsigned task = 0;
+            if (lane == 0) task = atomicAdd(&a.info->work[a.work_slot], 1u);
+            task = __shfl_sync(0xffffffffu, task, 0);
+            g = (int)(task >> a.part_log2);
+            part = (int)(task & (unsigned)(parts - 1));
             if (g >= G) {
                 first = 0;
                 close_cells(kWsDone);
@@ -551,7 +577,7 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                 flo[kk] = __shfl_sync(0xffffffffu, fb, kk);
                 fhi[kk] = __shfl_sync(0xffffffffu, fb, kk + 3);
             }
-            if (LEARNED && lane == 0) {
+            if (LEARNED && lane == 0 && part == 0) {
                 // the group's record: box centre, reference-relative (as
                 // k_walk forms it), and the frame the network's rows need
                 float xc[3];
@@ -566,17 +592,19 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
             const bool fast_side = ((__float_as_int(Lf) >> 23) & 255) > kMaxLevel + 1;
             bool overflow = false;
             int sp = 0;  // opened cells whose children are to be tested
+            int shared_min;  // all parts of a group walk cells of more bodies
             int ln = 0;  // opened leaves whose bodies are not listed yet
             {
                 // the system's root: holds every body, always opened
                 const int4 rb = nt.b[sysid];
+                shared_min = rb.y / kWsSharedFrac;
                 if ((rb.w >> 8) != 0) {
                     if (lane == 0) {
                         stk[0] = (uint32_t)rb.z;
-                        stn[0] = (uint8_t)(rb.w >> 8);
+                        stn[0] = (uint8_t)((rb.w >> 8) | (parts > 1 ? kWsShared : 0));
                     }
                     sp = 1;
-                } else {
+                } else if (part == 0) {
                     if (lane == 0) {
                         leaves[0] = make_int2(rb.x, rb.y);
                         if (list_stats) hsh = mix64(2ull * sysid + 2ull);
@@ -629,7 +657,7 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                 // lane are independent.
                 const int np = min(sp, 8);
                 sp -= np;
-                int v[2];
+                int v[2], stn8[2], push[2];
                 int4 nbd[2];
                 float4 src[2];
                 float band_e2[2];
@@ -637,7 +665,8 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
 #pragma unroll
                 for (int u = 0; u < 2; u++) {
                     const int e = slot8 + 4 * u;
-                    const bool have = e < np && child8 < (int)stn[sp + min(e, np - 1)];
+                    stn8[u] = (int)stn[sp + min(e, np - 1)];
+                    const bool have = e < np && child8 < (stn8[u] & 15);
                     v[u] = have ? (int)stk[sp + e] + child8 : (int)sysid;  // (the other lanes read a root's records)
                     nbd[u] = __ldg(&nt.b[v[u]]);
                     const float4 na = __ldg(&nt.a[v[u]]);
@@ -665,6 +694,18 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                     const bool open = have && !acc[u];
                     oint[u] = open && (nbd[u].w >> 8) != 0;
                     oleaf[u] = open && (nbd[u].w >> 8) == 0;
+                    push[u] = nbd[u].w >> 8;
+                    if (stn8[u] & kWsShared) {  // below a cell that all parts walk
+                        // (the cell's coordinates on its level's grid: siblings
+                        // differ, and a system's place in a batch is no matter)
+                        const int sh = kMaxLevel + 1 - (nbd[u].w & 255);
+                        const int own = (cc.x >> sh) + 2 * (cc.y >> sh) + 4 * (cc.z >> sh);
+                        const bool mine = (own & (parts - 1)) == part;
+                        acc[u] = acc[u] && mine;
+                        oleaf[u] = oleaf[u] && mine;
+                        if (nbd[u].y > shared_min) push[u] |= kWsShared;
+                        else oint[u] = oint[u] && mine;
+                    }
                 }
                 const unsigned om0 = __ballot_sync(0xffffffffu, oint[0]), om1 = __ballot_sync(0xffffffffu, oint[1]);
                 const unsigned lm0 = __ballot_sync(0xffffffffu, oleaf[0]), lm1 = __ballot_sync(0xffffffffu, oleaf[1]);
@@ -681,7 +722,7 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                     if (oint[u]) {
                         const int q = sp + (u ? no0 + __popc(om1 & lt) : __popc(om0 & lt));
                         stk[q] = (uint32_t)nbd[u].z;
-                        stn[q] = (uint8_t)(nbd[u].w >> 8);
+                        stn[q] = (uint8_t)push[u];
                     }
                     if (oleaf[u]) {
                         leaves[ln + (u ? nl0 + __popc(lm1 & lt) : __popc(lm0 & lt))] = make_int2(nbd[u].x, nbd[u].y);
@@ -742,9 +783,15 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                 atomicAdd(&a.info->interactions, (unsigned long long)gc * (unsigned long long)(Lc + Lb));
                 atomicAdd(&a.info->cells, (unsigned long long)gc * (unsigned long long)Lc);
                 atomicAdd(&a.info->bodies, (unsigned long long)gc * (unsigned long long)Lb);
-                if (a.ncell) a.ncell[g] = Lc;
-                if (a.nbody) a.nbody[g] = Lb;
-                if (a.hash) a.hash[g] = hsh;
+                if (parts > 1) {  // (zeroed before the launch)
+                    if (a.ncell) atomicAdd(&a.ncell[g], Lc);
+                    if (a.nbody) atomicAdd(&a.nbody[g], Lb);
+                    if (a.hash) atomicAdd(&a.hash[g], hsh);
+                } else {
+                    if (a.ncell) a.ncell[g] = Lc;
+                    if (a.nbody) a.nbody[g] = Lb;
+                    if (a.hash) a.hash[g] = hsh;
+                }
             }
             __syncwarp();
         }
@@ -753,10 +800,6 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
     }
 
     // ---------------------------------------------------------------- consumer
-    const int c = (warp - teams) % C;
-    float* pos = reinterpret_cast<float*>(after + (size_t)c * ws_pos_bytes(nb));
-    float* comb = reinterpret_cast<float*>(after + (size_t)C * ws_pos_bytes(nb));
-    int groups = 0;
     for (int k = 0;;) {
         bool ok = mbar_wait(&t.full[k % kWsSlots], (k / kWsSlots) & 1);
         if (ok) {
@@ -764,6 +807,7 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
             if (h->flags & kWsDone) return;
             const int gfirst = h->gfirst, ng = h->gend - h->gfirst;
             const double gx = h->ref[0], gy = h->ref[1], gz = h->ref[2];
+            const int g = h->group, part = a.part_log2 ? h->part : -1;
             // positions of every body slot (slots past the group repeat its
             // first body; their sums are dropped)
             const int slots = ng <= 32 ? 32 : (ng <= 64 ? 64 : nb);
@@ -778,10 +822,7 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                 pos[5 * nb + i] = (float)((double)q.z - gz);
             }
             __syncwarp();
-            float* cb = comb + (groups & 1) * (size_t)C * 8 * nb;
-            const int cph = groups & 1;
-            groups++;
-#define TC_WS_GROUP(K, S) consume_group<K, S, TILE, PRECISE, POT>(t, k, c, C, pos, nb, cb, cph, gfirst, ng, a)
+#define TC_WS_GROUP(K, S) consume_group<K, S, TILE, PRECISE, POT>(t, k, pos, nb, part, gfirst, ng, a)
             if (ng <= 16) k = TC_WS_GROUP(1, 2);
             else if (ng <= 32) k = TC_WS_GROUP(1, 1);
             else if (ng <= 40) k = TC_WS_GROUP(5, 4);
@@ -791,6 +832,7 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
             else k = TC_WS_GROUP(4, 1);
 #undef TC_WS_GROUP
             ok = k >= 0;
+            if (ok && part >= 0) add_parts<POT>(g, gfirst, ng, a);
         }
         if (!ok) {
             if (lane == 0) atomicOr(&a.info->err, kErrWorkLoop);
@@ -799,9 +841,9 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
     }
 }
 
-// a launch's team, block and shared memory
+// a launch's block and shared memory
 struct WsShape {
-    int C, threads, nb, stack;
+    int threads, nb, stack;
     size_t smem;
 };
 constexpr size_t kWsSmemMax = 227 * 1024;
@@ -809,18 +851,15 @@ constexpr size_t kWsSmemMax = 227 * 1024;
 __host__ __forceinline__ WsShape ws_shape(const WalkConfig& c, int tile)
 {
     WsShape w;
-    const int pairs = c.warps < 1 ? 1 : (c.warps > kWsMaxPairs ? kWsMaxPairs : c.warps);
-    w.C = c.consumers < 1 ? 1 : c.consumers;
-    while (w.C > 1 && (1 + w.C) > 2 * pairs) w.C = (w.C - 1) / 2;  // 7 -> 3 -> 1
-    const int teams = 2 * pairs / (1 + w.C);
-    w.threads = teams * (1 + w.C) * 32;
+    const int teams = c.warps < 1 ? 1 : (c.warps > kWsMaxPairs ? kWsMaxPairs : c.warps);
+    w.threads = teams * 64;
     w.nb = ws_body_slots(c.gmax);
     // a stack that leaves no room for the ring is cut (an entry stands for
     // all the children of a cell, so it holds several times as many nodes
     // as one entry per node)
     w.stack = (c.stack + 3) & ~3;
-    while (w.stack > 64 && ws_team_bytes(tile, w.stack, w.C, w.nb) * teams > kWsSmemMax) w.stack -= 16;
-    w.smem = ws_team_bytes(tile, w.stack, w.C, w.nb) * teams;
+    while (w.stack > 64 && ws_team_bytes(tile, w.stack, w.nb) * teams > kWsSmemMax) w.stack -= 16;
+    w.smem = ws_team_bytes(tile, w.stack, w.nb) * teams;
     return w;
 }
 
@@ -850,8 +889,9 @@ cudaError_t launch_ws_t(const WalkArgs& a, const WalkConfig& c, int grid, size_t
     // quadrupole terms (those run on k_walk); its learned walk records band cells
     if (a.list_cells || a.pair_body || a.gseg) return cudaErrorInvalidValue;
     if (LEARNED && (!a.band || !a.band_n || !a.grec)) return cudaErrorInvalidValue;
+    if (a.part_log2 && (!a.part_sum || !a.part_done)) return cudaErrorInvalidValue;
     const WsShape w = ws_shape(c, TILE);
-    k_walk_ws<TILE, PRECISE, POT, LEARNED><<<grid, w.threads, smem, s>>>(a, w.stack, w.C, w.nb);
+    k_walk_ws<TILE, PRECISE, POT, LEARNED><<<grid, w.threads, smem, s>>>(a, w.stack, w.nb);
     count_launches(1);
     return cudaGetLastError();
 }

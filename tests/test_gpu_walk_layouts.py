@@ -1,6 +1,5 @@
 """The split walk's body layouts (bodies per lane x list slices, chosen by a
-group's size) and its consumers per producer (chosen by n), at the sizes where
-either changes, against FP64 direct sums."""
+group's size) at the sizes where they change, against FP64 direct sums."""
 import numpy as np
 import pytest
 
@@ -35,8 +34,8 @@ def _check(ctx, p, m, off, eps, theta, pot):
 @pytest.mark.parametrize("gmax,repeat", [(64, 1), (64, 24), (64, 110), (128, 1), (128, 60)])
 @pytest.mark.parametrize("precise,pot,tile", [(1, 0, 128), (1, 1, 64), (0, 1, 256)])
 def test_group_sizes(gmax, repeat, precise, pot, tile):
-    """One group per system: every layout, with seven, three and one consumer
-    per producer as the bodies grow in number; theta = 0 sums every body."""
+    """One group per system: every layout, with eight, two and one part per
+    group as the bodies grow in number; theta = 0 sums every body."""
     from paper_1211_2293_gb300 import tc
 
     sizes = (EDGES64 if gmax == 64 else EDGES128) * repeat
@@ -51,8 +50,7 @@ def test_group_sizes(gmax, repeat, precise, pot, tile):
 @pytest.mark.parametrize("n", [700, 1500, 4000])
 @pytest.mark.parametrize("warps", [1, 2, 3, 4])
 def test_lists_of_many_tiles(n, warps):
-    """Groups whose list spans many tiles, shared by as many consumers as the
-    block has room for."""
+    """Groups whose list spans many tiles, with one to four teams in a block."""
     from paper_1211_2293_gb300 import tc
 
     p, _, m = inputs.plummer(n, seed=n, with_velocity=False)
