@@ -299,10 +299,10 @@ int tc_direct_static(const float *pos, const float *mass, int64_t n, const int64
  * one P2P.  theta >= 0 (0: every pair is P2P, the direct sum), eps > 0.
  * The accelerations replace the context's (tc_get_acc; no potential), and
  * tc_ctx_step refuses them (TC_ESTATE): a step integrates with the treecode.
- * Synchronises (it reads the tree's level ranges and checks its scratch).
+ * Synchronises (it checks the build before, and its scratch after).
  * Scratch is kept in the context and grows as needed: a pass whose lists
  * outgrew it is rerun.  TC_EDEVICE when a cell's refinement stack overflows
- * (2048 sources; theta far below 0.2 on strongly clustered bodies). */
+ * (some 2500 sources; theta far below 0.2 on strongly clustered bodies). */
 int tc_ctx_fmm(tc_ctx *ctx, float theta, float eps, float G);
 /* Pair counts of the last tc_ctx_fmm (M2L, P2P, self pairs of leaves
  * included) and two order-independent hashes of the pair sets: the sums

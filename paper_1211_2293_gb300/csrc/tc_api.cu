@@ -153,21 +153,19 @@ struct tc_ctx {
     // source lists (per node: offset and count into the pool of its level's
     // parity), per-warp slabs, counters, level starts
     bool forces_fmm = false;
-    int32_t* fmm_parent = nullptr;
     float* fmm_loc = nullptr;
     int64_t* fmm_off = nullptr;
-    int32_t* fmm_cnt = nullptr;
+    int32_t* fmm_cnt = nullptr;             // per node: list entries, then children done
     unsigned long long* fmm_rec = nullptr;  // 4 per node
     double* fmm_rad = nullptr;               // acceptance radii (FP64)
     int4* fmm_fnode = nullptr;               // 3 per node: the FMM's gathered cell records
     int64_t fmm_cap_m = 0;
-    int32_t* fmm_pool[2] = {nullptr, nullptr};
+    int32_t* fmm_pool = nullptr;
     int64_t fmm_pool_cap = 0;
     int32_t* fmm_slab = nullptr;
     int64_t fmm_slab_cap = 0;
     int64_t fmm_slab_warps = 0;
     unsigned long long* fmm_ctr = nullptr;
-    int64_t* fmm_lstart = nullptr;
     unsigned long long fmm_stats[4] = {0, 0, 0, 0};
     bool fmm_records = false;  // the last pass kept hashes and per-node records
 
@@ -1199,32 +1197,22 @@ int tc_ctx_fmm(tc_ctx* c, float theta, float eps, float G)
     if (!finite(G)) return fail(c, TC_EINVAL, "tc_fmm: G must be finite");
     int r = check_device(c);  // synchronises: the last build's node count, no pending error
     if (r) return r;
-    const int64_t M = c->info_h->M;
     cudaStream_t s = c->stream;
     if (c->fmm_cap_m < c->cap_m) {
-        TC_GROW(c, c->fmm_parent, c->cap_m);
         TC_GROW(c, c->fmm_loc, c->cap_m * fmm_loc_width());
         TC_GROW(c, c->fmm_off, c->cap_m);
-        TC_GROW(c, c->fmm_cnt, c->cap_m);
+        TC_GROW(c, c->fmm_cnt, 2 * c->cap_m);
         TC_GROW(c, c->fmm_rec, 4 * c->cap_m);
         TC_GROW(c, c->fmm_rad, c->cap_m);
         TC_GROW(c, c->fmm_fnode, 3 * c->cap_m);
         c->fmm_cap_m = c->cap_m;
     }
     if (!c->fmm_ctr) TC_GROW(c, c->fmm_ctr, 8);
-    if (!c->fmm_lstart) TC_GROW(c, c->fmm_lstart, kFmmLevelSlots);
-    launch_fmm_level_starts(c->info, c->cap_m, c->nt, c->fmm_lstart, s);
-    TC_CUDA(c, cudaGetLastError());
-    int64_t ls[kFmmLevelSlots];
-    TC_CUDA(c, cudaMemcpyAsync(ls, c->fmm_lstart, sizeof(ls), cudaMemcpyDeviceToHost, s));
-    TC_CUDA(c, cudaStreamSynchronize(s));
-    int depth = 0;
-    while (depth < kMaxLevel && ls[depth + 1] < M) depth++;
-    // the pools and slabs start at an estimate and grow to what an attempt
+    // the pool and slabs start at an estimate and grow to what an attempt
     // that overflowed them counted; the overflowing attempt is discarded
     // (TC_FMM_POOL / TC_FMM_SLAB, in entries, override the first estimate
     // of a context, to exercise the regrowth)
-    int64_t want_pool = std::max<int64_t>(c->fmm_pool_cap, 32 * c->cap_m + 65536);
+    int64_t want_pool = std::max<int64_t>(c->fmm_pool_cap, 64 * c->cap_m + 131072);
     int64_t want_slab = std::max<int64_t>(c->fmm_slab_cap, 4096);
     if (c->fmm_pool_cap == 0)
         if (const char* env = getenv("TC_FMM_POOL")) want_pool = std::max<long long>(1, atoll(env));
@@ -1234,8 +1222,7 @@ int tc_ctx_fmm(tc_ctx* c, float theta, float eps, float G)
     unsigned long long ctr[8];
     for (int attempt = 0;; attempt++) {
         if (want_pool > c->fmm_pool_cap) {
-            TC_GROW(c, c->fmm_pool[0], want_pool);
-            TC_GROW(c, c->fmm_pool[1], want_pool);
+            TC_GROW(c, c->fmm_pool, want_pool);
             c->fmm_pool_cap = want_pool;
         }
         const int64_t warps = fmm_slab_warps();
@@ -1245,8 +1232,7 @@ int tc_ctx_fmm(tc_ctx* c, float theta, float eps, float G)
             c->fmm_slab_warps = warps;
         }
         TC_CUDA(c, cudaMemsetAsync(c->fmm_ctr, 0, 8 * sizeof(unsigned long long), s));
-        TC_CUDA(c, cudaMemsetAsync(c->fmm_cnt, 0, c->cap_m * sizeof(int32_t), s));
-        TC_CUDA(c, cudaMemsetAsync(c->fmm_off, 0, c->cap_m * sizeof(int64_t), s));
+        TC_CUDA(c, cudaMemsetAsync(c->fmm_cnt, 0, 2 * c->cap_m * sizeof(int32_t), s));
         FmmLaunch p{};
         p.body = c->body;
         p.perm = c->perm;
@@ -1255,10 +1241,9 @@ int tc_ctx_fmm(tc_ctx* c, float theta, float eps, float G)
         p.info = c->info;
         p.err = &c->info->err;
         p.cap_m = c->cap_m;
-        p.parent = c->fmm_parent;
+        p.pend = reinterpret_cast<uint32_t*>(c->fmm_cnt + c->cap_m);
         p.loc = c->fmm_loc;
-        p.pool[0] = c->fmm_pool[0];
-        p.pool[1] = c->fmm_pool[1];
+        p.pool = c->fmm_pool;
         p.pool_cap = c->fmm_pool_cap;
         p.slab = c->fmm_slab;
         p.slab_cap = c->fmm_slab_cap;
@@ -1273,14 +1258,14 @@ int tc_ctx_fmm(tc_ctx* c, float theta, float eps, float G)
         p.theta = theta;
         p.eps = eps;
         p.G = G;
-        cudaError_t e = launch_fmm(p, ls, depth, s);
+        cudaError_t e = launch_fmm(p, s);
         if (e != cudaSuccess) return fail(c, TC_ECUDA, "fmm launch: %s", cudaGetErrorString(e));
         TC_CUDA(c, cudaMemcpyAsync(ctr, c->fmm_ctr, sizeof(ctr), cudaMemcpyDeviceToHost, s));
         TC_CUDA(c, cudaStreamSynchronize(s));
         TC_CUDA(c, cudaMemcpy(c->info_h, c->info, sizeof(Info), cudaMemcpyDeviceToHost));
         const int32_t err = c->info_h->err;
         const int32_t grow_bits = kErrFmmPool | kErrFmmSlab;
-        // a level that overflowed handed its children short lists, so deeper
+        // a cell that overflowed handed its children short lists, so deeper
         // levels may need more than this pass counted: grow at least 2x
         if ((err & grow_bits) && !(err & ~grow_bits) && attempt < 16) {
             TC_CUDA(c, cudaMemsetAsync(&c->info->err, 0, sizeof(int32_t), s));

@@ -383,16 +383,13 @@ void launch_direct(const float* pos, const float* mass, const uint32_t* sys_of, 
                    const int64_t* idx, int64_t n, int64_t ns, float eps2, float G, double* part, double* acc,
                    double* pot, cudaStream_t s);
 
-// fast multipole method (tc_fmm.cu).  Level starts: lstart[l] is the first
-// breadth-first index of level l, lstart[l] = M past the deepest level
-// (kFmmLevelSlots entries).  launch_fmm launches the parent table and one
-// kernel per level 0..depth; its scratch: loc (cap_m x fmm_loc_width()
-// floats), near_off / near_cnt (cap_m), two pools of pool_cap entries, a slab
-// of slab_cap entries for each of fmm_slab_warps() warps, ctr (8 counters:
-// pool fill per level parity, pool need, slab need, M2L pairs, P2P pairs and
-// their two hashes; zero the last six before the launch); rec: per node its
-// M2L and P2P pairs as target and their hashes.
-constexpr int kFmmLevelSlots = kMaxLevel + 3;
+// fast multipole method (tc_fmm.cu): the radii, then the walk of every cell.
+// Scratch: loc (cap_m x fmm_loc_width() floats), near_off, near_cnt and pend
+// (cap_m; the last two zero before the launch), a pool of pool_cap entries, a
+// slab of slab_cap entries for each of fmm_slab_warps() warps, ctr (8
+// counters: pool fill, tickets, pool need, slab need, M2L pairs, P2P pairs
+// and their two hashes; zero before the launch); rec: per node its M2L and
+// P2P pairs as target and their hashes.
 struct FmmLaunch {
     const float4* body;
     const uint32_t* perm;
@@ -401,9 +398,9 @@ struct FmmLaunch {
     const Info* info;
     int32_t* err;
     int64_t cap_m;
-    int32_t* parent;
+    uint32_t* pend;
     float* loc;
-    int32_t* pool[2];
+    int32_t* pool;
     int64_t pool_cap;
     int32_t* slab;
     int64_t slab_cap;
@@ -419,7 +416,6 @@ struct FmmLaunch {
 };
 int64_t fmm_slab_warps();
 int fmm_loc_width();
-void launch_fmm_level_starts(const Info* info, int64_t cap_m, NodeTables nt, int64_t* lstart, cudaStream_t s);
-cudaError_t launch_fmm(const FmmLaunch& p, const int64_t* lstart_h, int depth, cudaStream_t s);
+cudaError_t launch_fmm(const FmmLaunch& p, cudaStream_t s);
 
 }  // namespace tc
