@@ -366,8 +366,9 @@ int ensure_nodes(tc_ctx* c, int64_t M)
 // device error word -> status (synchronises); clears the word it reports
 int check_device(tc_ctx* c)
 {
+    // one wait for the stream and the word (pinned host memory)
+    TC_CUDA(c, cudaMemcpyAsync(c->info_h, c->info, sizeof(Info), cudaMemcpyDeviceToHost, c->stream));
     TC_CUDA(c, cudaStreamSynchronize(c->stream));
-    TC_CUDA(c, cudaMemcpy(c->info_h, c->info, sizeof(Info), cudaMemcpyDeviceToHost));
     int32_t e = c->info_h->err;
     if (e) {
         TC_CUDA(c, cudaMemsetAsync(&c->info->err, 0, sizeof(int32_t), c->stream));
@@ -944,8 +945,9 @@ int tc_set_stream(tc_ctx* c, void* stream)
     return TC_OK;
 }
 
-int tc_ctx_build_batch(tc_ctx* c, const float* pos, const float* mass, const int64_t* offsets, int64_t nsys,
-                       int leaf_max)
+// offsets: host memory (on_host), or either
+static int build_systems(tc_ctx* c, const float* pos, const float* mass, const int64_t* offsets, int64_t nsys,
+                         int leaf_max, bool on_host)
 {
     if (!c) return fail(c, TC_EINVAL, "tc_build: null context");
     if (!pos || !mass || !offsets) return fail(c, TC_EINVAL, "tc_build: null pos, mass or offsets");
@@ -953,7 +955,8 @@ int tc_ctx_build_batch(tc_ctx* c, const float* pos, const float* mass, const int
     if (leaf_max < 1 || leaf_max > kLeafMaxLimit)
         return fail(c, TC_EINVAL, "tc_build: leaf_max must be in [1, %d] (got %d)", kLeafMaxLimit, leaf_max);
     std::vector<int64_t> off(nsys + 1);
-    TC_CUDA(c, cudaMemcpy(off.data(), offsets, (nsys + 1) * sizeof(int64_t), cudaMemcpyDefault));
+    if (on_host) std::copy(offsets, offsets + nsys + 1, off.begin());
+    else TC_CUDA(c, cudaMemcpy(off.data(), offsets, (nsys + 1) * sizeof(int64_t), cudaMemcpyDefault));
     if (off[0] != 0) return fail(c, TC_EINVAL, "tc_build: offsets[0] must be 0");
     for (int64_t s = 0; s < nsys; s++)
         if (off[s + 1] <= off[s]) return fail(c, TC_EINVAL, "tc_build: system %lld holds no body", (long long)s);
@@ -974,12 +977,18 @@ int tc_ctx_build_batch(tc_ctx* c, const float* pos, const float* mass, const int
     return build_tree(c, true, c->stream);
 }
 
+int tc_ctx_build_batch(tc_ctx* c, const float* pos, const float* mass, const int64_t* offsets, int64_t nsys,
+                       int leaf_max)
+{
+    return build_systems(c, pos, mass, offsets, nsys, leaf_max, false);
+}
+
 int tc_ctx_build(tc_ctx* c, const float* pos, const float* mass, int64_t n, int leaf_max)
 {
     if (!c) return fail(c, TC_EINVAL, "tc_build: null context");
     if (n < 1 || n >= (int64_t)1 << 31) return fail(c, TC_EINVAL, "tc_build: n must be in [1, 2^31) (got %lld)", (long long)n);
     const int64_t off[2] = {0, n};
-    return tc_ctx_build_batch(c, pos, mass, off, 1, leaf_max);
+    return build_systems(c, pos, mass, off, 1, leaf_max, true);
 }
 
 int tc_ctx_set_velocity(tc_ctx* c, const float* vel)
@@ -1025,12 +1034,9 @@ int tc_get_acc(tc_ctx* c, float* acc, float* pot)
     if (!c) return fail(c, TC_EINVAL, "tc_get_acc: null context");
     if (!c->have_forces) return fail(c, TC_ESTATE, "tc_get_acc: no forces computed");
     if (pot && !c->forces_pot) return fail(c, TC_ESTATE, "tc_get_acc: potential not computed (want_pot = 0)");
-    int r = check_device(c);
-    if (r) return r;
     if (acc) TC_CUDA(c, cudaMemcpyAsync(acc, c->acc, 3 * c->n * sizeof(float), cudaMemcpyDefault, c->stream));
     if (pot) TC_CUDA(c, cudaMemcpyAsync(pot, c->pot, c->n * sizeof(float), cudaMemcpyDefault, c->stream));
-    TC_CUDA(c, cudaStreamSynchronize(c->stream));
-    return TC_OK;
+    return check_device(c);  // waits for the copies too
 }
 
 int tc_get_state(tc_ctx* c, float* pos, float* vel)
