@@ -82,11 +82,13 @@ typedef struct tc_ctx tc_ctx;
  *             one launch, gmax / 32 bodies per lane for every group.  Lists
  *             and forces are the same in both.  The split walk lays every
  *             group out over its lanes by its own size in one launch.
- *   split     1: the monopole walks (learned = 0, quadrupole = 0) run with
- *             the tree walk and the force loop on different warps: a
- *             producer warp walks and fills a ring of list tiles in shared
- *             memory, a consumer warp (several in small systems) sums them
- *             (the default); the learned walk stays on one warp per group
+ *   split     1: the monopole walks, and the quadrupole walk of groups of up
+ *             to 64 bodies, run with the tree walk and the force loop on
+ *             different warps: a producer warp walks and fills a ring of list
+ *             tiles in shared memory (the quadrupole walk's are of 32 cells
+ *             and 64 bodies whatever `tile` says), a consumer warp sums them
+ *             (the default; in small systems several such pairs share a
+ *             group's list); the learned walk stays on one warp per group
  *             with the network evaluated inside the walk.  2: the learned
  *             walk also splits, its band cells recorded by the producers and
  *             the network run on all of them after the walk.  0: every warp

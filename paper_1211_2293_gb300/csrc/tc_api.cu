@@ -587,10 +587,13 @@ int prepare_forces(tc_ctx* c)
     wc.tile = c->cfg.tile;
     wc.learned = c->cfg.learned && c->have_mlp;
     wc.quadw = c->cfg.quadrupole;
-    // split 1: producer/consumer walks for the monopole walks, the learned
-    // walk keeps the network inside the one-warp walk; 2: the learned walk
-    // too, the network then evaluated after the walk
-    wc.split = (!wc.quadw && (c->cfg.split == 2 || (c->cfg.split == 1 && !wc.learned))) ? 1 : 0;
+    // split 1: producer/consumer walks for the monopole walks and the
+    // quadrupole walk of groups of up to 64 bodies (tc_walk_ws.cuh measures
+    // both sides; four bodies a lane leave it no registers), the learned walk
+    // keeps the network inside the one-warp walk; 2: the learned walk too, the
+    // network then evaluated after the walk
+    wc.split = wc.quadw ? (c->cfg.split != 0 && !wc.learned && c->cfg.gmax <= 64)
+                        : (c->cfg.split == 2 || (c->cfg.split == 1 && !wc.learned));
     // one launch per size class: one warp per group only (the split walk
     // lays each group out over its lanes by its own size)
     wc.classes = (c->cfg.gmax > 32 && !wc.split) ? c->cfg.classes : 0;

@@ -23,6 +23,7 @@ TC_WALK_DECL_B(4)
 #define TC_WALK_WS_DECL(T)                                                                            \
     cudaError_t prepare_walk_ws_t##T(const WalkConfig& c, int num_sms, int* grid, size_t* smem);      \
     cudaError_t launch_walk_ws_t##T(const WalkArgs& a, const WalkConfig& c, int grid, size_t smem, cudaStream_t s);
+TC_WALK_WS_DECL(32)
 TC_WALK_WS_DECL(64)
 TC_WALK_WS_DECL(128)
 TC_WALK_WS_DECL(256)
@@ -67,6 +68,7 @@ int bodies_per_lane(int gmax)
 
 cudaError_t prepare_walk(const WalkConfig& c, int num_sms, int* grid, size_t* smem)
 {
+    if (c.split && c.quadw) return prepare_walk_ws_t32(c, num_sms, grid, smem);
     if (c.split) TC_WALK_WS_PICK(prepare_walk, c, num_sms, grid, smem)
     TC_WALK_PICK(prepare_walk, c, num_sms, grid, smem)
 }
@@ -82,6 +84,7 @@ cudaError_t launch_walk(const WalkArgs& a, const WalkConfig& c, int grid, size_t
         cudaMemsetAsync(&a.info->work[0], 0,
                         a.list_cells ? sizeof(a.info->work)
                                      : sizeof(a.info->work) + 3 * sizeof(unsigned long long), s);
+    if (c.split && c.quadw) return launch_walk_ws_t32(a, c, grid, smem, s);
     if (c.split) TC_WALK_WS_PICK(launch_walk, a, c, grid, smem, s)
     TC_WALK_PICK(launch_walk, a, c, grid, smem, s)
 }

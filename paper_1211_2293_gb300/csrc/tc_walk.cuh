@@ -187,11 +187,43 @@ __device__ __forceinline__ void put_quad(float* qtile, int k, const float* q6)
     t[14] = 0.f;
 }
 
-// The cell loop with quadrupole terms: per pair of cells and body, with
-// d = com - x, rho^2 = |d|^2 + eps^2 and Q the cell's second moments about
-// its centre of mass (second-order expansion of the softened potential):
+// Quadrupole terms: a pair of cells at (x, y, z) of masses m and one body,
+// with d = com - x, rho^2 = |d|^2 + eps^2 and Q = {xx, xy, xz, yy, yz, zz} the
+// cells' second moments about their centres of mass, tr its trace (trm15:
+// times -1.5)
+// (second-order expansion of the softened potential):
 //   a += (m rho^-3 + 7.5 d.Qd rho^-7 - 1.5 tr Q rho^-5) d - 3 rho^-5 Qd
 //   pot -= m rho^-1 + 0.5 (3 d.Qd rho^-5 - tr Q rho^-3)
+template <bool POT>
+__device__ __forceinline__ void quad_term(f2 x, f2 y, f2 z, f2 m, const f2 (&Q)[6], f2 trm15, f2 X, f2 Y, f2 Z,
+                                          f2 E2, f2& ax, f2& ay, f2& az, f2& ph)
+{
+    const f2 K75 = f2pack(7.5f, 7.5f), Km3 = f2pack(-3.f, -3.f);
+    const f2 K15 = f2pack(1.5f, 1.5f), K3rd = f2pack(1.f / 3.f, 1.f / 3.f);
+    const f2 dx = f2sub(x, X);
+    const f2 dy = f2sub(y, Y);
+    const f2 dz = f2sub(z, Z);
+    const f2 r2 = f2fma(dz, dz, f2fma(dy, dy, f2fma(dx, dx, E2)));
+    float r2a, r2b;
+    f2unpack(r2, r2a, r2b);
+    const f2 ri = f2pack(rsqrt_sfu(r2a), rsqrt_sfu(r2b));
+    const f2 ri2 = f2mul(ri, ri);
+    const f2 ri3 = f2mul(ri2, ri);
+    const f2 qx = f2fma(Q[2], dz, f2fma(Q[1], dy, f2mul(Q[0], dx)));
+    const f2 qy = f2fma(Q[4], dz, f2fma(Q[3], dy, f2mul(Q[1], dx)));
+    const f2 qz = f2fma(Q[5], dz, f2fma(Q[4], dy, f2mul(Q[2], dx)));
+    const f2 u = f2mul(f2fma(dz, qz, f2fma(dy, qy, f2mul(dx, qx))), ri2);  // d.Qd rho^-2
+    // coefficient of d: rho^-3 (m + rho^-2 (7.5 d.Qd rho^-2 - 1.5 tr))
+    const f2 cd = f2mul(f2fma(f2fma(K75, u, trm15), ri2, m), ri3);
+    const f2 s3 = f2mul(Km3, f2mul(ri3, ri2));
+    ax = f2fma(dx, cd, f2fma(qx, s3, ax));
+    ay = f2fma(dy, cd, f2fma(qy, s3, ay));
+    az = f2fma(dz, cd, f2fma(qz, s3, az));
+    // rho^-1 (m + rho^-2 (1.5 d.Qd rho^-2 - 0.5 tr))
+    if (POT) ph = f2sub(ph, f2mul(f2fma(f2fma(K15, u, f2mul(K3rd, trm15)), ri2, m), ri));
+}
+
+// The cell loop with quadrupole terms
 template <int B, bool POT, int UNROLL>
 __device__ __forceinline__ void sum_tile_quad(const float* __restrict__ tile, const float* __restrict__ qtile,
                                               int npairs, const f2 (&X)[B], const f2 (&Y)[B], const f2 (&Z)[B],
@@ -199,8 +231,6 @@ __device__ __forceinline__ void sum_tile_quad(const float* __restrict__ tile, co
 {
     const ulonglong2* t2 = reinterpret_cast<const ulonglong2*>(tile);
     const ulonglong2* q2 = reinterpret_cast<const ulonglong2*>(qtile);
-    const f2 K75 = f2pack(7.5f, 7.5f), Km15 = f2pack(-1.5f, -1.5f), Km3 = f2pack(-3.f, -3.f);
-    const f2 K15 = f2pack(1.5f, 1.5f), Kmh = f2pack(-0.5f, -0.5f);
 #pragma unroll(UNROLL)
     for (int p = 0; p < npairs; p++) {
         const ulonglong2 xy = t2[2 * p];
@@ -209,35 +239,11 @@ __device__ __forceinline__ void sum_tile_quad(const float* __restrict__ tile, co
         const ulonglong2 qb = q2[4 * p + 1];  // Qxz, Qyy
         const ulonglong2 qc = q2[4 * p + 2];  // Qyz, Qzz
         const ulonglong2 qd = q2[4 * p + 3];  // tr Q, 0
+        const f2 Q[6] = {qa.x, qa.y, qb.x, qb.y, qc.x, qc.y};
+        const f2 trm15 = f2mul(f2pack(-1.5f, -1.5f), qd.x);
 #pragma unroll
-        for (int b = 0; b < B; b++) {
-            const f2 dx = f2sub(xy.x, X[b]);
-            const f2 dy = f2sub(xy.y, Y[b]);
-            const f2 dz = f2sub(zm.x, Z[b]);
-            const f2 r2 = f2fma(dz, dz, f2fma(dy, dy, f2fma(dx, dx, E2)));
-            float r2a, r2b;
-            f2unpack(r2, r2a, r2b);
-            const f2 ri = f2pack(rsqrt_sfu(r2a), rsqrt_sfu(r2b));
-            const f2 ri2 = f2mul(ri, ri);
-            const f2 ri3 = f2mul(ri2, ri);
-            const f2 ri5 = f2mul(ri3, ri2);
-            const f2 ri7 = f2mul(ri5, ri2);
-            const f2 qx = f2fma(qb.x, dz, f2fma(qa.y, dy, f2mul(qa.x, dx)));
-            const f2 qy = f2fma(qc.x, dz, f2fma(qb.y, dy, f2mul(qa.y, dx)));
-            const f2 qz = f2fma(qc.y, dz, f2fma(qc.x, dy, f2mul(qb.x, dx)));
-            const f2 dqd = f2fma(dz, qz, f2fma(dy, qy, f2mul(dx, qx)));
-            const f2 trr5 = f2mul(qd.x, ri5);
-            // coefficient of d: m rho^-3 + 7.5 d.Qd rho^-7 - 1.5 tr rho^-5
-            const f2 cd = f2fma(K75, f2mul(dqd, ri7), f2fma(Km15, trr5, f2mul(zm.y, ri3)));
-            const f2 s3 = f2mul(Km3, ri5);
-            ax[b] = f2fma(dx, cd, f2fma(qx, s3, ax[b]));
-            ay[b] = f2fma(dy, cd, f2fma(qy, s3, ay[b]));
-            az[b] = f2fma(dz, cd, f2fma(qz, s3, az[b]));
-            if (POT) {
-                // m rho^-1 + 1.5 d.Qd rho^-5 - 0.5 tr rho^-3
-                ph[b] = f2sub(ph[b], f2fma(K15, f2mul(dqd, ri5), f2fma(Kmh, f2mul(qd.x, ri3), f2mul(zm.y, ri))));
-            }
-        }
+        for (int b = 0; b < B; b++)
+            quad_term<POT>(xy.x, xy.y, zm.x, zm.y, Q, trm15, X[b], Y[b], Z[b], E2, ax[b], ay[b], az[b], ph[b]);
     }
 }
 

@@ -74,14 +74,30 @@ namespace tc {
 
 namespace {
 
+// The quadrupole walk (precise, gmax up to 64) is the walk with list tiles of
+// 32 cells: ten planes hold a cell with its second moments, fetched by
+// cp.async as the bodies are (the trace is summed in the loop), and a slot of
+// that size 64 to 95 bodies.  Bound by the loop: 97 cycles per pair of cells
+// and body, where its 32 packed operations take 80 with the register reads of
+// the FMAs.  Plummer spheres at theta 0.68, us, one-warp walk / this: 10^4
+// bodies 365 / 59, 10^5 251 / 231, 10^6 1941 / 1865, 4 10^6 7909 / 7710.
+// (Cell loop unrolled twice: 1971 at 10^6, it no longer fits the instruction
+// cache with the others.)
+constexpr int kWsQuadTile = 32;
+__host__ __device__ constexpr bool ws_quad(int tile) { return tile == kWsQuadTile; }
+
 // tiles per team: two open, the others in flight
-__host__ __device__ constexpr int ws_slots(int tile) { return tile > 128 ? 5 : 6; }
+__host__ __device__ constexpr int ws_slots(int tile) { return tile > 128 || ws_quad(tile) ? 5 : 6; }
 constexpr int kWsMaxPairs = 4;                   // pairs per block (block = 2 x pairs warps)
 constexpr long long kWsWaitCycles = 1ll << 31;   // about 1 s of SM clock
 
 // entries of a plane: a step adds at most 64 to a tile that was not full,
 // and the count is padded to a multiple of 16 (four slices of quads)
 __host__ __device__ constexpr int ws_cap(int tile) { return tile + 64; }
+__host__ __device__ constexpr int ws_planes(int tile) { return ws_quad(tile) ? 10 : 4; }
+// of a body tile: entries at which it is handed over, entries of a plane
+__host__ __device__ constexpr int ws_body_tile(int tile) { return ws_quad(tile) ? 64 : tile; }
+__host__ __device__ constexpr int ws_body_cap(int tile) { return ws_quad(tile) ? 128 : ws_cap(tile); }
 
 // slot header (64 bytes at the front of a slot)
 struct WsHdr {
@@ -100,7 +116,7 @@ enum : int32_t { kWsFirst = 1, kWsLast = 2, kWsDone = 4, kWsAbort = 8, kWsBodies
 // the walk stack (first child and number of children of each opened cell),
 // the opened leaves, the consumer's body positions (absolute and
 // reference-relative).  nb: body slots of a group (64, or 128 for gmax 128).
-__host__ __device__ constexpr size_t ws_slot_bytes(int tile) { return sizeof(WsHdr) + (size_t)4 * ws_cap(tile) * 4; }
+__host__ __device__ constexpr size_t ws_slot_bytes(int tile) { return sizeof(WsHdr) + (size_t)ws_planes(tile) * ws_cap(tile) * 4; }
 __host__ __device__ constexpr size_t ws_pos_bytes(int nb) { return (size_t)6 * nb * 4; }
 constexpr int kWsShared = 128;     // of a stack entry's number of children: all parts walk it
 constexpr int kWsSharedFrac = 64;  // cells of more than this fraction of a system (16 to 128 measure alike)
@@ -184,10 +200,13 @@ __device__ __forceinline__ int consume_group(const WsTeam& t, int k, const float
                                              int gfirst, int ng, const WalkArgs& a)
 {
     constexpr int L = 32 / S;                      // lanes of a slice
-    constexpr int CAP = ws_cap(TILE);
+    constexpr bool QUADW = ws_quad(TILE);
+    constexpr int CAP = ws_body_cap(TILE);  // (of all tiles but the quadrupole walk's cells)
     constexpr int kWsSlots = ws_slots(TILE);
     constexpr int kUnroll = K >= 3 ? 1 : (K == 2 ? 2 : 4);  // about eight pairs of sources and bodies in flight
-    constexpr int kFold = (TILE + 32) / 2;                // pairs summed between two compensations
+    // pairs summed between two compensations (the quadrupole walk: as the
+    // one-warp walk's smallest tiles)
+    constexpr int kFold = QUADW ? 48 : (TILE + 32) / 2;
     const int lane = threadIdx.x & 31;
     const int sl = lane / L, j = lane % L;
     const f2 E2 = f2pack(a.eps2, a.eps2);
@@ -235,6 +254,22 @@ __device__ __forceinline__ int consume_group(const WsTeam& t, int k, const float
                 Z[b] = f2pack(z, z);
             }
             const float* p = t.tile(slot) + 4 * sl;
+            if (QUADW && !(flags & kWsBodies)) {
+                constexpr int QC = ws_cap(TILE);
+#pragma unroll 1
+                for (int r = 0; r < rounds; r++, p += 4 * S) {
+#pragma unroll
+                    for (int hh = 0; hh < 2; hh++) {
+                        const auto plane = [&](int k) { return *reinterpret_cast<const f2*>(p + k * QC + 2 * hh); };
+                        const f2 Q[6] = {plane(4), plane(5), plane(6), plane(7), plane(8), plane(9)};
+                        const f2 tr = f2mul(f2pack(-1.5f, -1.5f), f2add(f2add(Q[0], Q[3]), Q[5]));
+                        const f2 x2 = plane(0), y2 = plane(1), z2 = plane(2), m2 = plane(3);
+#pragma unroll
+                        for (int b = 0; b < K; b++)
+                            quad_term<POT>(x2, y2, z2, m2, Q, tr, X[b], Y[b], Z[b], E2, ax[b], ay[b], az[b], ph[b]);
+                    }
+                }
+            } else
 #pragma unroll(kUnroll)
             for (int r = 0; r < rounds; r++, p += 4 * S) {
                 const ulonglong2 xx = *reinterpret_cast<const ulonglong2*>(p);
@@ -375,9 +410,11 @@ __device__ __forceinline__ unsigned ws_incl_scan(unsigned x)
 template <int TILE, bool PRECISE, bool POT, bool LEARNED>
 __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a, int stack_cap, int nb)
 {
-    constexpr int kTile = TILE;
-    constexpr int CAP = ws_cap(TILE);
+    constexpr bool QUADW = ws_quad(TILE);
+    constexpr int kTile = TILE, kBodyTile = ws_body_tile(TILE);
+    constexpr int CAP = ws_cap(TILE), BCAP = ws_body_cap(TILE);
     constexpr int kWsSlots = ws_slots(TILE);
+    static_assert(4 * BCAP <= ws_planes(TILE) * CAP && kBodyTile + 32 <= BCAP && (!QUADW || PRECISE), "tile layout");
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -432,10 +469,14 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
             float* tile = t.tile(slot);
             const int n16 = (n + 15) & ~15;
             if (n + lane < n16) {  // massless padding
+                const int cap = flags & kWsBodies ? BCAP : CAP;
                 tile[n + lane] = 0.f;
-                tile[CAP + n + lane] = 0.f;
-                tile[2 * CAP + n + lane] = 0.f;
-                tile[3 * CAP + n + lane] = 0.f;
+                tile[cap + n + lane] = 0.f;
+                tile[2 * cap + n + lane] = 0.f;
+                tile[3 * cap + n + lane] = 0.f;
+                if (QUADW && !(flags & kWsBodies))
+#pragma unroll
+                    for (int i = 4; i < 10; i++) tile[i * CAP + n + lane] = 0.f;
             }
             if (lane == 0) {
                 WsHdr* h = t.hdr(slot);
@@ -453,7 +494,7 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                 t.seq[k % kWsSlots] = slot;
             }
             first = 0;
-            if (flags & kWsBodies) mbar_track_copies(&t.full[k % kWsSlots]);
+            if (QUADW || (flags & kWsBodies)) mbar_track_copies(&t.full[k % kWsSlots]);
             __syncwarp();
             if (lane == 0) mbar_arrive(&t.full[k % kWsSlots]);
             handed = (handed << 4) | (uint32_t)slot;
@@ -634,13 +675,13 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                         const float* src4 = reinterpret_cast<const float*>(&a.body[r[__popc(starts & le)] + o + lane]);
                         float* q = btile + bn + lane;
                         cp_async4(q, src4);
-                        cp_async4(q + CAP, src4 + 1);
-                        cp_async4(q + 2 * CAP, src4 + 2);
-                        cp_async4(q + 3 * CAP, src4 + 3);
+                        cp_async4(q + BCAP, src4 + 1);
+                        cp_async4(q + 2 * BCAP, src4 + 2);
+                        cp_async4(q + 3 * BCAP, src4 + 3);
                     }
                     r += __popc(starts);
                     bn += min(32, T - o);
-                    if (bn >= kTile) {
+                    if (bn >= kBodyTile) {
                         close_bodies(0);
                         if (!alive) break;
                     }
@@ -734,6 +775,11 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                         q[CAP] = src[u].y;
                         q[2 * CAP] = src[u].z;
                         q[3 * CAP] = src[u].w;
+                        if (QUADW) {
+                            const float* q6 = nt.quad + 6 * (int64_t)v[u];
+#pragma unroll
+                            for (int i = 0; i < 6; i++) cp_async4(q + (4 + i) * CAP, q6 + i);
+                        }
                         if (list_stats) hsh += mix64(2ull * (unsigned)v[u] + 1ull);
                     }
                 }
@@ -825,9 +871,9 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
 #define TC_WS_GROUP(K, S) consume_group<K, S, TILE, PRECISE, POT>(t, k, pos, nb, part, gfirst, ng, a)
             if (ng <= 16) k = TC_WS_GROUP(1, 2);
             else if (ng <= 32) k = TC_WS_GROUP(1, 1);
-            else if (ng <= 40) k = TC_WS_GROUP(5, 4);
+            else if (!ws_quad(TILE) && ng <= 40) k = TC_WS_GROUP(5, 4);
             else if (ng <= 48) k = TC_WS_GROUP(3, 2);
-            else if (ng <= 64) k = TC_WS_GROUP(2, 1);
+            else if (ws_quad(TILE) || ng <= 64) k = TC_WS_GROUP(2, 1);
             else if (ng <= 96) k = TC_WS_GROUP(3, 1);
             else k = TC_WS_GROUP(4, 1);
 #undef TC_WS_GROUP

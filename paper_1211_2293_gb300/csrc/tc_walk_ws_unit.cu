@@ -1,11 +1,12 @@
 // tc_walk_ws_unit.cu -- the walk on producer and consumer warps for list
 // tiles of TC_WALK_TILE entries, every mode.  The build compiles this file
-// once per tile in {64, 128, 256}, defining the macro.
+// once per tile in {64, 128, 256}, defining the macro, and once with 32, the
+// quadrupole walk.
 #include "tc_walk.cuh"
 #include "tc_walk_ws.cuh"
 
 #if !defined(TC_WALK_TILE)
-#error "compile with -DTC_WALK_TILE=<64|128|256>"
+#error "compile with -DTC_WALK_TILE=<32|64|128|256>"
 #endif
 
 #define TC_PASTE2(a, b) a##b
@@ -13,6 +14,21 @@
 
 namespace tc {
 
+#if TC_WALK_TILE == 32
+cudaError_t prepare_walk_ws_t32(const WalkConfig& c, int num_sms, int* grid, size_t* smem)
+{
+    if (!c.quadw || c.learned || !c.precise || c.gmax > 64) return cudaErrorInvalidValue;
+    if (c.want_pot) return prepare_ws_t<32, true, true, false>(c, num_sms, grid, smem);
+    return prepare_ws_t<32, true, false, false>(c, num_sms, grid, smem);
+}
+
+cudaError_t launch_walk_ws_t32(const WalkArgs& a, const WalkConfig& c, int grid, size_t smem, cudaStream_t s)
+{
+    if (!c.quadw || c.learned || !c.precise || c.gmax > 64) return cudaErrorInvalidValue;
+    if (c.want_pot) return launch_ws_t<32, true, true, false>(a, c, grid, smem, s);
+    return launch_ws_t<32, true, false, false>(a, c, grid, smem, s);
+}
+#else
 // precise or plain, with or without the potential; the learned walk (precise,
 // no potential) records its band cells for k_band_eval
 cudaError_t TC_UNIT_NAME(prepare_walk_ws_t, TC_WALK_TILE)(const WalkConfig& c, int num_sms, int* grid, size_t* smem)
@@ -37,5 +53,7 @@ cudaError_t TC_UNIT_NAME(launch_walk_ws_t, TC_WALK_TILE)(const WalkArgs& a, cons
     if (pot) return launch_ws_t<TC_WALK_TILE, false, true, false>(a, c, grid, smem, s);
     return launch_ws_t<TC_WALK_TILE, false, false, false>(a, c, grid, smem, s);
 }
+
+#endif
 
 }  // namespace tc
