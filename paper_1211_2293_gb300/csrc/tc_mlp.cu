@@ -129,6 +129,35 @@ __device__ __forceinline__ void colsum_c(float* G, int nb, const float (&c)[4], 
     }
 }
 
+// the same of all eight column blocks: each exchange halves the values a lane
+// still sums (the same pairs are added as above, 14 shuffles instead of 48)
+__device__ __forceinline__ void colsum_c8(float* G, const float (&c)[8][4], int lane, bool first)
+{
+    float v[16];
+#pragma unroll
+    for (int nb = 0; nb < 8; nb++) {
+        v[2 * nb] = c[nb][0] + c[nb][2];
+        v[2 * nb + 1] = c[nb][1] + c[nb][3];
+    }
+#pragma unroll
+    for (int h = 8, o = 4; h > 1; h >>= 1, o <<= 1)
+#pragma unroll
+        for (int i = 0; i < h; i++) {
+            const bool up = (lane & o) != 0;
+            const float got = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[h + i], o);
+            v[i] = (up ? v[h + i] : v[i]) + got;
+        }
+    const int nb = (lane & 4) | ((lane >> 2) & 2) | (lane >> 4);
+    float2* p = reinterpret_cast<float2*>(&G[nb * 8 + 2 * (lane & 3)]);
+    float2 x = make_float2(v[0], v[1]);
+    if (!first) {
+        const float2 y = *p;
+        x.x += y.x;
+        x.y += y.y;
+    }
+    *p = x;
+}
+
 // what a lane holds of a tile's rows before the network runs: row r0 = tile x
 // 16 + g and r0 + 8, features 2q, 2q + 1, 2q + 8, 2q + 9 of each, the targets
 // of its output columns 2q, 2q + 1 and the loss weights (rows past B: zero)
@@ -139,17 +168,23 @@ struct TrainRows {
     bool v[2];
 };
 
+// a lane's two row indices of a tile (-1 past B)
+__device__ __forceinline__ int2 train_index(const int32_t* __restrict__ idx, int B, int tile, int lane)
+{
+    const int row = tile * 16 + (lane >> 2);
+    return make_int2(row < B ? idx[row] : -1, row + 8 < B ? idx[row + 8] : -1);
+}
+
 __device__ __forceinline__ TrainRows train_rows(const float* __restrict__ X, const float* __restrict__ T,
-                                                const float* __restrict__ W, const int32_t* __restrict__ idx, int B,
-                                                int tile, int lane)
+                                                const float* __restrict__ W, int2 index, int lane)
 {
     TrainRows r;
-    const int g = lane >> 2, q = lane & 3;
+    const int q = lane & 3;
 #pragma unroll
     for (int h = 0; h < 2; h++) {
-        const int row = tile * 16 + g + 8 * h;
-        r.v[h] = row < B;
-        const int64_t i = r.v[h] ? idx[row] : 0;
+        const int at = h ? index.y : index.x;
+        r.v[h] = at >= 0;
+        const int64_t i = r.v[h] ? at : 0;
         const float2 z = make_float2(0.f, 0.f);
         const float2 lo = r.v[h] ? *reinterpret_cast<const float2*>(&X[i * kMlpInPad + 2 * q]) : z;
         const float2 hi = r.v[h] ? *reinterpret_cast<const float2*>(&X[i * kMlpInPad + 2 * q + 8]) : z;
@@ -164,10 +199,18 @@ __device__ __forceinline__ TrainRows train_rows(const float* __restrict__ X, con
     return r;
 }
 
-// Forward and backward of one 16-row tile on one warp; the gradient into gs
-// (the warp's partial, kGPad floats), the weighted squared errors onto lsum.
-__device__ __forceinline__ void train_tile(const MlpDev& m, const TrainRows& r, __nv_bfloat16* st, float* gs, bool first,
-                                           float inv_b, float& lsum, int lane)
+__device__ __forceinline__ TrainRows train_rows(const float* __restrict__ X, const float* __restrict__ T,
+                                                const float* __restrict__ W, const int32_t* __restrict__ idx, int B,
+                                                int tile, int lane)
+{
+    return train_rows(X, T, W, train_index(idx, B, tile, lane), lane);
+}
+
+// Forward and backward of one 16-row tile on one warp: the matrices of the
+// gradient's products into st, the gradients of the biases into b1, b2, b3,
+// the weighted squared errors onto lsum.
+__device__ __forceinline__ void tile_backward(const MlpDev& m, const TrainRows& r, __nv_bfloat16* st, float* b1, float* b2,
+                                              float* b3, bool first, float inv_b, float& lsum, int lane)
 {
     const int g = lane >> 2, q = lane & 3;
     uint32_t x[4];
@@ -197,19 +240,7 @@ __device__ __forceinline__ void train_tile(const MlpDev& m, const TrainRows& r, 
         store_c(st + kStH2, kLdH, nb, h2[nb], lane);
     }
     store_c(st + kStDY, kLdY, 0, dy, lane);
-    __syncwarp();
-    colsum_c(gs + kGB3, 0, dy, lane, first);
-    // dW3 = H2^T dY
-    uint32_t by[2];
-    load_bs(by, st + kStDY, kLdY, 0, lane);
-#pragma unroll
-    for (int mt = 0; mt < 4; mt++) {
-        uint32_t a[4];
-        load_at(a, st + kStH2, kLdH, mt, lane);
-        float c[4] = {0.f, 0.f, 0.f, 0.f};
-        mma_bf16(c, a, by);
-        add_c(gs + kGW3, kMlpOutPad, mt, 0, c, lane, first);
-    }
+    colsum_c(b3, 0, dy, lane, first);
     // dH2 = dY W3^T * [H2 > 0]; dY padded to a 16-deep k-step with zeros
     float dh2[8][4];
     {
@@ -224,7 +255,6 @@ __device__ __forceinline__ void train_tile(const MlpDev& m, const TrainRows& r, 
             store_c(st + kStDH2, kLdH, nb, dh2[nb], lane);
         }
     }
-    __syncwarp();
     // dH1 = dH2 W2^T * [H1 > 0]
     float dh1[8][4];
 #pragma unroll
@@ -246,10 +276,26 @@ __device__ __forceinline__ void train_tile(const MlpDev& m, const TrainRows& r, 
         for (int e = 0; e < 4; e++) dh1[nb][e] = h1[nb][e] > 0.f ? dh1[nb][e] : 0.f;
         store_c(st + kStDH1, kLdH, nb, dh1[nb], lane);
     }
+    colsum_c8(b2, dh2, lane, first);
+    colsum_c8(b1, dh1, lane, first);
+    __syncwarp();
+}
+
+// The same with the whole gradient into gs (the warp's partial, kGPad floats).
+__device__ __forceinline__ void train_tile(const MlpDev& m, const TrainRows& r, __nv_bfloat16* st, float* gs, bool first,
+                                           float inv_b, float& lsum, int lane)
+{
+    tile_backward(m, r, st, gs + kGB1, gs + kGB2, gs + kGB3, first, inv_b, lsum, lane);
+    // dW3 = H2^T dY
+    uint32_t by[2];
+    load_bs(by, st + kStDY, kLdY, 0, lane);
 #pragma unroll
-    for (int nb = 0; nb < 8; nb++) {
-        colsum_c(gs + kGB2, nb, dh2[nb], lane, first);
-        colsum_c(gs + kGB1, nb, dh1[nb], lane, first);
+    for (int mt = 0; mt < 4; mt++) {
+        uint32_t a[4];
+        load_at(a, st + kStH2, kLdH, mt, lane);
+        float c[4] = {0.f, 0.f, 0.f, 0.f};
+        mma_bf16(c, a, by);
+        add_c(gs + kGW3, kMlpOutPad, mt, 0, c, lane, first);
     }
     // dW2 = H1^T dH2
 #pragma unroll
@@ -483,7 +529,7 @@ constexpr int kUpdateLanes = 2;
 // 15 / 17 us a step) add the partials in their order and one of them keeps
 // the master parameter and its Adam moments in registers through the pass
 // and writes the BF16 copies the next step reads.  The next step's rows are
-// loaded before the barriers.  Same operations in the same order as the
+// loaded before the barriers.  (Mini-batches above kClusterRows.)  Same operations in the same order as the
 // single kernels: the same network bit for bit.
 __global__ void __launch_bounds__(kTrainWarps * 32) k_mlp_epoch(const float* __restrict__ X, const float* __restrict__ T,
                                                                  const float* __restrict__ W,
@@ -545,6 +591,247 @@ __global__ void __launch_bounds__(kTrainWarps * 32) k_mlp_epoch(const float* __r
     } else if (own) {
         *loss = pe;
     }
+}
+
+// The same pass on one cluster of eight blocks, for mini-batches whose tiles
+// its 64 warps do in a few rounds.  A step at two grid barriers is mostly
+// their latency and the partials' way through L2; here everything stays in
+// the cluster's shared memory.  Block j takes the tiles k = j mod 8 (the
+// order of reduce_element's eight sums): its warps do a tile each, then each
+// takes a column block of the weights' gradients over the tiles in turn, so
+// the block's sum comes out in registers.  Every block then owns an eighth of
+// the parameters: it adds the eight blocks' sums (distributed shared memory),
+// updates, and stores the parameter in all eight blocks, which turn them into
+// the BF16 copies the next step reads.  Same operations, same order, same
+// network.  Bound by mma.sync, which takes some 27 cycles a scheduler
+// here: 7.3 of a step's 17 thousand cycles are forward and backward, two tiles
+// a scheduler, 2.6 the gradient's products, 2.2 the two cluster barriers.  The
+// sums' and parameters' exchange was 3.9 when each of a thread's three
+// elements was read, updated and stored in turn, and the row indices of the
+// next tile cost their latency when they were not loaded a tile ahead.
+// Training on 2^18 pairs, us a step in all, grid barriers / cluster: 256 rows
+// 9.5 / 6.7, 1024 14.0 / 10.1, 4096 28.7 / 28.2, 8192 47 / 52.
+constexpr int kClusterRows = 4096;
+constexpr int kClusterBlocks = kReduceSlices, kClusterWarps = 8;
+constexpr int kOwn = (kMlpNParam + 1 + kClusterBlocks - 1) / kClusterBlocks;  // elements a block updates
+constexpr int kOwnThread = (kOwn + kClusterWarps * 32 - 1) / (kClusterWarps * 32);
+constexpr int kSideB2 = kMlpHid, kSideB3 = 2 * kMlpHid, kSideLoss = kSideB3 + kMlpOut;  // per tile: biases' gradients, loss
+// packed order with the rows of W2 ld apart (72 and 68: the accesses below
+// meet no bank conflicts)
+constexpr int kLdSum = 72, kLdP = 68;
+__device__ __forceinline__ int padded(int e, int ld)
+{
+    return e < kPW2 ? e : (e < kPB2 ? e + ((e - kPW2) / kMlpHid) * (ld - kMlpHid) : e + kMlpHid * (ld - kMlpHid));
+}
+struct ClusterShared {
+    MlpDev m;
+    float sum[(kMlpNParam + 1 + kMlpHid * (kLdSum - kMlpHid) + 3) & ~3];  // the block's sums
+    float p[(kMlpNParam + kMlpHid * (kLdP - kMlpHid) + 3) & ~3];          // the new parameters
+    float side[kClusterWarps][2 * kMlpHid + kMlpOutPad];
+    __nv_bfloat16 st[kClusterWarps][kStSize];
+};
+static_assert(kSideLoss < 2 * kMlpHid + kMlpOutPad && kStSize % 8 == 0 && sizeof(ClusterShared) <= 227 * 1024,
+              "the cluster kernel's shared memory");
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+// the address of this block's shared p in block `rank` of the cluster
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank)
+{
+    uint32_t d;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(d)
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return d;
+}
+
+// all parameters (padded order, shared memory) into the model's parts that a
+// step reads, as put_parameter does one by one
+__device__ __forceinline__ void put_parameters(MlpDev& m, const float* p)
+{
+    for (int i = threadIdx.x; i < 8 * 32; i += blockDim.x) {
+        const int l = i & 31, n = (i >> 5) * 8 + (l >> 2), k = 2 * (l & 3);
+        const auto w = [&](int r) { return r < kMlpIn ? p[r * kMlpHid + n] : 0.f; };
+        m.frag.f1[i >> 5][l] = make_uint2(pack_bf16(w(k), w(k + 1)), pack_bf16(w(k + 8), w(k + 9)));
+    }
+    for (int i = threadIdx.x; i < 4 * 8 * 32; i += blockDim.x) {
+        const int l = i & 31, n = ((i >> 5) & 7) * 8 + (l >> 2), k = (i >> 8) * 16 + 2 * (l & 3);
+        const auto w = [&](int r) { return p[kPW2 + r * kLdP + n]; };
+        m.frag.f2[i >> 8][(i >> 5) & 7][l] = make_uint2(pack_bf16(w(k), w(k + 1)), pack_bf16(w(k + 8), w(k + 9)));
+    }
+    for (int i = threadIdx.x; i < kMlpHid * kMlpHid / 4; i += blockDim.x) {
+        const float4 v = *reinterpret_cast<const float4*>(&p[kPW2 + (i >> 4) * kLdP + 4 * (i & 15)]);
+        reinterpret_cast<uint2*>(m.w2)[i] = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+    }
+    constexpr int kAfter = kMlpHid * (kLdP - kMlpHid);  // the padding before what follows W2
+    for (int i = threadIdx.x; i < kMlpHid * kMlpOut; i += blockDim.x) {
+        const int k = i / kMlpOut, n = i % kMlpOut;
+        const __nv_bfloat16 v = __float2bfloat16_rn(p[kPW3 + kAfter + i]);
+        reinterpret_cast<__nv_bfloat16*>(&m.frag.f3[k >> 4][n * 4 + ((k & 7) >> 1)])[2 * ((k >> 3) & 1) + (k & 1)] = v;
+        m.w3[k * kMlpOutPad + n] = v;
+    }
+    for (int i = threadIdx.x; i < kMlpHid; i += blockDim.x) {
+        reinterpret_cast<float*>(m.frag.b1)[i] = p[kPB1 + i];
+        reinterpret_cast<float*>(m.frag.b2)[i] = p[kPB2 + kAfter + i];
+    }
+    if (threadIdx.x < kMlpOut) reinterpret_cast<float*>(m.frag.b3)[threadIdx.x] = p[kPB3 + kAfter + threadIdx.x];
+}
+
+__global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(kClusterWarps * 32)
+    k_mlp_cluster(const float* __restrict__ X, const float* __restrict__ T, const float* __restrict__ W,
+                  const int32_t* __restrict__ idx, int n, int batch, MlpDev* model, float* params, float* mom, float* vel,
+                  const float* __restrict__ sched, float b1, float b2, float eps, float* loss)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    ClusterShared& S = *reinterpret_cast<ClusterShared*>(smem);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
+    const int cta = blockIdx.x;  // (one cluster: its rank)
+    // the elements this thread updates; the one past the parameters is the loss
+    float pe[kOwnThread], me[kOwnThread], ve[kOwnThread];
+    const auto own = [&](int i) {
+        const int o = threadIdx.x + i * kClusterWarps * 32;
+        const int e = cta * kOwn + o;
+        return o < kOwn && e <= kMlpNParam ? e : -1;
+    };
+#pragma unroll
+    for (int i = 0; i < kOwnThread; i++) {
+        const int e = own(i);
+        pe[i] = me[i] = ve[i] = 0.f;
+        if (e >= 0 && e < kMlpNParam) pe[i] = params[e], me[i] = mom[e], ve[i] = vel[e];
+        else if (e >= 0) pe[i] = *loss;
+    }
+    load_model(S.m, model);
+    __syncthreads();
+    // a warp's tiles follow each other through the rounds of all steps: the
+    // rows of the next one are loaded while this one's products run, the
+    // indices of the one after it before that
+    int fb = 0, ft = 0;  // the tile whose indices are loaded next: its step's first row, its round's first tile
+    const auto next_index = [&]() {
+        if (fb >= n) return make_int2(-1, -1);
+        const int B = min(batch, n - fb);
+        const int2 x = train_index(idx + fb, B, cta + kClusterBlocks * (ft + w), lane);
+        ft += kClusterWarps;
+        if (kClusterBlocks * ft + cta >= (B + 15) / 16) {
+            ft = 0;
+            fb += batch;
+        }
+        return x;
+    };
+    TrainRows r = train_rows(X, T, W, next_index(), lane);
+    int2 index = next_index();
+    for (int b0 = 0, step = 0; b0 < n; b0 += batch, step++) {
+        const int B = min(batch, n - b0), ntiles = (B + 15) / 16;
+        const float inv_b = 1.0f / (float)B;
+        const int mine = ntiles > cta ? (ntiles - cta - 1) / kClusterBlocks + 1 : 0;  // this block's tiles
+        const float lr = sched[3 * step], c1 = sched[3 * step + 1], c2 = sched[3 * step + 2];  // (needed after the sums)
+        float acc1[4], acc2[4][4], acc3[4], side = 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; k++) acc1[k] = acc3[k] = acc2[0][k] = acc2[1][k] = acc2[2][k] = acc2[3][k] = 0.f;
+        for (int t0 = 0; t0 < mine; t0 += kClusterWarps) {
+            if (t0 > 0) __syncthreads();  // the last round's matrices are read
+            if (t0 + w < mine) {
+                float lsum = 0.f;
+                tile_backward(S.m, r, S.st[w], S.side[w], S.side[w] + kSideB2, S.side[w] + kSideB3, true, inv_b, lsum, lane);
+#pragma unroll
+                for (int o = 16; o; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+                if (lane == 0) S.side[w][kSideLoss] = lsum * inv_b;
+            }
+            r = train_rows(X, T, W, index, lane);
+            index = next_index();
+            __syncthreads();
+            const int nt = min(mine - t0, kClusterWarps);
+            for (int i = 0; i < nt; i++) {
+                const __nv_bfloat16* st = S.st[i];
+                uint32_t a[4], b[2];
+                load_bs(b, st + kStDH2, kLdH, w, lane);  // dW2 = H1^T dH2, columns 8 w ..
+#pragma unroll
+                for (int mt = 0; mt < 4; mt++) {
+                    load_at(a, st + kStH1, kLdH, mt, lane);
+                    float c[4] = {0.f, 0.f, 0.f, 0.f};
+                    mma_bf16(c, a, b);
+#pragma unroll
+                    for (int k = 0; k < 4; k++) acc2[mt][k] += c[k];
+                }
+                load_bs(b, st + kStDH1, kLdH, w, lane);  // dW1 = X^T dH1
+                load_at(a, st + kStX, kLdX, 0, lane);
+                {
+                    float c[4] = {0.f, 0.f, 0.f, 0.f};
+                    mma_bf16(c, a, b);
+#pragma unroll
+                    for (int k = 0; k < 4; k++) acc1[k] += c[k];
+                }
+                if (w < 4) {  // dW3 = H2^T dY, rows 16 w ..
+                    load_bs(b, st + kStDY, kLdY, 0, lane);
+                    load_at(a, st + kStH2, kLdH, w, lane);
+                    float c[4] = {0.f, 0.f, 0.f, 0.f};
+                    mma_bf16(c, a, b);
+#pragma unroll
+                    for (int k = 0; k < 4; k++) acc3[k] += c[k];
+                }
+                if (threadIdx.x <= kSideLoss) side += S.side[i][threadIdx.x];
+            }
+        }
+        // the block's sums
+        constexpr int kAfter = kMlpHid * (kLdSum - kMlpHid);
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int row = g + 8 * h, col = w * 8 + 2 * q;
+            if (row < kMlpIn) *reinterpret_cast<float2*>(&S.sum[row * kMlpHid + col]) = make_float2(acc1[2 * h], acc1[2 * h + 1]);
+#pragma unroll
+            for (int mt = 0; mt < 4; mt++)
+                *reinterpret_cast<float2*>(&S.sum[kPW2 + (mt * 16 + row) * kLdSum + col]) =
+                    make_float2(acc2[mt][2 * h], acc2[mt][2 * h + 1]);
+#pragma unroll
+            for (int k = 0; k < 2; k++)
+                if (w < 4 && 2 * q + k < kMlpOut) S.sum[kPW3 + kAfter + (w * 16 + row) * kMlpOut + 2 * q + k] = acc3[2 * h + k];
+        }
+        if (threadIdx.x < kSideB2) S.sum[kPB1 + threadIdx.x] = side;
+        else if (threadIdx.x < kSideB3) S.sum[kPB2 + kAfter + threadIdx.x - kSideB2] = side;
+        else if (threadIdx.x < kSideLoss) S.sum[kPB3 + kAfter + threadIdx.x - kSideB3] = side;
+        else if (threadIdx.x == kSideLoss) S.sum[kMlpNParam + kAfter] = side;
+        cluster_sync();
+        float s[kOwnThread][kClusterBlocks];
+#pragma unroll
+        for (int i = 0; i < kOwnThread; i++) {
+            const int e = own(i);
+            const float* from = &S.sum[padded(e < 0 ? 0 : e, kLdSum)];
+#pragma unroll
+            for (int j = 0; j < kClusterBlocks; j++)
+                asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(s[i][j]) : "r"(cluster_addr(from, j)) : "memory");
+        }
+#pragma unroll
+        for (int i = 0; i < kOwnThread; i++) {
+            const int e = own(i);
+            float t = s[i][0];
+#pragma unroll
+            for (int j = 1; j < kClusterBlocks; j++) t += s[i][j];
+            if (e == kMlpNParam) pe[i] += t;
+            else if (e >= 0) adam_update(pe[i], me[i], ve[i], t, lr, b1, b2, eps, c1, c2);
+        }
+#pragma unroll
+        for (int i = 0; i < kOwnThread; i++) {
+            const int e = own(i);
+            if (e < 0 || e == kMlpNParam) continue;
+            const float* to = &S.p[padded(e, kLdP)];
+#pragma unroll
+            for (int j = 0; j < kClusterBlocks; j++)
+                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(to, j)), "f"(pe[i]) : "memory");
+        }
+        cluster_sync();
+        put_parameters(S.m, S.p);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < kOwnThread; i++) {
+        const int e = own(i);
+        if (e >= 0 && e < kMlpNParam) params[e] = pe[i], mom[e] = me[i], vel[e] = ve[i];
+        else if (e >= 0) *loss = pe[i];
+    }
+    if (cta == 0)
+        for (int i = threadIdx.x; i < (int)(sizeof(MlpDev) / 16); i += blockDim.x)
+            reinterpret_cast<uint4*>(model)[i] = reinterpret_cast<const uint4*>(&S.m)[i];
 }
 
 // packed FP32 parameters + feature/output maps -> device BF16 model: the
@@ -915,6 +1202,16 @@ cudaError_t launch_mlp_epoch(const float* X, const float* T, const float* W, con
                              float* part, float* loss, uint32_t* bar, int32_t* err, cudaStream_t s)
 {
     const size_t smem = mlp_train_smem();
+    float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+    if (batch <= kClusterRows) {
+        const cudaError_t e = cudaFuncSetAttribute(k_mlp_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)sizeof(ClusterShared));
+        if (e != cudaSuccess) return e;
+        k_mlp_cluster<<<kClusterBlocks, kClusterWarps * 32, sizeof(ClusterShared), s>>>(
+            X, T, W, idx, n, batch, (MlpDev*)model, params, mom, vel, sched, b1, b2, eps, loss);
+        count_launches(1);
+        return cudaGetLastError();
+    }
     cudaError_t e = cudaFuncSetAttribute(k_mlp_epoch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(bar, 0, sizeof(uint32_t), s);
@@ -926,7 +1223,6 @@ cudaError_t launch_mlp_epoch(const float* X, const float* T, const float* W, con
     if (blocks > grid) grid = blocks;
     float* lpart = part + (int64_t)max_blocks * kTrainWarps * kGPad;
     MlpDev* mdl = (MlpDev*)model;
-    float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     void* args[] = {&X, &T, &W, &idx, &n, &batch, &max_blocks, &mdl, &params, &mom, &vel, &sched,
                     &b1, &b2, &eps, &part, &lpart, &loss, &bar, &err};
     e = cudaLaunchCooperativeKernel((const void*)k_mlp_epoch, dim3(grid), dim3(threads), args, smem, s);
