@@ -88,10 +88,10 @@ typedef struct tc_ctx tc_ctx;
  *             tiles in shared memory (the quadrupole walk's are of 32 cells
  *             and 64 bodies whatever `tile` says), a consumer warp sums them
  *             (the default; in small systems several such pairs share a
- *             group's list); the learned walk stays on one warp per group
- *             with the network evaluated inside the walk.  2: the learned
- *             walk also splits, its band cells recorded by the producers and
- *             the network run on all of them after the walk.  0: every warp
+ *             group's list); in the learned walk the producers run the
+ *             network on the band cells they meet.  2: they record the band
+ *             cells instead, and the network runs on all of them after the
+ *             walk.  0: every warp
  *             walks and sums its own groups.  Same lists; the sums take the
  *             entries in another order (rounding-level differences). */
 typedef struct {

@@ -587,19 +587,17 @@ int prepare_forces(tc_ctx* c)
     wc.tile = c->cfg.tile;
     wc.learned = c->cfg.learned && c->have_mlp;
     wc.quadw = c->cfg.quadrupole;
-    // split 1: producer/consumer walks for the monopole walks and the
-    // quadrupole walk of groups of up to 64 bodies (tc_walk_ws.cuh measures
-    // both sides; four bodies a lane leave it no registers), the learned walk
-    // keeps the network inside the one-warp walk; 2: the learned walk too, the
-    // network then evaluated after the walk
-    wc.split = wc.quadw ? (c->cfg.split != 0 && !wc.learned && c->cfg.gmax <= 64)
-                        : (c->cfg.split == 2 || (c->cfg.split == 1 && !wc.learned));
+    // split 1: producer/consumer walks, the quadrupole's for groups of up to
+    // 64 bodies (tc_walk_ws.cuh measures both sides; four bodies a lane leave
+    // it no registers); 2: the learned walk's network evaluated after the walk
+    wc.split = c->cfg.split != 0 && !(wc.quadw && (wc.learned || c->cfg.gmax > 64));
+    wc.record = wc.learned && wc.split && c->cfg.split == 2;
     // one launch per size class: one warp per group only (the split walk
     // lays each group out over its lanes by its own size)
     wc.classes = (c->cfg.gmax > 32 && !wc.split) ? c->cfg.classes : 0;
     wc.part_log2 = wc.split ? walk_parts(c) : 0;
     if (wc.part_log2) {
-        const int64_t want = ((int64_t)8 << wc.part_log2) * c->n;
+        const int64_t want = ((int64_t)kPartPlanes << wc.part_log2) * c->n;
         if (want > c->cap_part) {
             TC_GROW(c, c->part_sum, want);
             c->cap_part = want;
@@ -610,7 +608,7 @@ int prepare_forces(tc_ctx* c)
     if (c->cap_m < st) st = c->cap_m < 32 ? 32 : c->cap_m;  // a stack of M entries cannot overflow
     st = (st + 3) & ~(int64_t)3;                            // keeps every warp's tiles 16-byte aligned
     wc.stack = (int)st;
-    if (wc.learned && wc.split) {
+    if (wc.record) {
         // the band-cell record: 12 cells per body (the learned workloads
         // record 2 to 7) plus a chunk per producer warp of every size-class
         // launch (each keeps a partly filled chunk); a walk that records
@@ -674,7 +672,7 @@ int run_forces(tc_ctx* c, float theta, float eps, float G, cudaStream_t s)
     a.G = G;
     a.inv_eps = 1.0f / eps;
     a.eps = eps;
-    const bool deferred = c->walk_cfg.learned && c->walk_cfg.split;
+    const bool deferred = c->walk_cfg.record;
     if (c->walk_cfg.learned) {
         a.mlp = c->mlp_dev;
         a.band2 = c->mlp_band * c->mlp_band;

@@ -265,7 +265,8 @@ struct WalkArgs {
     const int32_t* gseg;
     int work_slot;  // this launch's work-queue counter, info->work[work_slot]
     // split walk: 2^part_log2 parts per group; a part's compensated sums in
-    // part_sum[((8 part) + 2 component (+ 1: compensation)) part_stride + body],
+    // part_sum[(kPartPlanes part + 2 component (+ 1: compensation)) part_stride + body]
+    // (the learned correction in planes 6 to 8),
     // the parts done so far in part_done[group] (zero before and after)
     int part_log2;
     float* part_sum;
@@ -283,6 +284,7 @@ struct WalkArgs {
     float4* grec;
 };
 constexpr int kBandChunk = 256;
+constexpr int kPartPlanes = 9;
 struct WalkConfig {
     int gmax;         // 32, 64 or 128
     int warps;        // warps per block
@@ -297,6 +299,7 @@ struct WalkConfig {
     int classes;      // 1: one launch per group size class (the smaller beside the largest); 0: one launch
     int split;        // 1: monopole walks on producer/consumer warps (k_walk_ws)
     int part_log2;    // split: each group is walked in 2^part_log2 parts
+    int record;       // split, learned: the band cells are recorded for a launch after the walk
 };
 // host-side preparation of the walk kernel's launch (attributes, occupancy);
 // call before a stream capture

@@ -105,9 +105,9 @@ struct WsHdr {
     int32_t n;      // entries, padded to a multiple of 16 with massless ones
     int32_t gfirst, gend;
     int32_t group, part;
-    int32_t pad[2];
+    float corr[3];  // the learned correction (at the group's last position)
+    int32_t pad;
     double ref[3];  // centre of the group's reference cube (absolute, FP64)
-    double pad2;
 };
 static_assert(sizeof(WsHdr) == 64, "slot header");
 enum : int32_t { kWsFirst = 1, kWsLast = 2, kWsDone = 4, kWsAbort = 8, kWsBodies = 16 };
@@ -115,16 +115,18 @@ enum : int32_t { kWsFirst = 1, kWsLast = 2, kWsDone = 4, kWsAbort = 8, kWsBodies
 // One team's shared memory: barriers and slot numbers (128 bytes), the ring,
 // the walk stack (first child and number of children of each opened cell),
 // the opened leaves, the consumer's body positions (absolute and
-// reference-relative).  nb: body slots of a group (64, or 128 for gmax 128).
+// reference-relative), and where the producer runs the network its pending
+// cells and rows (the block's copy of the network lies in front of the teams).
+// nb: body slots of a group (64, or 128 for gmax 128).
 __host__ __device__ constexpr size_t ws_slot_bytes(int tile) { return sizeof(WsHdr) + (size_t)ws_planes(tile) * ws_cap(tile) * 4; }
 __host__ __device__ constexpr size_t ws_pos_bytes(int nb) { return (size_t)6 * nb * 4; }
 constexpr int kWsShared = 128;     // of a stack entry's number of children: all parts walk it
 constexpr int kWsSharedFrac = 64;  // cells of more than this fraction of a system (16 to 128 measure alike)
 constexpr int kWsLeaves = 96;  // opened leaves: up to 31 left over + 64 of a step
-__host__ __device__ constexpr size_t ws_team_bytes(int tile, int stack, int nb)
+__host__ __device__ constexpr size_t ws_team_bytes(int tile, int stack, int nb, bool rows)
 {
     return 128 + ws_slots(tile) * ws_slot_bytes(tile) + (size_t)stack * 4 + ((stack + 15) & ~15) + kWsLeaves * 8 +
-           32 * 4 + ws_pos_bytes(nb);
+           32 * 4 + ws_pos_bytes(nb) + (rows ? (kPend + 32 * kRowW) * 4 : 0);
 }
 static_assert(2 * 8 * ws_slots(64) + 4 * ws_slots(64) <= 128 && 2 * 8 * ws_slots(256) + 4 * ws_slots(256) <= 128,
               "a team's barriers and slot numbers");
@@ -195,7 +197,7 @@ struct WsTeam {
 // positions from the warp's shared-memory copy, K bodies per lane, S slices.  Starts at position k
 // (whose full barrier has been waited for) and returns the position after
 // the group's last tile, or -1 when a wait ran out.
-template <int K, int S, int TILE, bool PRECISE, bool POT>
+template <int K, int S, int TILE, bool PRECISE, bool POT, int LEARNED>
 __device__ __forceinline__ int consume_group(const WsTeam& t, int k, const float* __restrict__ pos, int nb, int part,
                                              int gfirst, int ng, const WalkArgs& a)
 {
@@ -229,10 +231,15 @@ __device__ __forceinline__ int consume_group(const WsTeam& t, int k, const float
     };
     int pairs = 0;
     int flags;
+    float corr[3] = {0.f, 0.f, 0.f};
     for (;;) {
         const int slot = t.seq[k % kWsSlots];
         const WsHdr* h = t.hdr(slot);
         flags = h->flags;
+        if (LEARNED == 2 && (flags & kWsLast)) {
+#pragma unroll
+            for (int v = 0; v < 3; v++) corr[v] = h->corr[v];
+        }
         const int rounds = (h->n >> 2) / S;        // n is a multiple of 4 S
         if (rounds > 0) {
             if (PRECISE) {
@@ -322,7 +329,7 @@ __device__ __forceinline__ int consume_group(const WsTeam& t, int k, const float
         }
     }
     if (part >= 0) {
-        float* o = a.part_sum + (int64_t)part * 8 * a.part_stride + gfirst;
+        float* o = a.part_sum + (int64_t)part * kPartPlanes * a.part_stride + gfirst;
 #pragma unroll
         for (int b = 0; b < K; b++) {
             const int i = j + b * L;
@@ -337,18 +344,23 @@ __device__ __forceinline__ int consume_group(const WsTeam& t, int k, const float
                 o[6 * a.part_stride + i] = sp[b];
                 o[7 * a.part_stride + i] = cp[b];
             }
+            if (LEARNED == 2) {
+#pragma unroll
+                for (int v = 0; v < 3; v++) o[(6 + v) * a.part_stride + i] = corr[v];
+            }
         }
         return k;
     }
+    const auto with = [&](float f, int v) { return LEARNED == 2 ? f + corr[v] : f; };
     if (flags & kWsAbort) return k;
 #pragma unroll
     for (int b = 0; b < K; b++) {
         const int i = j + b * L;
         if (b % S != sl || i >= ng) continue;
         const int64_t o = a.perm[gfirst + i];
-        a.acc[3 * o + 0] = a.G * (sx[b] + cx[b]);
-        a.acc[3 * o + 1] = a.G * (sy[b] + cy[b]);
-        a.acc[3 * o + 2] = a.G * (sz[b] + cz[b]);
+        a.acc[3 * o + 0] = with(a.G * (sx[b] + cx[b]), 0);
+        a.acc[3 * o + 1] = with(a.G * (sy[b] + cy[b]), 1);
+        a.acc[3 * o + 2] = with(a.G * (sz[b] + cz[b]), 2);
         // (the potential drops the body's own term, -m_i / eps, summed with the list)
         if (POT) a.pot[o] = a.G * ((sp[b] + cp[b]) + a.body[gfirst + i].w * rsqrtf(a.eps2));
     }
@@ -357,7 +369,7 @@ __device__ __forceinline__ int consume_group(const WsTeam& t, int k, const float
 
 // A part of group g has been summed (the sums are in memory): the warp of
 // the group's last part adds the parts' sums in their order.
-template <bool POT>
+template <bool POT, int LEARNED>
 __device__ __forceinline__ void add_parts(int g, int gfirst, int ng, const WalkArgs& a)
 {
     const int lane = threadIdx.x & 31;
@@ -374,18 +386,24 @@ __device__ __forceinline__ void add_parts(int g, int gfirst, int ng, const WalkA
         float s[POT ? 4 : 3], c[POT ? 4 : 3];
 #pragma unroll
         for (int v = 0; v < (POT ? 4 : 3); v++) s[v] = c[v] = 0.f;
+        float corr[3] = {0.f, 0.f, 0.f};
         const float* o = a.part_sum + gfirst + i;
-        for (int p = 0; p < parts; p++, o += 8 * a.part_stride) {
+        for (int p = 0; p < parts; p++, o += kPartPlanes * a.part_stride) {
+            if (LEARNED == 2) {
+#pragma unroll
+                for (int v = 0; v < 3; v++) corr[v] += __ldcg(o + (6 + v) * a.part_stride);
+            }
 #pragma unroll
             for (int v = 0; v < (POT ? 4 : 3); v++) {
                 c[v] = __fadd_rn(c[v], __ldcg(o + (2 * v + 1) * a.part_stride));
                 two_sum_acc(s[v], c[v], __ldcg(o + 2 * v * a.part_stride));
             }
         }
+        const auto with = [&](float f, int v) { return LEARNED == 2 ? f + corr[v] : f; };
         const int64_t b = a.perm[gfirst + i];
-        a.acc[3 * b + 0] = a.G * (s[0] + c[0]);
-        a.acc[3 * b + 1] = a.G * (s[1] + c[1]);
-        a.acc[3 * b + 2] = a.G * (s[2] + c[2]);
+        a.acc[3 * b + 0] = with(a.G * (s[0] + c[0]), 0);
+        a.acc[3 * b + 1] = with(a.G * (s[1] + c[1]), 1);
+        a.acc[3 * b + 2] = with(a.G * (s[2] + c[2]), 2);
         if (POT) a.pot[b] = a.G * ((s[POT ? 3 : 0] + c[POT ? 3 : 0]) + a.body[gfirst + i].w * rsqrtf(a.eps2));
     }
     __syncwarp();
@@ -403,11 +421,17 @@ __device__ __forceinline__ unsigned ws_incl_scan(unsigned x)
     return x;
 }
 
-// LEARNED: the producer also records the group's band cells (accepted, two
-// bodies or more, s >= band d) for the network, which runs after the walk
-// (k_band_eval) as (node, group) pairs, and each group's record (box centre
-// and frame)
-template <int TILE, bool PRECISE, bool POT, bool LEARNED>
+// LEARNED: band cells (accepted, two bodies or more, s >= band d) go through
+// the correction's network.  1: the producer records them, and the group's
+// record (box centre and frame), for k_band_eval after the walk; 2: the
+// producer runs the network on 32 of them at a time, as k_walk does, and hands
+// the group's correction over with its last tile.  The mma.sync of a call take
+// a scheduler's tensor unit 2.4 thousand cycles, six calls a group: the
+// producers are then as long at a group as the consumers.  Plummer spheres at
+// theta 0.67, band 0.55, us, one-warp walk / recorded / in the producers: 5000
+// bodies 154 / 79 / 48, 20000 182 / 100 / 77, 300000 446 / 424 / 414, 2^22
+// 5326 / 5273 / 5205.
+template <int TILE, bool PRECISE, bool POT, int LEARNED>
 __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a, int stack_cap, int nb)
 {
     constexpr bool QUADW = ws_quad(TILE);
@@ -421,8 +445,8 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
     const int teams = (int)(blockDim.x >> 6);
     const bool producer = warp < teams;
     const int team = producer ? warp : warp - teams;
-    const size_t team_bytes = ws_team_bytes(TILE, stack_cap, nb);
-    unsigned char* base = smem + (size_t)team * team_bytes;
+    const size_t team_bytes = ws_team_bytes(TILE, stack_cap, nb, LEARNED == 2);
+    unsigned char* base = smem + (LEARNED == 2 ? mlp_frag_bytes() : 0) + (size_t)team * team_bytes;
     WsTeam t;
     t.full = reinterpret_cast<uint64_t*>(base);
     t.empty = t.full + kWsSlots;
@@ -434,9 +458,15 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
     int32_t* row = reinterpret_cast<int32_t*>(leaves + kWsLeaves);
     uint8_t* stn = reinterpret_cast<uint8_t*>(row + 32);
     float* pos = reinterpret_cast<float*>(stn + ((stack_cap + 15) & ~15));
+    uint32_t* pend = reinterpret_cast<uint32_t*>(pos + 6 * nb);  // LEARNED 2
+    uint32_t* rows = pend + kPend;
+    MlpFrag* mlp = reinterpret_cast<MlpFrag*>(smem);
 
     const Info* info = a.info;
     if (info->err & kErrCapacity) return;  // the build stopped: no tree to walk (uniform: no barrier used yet)
+    if (LEARNED == 2)  // the inference part at the front of the device model
+        for (int i = threadIdx.x; i < (int)(sizeof(MlpFrag) / 4); i += blockDim.x)
+            reinterpret_cast<uint32_t*>(mlp)[i] = reinterpret_cast<const uint32_t*>(a.mlp)[i];
     if (producer && lane == 0) {
         for (int s = 0; s < kWsSlots; s++) {
             mbar_init(&t.full[s], 1);
@@ -462,6 +492,7 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
         const int parts = 1 << a.part_log2;
         int part = 0;
         double gx = 0, gy = 0, gz = 0;
+        float corr[3] = {0.f, 0.f, 0.f};  // LEARNED 2: this group's (or part's)
         bool alive = true;
         // hands a slot's tile of n entries over (flags: kind, last, ...) and
         // takes the next free slot in its place (-1: a wait ran out)
@@ -482,6 +513,7 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                 WsHdr* h = t.hdr(slot);
                 h->flags = flags | first;
                 h->n = n16;
+                if (LEARNED == 2) h->corr[0] = corr[0], h->corr[1] = corr[1], h->corr[2] = corr[2];
                 if (first) {
                     h->gfirst = gfirst;
                     h->gend = gend;
@@ -564,7 +596,7 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                 first = 0;
                 close_cells(kWsDone);
                 // the unused tail of the chunk: no cell
-                if (LEARNED && cbase >= 0)
+                if (LEARNED == 1 && cbase >= 0)
                     for (int i = cused + lane; i < kBandChunk; i += 32) a.band[cbase + i] = make_int2(-1, 0);
                 break;
             }
@@ -618,12 +650,15 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                 flo[kk] = __shfl_sync(0xffffffffu, fb, kk);
                 fhi[kk] = __shfl_sync(0xffffffffu, fb, kk + 3);
             }
-            if (LEARNED && lane == 0 && part == 0) {
-                // the group's record: box centre, reference-relative (as
-                // k_walk forms it), and the frame the network's rows need
-                float xc[3];
+            // the group's box centre, reference-relative (as k_walk forms it)
+            float xc[3];
 #pragma unroll
-                for (int kk = 0; kk < 3; kk++) xc[kk] = 0.5f * (fmaf(klof[kk], uf, flo[kk]) + fmaf(khif[kk], uf, fhi[kk]));
+            for (int kk = 0; kk < 3; kk++) xc[kk] = 0.5f * (fmaf(klof[kk], uf, flo[kk]) + fmaf(khif[kk], uf, fhi[kk]));
+            int qn = 0, nevals = 0;  // LEARNED 2: pending band cells, cells evaluated
+            corr[0] = corr[1] = corr[2] = 0.f;
+            if (LEARNED == 1 && lane == 0 && part == 0) {
+                // the group's record: the centre and the frame the network's
+                // rows need
                 a.grec[2 * (int64_t)g] = make_float4(xc[0], xc[1], xc[2], uf);
                 a.grec[2 * (int64_t)g + 1] =
                     make_float4(__int_as_float(rc.x), __int_as_float(rc.y), __int_as_float(rc.z), Lf);
@@ -796,7 +831,25 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                             const float sz = pow2_down(Lf, nbd[u].w & 255, fast_side);
                             band = sz * sz >= a.band2 * band_e2[u];
                         }
-                        band_append(band, v[u], g);
+                        if (LEARNED == 1) {
+                            band_append(band, v[u], g);
+                            continue;
+                        }
+                        const unsigned bm = __ballot_sync(0xffffffffu, band);
+                        if (!bm) continue;
+                        if (band) pend[qn + __popc(bm & lt)] = (uint32_t)v[u];
+                        qn += __popc(bm);
+                        __syncwarp();
+                        if (qn >= 32) {
+                            learned_rows(*mlp, pend, 32, rows, nt, rc, uf, Lf, 1.0f / Lf, xc, a.eps, 0.f, a.G, corr, lane);
+                            nevals += 32;
+                            // the cells past the first 32 to the front (read all, then write)
+                            const uint32_t t32 = lane < qn - 32 ? pend[32 + lane] : 0u;
+                            __syncwarp();
+                            if (lane < qn - 32) pend[lane] = t32;
+                            qn -= 32;
+                            __syncwarp();
+                        }
                     }
                 }
                 __syncwarp();
@@ -819,6 +872,17 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
             }
             if (cn > 0) close_cells(0);
             if (!alive) break;
+            if (LEARNED == 2) {
+                if (qn > 0) {
+                    learned_rows(*mlp, pend, qn, rows, nt, rc, uf, Lf, 1.0f / Lf, xc, a.eps, 0.f, a.G, corr, lane);
+                    nevals += qn;
+                }
+#pragma unroll
+                for (int kk = 0; kk < 3; kk++)
+#pragma unroll
+                    for (int o = 16; o; o >>= 1) corr[kk] += __shfl_xor_sync(0xffffffffu, corr[kk], o);
+                if (lane == 0 && a.mlp_evals) atomicAdd(a.mlp_evals, (unsigned long long)nevals);
+            }
             close_bodies(kWsLast);
             if (list_stats) {
 #pragma unroll
@@ -868,7 +932,7 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
                 pos[5 * nb + i] = (float)((double)q.z - gz);
             }
             __syncwarp();
-#define TC_WS_GROUP(K, S) consume_group<K, S, TILE, PRECISE, POT>(t, k, pos, nb, part, gfirst, ng, a)
+#define TC_WS_GROUP(K, S) consume_group<K, S, TILE, PRECISE, POT, LEARNED>(t, k, pos, nb, part, gfirst, ng, a)
             if (ng <= 16) k = TC_WS_GROUP(1, 2);
             else if (ng <= 32) k = TC_WS_GROUP(1, 1);
             else if (!ws_quad(TILE) && ng <= 40) k = TC_WS_GROUP(5, 4);
@@ -878,7 +942,7 @@ __global__ void __launch_bounds__(2 * 32 * kWsMaxPairs, 2) k_walk_ws(WalkArgs a,
             else k = TC_WS_GROUP(4, 1);
 #undef TC_WS_GROUP
             ok = k >= 0;
-            if (ok && part >= 0) add_parts<POT>(g, gfirst, ng, a);
+            if (ok && part >= 0) add_parts<POT, LEARNED>(g, gfirst, ng, a);
         }
         if (!ok) {
             if (lane == 0) atomicOr(&a.info->err, kErrWorkLoop);
@@ -894,7 +958,7 @@ struct WsShape {
 };
 constexpr size_t kWsSmemMax = 227 * 1024;
 
-__host__ __forceinline__ WsShape ws_shape(const WalkConfig& c, int tile)
+__host__ __forceinline__ WsShape ws_shape(const WalkConfig& c, int tile, bool rows)
 {
     WsShape w;
     const int teams = c.warps < 1 ? 1 : (c.warps > kWsMaxPairs ? kWsMaxPairs : c.warps);
@@ -904,15 +968,22 @@ __host__ __forceinline__ WsShape ws_shape(const WalkConfig& c, int tile)
     // all the children of a cell, so it holds several times as many nodes
     // as one entry per node)
     w.stack = (c.stack + 3) & ~3;
-    while (w.stack > 64 && ws_team_bytes(tile, w.stack, w.nb) * teams > kWsSmemMax) w.stack -= 16;
-    w.smem = ws_team_bytes(tile, w.stack, w.nb) * teams;
+    const auto bytes = [&](int stack) {
+        return ws_team_bytes(tile, stack, w.nb, rows) * teams + (rows ? mlp_frag_bytes() : 0);
+    };
+    while (w.stack > 64 && bytes(w.stack) > kWsSmemMax) w.stack -= 16;
+    // the network and its rows take the room of a second block on the SM;
+    // a stack of more than 512 opened cells gives way
+    if (rows && bytes(512) <= kWsSmemMax / 2 - 1024)
+        while (w.stack > 512 && bytes(w.stack) > kWsSmemMax / 2 - 1024) w.stack -= 16;
+    w.smem = bytes(w.stack);
     return w;
 }
 
-template <int TILE, bool PRECISE, bool POT, bool LEARNED>
+template <int TILE, bool PRECISE, bool POT, int LEARNED>
 cudaError_t prepare_ws_t(const WalkConfig& c, int num_sms, int* grid, size_t* smem_out)
 {
-    const WsShape w = ws_shape(c, TILE);
+    const WsShape w = ws_shape(c, TILE, LEARNED == 2);
     const int threads = w.threads;
     const size_t smem = w.smem;
     auto kern = k_walk_ws<TILE, PRECISE, POT, LEARNED>;
@@ -928,15 +999,16 @@ cudaError_t prepare_ws_t(const WalkConfig& c, int num_sms, int* grid, size_t* sm
     return cudaSuccess;
 }
 
-template <int TILE, bool PRECISE, bool POT, bool LEARNED>
+template <int TILE, bool PRECISE, bool POT, int LEARNED>
 cudaError_t launch_ws_t(const WalkArgs& a, const WalkConfig& c, int grid, size_t smem, cudaStream_t s)
 {
     // the split walk has no list export, training pairs, size classes or
-    // quadrupole terms (those run on k_walk); its learned walk records band cells
+    // quadrupole terms of large groups (those run on k_walk)
     if (a.list_cells || a.pair_body || a.gseg) return cudaErrorInvalidValue;
-    if (LEARNED && (!a.band || !a.band_n || !a.grec)) return cudaErrorInvalidValue;
+    if (LEARNED == 1 && (!a.band || !a.band_n || !a.grec)) return cudaErrorInvalidValue;
+    if (LEARNED == 2 && !a.mlp) return cudaErrorInvalidValue;
     if (a.part_log2 && (!a.part_sum || !a.part_done)) return cudaErrorInvalidValue;
-    const WsShape w = ws_shape(c, TILE);
+    const WsShape w = ws_shape(c, TILE, LEARNED == 2);
     k_walk_ws<TILE, PRECISE, POT, LEARNED><<<grid, w.threads, smem, s>>>(a, w.stack, w.nb);
     count_launches(1);
     return cudaGetLastError();

@@ -18,28 +18,30 @@ namespace tc {
 cudaError_t prepare_walk_ws_t32(const WalkConfig& c, int num_sms, int* grid, size_t* smem)
 {
     if (!c.quadw || c.learned || !c.precise || c.gmax > 64) return cudaErrorInvalidValue;
-    if (c.want_pot) return prepare_ws_t<32, true, true, false>(c, num_sms, grid, smem);
-    return prepare_ws_t<32, true, false, false>(c, num_sms, grid, smem);
+    if (c.want_pot) return prepare_ws_t<32, true, true, 0>(c, num_sms, grid, smem);
+    return prepare_ws_t<32, true, false, 0>(c, num_sms, grid, smem);
 }
 
 cudaError_t launch_walk_ws_t32(const WalkArgs& a, const WalkConfig& c, int grid, size_t smem, cudaStream_t s)
 {
     if (!c.quadw || c.learned || !c.precise || c.gmax > 64) return cudaErrorInvalidValue;
-    if (c.want_pot) return launch_ws_t<32, true, true, false>(a, c, grid, smem, s);
-    return launch_ws_t<32, true, false, false>(a, c, grid, smem, s);
+    if (c.want_pot) return launch_ws_t<32, true, true, 0>(a, c, grid, smem, s);
+    return launch_ws_t<32, true, false, 0>(a, c, grid, smem, s);
 }
 #else
 // precise or plain, with or without the potential; the learned walk (precise,
-// no potential) records its band cells for k_band_eval
+// no potential) evaluates its band cells or
+// records them for k_band_eval
 cudaError_t TC_UNIT_NAME(prepare_walk_ws_t, TC_WALK_TILE)(const WalkConfig& c, int num_sms, int* grid, size_t* smem)
 {
     const bool p = c.precise != 0, pot = c.want_pot != 0;
     if (c.quadw || (c.learned && (!p || pot))) return cudaErrorInvalidValue;
-    if (c.learned) return prepare_ws_t<TC_WALK_TILE, true, false, true>(c, num_sms, grid, smem);
-    if (p && pot) return prepare_ws_t<TC_WALK_TILE, true, true, false>(c, num_sms, grid, smem);
-    if (p) return prepare_ws_t<TC_WALK_TILE, true, false, false>(c, num_sms, grid, smem);
-    if (pot) return prepare_ws_t<TC_WALK_TILE, false, true, false>(c, num_sms, grid, smem);
-    return prepare_ws_t<TC_WALK_TILE, false, false, false>(c, num_sms, grid, smem);
+    if (c.learned && c.record) return prepare_ws_t<TC_WALK_TILE, true, false, 1>(c, num_sms, grid, smem);
+    if (c.learned) return prepare_ws_t<TC_WALK_TILE, true, false, 2>(c, num_sms, grid, smem);
+    if (p && pot) return prepare_ws_t<TC_WALK_TILE, true, true, 0>(c, num_sms, grid, smem);
+    if (p) return prepare_ws_t<TC_WALK_TILE, true, false, 0>(c, num_sms, grid, smem);
+    if (pot) return prepare_ws_t<TC_WALK_TILE, false, true, 0>(c, num_sms, grid, smem);
+    return prepare_ws_t<TC_WALK_TILE, false, false, 0>(c, num_sms, grid, smem);
 }
 
 cudaError_t TC_UNIT_NAME(launch_walk_ws_t, TC_WALK_TILE)(const WalkArgs& a, const WalkConfig& c, int grid, size_t smem,
@@ -47,11 +49,12 @@ cudaError_t TC_UNIT_NAME(launch_walk_ws_t, TC_WALK_TILE)(const WalkArgs& a, cons
 {
     const bool p = c.precise != 0, pot = c.want_pot != 0;
     if (c.quadw || (c.learned && (!p || pot))) return cudaErrorInvalidValue;
-    if (c.learned) return launch_ws_t<TC_WALK_TILE, true, false, true>(a, c, grid, smem, s);
-    if (p && pot) return launch_ws_t<TC_WALK_TILE, true, true, false>(a, c, grid, smem, s);
-    if (p) return launch_ws_t<TC_WALK_TILE, true, false, false>(a, c, grid, smem, s);
-    if (pot) return launch_ws_t<TC_WALK_TILE, false, true, false>(a, c, grid, smem, s);
-    return launch_ws_t<TC_WALK_TILE, false, false, false>(a, c, grid, smem, s);
+    if (c.learned && c.record) return launch_ws_t<TC_WALK_TILE, true, false, 1>(a, c, grid, smem, s);
+    if (c.learned) return launch_ws_t<TC_WALK_TILE, true, false, 2>(a, c, grid, smem, s);
+    if (p && pot) return launch_ws_t<TC_WALK_TILE, true, true, 0>(a, c, grid, smem, s);
+    if (p) return launch_ws_t<TC_WALK_TILE, true, false, 0>(a, c, grid, smem, s);
+    if (pot) return launch_ws_t<TC_WALK_TILE, false, true, 0>(a, c, grid, smem, s);
+    return launch_ws_t<TC_WALK_TILE, false, false, 0>(a, c, grid, smem, s);
 }
 
 #endif
