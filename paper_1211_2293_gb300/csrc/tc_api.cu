@@ -468,6 +468,15 @@ int setup_systems(tc_ctx* c, const int64_t* off, int nsys)
     return TC_OK;
 }
 
+// Bodies up to which the kernels of a synchronised build (and of the groups'
+// ordering) overlap their predecessor's end: a dozen short kernels in a row,
+// each of which starts a microsecond or two earlier.  Builds in us, one after
+// the other / overlapping: 4096 bodies 96 / 81, 10007 131 / 103, 10^5 146 /
+// 139, 500000 233 / 214, 700000 262 / 272, 10^6 299 / 306, 2^22 743 / 737.  A
+// captured step keeps plain launches: four steps of 10007 bodies take 709 us,
+// 731 with the overlaps as edges of the graph.
+constexpr int64_t kChainBodies = kClimbBodies;
+
 // The build from c->pos / c->mass (already on the device), on stream s.
 // synced: validate the input and size the node table (one synchronisation);
 // otherwise no host interaction at all (the form captured in a step graph),
@@ -475,6 +484,7 @@ int setup_systems(tc_ctx* c, const int64_t* off, int nsys)
 int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
 {
     const int64_t n = c->n;
+    const ChainStream cs(s, synced && n <= kChainBodies);
     cudaEvent_t t0 = phase_begin(c, s, 0);
     // The passes sort only the key digits of the levels down to the last
     // synchronised build's depth + kSortMarginLevels; runs of equal top
@@ -501,27 +511,27 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
     c->sb.tiles = c->sb.ghist + kSortMaxPasses * 256;
     c->scan = reinterpret_cast<unsigned long long*>(c->sb.tiles + 16);
     c->sb.status = c->scan + build_scan_words(n);
-    launch_build_init(c->zero, (zero_words(n, status) + 1) / 2, c->sysp, c->nsys, c->info, synced, s);
-    launch_bbox(c->pos, c->chunks, c->nchunks, c->sysp, &c->info->err, s);
+    launch_build_init(c->zero, (zero_words(n, status) + 1) / 2, c->sysp, c->nsys, c->info, synced, cs);
+    launch_bbox(c->pos, c->chunks, c->nchunks, c->sysp, &c->info->err, cs);
     // the keys go where the passes (and the completion) end in keys / perm
     const int moves = one_block ? 1 : plan.npass + (low_bit > 0 ? 1 : 0);
     uint64_t *ka = moves % 2 ? c->sb.keys_alt : c->keys, *kb = moves % 2 ? c->keys : c->sb.keys_alt;
     uint32_t *va = moves % 2 ? c->sb.vals_alt : c->perm, *vb = moves % 2 ? c->perm : c->sb.vals_alt;
     launch_keys(c->pos, c->mass, n, c->sys_of, c->sysp, ka, va, plan, one_block ? nullptr : c->sb.ghist, &c->info->err,
-                s);
+                cs);
     const int64_t run_max = synced ? kSortRunMaxSynced : kSortRunMax;
     if (one_block) {
-        launch_sort_block(ka, va, kb, vb, n, plan, c->sys_of, c->pos, c->mass, c->body, run_max, &c->info->err, s);
+        launch_sort_block(ka, va, kb, vb, n, plan, c->sys_of, c->pos, c->mass, c->body, run_max, &c->info->err, cs);
     } else {
-        launch_sort_passes(ka, va, kb, vb, n, plan, c->sys_of, c->sb, s);
+        launch_sort_passes(ka, va, kb, vb, n, plan, c->sys_of, c->sb, cs);
         if (low_bit > 0)
             launch_sort_runs(c->sb.keys_alt, c->sb.vals_alt, c->keys, c->perm, n, low_bit, c->nsys > 1 ? c->sys_of : nullptr,
-                             c->pos, c->mass, c->body, run_max, &c->info->err, s);
+                             c->pos, c->mass, c->body, run_max, &c->info->err, cs);
         else
-            launch_gather(c->pos, c->mass, c->perm, n, c->body, s);
+            launch_gather(c->pos, c->mass, c->perm, n, c->body, cs);
     }
     launch_node_levels(c->keys, c->sys_of, n, c->leaf_max, c->w, c->delta, c->top, c->gref_at, c->lcnt, c->scan,
-                       synced ? -1 : c->cap_m, c->info, s);
+                       synced ? -1 : c->cap_m, c->info, cs);
     int depth = -1;
     if (synced) {
         // one round trip: the error word, the number of nodes and the depth
@@ -543,10 +553,10 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
         c->depth_hint = depth;
         c->depth_hint_n = n;
     }
-    launch_emit_nodes(c->keys, c->delta, c->top, c->sys_of, n, c->lcnt, c->info, c->lstart, c->nt, s);
+    launch_emit_nodes(c->keys, c->delta, c->top, c->sys_of, n, c->lcnt, c->info, c->lstart, c->nt, cs);
     launch_moments(c->body, c->delta, n, c->nsys, c->cap_m, depth, c->depth_hint, c->lstart, c->sysp, c->info, c->nt,
-                   c->cfg.quad != 0, s);
-    launch_groups(c->cap_m, c->info, c->nt, c->cfg.gmax, n, c->gref_at, c->scan, c->gfirst, c->gref, c->part_done, s);
+                   c->cfg.quad != 0, cs);
+    launch_groups(c->cap_m, c->info, c->nt, c->cfg.gmax, n, c->gref_at, c->scan, c->gfirst, c->gref, c->part_done, cs);
     c->gorder_ready = false;
     TC_CUDA(c, cudaGetLastError());
     phase_end(c, 0, t0, s);
@@ -651,7 +661,7 @@ int prepare_forces(tc_ctx* c)
     return TC_OK;
 }
 
-int run_forces(tc_ctx* c, float theta, float eps, float G, cudaStream_t s)
+int run_forces(tc_ctx* c, float theta, float eps, float G, cudaStream_t s, bool chain = false)
 {
     WalkArgs a{};
     a.body = c->body;
@@ -698,7 +708,7 @@ int run_forces(tc_ctx* c, float theta, float eps, float G, cudaStream_t s)
     const bool ordered =
         c->walk_ncls > 0 || (c->walk_cfg.split && (double)c->n / (0.7 * c->cfg.gmax) > (double)c->num_sms);
     if (ordered) {
-        if (!c->gorder_ready) launch_group_order(c->gfirst, c->info, c->gorder, c->gseg, c->gseg + 4, s);
+        if (!c->gorder_ready) launch_group_order(c->gfirst, c->info, c->gorder, c->gseg, c->gseg + 4, {s, chain});
         c->gorder_ready = true;
         a.glist = c->gorder;
     }
@@ -1010,7 +1020,7 @@ int tc_ctx_forces(tc_ctx* c, float theta, float eps, float G)
     if (c->cfg.learned && !c->have_mlp) return fail(c, TC_ESTATE, "tc_forces: learned = 1 but no model is set");
     int r = prepare_forces(c);
     if (r) return r;
-    return run_forces(c, theta, eps, G, c->stream);
+    return run_forces(c, theta, eps, G, c->stream, c->n <= kChainBodies);
 }
 
 int tc_ctx_step(tc_ctx* c, float dt)

@@ -42,6 +42,7 @@
 // the tree is the order of (level, first body).
 #include "tc_internal.cuh"
 #include "tc_lookback.cuh"
+#include "tc_pdl.cuh"
 
 // With several systems, cd() of two bodies of different systems is taken as
 // -1 (no common cube), so delta_s = -1 at the first body of every system and
@@ -88,9 +89,10 @@ __device__ __forceinline__ bool capacity_failed(const Info* info)
 }
 
 // ------------------------------------------------------------------ systems
-__global__ void k_sys_ids(const int64_t* __restrict__ off, int nsys, int64_t n, uint32_t* __restrict__ sys_of,
-                          SysParams* __restrict__ sysp)
+__global__ void k_sys_ids(const int64_t* off, int nsys, int64_t n, uint32_t* sys_of,
+                          SysParams* sysp)
 {
+    pdl_begin();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < nsys) {
         sysp[i].first = (int32_t)off[i];
@@ -130,9 +132,10 @@ __device__ __forceinline__ float warp_max(float x)
     return x;
 }
 
-__global__ void k_build_init(uint4* __restrict__ zero, int64_t nzero, SysParams* __restrict__ sysp, int nsys, Info* info,
+__global__ void k_build_init(uint4* zero, int64_t nzero, SysParams* sysp, int nsys, Info* info,
                              int reset_err)
 {
+    pdl_begin();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = t; i < nzero; i += stride) zero[i] = make_uint4(0u, 0u, 0u, 0u);
     for (int64_t s = t; s < nsys; s += stride) {
@@ -187,9 +190,10 @@ __device__ void sys_cube(SysParams& P)
 
 // one block per chunk (system, start, end, chunks of the system); the block
 // that completes a system's last chunk forms its root cube
-__global__ void __launch_bounds__(kBboxThreads) k_bbox(const float* __restrict__ pos, const int4* __restrict__ chunks,
-                                                       SysParams* __restrict__ sysp, int32_t* __restrict__ err)
+__global__ void __launch_bounds__(kBboxThreads) k_bbox(const float* pos, const int4* chunks,
+                                                       SysParams* sysp, int32_t* err)
 {
+    pdl_begin();
     __shared__ float sm[6][kBboxThreads / 32];
     const int4 ch = chunks[blockIdx.x];
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
@@ -247,11 +251,12 @@ constexpr int kKeyRounds = 4;  // bodies of a thread whose loads are in flight t
 
 // also (ghist not null) the digit counts of the sort's passes, per block in
 // shared memory
-__global__ void __launch_bounds__(256) k_keys(const float* __restrict__ pos, const float* __restrict__ mass, int64_t n,
-                                              const uint32_t* __restrict__ sys_of, const SysParams* __restrict__ sysp,
-                                              uint64_t* __restrict__ keys, uint32_t* __restrict__ idx, SortPlan plan,
-                                              uint32_t* __restrict__ ghist, int32_t* err)
+__global__ void __launch_bounds__(256) k_keys(const float* pos, const float* mass, int64_t n,
+                                              const uint32_t* sys_of, const SysParams* sysp,
+                                              uint64_t* keys, uint32_t* idx, SortPlan plan,
+                                              uint32_t* ghist, int32_t* err)
 {
+    pdl_begin();
     __shared__ uint32_t h[kSortMaxPasses][256];
     const int npass = ghist ? plan.npass : 0;
     for (int p = 0; p < npass; p++) h[p][threadIdx.x] = 0u;
@@ -304,9 +309,10 @@ __global__ void __launch_bounds__(256) k_keys(const float* __restrict__ pos, con
     }
 }
 
-__global__ void k_gather(const float* __restrict__ pos, const float* __restrict__ mass,
-                         const uint32_t* __restrict__ perm, int64_t n, float4* __restrict__ body)
+__global__ void k_gather(const float* pos, const float* mass,
+                         const uint32_t* perm, int64_t n, float4* body)
 {
+    pdl_begin();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     const int64_t i = perm[k];
@@ -355,7 +361,7 @@ __device__ __forceinline__ uint32_t set_levels(int d, int t)
 // per level, the block's nodes -> cnt[l][block]; the deepest level of the
 // forest (a block maximum, then one atomic a block)
 __device__ __forceinline__ void count_levels(const int (&d)[kNodeRounds], const int (&t)[kNodeRounds],
-                                             uint32_t* __restrict__ cnt, int32_t* depth)
+                                             uint32_t* cnt, int32_t* depth)
 {
     __shared__ uint32_t wc[kNodeThreads / 32][kLevels];
     __shared__ int wmax[kNodeThreads / 32];
@@ -382,9 +388,10 @@ __device__ __forceinline__ void count_levels(const int (&d)[kNodeRounds], const 
     }
 }
 
-__global__ void k_window(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ sys_of, int64_t n,
-                         int leaf_max, int8_t* __restrict__ w)
+__global__ void k_window(const uint64_t* keys, const uint32_t* sys_of, int64_t n,
+                         int leaf_max, int8_t* w)
 {
+    pdl_begin();
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     w[j] = (j + leaf_max < n && sys_of[j] == sys_of[j + leaf_max])
@@ -393,13 +400,14 @@ __global__ void k_window(const uint64_t* __restrict__ keys, const uint32_t* __re
 }
 
 // leaf_max > kTileWindow: the window digits come from k_window
-__global__ void __launch_bounds__(kNodeThreads) k_node_levels(const uint64_t* __restrict__ keys,
-                                                              const uint32_t* __restrict__ sys_of,
-                                                              const int8_t* __restrict__ w, int64_t n, int leaf_max,
-                                                              int8_t* __restrict__ delta, int8_t* __restrict__ top,
-                                                              int32_t* __restrict__ gref_at, uint32_t* __restrict__ cnt,
-                                                              int32_t* __restrict__ depth)
+__global__ void __launch_bounds__(kNodeThreads) k_node_levels(const uint64_t* keys,
+                                                              const uint32_t* sys_of,
+                                                              const int8_t* w, int64_t n, int leaf_max,
+                                                              int8_t* delta, int8_t* top,
+                                                              int32_t* gref_at, uint32_t* cnt,
+                                                              int32_t* depth)
 {
+    pdl_begin();
     int d[kNodeRounds], t[kNodeRounds];
 #pragma unroll
     for (int r = 0; r < kNodeRounds; r++) {
@@ -424,14 +432,15 @@ __global__ void __launch_bounds__(kNodeThreads) k_node_levels(const uint64_t* __
 // and systems of [b0 - leaf_max, b0 + kNodeBlock + leaf_max) in shared memory,
 // forms the window digits cd(key_j, key_j+leaf_max) there, and takes each
 // body's window maximum from them.
-__global__ void __launch_bounds__(kNodeThreads) k_node_levels_tiled(const uint64_t* __restrict__ keys,
-                                                                    const uint32_t* __restrict__ sys_of, int64_t n,
-                                                                    int leaf_max, int8_t* __restrict__ delta,
-                                                                    int8_t* __restrict__ top,
-                                                                    int32_t* __restrict__ gref_at,
-                                                                    uint32_t* __restrict__ cnt,
-                                                                    int32_t* __restrict__ depth)
+__global__ void __launch_bounds__(kNodeThreads) k_node_levels_tiled(const uint64_t* keys,
+                                                                    const uint32_t* sys_of, int64_t n,
+                                                                    int leaf_max, int8_t* delta,
+                                                                    int8_t* top,
+                                                                    int32_t* gref_at,
+                                                                    uint32_t* cnt,
+                                                                    int32_t* depth)
 {
+    pdl_begin();
     __shared__ uint64_t sk[kNodeBlock + 2 * kTileWindow];
     __shared__ uint32_t ss[kNodeBlock + 2 * kTileWindow];
     __shared__ int8_t sw[kNodeBlock + kTileWindow];
@@ -516,10 +525,11 @@ __device__ __forceinline__ uint32_t scan_tile(uint32_t x, int64_t tile, unsigned
     return pre_sh + before + incl - x;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_levels(uint32_t* __restrict__ cnt, int64_t ncnt,
+__global__ void __launch_bounds__(kScanThreads) k_scan_levels(uint32_t* cnt, int64_t ncnt,
                                                               unsigned long long* st, uint32_t* counter, int64_t cap_m,
                                                               Info* info)
 {
+    pdl_begin();
     __shared__ int tile_sh;
     if (threadIdx.x == 0) tile_sh = (int)atomicAdd(counter, 1u);
     __syncthreads();
@@ -553,13 +563,14 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_levels(uint32_t* __restri
 // starts at or before s.  fam = 1 marks a node that follows a sibling (the
 // topmost one starting at its body), so the children of a cell are its first
 // child and the marked nodes right after it.  Counts follow bottom-up.
-__global__ void __launch_bounds__(kNodeThreads) k_emit_nodes(const uint64_t* __restrict__ keys,
-                                                             const int8_t* __restrict__ delta,
-                                                             const int8_t* __restrict__ top,
-                                                             const uint32_t* __restrict__ sys_of, int64_t n,
-                                                             const uint32_t* __restrict__ offs, const Info* info,
-                                                             uint32_t* __restrict__ lstart, NodeTables nt)
+__global__ void __launch_bounds__(kNodeThreads) k_emit_nodes(const uint64_t* keys,
+                                                             const int8_t* delta,
+                                                             const int8_t* top,
+                                                             const uint32_t* sys_of, int64_t n,
+                                                             const uint32_t* offs, const Info* info,
+                                                             uint32_t* lstart, NodeTables nt)
 {
+    pdl_begin();
     if (capacity_failed(info)) return;
     __shared__ uint32_t wc[kNodeSets][kLevels];
     __shared__ uint4 list[kNodeThreads / 32][64];
@@ -656,7 +667,7 @@ __global__ void __launch_bounds__(kNodeThreads) k_emit_nodes(const uint64_t* __r
 }
 
 // children of the cell whose first child is cf: cf and the marked nodes after it
-__device__ __forceinline__ int family(const uint8_t* __restrict__ fam, int64_t cf, int64_t M)
+__device__ __forceinline__ int family(const uint8_t* fam, int64_t cf, int64_t M)
 {
     unsigned marks = 0;
 #pragma unroll
@@ -782,7 +793,7 @@ __device__ __forceinline__ T ld(const T* p)
 // children are issued before the first sum: in turn they were most of a
 // level's time.
 template <bool QUAD, bool CG>
-__device__ __forceinline__ void level_node(int64_t v, int4 pb, int nch, SysParams* __restrict__ sysp,
+__device__ __forceinline__ void level_node(int64_t v, int4 pb, int nch, SysParams* sysp,
                                            const NodeTables& nt)
 {
     float4 h[8], lo[8];
@@ -840,9 +851,10 @@ __device__ __forceinline__ void level_node(int64_t v, int4 pb, int nch, SysParam
 // child computes the cell and goes on to its parent, so no launch per level
 // follows.
 template <bool QUAD, bool CLIMB>
-__global__ void k_leaf_nodes(const float4* __restrict__ body, const int8_t* __restrict__ delta, int64_t n,
-                             SysParams* __restrict__ sysp, const Info* info, NodeTables nt)
+__global__ void k_leaf_nodes(const float4* body, const int8_t* delta, int64_t n,
+                             SysParams* sysp, const Info* info, NodeTables nt)
 {
+    pdl_begin();
     if (capacity_failed(info)) return;
     const int64_t M = info->M;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < M; v += (int64_t)gridDim.x * blockDim.x) {
@@ -937,9 +949,10 @@ __global__ void k_leaf_nodes(const float4* __restrict__ body, const int8_t* __re
 
 // internal cells of level `lev`: [level_start[lev], level_start[lev + 1])
 template <bool QUAD>
-__global__ void k_level_moments(int lev, const uint32_t* __restrict__ level_start, SysParams* __restrict__ sysp,
+__global__ void k_level_moments(int lev, const uint32_t* level_start, SysParams* sysp,
                                 const Info* info, NodeTables nt)
 {
+    pdl_begin();
     if (capacity_failed(info)) return;
     const int64_t start = level_start[lev];
     const int64_t end = level_start[lev + 1];
@@ -955,10 +968,11 @@ __global__ void k_level_moments(int lev, const uint32_t* __restrict__ level_star
 // cells
 template <bool QUAD>
 __global__ void __launch_bounds__(512) k_level_moments_block(int lev_hi, int lev_lo,
-                                                             const uint32_t* __restrict__ level_start,
-                                                             SysParams* __restrict__ sysp, const Info* info,
+                                                             const uint32_t* level_start,
+                                                             SysParams* sysp, const Info* info,
                                                              NodeTables nt)
 {
+    pdl_begin();
     if (capacity_failed(info)) return;
     for (int lev = lev_hi - 1; lev >= lev_lo; lev--) {
         const int64_t start = level_start[lev];
@@ -982,8 +996,9 @@ __global__ void __launch_bounds__(512) k_level_moments_block(int lev_hi, int lev
 // reference cube (itself, the leaf it was cut from, or the common parent of
 // the packed children); the walk measures positions from that cube's centre.
 // gref_at[s] = the reference cube + 1 of the group that starts at body s (0: none)
-__global__ void k_group_marks(const Info* info, const NodeTables nt, int gmax, int32_t* __restrict__ gref_at)
+__global__ void k_group_marks(const Info* info, const NodeTables nt, int gmax, int32_t* gref_at)
 {
+    pdl_begin();
     if (capacity_failed(info)) return;
     const int64_t M = info->M;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < M; v += (int64_t)gridDim.x * blockDim.x) {
@@ -1023,11 +1038,12 @@ __global__ void k_group_marks(const Info* info, const NodeTables nt, int gmax, i
 }
 
 // the marked bodies in order -> the group table, one pass
-__global__ void __launch_bounds__(kScanThreads) k_group_table(const int32_t* __restrict__ gref_at, int64_t n,
+__global__ void __launch_bounds__(kScanThreads) k_group_table(const int32_t* gref_at, int64_t n,
                                                               unsigned long long* st, uint32_t* counter,
-                                                              int32_t* __restrict__ gfirst, int32_t* __restrict__ gref,
-                                                              int32_t* __restrict__ part_done, Info* info)
+                                                              int32_t* gfirst, int32_t* gref,
+                                                              int32_t* part_done, Info* info)
 {
+    pdl_begin();
     __shared__ int tile_sh;
     __shared__ int32_t mark[kScanTile];
     if (threadIdx.x == 0) tile_sh = (int)atomicAdd(counter, 1u);
@@ -1074,7 +1090,7 @@ __global__ void __launch_bounds__(kScanThreads) k_group_table(const int32_t* __r
 constexpr int kSplitBlocks = 256;
 constexpr int kSplitThreads = 256;
 
-__device__ __forceinline__ int group_class(const int32_t* __restrict__ gfirst, int64_t g)
+__device__ __forceinline__ int group_class(const int32_t* gfirst, int64_t g)
 {
     const int n = gfirst[g + 1] - gfirst[g];
     if (n > 64) return n > 96 ? 0 : 1;
@@ -1097,9 +1113,10 @@ __device__ __forceinline__ int warp_sum_i(int v)
     return v;
 }
 
-__global__ void __launch_bounds__(kSplitThreads) k_order_count(const int32_t* __restrict__ gfirst, const Info* info,
-                                                               int32_t* __restrict__ bcount)
+__global__ void __launch_bounds__(kSplitThreads) k_order_count(const int32_t* gfirst, const Info* info,
+                                                               int32_t* bcount)
 {
+    pdl_begin();
     __shared__ int cnt[kGroupClasses];
     const int tid = threadIdx.x, lane = tid & 31;
     if (tid < kGroupClasses) cnt[tid] = 0;
@@ -1118,10 +1135,11 @@ __global__ void __launch_bounds__(kSplitThreads) k_order_count(const int32_t* __
     if (tid < kGroupClasses) bcount[kGroupClasses * blockIdx.x + tid] = cnt[tid];
 }
 
-__global__ void __launch_bounds__(kSplitThreads) k_order_scatter(const int32_t* __restrict__ gfirst, const Info* info,
-                                                                 const int32_t* __restrict__ bcount,
-                                                                 int32_t* __restrict__ order, int32_t* __restrict__ seg)
+__global__ void __launch_bounds__(kSplitThreads) k_order_scatter(const int32_t* gfirst, const Info* info,
+                                                                 const int32_t* bcount,
+                                                                 int32_t* order, int32_t* seg)
 {
+    pdl_begin();
     constexpr int W = kSplitThreads / 32, NC = kGroupClasses;
     __shared__ int red[W][2 * NC];
     __shared__ int wcnt[W][NC];
@@ -1209,40 +1227,40 @@ inline unsigned gsgrid(int64_t cap, int t)
 
 }  // namespace
 
-void launch_sys_ids(const int64_t* offsets, int nsys, int64_t n, uint32_t* sys_of, SysParams* sysp, cudaStream_t s)
+void launch_sys_ids(const int64_t* offsets, int nsys, int64_t n, uint32_t* sys_of, SysParams* sysp, ChainStream s)
 {
     const int64_t m = n > nsys ? n : nsys;
-    k_sys_ids<<<nblk(m, 256), 256, 0, s>>>(offsets, nsys, n, sys_of, sysp);
+    pdl_launch(k_sys_ids, nblk(m, 256), 256, 0, s, offsets, nsys, n, sys_of, sysp);
     count_launches(1);
 }
 
 void launch_build_init(uint4* zero, int64_t nzero, SysParams* sysp, int nsys, Info* info, bool reset_err,
-                       cudaStream_t s)
+                       ChainStream s)
 {
     const int64_t m = nzero > nsys ? nzero : nsys;
-    k_build_init<<<gsgrid(m, 256), 256, 0, s>>>(zero, nzero, sysp, nsys, info, reset_err);
+    pdl_launch(k_build_init, gsgrid(m, 256), 256, 0, s, zero, nzero, sysp, nsys, info, reset_err);
     count_launches(1);
 }
 
-void launch_bbox(const float* pos, const int4* chunks, int nchunks, SysParams* sysp, int32_t* err, cudaStream_t s)
+void launch_bbox(const float* pos, const int4* chunks, int nchunks, SysParams* sysp, int32_t* err, ChainStream s)
 {
-    k_bbox<<<nchunks, kBboxThreads, 0, s>>>(pos, chunks, sysp, err);
+    pdl_launch(k_bbox, nchunks, kBboxThreads, 0, s, pos, chunks, sysp, err);
     count_launches(1);
 }
 
 void launch_keys(const float* pos, const float* mass, int64_t n, const uint32_t* sys_of, const SysParams* sysp,
-                 uint64_t* keys, uint32_t* idx, const SortPlan& plan, uint32_t* ghist, int32_t* err, cudaStream_t s)
+                 uint64_t* keys, uint32_t* idx, const SortPlan& plan, uint32_t* ghist, int32_t* err, ChainStream s)
 {
     int64_t g = (n + 1023) / 1024;
     if (g > 6 * sm_count()) g = 6 * sm_count();
-    k_keys<<<(unsigned)g, 256, 0, s>>>(pos, mass, n, sys_of, sysp, keys, idx, plan, ghist, err);
+    pdl_launch(k_keys, g, 256, 0, s, pos, mass, n, sys_of, sysp, keys, idx, plan, ghist, err);
     count_launches(1);
 }
 
 void launch_gather(const float* pos, const float* mass, const uint32_t* perm, int64_t n, float4* body,
-                   cudaStream_t s)
+                   ChainStream s)
 {
-    k_gather<<<nblk(n, 256), 256, 0, s>>>(pos, mass, perm, n, body);
+    pdl_launch(k_gather, nblk(n, 256), 256, 0, s, pos, mass, perm, n, body);
     count_launches(1);
 }
 
@@ -1257,44 +1275,47 @@ int64_t build_scan_words(int64_t n) { return scan_tiles(level_counts_size(n)) + 
 
 void launch_node_levels(const uint64_t* keys, const uint32_t* sys_of, int64_t n, int leaf_max, int8_t* w,
                         int8_t* delta, int8_t* top, int32_t* gref_at, uint32_t* cnt, unsigned long long* scan,
-                        int64_t cap_m, Info* info, cudaStream_t s)
+                        int64_t cap_m, Info* info, ChainStream s)
 {
     const unsigned nb = nblk(n, kNodeBlock);
     if (leaf_max <= kTileWindow) {
-        k_node_levels_tiled<<<nb, kNodeThreads, 0, s>>>(keys, sys_of, n, leaf_max, delta, top, gref_at, cnt, &info->depth);
+        pdl_launch(k_node_levels_tiled, nb, kNodeThreads, 0, s, keys, sys_of, n, leaf_max, delta, top, gref_at, cnt,
+                   &info->depth);
         count_launches(1);
     } else {
-        k_window<<<nblk(n, 256), 256, 0, s>>>(keys, sys_of, n, leaf_max, w);
-        k_node_levels<<<nb, kNodeThreads, 0, s>>>(keys, sys_of, w, n, leaf_max, delta, top, gref_at, cnt, &info->depth);
+        pdl_launch(k_window, nblk(n, 256), 256, 0, s, keys, sys_of, n, leaf_max, w);
+        pdl_launch(k_node_levels, nb, kNodeThreads, 0, s, keys, sys_of, w, n, leaf_max, delta, top, gref_at, cnt,
+                   &info->depth);
         count_launches(2);
     }
     const int64_t nc = level_counts_size(n);
     uint32_t* counters = reinterpret_cast<uint32_t*>(scan + build_scan_words(n) - 1);
-    k_scan_levels<<<(unsigned)scan_tiles(nc), kScanThreads, 0, s>>>(cnt, nc, scan, counters, cap_m, info);
+    pdl_launch(k_scan_levels, scan_tiles(nc), kScanThreads, 0, s, cnt, nc, scan, counters, cap_m, info);
     count_launches(1);
 }
 
 void launch_emit_nodes(const uint64_t* keys, const int8_t* delta, const int8_t* top, const uint32_t* sys_of, int64_t n,
-                       const uint32_t* offs, const Info* info, uint32_t* lstart, NodeTables nt, cudaStream_t s)
+                       const uint32_t* offs, const Info* info, uint32_t* lstart, NodeTables nt, ChainStream s)
 {
-    k_emit_nodes<<<nblk(n, kNodeBlock), kNodeThreads, 0, s>>>(keys, delta, top, sys_of, n, offs, info, lstart, nt);
+    pdl_launch(k_emit_nodes, nblk(n, kNodeBlock), kNodeThreads, 0, s, keys, delta, top, sys_of, n, offs, info, lstart,
+               nt);
     count_launches(1);
 }
 
 void launch_moments(const float4* body, const int8_t* delta, int64_t n, int nsys, int64_t cap_m, int depth,
                     int depth_hint, const uint32_t* level_start, SysParams* sysp, const Info* info, NodeTables nt,
-                    bool quad, cudaStream_t s)
+                    bool quad, ChainStream s)
 {
     const unsigned g = gsgrid(cap_m, 128);
     const bool climb = n <= kClimbBodies;
     if (climb) {
-        if (quad) k_leaf_nodes<true, true><<<g, 128, 0, s>>>(body, delta, n, sysp, info, nt);
-        else k_leaf_nodes<false, true><<<g, 128, 0, s>>>(body, delta, n, sysp, info, nt);
+        if (quad) pdl_launch(k_leaf_nodes<true, true>, g, 128, 0, s, body, delta, n, sysp, info, nt);
+        else pdl_launch(k_leaf_nodes<false, true>, g, 128, 0, s, body, delta, n, sysp, info, nt);
         count_launches(1);
         return;
     }
-    if (quad) k_leaf_nodes<true, false><<<g, 128, 0, s>>>(body, delta, n, sysp, info, nt);
-    else k_leaf_nodes<false, false><<<g, 128, 0, s>>>(body, delta, n, sysp, info, nt);
+    if (quad) pdl_launch(k_leaf_nodes<true, false>, g, 128, 0, s, body, delta, n, sysp, info, nt);
+    else pdl_launch(k_leaf_nodes<false, false>, g, 128, 0, s, body, delta, n, sysp, info, nt);
     count_launches(1);
     // the level launches take a small grid (4 blocks per SM): most levels
     // hold few internal cells, the launches past the tree's depth none, and a
@@ -1302,8 +1323,8 @@ void launch_moments(const float4* body, const int8_t* delta, int64_t n, int nsys
     const unsigned glim = 4u * (unsigned)sm_count();
     const unsigned gl = g < glim ? g : glim;
     auto block = [&](int hi, int lo) {
-        if (quad) k_level_moments_block<true><<<1, 512, 0, s>>>(hi, lo, level_start, sysp, info, nt);
-        else k_level_moments_block<false><<<1, 512, 0, s>>>(hi, lo, level_start, sysp, info, nt);
+        if (quad) pdl_launch(k_level_moments_block<true>, 1, 512, 0, s, hi, lo, level_start, sysp, info, nt);
+        else pdl_launch(k_level_moments_block<false>, 1, 512, 0, s, hi, lo, level_start, sysp, info, nt);
         count_launches(1);
     };
     int top = depth < 0 ? kMaxLevel : depth;
@@ -1318,30 +1339,30 @@ void launch_moments(const float4* body, const int8_t* delta, int64_t n, int nsys
     while (few < top && ((int64_t)nsys << (3 * few)) <= 2048) few++;
     if (few < 2) few = 0;
     for (int lev = top - 1; lev >= few; lev--) {
-        if (quad) k_level_moments<true><<<gl, 128, 0, s>>>(lev, level_start, sysp, info, nt);
-        else k_level_moments<false><<<gl, 128, 0, s>>>(lev, level_start, sysp, info, nt);
+        if (quad) pdl_launch(k_level_moments<true>, gl, 128, 0, s, lev, level_start, sysp, info, nt);
+        else pdl_launch(k_level_moments<false>, gl, 128, 0, s, lev, level_start, sysp, info, nt);
         count_launches(1);
     }
     if (few) block(few, 0);
 }
 
 void launch_groups(int64_t cap_m, Info* info, const NodeTables nt, int gmax, int64_t n, int32_t* gref_at,
-                   unsigned long long* scan, int32_t* gfirst, int32_t* gref, int32_t* part_done, cudaStream_t s)
+                   unsigned long long* scan, int32_t* gfirst, int32_t* gref, int32_t* part_done, ChainStream s)
 {
-    k_group_marks<<<gsgrid(cap_m, 128), 128, 0, s>>>(info, nt, gmax, gref_at);
+    pdl_launch(k_group_marks, gsgrid(cap_m, 128), 128, 0, s, info, nt, gmax, gref_at);
     uint32_t* counters = reinterpret_cast<uint32_t*>(scan + build_scan_words(n) - 1);
-    k_group_table<<<(unsigned)scan_tiles(n), kScanThreads, 0, s>>>(
-        gref_at, n, scan + scan_tiles(level_counts_size(n)), counters + 1, gfirst, gref, part_done, info);
+    pdl_launch(k_group_table, scan_tiles(n), kScanThreads, 0, s, gref_at, n, scan + scan_tiles(level_counts_size(n)),
+               counters + 1, gfirst, gref, part_done, info);
     count_launches(2);
 }
 
 size_t group_order_scratch() { return (size_t)kGroupClasses * kSplitBlocks; }
 
 void launch_group_order(const int32_t* gfirst, const Info* info, int32_t* order, int32_t* seg, int32_t* scratch,
-                        cudaStream_t s)
+                        ChainStream s)
 {
-    k_order_count<<<kSplitBlocks, kSplitThreads, 0, s>>>(gfirst, info, scratch);
-    k_order_scatter<<<kSplitBlocks, kSplitThreads, 0, s>>>(gfirst, info, scratch, order, seg);
+    pdl_launch(k_order_count, kSplitBlocks, kSplitThreads, 0, s, gfirst, info, scratch);
+    pdl_launch(k_order_scatter, kSplitBlocks, kSplitThreads, 0, s, gfirst, info, scratch, order, seg);
     count_launches(2);
 }
 

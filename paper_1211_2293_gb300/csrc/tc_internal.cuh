@@ -49,6 +49,14 @@ struct SysParams {
 
 // Per-context scalars kept in device memory (written by kernels, read by
 // kernels and, at synchronisation points, by the host).
+// a stream, and whether a kernel launched on it may come while the kernel
+// before it still runs (tc_pdl.cuh)
+struct ChainStream {
+    cudaStream_t s;
+    bool chain;
+    ChainStream(cudaStream_t stream, bool c = false) : s(stream), chain(c) {}
+};
+
 struct Info {
     int32_t err;       // error bits
     int32_t depth;     // deepest level of the forest
@@ -143,7 +151,7 @@ struct SortPlan {
 // digit counts of every pass; b.tiles and radix_status_words(n, npass) words
 // of b.status are zero.
 void launch_sort_passes(uint64_t* ka, uint32_t* va, uint64_t* kb, uint32_t* vb, int64_t n, const SortPlan& plan,
-                        const uint32_t* sys_of, const SortBufs& b, cudaStream_t s);
+                        const uint32_t* sys_of, const SortBufs& b, ChainStream s);
 int64_t radix_status_words(int64_t n, int npass);
 int64_t radix_status_words(int64_t n);  // enough for any sort of up to n items
 // After passes over bits [low_bit, 63): every run of items with equal top
@@ -156,13 +164,13 @@ constexpr int64_t kSortRunMaxSynced = 1024;  // a synchronised build re-sorts ev
 constexpr int kSortMarginLevels = 2;  // levels below the last synchronised depth a step's sort orders
 void launch_sort_runs(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout, int64_t n,
                       int low_bit, const uint32_t* sys_of, const float* pos, const float* mass, float4* body,
-                      int64_t run_max, int32_t* err, cudaStream_t s);
+                      int64_t run_max, int32_t* err, ChainStream s);
 // Up to kBlockSortMax items: the passes, the completion (low_bit > 0) and the
 // bodies in one launch of one block; no digit counts or scratch needed.
 constexpr int64_t kBlockSortMax = 4096;
 void launch_sort_block(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout, int64_t n,
                        const SortPlan& plan, const uint32_t* sys_of, const float* pos, const float* mass, float4* body,
-                       int64_t run_max, int32_t* err, cudaStream_t s);
+                       int64_t run_max, int32_t* err, ChainStream s);
 // A whole sort of (key, val) by bits [0, nbits) of key, in place.
 void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int nbits, SortBufs& b, cudaStream_t s);
 // self-test of the radix pass's bounded look-back (see tc_sort.cu)
@@ -173,19 +181,19 @@ int64_t sort_selftest_items();
 
 // build pieces
 void launch_sys_ids(const int64_t* offsets, int nsys, int64_t n, uint32_t* sys_of, SysParams* sysp,
-                    cudaStream_t s);
+                    ChainStream s);
 // start of a build: nzero 16-byte words of scratch zeroed, info->depth (and,
 // reset_err, info->err) too, the bounding boxes emptied
 void launch_build_init(uint4* zero, int64_t nzero, SysParams* sysp, int nsys, Info* info, bool reset_err,
-                       cudaStream_t s);
+                       ChainStream s);
 // bounding boxes, and each system's root cube once its last chunk is done;
 // chunks: (system, start, end, chunks of the system)
-void launch_bbox(const float* pos, const int4* chunks, int nchunks, SysParams* sysp, int32_t* err, cudaStream_t s);
+void launch_bbox(const float* pos, const int4* chunks, int nchunks, SysParams* sysp, int32_t* err, ChainStream s);
 // Morton keys, indices and (ghist not null) the digit counts of the plan's passes
 void launch_keys(const float* pos, const float* mass, int64_t n, const uint32_t* sys_of, const SysParams* sysp,
-                 uint64_t* keys, uint32_t* idx, const SortPlan& plan, uint32_t* ghist, int32_t* err, cudaStream_t s);
+                 uint64_t* keys, uint32_t* idx, const SortPlan& plan, uint32_t* ghist, int32_t* err, ChainStream s);
 void launch_gather(const float* pos, const float* mass, const uint32_t* perm, int64_t n,
-                   float4* body, cudaStream_t s);
+                   float4* body, ChainStream s);
 // The levels of the cubes that start at each sorted body (delta < l <= top),
 // their number per level and block of bodies, and the exclusive scan of those
 // (level by level, so the nodes' breadth-first places); zeroes gref_at;
@@ -195,11 +203,11 @@ int64_t level_counts_size(int64_t n);
 int64_t build_scan_words(int64_t n);
 void launch_node_levels(const uint64_t* keys, const uint32_t* sys_of, int64_t n, int leaf_max, int8_t* w,
                         int8_t* delta, int8_t* top, int32_t* gref_at, uint32_t* cnt, unsigned long long* scan,
-                        int64_t cap_m, Info* info, cudaStream_t s);
+                        int64_t cap_m, Info* info, ChainStream s);
 // the node records at those places (counts and children follow with the
 // moments) and lstart[0..22], the first node of each level
 void launch_emit_nodes(const uint64_t* keys, const int8_t* delta, const int8_t* top, const uint32_t* sys_of, int64_t n,
-                       const uint32_t* offs, const Info* info, uint32_t* lstart, NodeTables nt, cudaStream_t s);
+                       const uint32_t* offs, const Info* info, uint32_t* lstart, NodeTables nt, ChainStream s);
 // counts, children and moments: the leaves, then the internal cells, in the
 // same launch for up to kClimbBodies bodies, else level by level from
 // depth - 1 (depth < 0: the depth is known on the device only; with
@@ -209,10 +217,10 @@ void launch_emit_nodes(const uint64_t* keys, const int8_t* delta, const int8_t* 
 constexpr int64_t kClimbBodies = 1 << 19;  // (both ways timed: tc_build.cu, "moments")
 void launch_moments(const float4* body, const int8_t* delta, int64_t n, int nsys, int64_t cap_m, int depth,
                     int depth_hint, const uint32_t* level_start, SysParams* sysp, const Info* info, NodeTables nt,
-                    bool quad, cudaStream_t s);
+                    bool quad, ChainStream s);
 // the body groups: gfirst[0..G], gref[0..G), info->G
 void launch_groups(int64_t cap_m, Info* info, const NodeTables nt, int gmax, int64_t n, int32_t* gref_at,
-                   unsigned long long* scan, int32_t* gfirst, int32_t* gref, int32_t* part_done, cudaStream_t s);
+                   unsigned long long* scan, int32_t* gfirst, int32_t* gref, int32_t* part_done, ChainStream s);
 // the groups by the walk's layout of their bodies (kGroupClasses of them),
 // the largest first, stable: order[0, G); seg[0..3] = the ranges of groups of
 // more than 64, 33 to 64 and up to 32 bodies in it; scratch holds
@@ -220,7 +228,7 @@ void launch_groups(int64_t cap_m, Info* info, const NodeTables nt, int gmax, int
 constexpr int kGroupClasses = 7;
 size_t group_order_scratch();
 void launch_group_order(const int32_t* gfirst, const Info* info, int32_t* order, int32_t* seg, int32_t* scratch,
-                        cudaStream_t s);
+                        ChainStream s);
 // walk + force
 struct WalkArgs {
     const float4* body;        // Morton order (x, y, z, m)

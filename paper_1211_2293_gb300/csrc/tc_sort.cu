@@ -24,6 +24,7 @@
 
 #include "tc_internal.cuh"
 #include "tc_lookback.cuh"
+#include "tc_pdl.cuh"
 
 namespace tc {
 
@@ -41,9 +42,10 @@ __host__ __device__ constexpr int sort_tile(int items) { return kSortThreads * i
 int sort_items(int64_t n) { return n <= kSortSmall ? kItemsSmall : kItemsLarge; }
 
 // digit histograms of npass passes from bit shift0 up
-__global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint64_t* __restrict__ keys, int64_t n, int npass,
-                                                            uint32_t* __restrict__ ghist)
+__global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint64_t* keys, int64_t n, int npass,
+                                                            uint32_t* ghist)
 {
+    pdl_begin();
     __shared__ uint32_t h[8][256];
     for (int i = threadIdx.x; i < 8 * 256; i += kSortThreads) (&h[0][0])[i] = 0;
     __syncthreads();
@@ -85,10 +87,11 @@ __device__ __forceinline__ unsigned digit_peers(unsigned in, uint32_t d)
 // SYS: the digit holds bits of the system of the value's body (SortPlan)
 template <bool SYS, int ITEMS>
 __global__ void __launch_bounds__(kSortThreads, 3)
-    k_onesweep(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint64_t* __restrict__ kout,
-               uint32_t* __restrict__ vout, int64_t n, SortDigit dg, const uint32_t* __restrict__ ghist,
-               unsigned long long* status, uint32_t* tile_counter, int32_t* err, const uint32_t* __restrict__ sys_of)
+    k_onesweep(const uint64_t* kin, const uint32_t* vin, uint64_t* kout,
+               uint32_t* vout, int64_t n, SortDigit dg, const uint32_t* ghist,
+               unsigned long long* status, uint32_t* tile_counter, int32_t* err, const uint32_t* sys_of)
 {
+    pdl_begin();
     constexpr int TILE = sort_tile(ITEMS), WARP = 32 * ITEMS, H = ITEMS < 8 ? ITEMS : 8;
     extern __shared__ __align__(16) unsigned char dsm[];
     uint64_t* skey = reinterpret_cast<uint64_t*>(dsm);
@@ -313,7 +316,7 @@ int64_t radix_status_words(int64_t n, int npass)
 }
 
 void launch_sort_passes(uint64_t* ka, uint32_t* va, uint64_t* kb, uint32_t* vb, int64_t n, const SortPlan& plan,
-                        const uint32_t* sys_of, const SortBufs& b, cudaStream_t s)
+                        const uint32_t* sys_of, const SortBufs& b, ChainStream s)
 {
     sort_attributes();
     const int items = sort_items(n);
@@ -323,8 +326,8 @@ void launch_sort_passes(uint64_t* ka, uint32_t* va, uint64_t* kb, uint32_t* vb, 
         const SortDigit dg = plan.digit(p);
         unsigned long long* st = b.status + (size_t)p * nt * 256;
         auto go = [&](auto* kernel) {
-            kernel<<<(unsigned)nt, kSortThreads, dsm, s>>>(ka, va, kb, vb, n, dg, b.ghist + 256 * p, st, b.tiles + p, b.err,
-                                                          sys_of);
+            pdl_launch(kernel, nt, kSortThreads, dsm, s, ka, va, kb, vb, n, dg, b.ghist + 256 * p, st, b.tiles + p,
+                       b.err, sys_of);
         };
         if (items == kItemsLarge) dg.sys ? go(k_onesweep<true, kItemsLarge>) : go(k_onesweep<false, kItemsLarge>);
         else dg.sys ? go(k_onesweep<true, kItemsSmall>) : go(k_onesweep<false, kItemsSmall>);
@@ -345,8 +348,8 @@ namespace {
 
 constexpr int kShortRun = 32;
 
-__device__ __forceinline__ bool same_run(const uint64_t* __restrict__ k, const uint32_t* __restrict__ v,
-                                         const uint32_t* __restrict__ sys_of, int low_bit, int64_t i, int64_t j)
+__device__ __forceinline__ bool same_run(const uint64_t* k, const uint32_t* v,
+                                         const uint32_t* sys_of, int low_bit, int64_t i, int64_t j)
 {
     if ((k[i] >> low_bit) != (k[j] >> low_bit)) return false;
     return !sys_of || sys_of[v[i]] == sys_of[v[j]];
@@ -358,12 +361,13 @@ __device__ __forceinline__ bool before(uint64_t ka, uint32_t va, uint64_t kb, ui
 }
 
 // Also the bodies in that order: body[k] = (x, y, z, m) of the k-th item.
-__global__ void __launch_bounds__(256) k_sort_runs(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-                                                   uint64_t* __restrict__ kout, uint32_t* __restrict__ vout, int64_t n,
-                                                   int low_bit, const uint32_t* __restrict__ sys_of,
-                                                   const float* __restrict__ pos, const float* __restrict__ mass,
-                                                   float4* __restrict__ body, int64_t run_max, int32_t* __restrict__ err)
+__global__ void __launch_bounds__(256) k_sort_runs(const uint64_t* kin, const uint32_t* vin,
+                                                   uint64_t* kout, uint32_t* vout, int64_t n,
+                                                   int low_bit, const uint32_t* sys_of,
+                                                   const float* pos, const float* mass,
+                                                   float4* body, int64_t run_max, int32_t* err)
 {
+    pdl_begin();
     __shared__ int nlong;
     __shared__ int64_t longs[256 / kShortRun + 1];
     __shared__ long long en_sh;
@@ -441,11 +445,12 @@ constexpr size_t block_sort_smem(int items)
 
 template <int ITEMS>
 __global__ void __launch_bounds__(kBlockThreads, 1)
-    k_sort_block(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint64_t* __restrict__ kout,
-                 uint32_t* __restrict__ vout, int n, SortPlan plan, const uint32_t* __restrict__ sys_of,
-                 const float* __restrict__ pos, const float* __restrict__ mass, float4* __restrict__ body, int run_max,
-                 int32_t* __restrict__ err)
+    k_sort_block(const uint64_t* kin, const uint32_t* vin, uint64_t* kout,
+                 uint32_t* vout, int n, SortPlan plan, const uint32_t* sys_of,
+                 const float* pos, const float* mass, float4* body, int run_max,
+                 int32_t* err)
 {
+    pdl_begin();
     constexpr int WARP = 32 * ITEMS;
     extern __shared__ __align__(16) unsigned char dsm[];
     uint64_t* skey = reinterpret_cast<uint64_t*>(dsm);
@@ -592,24 +597,24 @@ static_assert(kBlockSortMax == kBlockThreads * kBlockItems, "one block's items")
 
 void launch_sort_block(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout, int64_t n,
                        const SortPlan& plan, const uint32_t* sys_of, const float* pos, const float* mass, float4* body,
-                       int64_t run_max, int32_t* err, cudaStream_t s)
+                       int64_t run_max, int32_t* err, ChainStream s)
 {
     sort_attributes();
     const int rm = (int)(run_max < 1 || run_max > kSortRunMax ? kSortRunMax : run_max);
-    k_sort_block<kBlockItems><<<1, kBlockThreads, block_sort_smem(kBlockItems), s>>>(kin, vin, kout, vout, (int)n, plan,
-                                                                                   sys_of, pos, mass, body, rm, err);
+    pdl_launch(k_sort_block<kBlockItems>, 1, kBlockThreads, block_sort_smem(kBlockItems), s, kin, vin, kout, vout,
+               (int)n, plan, sys_of, pos, mass, body, rm, err);
     count_launches(1);
 }
 
 void launch_sort_runs(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout, int64_t n,
                       int low_bit, const uint32_t* sys_of, const float* pos, const float* mass, float4* body,
-                      int64_t run_max, int32_t* err, cudaStream_t s)
+                      int64_t run_max, int32_t* err, ChainStream s)
 {
     if (run_max < 1 || run_max > kSortRunMax) run_max = kSortRunMax;
     int64_t g = (n + 255) / 256;
     if (g > 16 * sm_count()) g = 16 * sm_count();
-    k_sort_runs<<<(unsigned)(g < 1 ? 1 : g), 256, 0, s>>>(kin, vin, kout, vout, n, low_bit, sys_of, pos, mass, body, run_max,
-                                                          err);
+    pdl_launch(k_sort_runs, g < 1 ? 1 : g, 256, 0, s, kin, vin, kout, vout, n, low_bit, sys_of, pos, mass, body,
+               run_max, err);
     count_launches(1);
 }
 
@@ -622,7 +627,7 @@ void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int nbits, SortBu
     cudaMemsetAsync(b.status, 0, radix_status_words(n, plan.npass) * sizeof(unsigned long long), s);
     int64_t hb = (n + kSortThreads * 16 - 1) / (kSortThreads * 16);
     if (hb > 4 * sm_count()) hb = 4 * sm_count();
-    k_sort_hist<<<(unsigned)hb, kSortThreads, 0, s>>>(keys, n, plan.npass, b.ghist);
+    pdl_launch(k_sort_hist, hb, kSortThreads, 0, s, keys, n, plan.npass, b.ghist);
     count_launches(1);
     launch_sort_passes(keys, vals, b.keys_alt, b.vals_alt, n, plan, nullptr, b, s);
     if (plan.npass % 2) {
@@ -647,8 +652,8 @@ cudaError_t sort_wait_selftest(uint64_t* keys, uint32_t* vals, uint64_t* kout, u
     const uint32_t one = 1;  // the only block launched takes tile 1
     cudaMemcpyAsync(counter, &one, sizeof(one), cudaMemcpyHostToDevice, s);
     sort_attributes();
-    k_onesweep<false, kItemsLarge><<<1, kSortThreads, onesweep_smem(kItemsLarge), s>>>(
-        keys, vals, kout, vout, n, SortPlan::make(63, 0, 0).digit(0), hist, status, counter, err, nullptr);
+    pdl_launch(k_onesweep<false, kItemsLarge>, 1, kSortThreads, onesweep_smem(kItemsLarge), s, keys, vals, kout, vout,
+               n, SortPlan::make(63, 0, 0).digit(0), hist, status, counter, err, nullptr);
     count_launches(1);
     return cudaGetLastError();
 }
