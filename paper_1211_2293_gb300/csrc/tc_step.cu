@@ -113,9 +113,9 @@ __global__ void k_diag(const float* __restrict__ pos, const float* __restrict__ 
 // counted from its start); k_direct_reduce adds the slices in order.  With
 // one block per 256 targets and no slices, the 4096 sampled targets of an
 // accuracy check kept 16 of 152 SMs busy: 44.6 ms over 2^20 bodies, 1.9 of
-// 80 TFLOP/s; sliced 76 ways and packed 2.0 ms, 43 TFLOP/s.  A thread holds four targets as two packed pairs, so each
-// paired FP32 instruction serves two of them and the broadcast loads of a
-// source (stored twice, {x, x}) serve four; per target the operations and
+// 80 TFLOP/s; sliced and packed 1.9 ms, 45 TFLOP/s.  A thread holds four
+// targets as two packed pairs, so each paired FP32 instruction serves two of
+// them and the broadcast loads of a source (stored twice, {x, x}) serve four; per target the operations and
 // their order inside a tile are those of the scalar loop, bit for bit.  The
 // bound is the FP32 pipe (13 operations a pair of bodies).
 constexpr int kDirTile = 256;                       // sources per tile
@@ -399,13 +399,17 @@ void launch_diag(const float* pos, const float* vel, const float* mass, const fl
     count_launches(1);
 }
 
-// source slices of a direct sum: as many as fill the SMs once (kDirBlocksPerSm
-// resident blocks each) where few target blocks leave them idle, about four
-// waves of blocks where there are more, never more than there are tiles
+// Source slices of a direct sum: with few target blocks as many as fill the SMs
+// once (kDirBlocksPerSm resident blocks each); from eight target blocks on
+// three times as many, so that blocks that end early (a scheduler favours its
+// oldest warps) are replaced: 4096 targets of 2^20 / 2^18 bodies take 1910 /
+// 563 us, 1999 / 586 when filled once, 1962 / 577 with four times; 512 targets
+// of 2^20 464, 378 when filled once (the slices' sums to add).  Never more
+// than there are tiles.
 int direct_slices(int64_t n, int64_t ns)
 {
     const int64_t nbx = nblk(ns, kDirTargets), room = (int64_t)kDirBlocksPerSm * sm_count();
-    int64_t S = nbx * 4 <= room ? room / nbx : (4 * room) / nbx;
+    int64_t S = (nbx >= 8 ? 3 * room : room) / nbx;
     const int64_t tiles = (n + kDirTile - 1) / kDirTile;
     if (S > tiles) S = tiles;
     return (int)(S < 1 ? 1 : S);
