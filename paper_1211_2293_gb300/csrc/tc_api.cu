@@ -86,7 +86,7 @@ struct tc_ctx {
     int32_t* gseg = nullptr;    // 4 range ends of its size classes, then the ordering's scratch
     int32_t* part_done = nullptr;  // split walk: parts of each group done
     float* part_sum = nullptr;
-    int64_t cap_part = 0;
+    int64_t cap_part = 0, part_refused = INT64_MAX;
     bool gorder_ready = false;  // the order is that of the current groups
     int walk_ncls = 0;
     int depth_hint = -1;  // tree depth of the last build the host saw (-1: none)
@@ -608,11 +608,13 @@ int prepare_forces(tc_ctx* c)
     wc.part_log2 = wc.split ? walk_parts(c) : 0;
     if (wc.part_log2) {
         const int64_t want = ((int64_t)kPartPlanes << wc.part_log2) * c->n;
-        if (want > c->cap_part) {
-            TC_GROW(c, c->part_sum, want);
-            c->cap_part = want;
-            drop_graph(c);
+        if (want > c->cap_part && want < c->part_refused) {
+            c->cap_part = 0;
+            if (grow(c, &c->part_sum, want) == TC_OK) c->cap_part = want;
+            else c->part_refused = want;
         }
+        // a few megabytes; where they are not to be had the groups are walked whole
+        if (want > c->cap_part) wc.part_log2 = 0;
     }
     int64_t st = c->cfg.stack;
     if (c->cap_m < st) st = c->cap_m < 32 ? 32 : c->cap_m;  // a stack of M entries cannot overflow

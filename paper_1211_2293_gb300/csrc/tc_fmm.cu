@@ -406,6 +406,7 @@ struct P2PSum {
 // or child is found in FP32 and only that one is computed in FP64; where the
 // second comes within the FP32 values' error of the first, all are.  10^6
 // bodies: 92 us, 295 with a launch per level and FP64 throughout.
+constexpr float kRadiusTiny = 1e-24f;  // squares whose FP32 rounding is relative
 __global__ void __launch_bounds__(128) k_fmm_radius(const float4* __restrict__ body, const SysParams* __restrict__ sysp,
                                                     NodeTables nt, double* __restrict__ rad, int4* __restrict__ fnode,
                                                     uint32_t* __restrict__ pend, const Info* info)
@@ -450,7 +451,7 @@ __global__ void __launch_bounds__(128) k_fmm_radius(const float4* __restrict__ b
             }
         }
         double r2max = body2(far);
-        if (!(second < first * (1.f - 1e-5f)))  // (also infinities and NaN)
+        if (!(second < first * (1.f - 1e-5f) && first > kRadiusTiny))  // (also infinities, NaN and underflows)
             for (int i = b.x; i < b.x + b.y; i++) r2max = fmax(r2max, body2(i));
         record(v, b, nt.a[v], nt.c[v], sqrt(r2max));
         for (;;) {
@@ -492,7 +493,7 @@ __global__ void __launch_bounds__(128) k_fmm_radius(const float4* __restrict__ b
             }
             double r = sphere(far);
             const float side = ldexpf(uf, kMaxLevel + 1 - (b.w & 255));  // the cell's: what the offsets are rounded to
-            if (!(second < first * (1.f - 1e-5f) - 1e-6f * side))
+            if (!(second < first * (1.f - 1e-5f) - 1e-6f * side && side * side > kRadiusTiny))
                 for (int k = b.z; k < b.z + nch; k++) r = fmax(r, sphere(k));
             record(v, b, na, nc, r);
         }

@@ -70,3 +70,29 @@ def test_parts_of_systems():
         return ctx
 
     _compare(_both(make, lambda ctx: ctx.forces(0.5, EPS)), m)
+
+
+def test_parts_without_their_scratch(monkeypatch):
+    """Where the parts' sums find no memory the groups are walked whole."""
+    from paper_1211_2293_gb300 import tc
+
+    p, _, m = inputs.plummer(5000, seed=4, with_velocity=False)
+    free = tc.Context()
+    free.build(p, m, 8)
+    free.forces(0.6, EPS)
+    a0 = free.get_acc()
+    for cap in range(1, 64):  # the smallest cap (in 100 kB) that lets the build through
+        monkeypatch.setenv("TC_ALLOC_CAP_BYTES", str(100000 * cap))
+        ctx = tc.Context()
+        try:
+            ctx.build(p, m, 8)
+        except tc.TcError:
+            ctx.close()
+            continue
+        for _ in range(2):
+            ctx.forces(0.6, EPS)
+            a1 = ctx.get_acc()
+            assert np.all(np.linalg.norm(a1 - a0, axis=1) <= 4e-5 * np.linalg.norm(a0, axis=1).mean())
+        break
+    else:
+        pytest.fail("no cap let the build through")
