@@ -67,7 +67,7 @@ TRAIN_SEEDS = (3, 4, 5)  # networks trained from these seeds; the training spher
 PROFILE_TRAFFIC = os.path.join(ROOT, "profiles", "walk_uniform_1m.txt")
 PROFILE_TRAFFIC_PLUMMER = os.path.join(ROOT, "profiles", "walk_plummer_4m.txt")
 PROFILE_TRAFFIC_PLUMMER_ONEWARP = os.path.join(ROOT, "profiles", "walk_plummer_4m_onewarp.txt")
-WALK_SRC = [os.path.join(ROOT, "paper_1211_2293_gb300", "csrc", f) for f in ("tc_walk.cuh", "tc_walk_ws.cuh")]
+WALK_SRC = [os.path.join(ROOT, "paper_1211_2293_gb300", "csrc", f) for f in ("tc_walk.cuh", "tc_walk_ws.cuh", "tc_f32x2.cuh")]
 
 
 def walk_source_hash(paths=None):
