@@ -149,9 +149,8 @@ struct tc_ctx {
     SortBufs pair_sb{};
     int64_t pair_sort_cap = 0;
 
-    // fast multipole method: parent table, local expansions, unresolved
-    // source lists (per node: offset and count into the pool of its level's
-    // parity), per-warp slabs, counters, level starts
+    // fast multipole method: local expansions, unresolved source lists (per
+    // node: offset and count into the pool), per-warp slabs, counters
     bool forces_fmm = false;
     float* fmm_loc = nullptr;
     int64_t* fmm_off = nullptr;

@@ -1066,15 +1066,27 @@ __global__ void __launch_bounds__(kSumThreads) k_mlp_sums(const float* __restric
 // the model's maps from the sums: feature means and inverse standard
 // deviations (0 for a constant feature), output RMS (1 for an all-zero
 // output); and the factor-weight scale n / sum F^2
-__global__ void k_mlp_maps(const double* __restrict__ part, int nblocks, int64_t n, float* __restrict__ maps,
-                           float* __restrict__ wscale)
+// (one warp per j = 0..7 adds the blocks b = j mod 8, then the eight sums in
+// turn: one chain of FP64 additions per column took 56 us of 2^18 pairs' 2.6 ms,
+// 15)
+constexpr int kMapWarps = 8;
+__global__ void __launch_bounds__(32 * kMapWarps) k_mlp_maps(const double* __restrict__ part, int nblocks, int64_t n,
+                                                             float* __restrict__ maps, float* __restrict__ wscale)
 {
-    __shared__ double sums[kMlpSums];
-    const int k = threadIdx.x;
+    __shared__ double red[kMapWarps][kMlpSums], sums[kMlpSums];
+    const int k = threadIdx.x & 31, j = threadIdx.x >> 5;
     if (k < kMlpSums) {
         double v = 0.0;
-#pragma unroll 16
-        for (int b = 0; b < nblocks; b++) v += part[(int64_t)b * kMlpSums + k];
+#pragma unroll 8
+        for (int b = j; b < nblocks; b += kMapWarps) v += part[(int64_t)b * kMlpSums + k];
+        red[j][k] = v;
+    }
+    __syncthreads();
+    if (j > 0) return;
+    if (k < kMlpSums) {
+        double v = red[0][k];
+#pragma unroll
+        for (int w = 1; w < kMapWarps; w++) v += red[w][k];
         sums[k] = v;
     }
     __syncwarp();
@@ -1303,7 +1315,7 @@ void launch_mlp_maps(const float* X, const float* T, const float* F, int64_t n, 
 {
     const int nb = mlp_sum_blocks(n);
     k_mlp_sums<<<nb, kSumThreads, 0, s>>>(X, T, F, n, part);
-    k_mlp_maps<<<1, 32, 0, s>>>(part, nb, n, maps, wscale);
+    k_mlp_maps<<<1, 32 * kMapWarps, 0, s>>>(part, nb, n, maps, wscale);
     count_launches(2);
 }
 
