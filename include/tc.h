@@ -159,7 +159,8 @@ int tc_ctx_forces(tc_ctx *ctx, float theta, float eps, float G);
  * a prior tc_ctx_forces on the current positions.  Enqueue only: the rebuild
  * reuses the node table sized by the last tc_ctx_build / tc_set_state (with
  * 50% headroom); a tree that outgrows it stops the step on the device and
- * the next synchronising call reports TC_EDEVICE. */
+ * the next synchronising call reports TC_EDEVICE; from then on the context
+ * has no tree (see tc_set_state). */
 int tc_ctx_step(tc_ctx *ctx, float dt);
 
 /* Accelerations (n x 3) and, if pot != NULL and want_pot was set, the
@@ -170,10 +171,15 @@ int tc_get_acc(tc_ctx *ctx, float *acc, float *pot);
 /* Current positions / velocities (n x 3 each; either may be NULL). */
 int tc_get_state(tc_ctx *ctx, float *pos, float *vel);
 /* Replace positions and velocities (n x 3 each, n of the last build) and
- * rebuild the tree; forces must be recomputed before the next step. */
+ * rebuild the tree; forces must be recomputed before the next step.
+ * After a rebuild that failed (this call or tc_set_config reported an error,
+ * a step's rebuild stopped) the context holds the bodies but no tree and no
+ * forces: calls that need those return TC_ESTATE until tc_set_state or a
+ * build succeeds; after a failed tc_ctx_build only a build does. */
 int tc_set_state(tc_ctx *ctx, const float *pos, const float *vel);
 
-/* Sizes of the last build: bodies, nodes, groups (any may be NULL). */
+/* Sizes of the last build: bodies, and the nodes and groups of the last tree
+ * (any may be NULL). */
 int tc_get_sizes(tc_ctx *ctx, int64_t *n, int64_t *nnodes, int64_t *ngroups);
 
 /* Verification exports of the last build (any pointer may be NULL).

@@ -42,7 +42,9 @@ struct tc_ctx {
     int nchunks = 0, cap_chunks = 0;
     int64_t M = 0, cap_m = 0;  // nodes of the last synchronised build, node table capacity
     int leaf_max = 0;
-    bool built = false, have_forces = false, forces_pot = false;
+    // built: the bodies of a build are here (a failed tc_set_state keeps them);
+    // tree: the node and group tables are theirs
+    bool built = false, tree = false, have_forces = false, forces_pot = false;
     float theta = 0.f, eps = 0.f, Gc = 0.f;
 
     // state, original body order
@@ -370,6 +372,7 @@ int check_device(tc_ctx* c)
     TC_CUDA(c, cudaStreamSynchronize(c->stream));
     int32_t e = c->info_h->err;
     if (e) {
+        if (e & kErrCapacity) c->tree = c->have_forces = false;  // a rebuild stopped before its tables
         TC_CUDA(c, cudaMemsetAsync(&c->info->err, 0, sizeof(int32_t), c->stream));
         // a walk whose wait gave up leaves its groups' counts
         if (c->part_done) TC_CUDA(c, cudaMemsetAsync(c->part_done, 0, c->cap_n * sizeof(int32_t), c->stream));
@@ -483,6 +486,7 @@ constexpr int64_t kChainBodies = kClimbBodies;
 int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
 {
     const int64_t n = c->n;
+    if (synced) c->tree = c->have_forces = false;  // until it has succeeded
     const ChainStream cs(s, synced && n <= kChainBodies);
     cudaEvent_t t0 = phase_begin(c, s, 0);
     // The passes sort only the key digits of the levels down to the last
@@ -544,10 +548,10 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
             return build_tree(c, true, s, true);
         }
         if (c->info_h->err) return check_device(c);  // invalid input; clears the word
-        if (c->info_h->M < 1) return fail(c, TC_EDEVICE, "empty node table");
-        int r = ensure_nodes(c, c->info_h->M);
+        if (c->info_h->count < 1) return fail(c, TC_EDEVICE, "empty node table");
+        int r = ensure_nodes(c, c->info_h->count);
         if (r) return r;
-        c->M = c->info_h->M;
+        c->M = c->info_h->count;
         depth = c->info_h->depth;
         c->depth_hint = depth;
         c->depth_hint_n = n;
@@ -559,8 +563,8 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
     c->gorder_ready = false;
     TC_CUDA(c, cudaGetLastError());
     phase_end(c, 0, t0, s);
-    c->built = true;
     c->have_forces = false;
+    if (synced) c->built = c->tree = true;
     return TC_OK;
 }
 
@@ -928,7 +932,7 @@ int tc_set_config(tc_ctx* c, const tc_config* cfg)
         return fail(c, TC_EINVAL, "quadrupole = 1 needs precise = 1 and quad = 1");
     if (cfg->classes < 0 || cfg->classes > 1) return fail(c, TC_EINVAL, "classes must be 0 or 1 (got %d)", cfg->classes);
     if (cfg->split < 0 || cfg->split > 2) return fail(c, TC_EINVAL, "split must be 0, 1 or 2 (got %d)", cfg->split);
-    bool rebuild = c->built && (cfg->gmax != c->cfg.gmax || (cfg->quad != 0) != (c->cfg.quad != 0));
+    bool rebuild = c->tree && (cfg->gmax != c->cfg.gmax || (cfg->quad != 0) != (c->cfg.quad != 0));
     c->cfg = *cfg;
     c->cfg.precise = cfg->precise ? 1 : 0;
     c->cfg.want_pot = cfg->want_pot ? 1 : 0;
@@ -976,6 +980,7 @@ static int build_systems(tc_ctx* c, const float* pos, const float* mass, const i
     if (n >= (int64_t)1 << 31) return fail(c, TC_EINVAL, "tc_build: n must be below 2^31 (got %lld)", (long long)n);
     int r = ensure_bodies(c, n);
     if (r) return r;
+    c->built = c->tree = c->have_forces = false;  // until it has succeeded
     if (n != c->n) TC_CUDA(c, cudaMemsetAsync(c->vel, 0, 3 * n * sizeof(float), c->stream));
     c->n = n;
     c->leaf_max = leaf_max;
@@ -985,7 +990,6 @@ static int build_systems(tc_ctx* c, const float* pos, const float* mass, const i
     }
     TC_CUDA(c, cudaMemcpyAsync(c->pos, pos, 3 * n * sizeof(float), cudaMemcpyDefault, c->stream));
     TC_CUDA(c, cudaMemcpyAsync(c->mass, mass, n * sizeof(float), cudaMemcpyDefault, c->stream));
-    c->built = false;
     return build_tree(c, true, c->stream);
 }
 
@@ -1014,7 +1018,7 @@ int tc_ctx_set_velocity(tc_ctx* c, const float* vel)
 int tc_ctx_forces(tc_ctx* c, float theta, float eps, float G)
 {
     if (!c) return fail(c, TC_EINVAL, "tc_forces: null context");
-    if (!c->built) return fail(c, TC_ESTATE, "tc_forces: build the tree first");
+    if (!c->tree) return fail(c, TC_ESTATE, "tc_forces: build the tree first");
     if (!finite(theta) || theta < 0.f) return fail(c, TC_EINVAL, "tc_forces: theta must be finite and >= 0");
     if (!finite(eps) || eps <= 0.f) return fail(c, TC_EINVAL, "tc_forces: eps must be finite and > 0");
     if (!finite(G)) return fail(c, TC_EINVAL, "tc_forces: G must be finite");
@@ -1065,6 +1069,7 @@ int tc_set_state(tc_ctx* c, const float* pos, const float* vel)
     if (!c || !pos || !vel) return fail(c, TC_EINVAL, "tc_set_state: null argument");
     if (!c->built) return fail(c, TC_ESTATE, "tc_set_state: build first");
     TC_CUDA(c, cudaMemcpyAsync(c->pos, pos, 3 * c->n * sizeof(float), cudaMemcpyDefault, c->stream));
+    c->tree = c->have_forces = false;
     TC_CUDA(c, cudaMemcpyAsync(c->vel, vel, 3 * c->n * sizeof(float), cudaMemcpyDefault, c->stream));
     return build_tree(c, true, c->stream);
 }
@@ -1084,7 +1089,7 @@ int tc_get_sizes(tc_ctx* c, int64_t* n, int64_t* nnodes, int64_t* ngroups)
 int tc_get_systems(tc_ctx* c, int64_t* nsys, double* cubes)
 {
     if (!c) return fail(c, TC_EINVAL, "tc_get_systems: null context");
-    if (!c->built) return fail(c, TC_ESTATE, "tc_get_systems: build first");
+    if (!c->tree) return fail(c, TC_ESTATE, "tc_get_systems: build first");
     int r = check_device(c);
     if (r) return r;
     if (nsys) *nsys = c->nsys;
@@ -1103,7 +1108,7 @@ int tc_get_systems(tc_ctx* c, int64_t* nsys, double* cubes)
 int tc_get_cube(tc_ctx* c, double* out5)
 {
     if (!c || !out5) return fail(c, TC_EINVAL, "tc_get_cube: null argument");
-    if (!c->built) return fail(c, TC_ESTATE, "tc_get_cube: build first");
+    if (!c->tree) return fail(c, TC_ESTATE, "tc_get_cube: build first");
     std::vector<double> all(5 * (size_t)c->nsys);
     int r = tc_get_systems(c, nullptr, all.data());
     if (r) return r;
@@ -1114,7 +1119,7 @@ int tc_get_cube(tc_ctx* c, double* out5)
 int tc_get_tree(tc_ctx* c, uint32_t* perm, uint64_t* keys)
 {
     if (!c) return fail(c, TC_EINVAL, "tc_get_tree: null context");
-    if (!c->built) return fail(c, TC_ESTATE, "tc_get_tree: build first");
+    if (!c->tree) return fail(c, TC_ESTATE, "tc_get_tree: build first");
     if (perm) TC_CUDA(c, cudaMemcpyAsync(perm, c->perm, c->n * sizeof(uint32_t), cudaMemcpyDefault, c->stream));
     if (keys) TC_CUDA(c, cudaMemcpyAsync(keys, c->keys, c->n * sizeof(uint64_t), cudaMemcpyDefault, c->stream));
     return check_device(c);
@@ -1124,7 +1129,7 @@ int tc_get_nodes(tc_ctx* c, int32_t* level, uint64_t* prefix, int32_t* first, in
                  int32_t* nchild, double* mass, double* com, double* quad)
 {
     if (!c) return fail(c, TC_EINVAL, "tc_get_nodes: null context");
-    if (!c->built) return fail(c, TC_ESTATE, "tc_get_nodes: build first");
+    if (!c->tree) return fail(c, TC_ESTATE, "tc_get_nodes: build first");
     if (quad && !c->cfg.quad) return fail(c, TC_ESTATE, "tc_get_nodes: second moments not computed (quad = 0)");
     int r = check_device(c);
     if (r) return r;
@@ -1159,7 +1164,7 @@ int tc_get_nodes(tc_ctx* c, int32_t* level, uint64_t* prefix, int32_t* first, in
 int tc_get_groups(tc_ctx* c, int32_t* gfirst, int32_t* gcount, int32_t* gref)
 {
     if (!c) return fail(c, TC_EINVAL, "tc_get_groups: null context");
-    if (!c->built) return fail(c, TC_ESTATE, "tc_get_groups: build first");
+    if (!c->tree) return fail(c, TC_ESTATE, "tc_get_groups: build first");
     int r = check_device(c);
     if (r) return r;
     const int64_t G = c->info_h->G;
@@ -1209,7 +1214,7 @@ int tc_diag(tc_ctx* c, double* out8)
 int tc_ctx_fmm(tc_ctx* c, float theta, float eps, float G)
 {
     if (!c) return fail(c, TC_EINVAL, "tc_fmm: null context");
-    if (!c->built) return fail(c, TC_ESTATE, "tc_fmm: build the tree first");
+    if (!c->tree) return fail(c, TC_ESTATE, "tc_fmm: build the tree first");
     if (!finite(theta) || theta < 0.f) return fail(c, TC_EINVAL, "tc_fmm: theta must be finite and >= 0");
     if (!finite(eps) || eps <= 0.f) return fail(c, TC_EINVAL, "tc_fmm: eps must be finite and > 0");
     if (!finite(G)) return fail(c, TC_EINVAL, "tc_fmm: G must be finite");
@@ -1664,7 +1669,7 @@ int tc_mlp_pairs(tc_ctx* c, float theta, float eps, float band, float prob, uint
                  float* T, float* F, int64_t* body, int64_t* node, int64_t* npairs)
 {
     if (!c || !npairs) return fail(c, TC_EINVAL, "tc_mlp_pairs: null argument");
-    if (!c->built) return fail(c, TC_ESTATE, "tc_mlp_pairs: build first");
+    if (!c->tree) return fail(c, TC_ESTATE, "tc_mlp_pairs: build first");
     if (!c->cfg.quad) return fail(c, TC_ESTATE, "tc_mlp_pairs: the features need quad = 1");
     if (!finite(theta) || theta < 0.f || !finite(eps) || eps <= 0.f || !finite(band) || band < 0.f ||
         !(prob > 0.f && prob <= 1.f) || max_pairs < 1)
@@ -1785,7 +1790,7 @@ int tc_get_group_list(tc_ctx* c, int64_t group, float theta, int32_t* cells, int
                       int64_t* ncells, int64_t* nleaves)
 {
     if (!c || !ncells || !nleaves) return fail(c, TC_EINVAL, "tc_get_group_list: null argument");
-    if (!c->built) return fail(c, TC_ESTATE, "tc_get_group_list: build first");
+    if (!c->tree) return fail(c, TC_ESTATE, "tc_get_group_list: build first");
     if (!finite(theta) || theta < 0.f || cap < 0) return fail(c, TC_EINVAL, "tc_get_group_list: theta >= 0, cap >= 0");
     int r = check_device(c);
     if (r) return r;
@@ -1851,7 +1856,7 @@ int tc_get_group_list(tc_ctx* c, int64_t group, float theta, int32_t* cells, int
 int tc_autotune(tc_ctx* c, float theta, float eps, float G, int reps, tc_config* best_out, double* best_ms_out)
 {
     if (!c) return fail(c, TC_EINVAL, "tc_autotune: null context");
-    if (!c->built) return fail(c, TC_ESTATE, "tc_autotune: build first");
+    if (!c->tree) return fail(c, TC_ESTATE, "tc_autotune: build first");
     if (!finite(theta) || theta < 0.f || !finite(eps) || eps <= 0.f || !finite(G))
         return fail(c, TC_EINVAL, "tc_autotune: theta >= 0, eps > 0, finite G required");
     if (reps < 1) reps = 1;

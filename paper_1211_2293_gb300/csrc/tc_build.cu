@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(kNodeThreads) k_node_levels_tiled(const uint64
 }
 
 // Exclusive scan of the counts in place, one pass; the total is the number of
-// nodes.  A look-back that gave up raises kErrCapacity too, so nothing is
+// nodes (info->M follows with the records).  A look-back that gave up raises kErrCapacity too, so nothing is
 // placed by offsets that are not known.
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 16;
@@ -551,7 +551,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_levels(uint32_t* cnt, int
     if (threadIdx.x == 0) {
         if (!ok) atomicOr(&info->err, kErrWorkLoop | kErrCapacity);
         if (tile == gridDim.x - 1) {
-            info->M = total;
+            info->count = total;
             if (cap_m >= 0 && (int64_t)total > cap_m) atomicOr(&info->err, kErrCapacity);
         }
     }
@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(kNodeThreads) k_emit_nodes(const uint64_t* key
                                                              const int8_t* delta,
                                                              const int8_t* top,
                                                              const uint32_t* sys_of, int64_t n,
-                                                             const uint32_t* offs, const Info* info,
+                                                             const uint32_t* offs, Info* info,
                                                              uint32_t* lstart, NodeTables nt)
 {
     pdl_begin();
@@ -589,7 +589,8 @@ __global__ void __launch_bounds__(kNodeThreads) k_emit_nodes(const uint64_t* key
         sy[r] = s < n ? sys_of[s] : 0u;
     }
     if (blockIdx.x == 0 && threadIdx.x <= kLevels)  // the first node of each level
-        lstart[threadIdx.x] = threadIdx.x < kLevels ? offs[(int64_t)threadIdx.x * gridDim.x] : (uint32_t)info->M;
+        lstart[threadIdx.x] = threadIdx.x < kLevels ? offs[(int64_t)threadIdx.x * gridDim.x] : (uint32_t)info->count;
+    if (blockIdx.x == 0 && threadIdx.x == 0) info->M = info->count;
 #pragma unroll
     for (int r = 0; r < kNodeRounds; r++) {
         const uint32_t mine = set_levels(d[r], t[r]);
@@ -1037,7 +1038,8 @@ __global__ void k_group_marks(const Info* info, const NodeTables nt, int gmax, i
     }
 }
 
-// the marked bodies in order -> the group table, one pass
+// the marked bodies in order -> the group table, one pass (which stays as it is
+// where the build stopped)
 __global__ void __launch_bounds__(kScanThreads) k_group_table(const int32_t* gref_at, int64_t n,
                                                               unsigned long long* st, uint32_t* counter,
                                                               int32_t* gfirst, int32_t* gref,
@@ -1046,8 +1048,9 @@ __global__ void __launch_bounds__(kScanThreads) k_group_table(const int32_t* gre
     pdl_begin();
     __shared__ int tile_sh;
     __shared__ int32_t mark[kScanTile];
-    if (threadIdx.x == 0) tile_sh = (int)atomicAdd(counter, 1u);
+    if (threadIdx.x == 0) tile_sh = capacity_failed(info) ? -1 : (int)atomicAdd(counter, 1u);
     __syncthreads();
+    if (tile_sh < 0) return;
     const int64_t tile = tile_sh, t0 = tile * kScanTile;
 #pragma unroll
     for (int i = 0; i < kScanItems; i++) {
@@ -1295,7 +1298,7 @@ void launch_node_levels(const uint64_t* keys, const uint32_t* sys_of, int64_t n,
 }
 
 void launch_emit_nodes(const uint64_t* keys, const int8_t* delta, const int8_t* top, const uint32_t* sys_of, int64_t n,
-                       const uint32_t* offs, const Info* info, uint32_t* lstart, NodeTables nt, ChainStream s)
+                       const uint32_t* offs, Info* info, uint32_t* lstart, NodeTables nt, ChainStream s)
 {
     pdl_launch(k_emit_nodes, nblk(n, kNodeBlock), kNodeThreads, 0, s, keys, delta, top, sys_of, n, offs, info, lstart,
                nt);

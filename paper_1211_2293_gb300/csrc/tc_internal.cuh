@@ -60,8 +60,9 @@ struct ChainStream {
 struct Info {
     int32_t err;       // error bits
     int32_t depth;     // deepest level of the forest
-    int64_t M;         // number of nodes
-    int64_t G;         // number of groups
+    int64_t M;         // nodes in the node table
+    int64_t G;         // groups in the group table
+    int64_t count;     // nodes that the last build counted (M once they are in the table)
     uint32_t work[4];  // walk work-queue counters, one per launch of a force phase
     unsigned long long interactions;  // body-source interactions of the last walk
     unsigned long long cells;         // body-cell interactions (group size x accepted cells)
@@ -197,7 +198,7 @@ void launch_gather(const float* pos, const float* mass, const uint32_t* perm, in
 // The levels of the cubes that start at each sorted body (delta < l <= top),
 // their number per level and block of bodies, and the exclusive scan of those
 // (level by level, so the nodes' breadth-first places); zeroes gref_at;
-// info->M = nodes, kErrCapacity where cap_m >= 0 and M exceeds it.  cnt:
+// info->count = nodes, kErrCapacity where cap_m >= 0 and it exceeds that.  cnt:
 // level_counts_size(n) words; scan: build_scan_words(n) words, zeroed.
 int64_t level_counts_size(int64_t n);
 int64_t build_scan_words(int64_t n);
@@ -205,9 +206,10 @@ void launch_node_levels(const uint64_t* keys, const uint32_t* sys_of, int64_t n,
                         int8_t* delta, int8_t* top, int32_t* gref_at, uint32_t* cnt, unsigned long long* scan,
                         int64_t cap_m, Info* info, ChainStream s);
 // the node records at those places (counts and children follow with the
-// moments) and lstart[0..22], the first node of each level
+// moments), lstart[0..22], the first node of each level, and info->M; nothing
+// (so M stays that of the table) after kErrCapacity
 void launch_emit_nodes(const uint64_t* keys, const int8_t* delta, const int8_t* top, const uint32_t* sys_of, int64_t n,
-                       const uint32_t* offs, const Info* info, uint32_t* lstart, NodeTables nt, ChainStream s);
+                       const uint32_t* offs, Info* info, uint32_t* lstart, NodeTables nt, ChainStream s);
 // counts, children and moments: the leaves, then the internal cells, in the
 // same launch for up to kClimbBodies bodies, else level by level from
 // depth - 1 (depth < 0: the depth is known on the device only; with
