@@ -456,6 +456,7 @@ int setup_systems(tc_ctx* c, const int64_t* off, int nsys)
         for (int64_t a = off[s]; a < off[s + 1]; a += chunk)
             ch.push_back(make_int4(s, (int)a, (int)std::min(off[s + 1], a + chunk),
                                    (int)((off[s + 1] - off[s] + chunk - 1) / chunk)));
+    drop_graph(c);  // a captured step holds the number of chunks and counts on their table
     int r = ensure_systems(c, nsys, (int)ch.size());
     if (r) return r;
     c->off_h.assign(off, off + nsys + 1);
