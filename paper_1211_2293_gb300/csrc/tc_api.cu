@@ -173,6 +173,7 @@ struct tc_ctx {
     // the captured leapfrog step
     cudaGraphExec_t gexec = nullptr;
     std::string gkey;
+    int gdepth = -1;  // the tree depth its sort and moments count on (depth_hint)
     long long graph_kernels = 0;
 };
 
@@ -808,7 +809,11 @@ int step_graph(tc_ctx* c, float dt)
 {
     const bool timing = c->timing;
     const std::string key = graph_key(c, dt) + (timing ? "/timed" : "");
-    if (!c->gexec || key != c->gkey) {
+    // (a graph sorts the digits of the depth it was captured with: a deeper
+    // tree built since would meet long runs of equal digits, ranked in
+    // quadratic time or, past kSortRunMax bodies, refused at every replay; a
+    // shallower one is sorted all the same)
+    if (!c->gexec || key != c->gkey || c->depth_hint > c->gdepth) {
         drop_graph(c);
         if (!c->cap_stream) TC_CUDA(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
         int r = prepare_forces(c);
@@ -840,6 +845,7 @@ int step_graph(tc_ctx* c, float dt)
             return fail(c, TC_ECUDA, "step graph instantiation: %s", cudaGetErrorString(e));
         }
         c->gkey = key;
+        c->gdepth = c->depth_hint;
     }
     cudaEvent_t t0 = phase_begin(c, c->stream, 0);
     c->gorder_ready = false;  // the graph rebuilds the groups

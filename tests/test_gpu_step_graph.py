@@ -47,3 +47,32 @@ def test_other_split_of_the_same_bodies():
         out.append(got)
     for a, b in zip(*out):
         _same(a, b)
+
+
+@pytest.mark.parametrize("shallow_again", [False, True])
+def test_deeper_tree_built_since_the_capture(shallow_again):
+    """A step captured on an even cloud, then a state of as many bodies and
+    nodes with 20000 of them in a cube of side 1e-4, more than a step orders
+    within a run of equal digits: its steps sort the digits of that tree."""
+    from paper_1211_2293_gb300 import tc
+
+    n, tight = 40000, 20000
+    rng = np.random.default_rng(81)
+    p = rng.random((n, 3)).astype(np.float32)
+    q = p.copy()
+    q[:tight] = (0.3 + 1e-4 * rng.random((tight, 3))).astype(np.float32)
+    v, m = np.zeros_like(p), np.full(n, 1.0 / n, np.float32)
+    out = []
+    for graph in (0, 1):
+        ctx = tc.Context(graph=graph)
+        ctx.build(_dev(p), _dev(m), 16)
+        got = []
+        for x in (p, q, p) if shallow_again else (p, q):
+            ctx.set_state(_dev(x), _dev(v))
+            ctx.forces(0.7, 0.01)
+            for _ in range(2):
+                ctx.step(1e-6)
+            got.append(_state(ctx))
+        out.append(got)
+    for a, b in zip(*out):
+        _same(a, b)
