@@ -808,6 +808,10 @@ std::string graph_key(tc_ctx* c, float dt)
 int step_graph(tc_ctx* c, float dt)
 {
     const bool timing = c->timing;
+    // the walk of this configuration (list export, training pairs and another
+    // configuration leave theirs); it may drop the graph
+    int r = prepare_forces(c);
+    if (r) return r;
     const std::string key = graph_key(c, dt) + (timing ? "/timed" : "");
     // (a graph sorts the digits of the depth it was captured with: a deeper
     // tree built since would meet long runs of equal digits, ranked in
@@ -816,8 +820,6 @@ int step_graph(tc_ctx* c, float dt)
     if (!c->gexec || key != c->gkey || c->depth_hint > c->gdepth) {
         drop_graph(c);
         if (!c->cap_stream) TC_CUDA(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
-        int r = prepare_forces(c);
-        if (r) return r;
         c->timing = false;
         const long long k0 = launches_total();
         cudaStream_t s = c->cap_stream;
@@ -853,7 +855,7 @@ int step_graph(tc_ctx* c, float dt)
     count_launches((int)c->graph_kernels);
     phase_end(c, 0, t0, c->stream);  // (timing mode: kick + drift + rebuild)
     if (timing) {
-        int r = run_forces(c, c->theta, c->eps, c->Gc, c->stream);
+        r = run_forces(c, c->theta, c->eps, c->Gc, c->stream);
         if (r) return r;
         t0 = phase_begin(c, c->stream, 2);
         launch_kick(c->vel, c->acc, c->n, 0.5f * dt, c->info, c->stream);

@@ -76,3 +76,32 @@ def test_deeper_tree_built_since_the_capture(shallow_again):
         out.append(got)
     for a, b in zip(*out):
         _same(a, b)
+
+
+@pytest.mark.parametrize("cfg", [dict(quad=1, quadrupole=1), dict(want_pot=1, gmax=128)])
+@pytest.mark.parametrize("between", ["list", "other"])
+def test_timed_step_after_another_walk(cfg, between):
+    """With phase timing the walk follows the graph: it is the configuration's,
+    whatever walk ran between two steps."""
+    from paper_1211_2293_gb300 import tc
+
+    p, v, m = inputs.plummer(5000, 91)
+    out = []
+    for timing in (False, True):
+        ctx = tc.Context(**cfg)
+        ctx.set_timing(timing)
+        ctx.build(_dev(p), _dev(m), 8)
+        ctx.set_velocity(_dev(v))
+        ctx.forces(0.6, 0.01)
+        ctx.group_list(3, 0.3)  # (its scratch: a buffer that grows drops the graph)
+        ctx.step(1e-3)
+        if between == "list":
+            ctx.group_list(3, 0.9)
+        else:
+            keep = ctx.config()
+            ctx.set_config(quadrupole=0, split=0)
+            ctx.forces(0.6, 0.01)
+            ctx.set_config(**keep)
+        ctx.step(1e-3)
+        out.append(_state(ctx))
+    _same(*out)
