@@ -253,6 +253,10 @@ void drop_graph(tc_ctx* c)
     c->gkey.clear();
 }
 
+// A buffer of count elements in place of *p.  The old one goes first, so the
+// capacity that stands for a set of buffers is zero before the first of them
+// grows and set after the last: where one finds no memory the next call grows
+// all of them again.
 template <typename T>
 int grow(tc_ctx* c, T** p, int64_t count)
 {
@@ -296,6 +300,11 @@ int ensure_bodies(tc_ctx* c, int64_t n)
 {
     if (n <= c->cap_n) return TC_OK;
     int64_t cap = n;
+    // the last build's bodies, tree and forces go with their buffers; the node
+    // tables are sized with the first build at this capacity
+    c->built = c->tree = c->have_forces = false;
+    c->off_h.clear();
+    c->n = c->cap_n = c->cap_m = 0;
     TC_GROW(c, c->pos, 3 * cap);
     TC_GROW(c, c->vel, 3 * cap);
     TC_GROW(c, c->acc, 3 * cap);
@@ -326,18 +335,19 @@ int ensure_bodies(tc_ctx* c, int64_t n)
     TC_GROW(c, c->part_done, cap);
     TC_GROW(c, c->gseg, 4 + (int64_t)group_order_scratch());
     c->cap_n = cap;
-    c->cap_m = 0;  // node tables are sized with the first build at this capacity
     return TC_OK;
 }
 
 int ensure_systems(tc_ctx* c, int nsys, int nchunks)
 {
     if (nsys > c->cap_sys) {
+        c->cap_sys = 0;
         TC_GROW(c, c->sysp, nsys);
         TC_GROW(c, c->off_dev, nsys + 1);
         c->cap_sys = nsys;
     }
     if (nchunks > c->cap_chunks) {
+        c->cap_chunks = 0;
         TC_GROW(c, c->chunks, nchunks);
         c->cap_chunks = nchunks;
     }
@@ -348,6 +358,7 @@ int ensure_nodes(tc_ctx* c, int64_t M)
 {
     if (M <= c->cap_m) return TC_OK;
     const int64_t cap = M + M / 2 + 1024;  // headroom for the rebuilds of later steps
+    c->cap_m = 0;
     TC_GROW(c, c->nt.a, cap);
     TC_GROW(c, c->nt.b, cap);
     TC_GROW(c, c->nt.c, cap);
@@ -458,6 +469,7 @@ int setup_systems(tc_ctx* c, const int64_t* off, int nsys)
             ch.push_back(make_int4(s, (int)a, (int)std::min(off[s + 1], a + chunk),
                                    (int)((off[s + 1] - off[s] + chunk - 1) / chunk)));
     drop_graph(c);  // a captured step holds the number of chunks and counts on their table
+    c->off_h.clear();  // until the new ones are on the device
     int r = ensure_systems(c, nsys, (int)ch.size());
     if (r) return r;
     c->off_h.assign(off, off + nsys + 1);
@@ -637,13 +649,16 @@ int prepare_forces(tc_ctx* c)
             if (v > 0) want = v;
         }
         if (want != c->band_cap) {
-            if (want > c->band_cap) TC_GROW(c, c->band, want);
+            const bool more = want > c->band_cap;
+            c->band_cap = 0;
+            if (more) TC_GROW(c, c->band, want);
             c->band_cap = want;
             c->walk_ready = false;
             drop_graph(c);
         }
         if (!c->band_n) TC_GROW(c, c->band_n, 1);
         if (c->cap_n + 1 > c->band_gcap) {
+            c->band_gcap = 0;
             TC_GROW(c, c->grec, 2 * (c->cap_n + 1));
             TC_GROW(c, c->gcorr, 3 * (c->cap_n + 1));
             c->band_gcap = c->cap_n + 1;
@@ -1231,6 +1246,7 @@ int tc_ctx_fmm(tc_ctx* c, float theta, float eps, float G)
     if (r) return r;
     cudaStream_t s = c->stream;
     if (c->fmm_cap_m < c->cap_m) {
+        c->fmm_cap_m = 0;
         TC_GROW(c, c->fmm_loc, c->cap_m * fmm_loc_width());
         TC_GROW(c, c->fmm_off, c->cap_m);
         TC_GROW(c, c->fmm_cnt, 2 * c->cap_m);
@@ -1254,11 +1270,13 @@ int tc_ctx_fmm(tc_ctx* c, float theta, float eps, float G)
     unsigned long long ctr[8];
     for (int attempt = 0;; attempt++) {
         if (want_pool > c->fmm_pool_cap) {
+            c->fmm_pool_cap = 0;
             TC_GROW(c, c->fmm_pool, want_pool);
             c->fmm_pool_cap = want_pool;
         }
         const int64_t warps = fmm_slab_warps();
         if (want_slab > c->fmm_slab_cap || warps != c->fmm_slab_warps) {
+            c->fmm_slab_cap = 0;
             TC_GROW(c, c->fmm_slab, want_slab * warps);
             c->fmm_slab_cap = want_slab;
             c->fmm_slab_warps = warps;
@@ -1290,6 +1308,7 @@ int tc_ctx_fmm(tc_ctx* c, float theta, float eps, float G)
         p.theta = theta;
         p.eps = eps;
         p.G = G;
+        c->have_forces = false;  // (the pass writes where the last force phase's accelerations are)
         cudaError_t e = launch_fmm(p, s);
         if (e != cudaSuccess) return fail(c, TC_ECUDA, "fmm launch: %s", cudaGetErrorString(e));
         TC_CUDA(c, cudaMemcpyAsync(ctr, c->fmm_ctr, sizeof(ctr), cudaMemcpyDeviceToHost, s));
@@ -1307,10 +1326,7 @@ int tc_ctx_fmm(tc_ctx* c, float theta, float eps, float G)
                 want_slab = std::max<int64_t>((int64_t)(ctr[3] + ctr[3] / 4 + 256), 2 * c->fmm_slab_cap);
             continue;
         }
-        if (err) {
-            c->have_forces = false;
-            return check_device(c);  // reports and clears the error word
-        }
+        if (err) return check_device(c);  // reports and clears the error word
         break;
     }
     phase_end(c, 1, t0, s);
@@ -1365,6 +1381,7 @@ int tc_direct(tc_ctx* c, const int64_t* idx, int64_t ns, float eps, float G, dou
         if (hidx[k] < 0 || hidx[k] >= c->n)
             return fail(c, TC_EINVAL, "tc_direct: index %lld out of range", (long long)hidx[k]);
     if (ns > c->cap_idx) {
+        c->cap_idx = 0;
         TC_GROW(c, c->idx_dev, ns);
         TC_GROW(c, c->dir_out, 4 * ns);
         c->cap_idx = ns;
@@ -1437,7 +1454,7 @@ constexpr int kMlpNModel = kMlpNParamHost + 2 * 13 + 3;  // parameters + feature
 
 int mlp_alloc(tc_ctx* c)
 {
-    if (c->mlp_params) return TC_OK;
+    if (c->mlp_bad) return TC_OK;  // (the last of them)
     TC_GROW(c, c->mlp_params, kMlpNParamHost);
     TC_GROW(c, c->mlp_maps, 32);
     TC_GROW(c, *(char**)&c->mlp_dev, (int64_t)mlp_dev_size());
@@ -1456,6 +1473,7 @@ int mlp_alloc(tc_ctx* c)
 int mlp_scratch(tc_ctx* c, int64_t n)
 {
     if (n <= c->mlp_cap) return TC_OK;
+    c->mlp_cap = 0;
     TC_GROW(c, c->mlp_x, n * 16);
     TC_GROW(c, c->mlp_t, n * 3);
     TC_GROW(c, c->mlp_w, n);
@@ -1560,6 +1578,7 @@ static int mlp_part(tc_ctx* c, int blocks)
 {
     const int64_t want = mlp_train_part_floats(blocks);
     if (want > c->mlp_part_cap) {
+        c->mlp_part_cap = 0;
         TC_GROW(c, c->mlp_part, want);
         c->mlp_part_cap = want;
     }
@@ -1684,6 +1703,7 @@ int tc_mlp_pairs(tc_ctx* c, float theta, float eps, float band, float prob, uint
         !(prob > 0.f && prob <= 1.f) || max_pairs < 1)
         return fail(c, TC_EINVAL, "tc_mlp_pairs: theta >= 0, eps > 0, band >= 0, 0 < prob <= 1, max_pairs >= 1");
     if (max_pairs > c->pair_cap) {
+        c->pair_cap = 0;
         TC_GROW(c, c->pair_b, max_pairs);
         TC_GROW(c, c->pair_v, max_pairs);
         TC_GROW(c, c->pair_n, 1);
@@ -1691,6 +1711,7 @@ int tc_mlp_pairs(tc_ctx* c, float theta, float eps, float band, float prob, uint
     }
     if (max_pairs > c->pair_sort_cap) {
         const int64_t cap = max_pairs;
+        c->pair_sort_cap = 0;
         TC_GROW(c, c->pair_key, cap);
         TC_GROW(c, c->pair_val, cap);
         TC_GROW(c, c->pair_sb.keys_alt, cap);
@@ -1806,6 +1827,7 @@ int tc_get_group_list(tc_ctx* c, int64_t group, float theta, int32_t* cells, int
     if (group < 0 || group >= c->info_h->G) return fail(c, TC_EINVAL, "tc_get_group_list: no group %lld", (long long)group);
     const int64_t want = cap < 1 ? 1 : cap;
     if (want > c->list_cap) {
+        c->list_cap = 0;
         TC_GROW(c, c->list_buf, 2 * want);
         c->list_cap = want;
     }
