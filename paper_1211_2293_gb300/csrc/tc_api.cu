@@ -418,6 +418,15 @@ int check_device(tc_ctx* c)
 
 bool finite(float x) { return std::isfinite(x); }
 
+// work enqueued on s goes into a graph (a step's, or one the caller captures)
+bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(s, &st);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && st != cudaStreamCaptureStatusNone;
+}
+
 cudaEvent_t take_event(tc_ctx* c)
 {
     if (c->ev_used == c->ev_pool.size()) {
@@ -593,13 +602,22 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
 // step and a direct call sum alike.  A stack set below the default is kept as
 // the limit of whole walks.
 constexpr int kDefaultStack = 1024;
+constexpr double kPartTasks = 20.0;  // per SM
 int walk_parts(const tc_ctx* c)
 {
     if (c->cfg.stack < kDefaultStack) return 0;
     const double groups = std::max((double)c->n / (0.7 * c->cfg.gmax), (double)c->nsys);
     int log2 = 0;
-    while (log2 < 3 && groups * (2 << log2) <= 20.0 * c->num_sms) log2++;
+    while (log2 < 3 && groups * (2 << log2) <= kPartTasks * c->num_sms) log2++;
     return log2;
+}
+// the sums of any parts of up to cap_n bodies in groups of up to 128 (10 MB at
+// most on 152 SMs): one size whatever is built and configured in between, so
+// that a force phase the caller captured keeps its buffer
+int64_t part_floats(const tc_ctx* c)
+{
+    const int64_t bodies = std::min<int64_t>(8 * c->cap_n, (int64_t)(kPartTasks * c->num_sms * 0.7 * 128) + 1);
+    return kPartPlanes * bodies;
 }
 
 int prepare_forces(tc_ctx* c)
@@ -624,13 +642,14 @@ int prepare_forces(tc_ctx* c)
     wc.classes = (c->cfg.gmax > 32 && !wc.split) ? c->cfg.classes : 0;
     wc.part_log2 = wc.split ? walk_parts(c) : 0;
     if (wc.part_log2) {
-        const int64_t want = ((int64_t)kPartPlanes << wc.part_log2) * c->n;
-        if (want > c->cap_part && want < c->part_refused) {
+        const int64_t want = part_floats(c);
+        if (want > c->cap_part && want < c->part_refused && !capturing(c->stream)) {
             c->cap_part = 0;
             if (grow(c, &c->part_sum, want) == TC_OK) c->cap_part = want;
             else c->part_refused = want;
         }
-        // a few megabytes; where they are not to be had the groups are walked whole
+        // where they are not to be had, or the caller captures the first
+        // force phase, the groups are walked whole
         if (want > c->cap_part) wc.part_log2 = 0;
     }
     int64_t st = c->cfg.stack;
@@ -730,8 +749,12 @@ int run_forces(tc_ctx* c, float theta, float eps, float G, cudaStream_t s, bool 
     const bool ordered =
         c->walk_ncls > 0 || (c->walk_cfg.split && (double)c->n / (0.7 * c->cfg.gmax) > (double)c->num_sms);
     if (ordered) {
-        if (!c->gorder_ready) launch_group_order(c->gfirst, c->info, c->gorder, c->gseg, c->gseg + 4, {s, chain});
-        c->gorder_ready = true;
+        // (a graph orders the groups it meets when it runs, and orders none
+        // by being captured)
+        const bool graph = capturing(s);
+        if (graph || !c->gorder_ready)
+            launch_group_order(c->gfirst, c->info, c->gorder, c->gseg, c->gseg + 4, {s, chain && !graph});
+        if (!graph) c->gorder_ready = true;
         a.glist = c->gorder;
     }
     if (c->walk_cfg.part_log2) {
