@@ -54,7 +54,9 @@ typedef struct tc_ctx tc_ctx;
  *   want_pot  1: also compute the potential (tc_get_acc's pot, tc_diag's PE)
  *   verify    1: record per-group list lengths and hashes (tc_get_lists)
  *   stack     walk stack entries per walking warp (shared memory), 64..8192;
- *             an entry is a node, in the split walk an opened cell
+ *             an entry is a node, in the split walk an opened cell (as many
+ *             as fit beside its list tiles; of a setting up to the default
+ *             of 1024 the learned split walk takes 512 or more)
  *   blocks_per_sm  0 = as many as fit, else a cap
  *   quad      1: also reduce the cells' second moments about the centre of
  *             mass (FP32, within (leaf_max + 128) 2^-25 M s^2; the learned

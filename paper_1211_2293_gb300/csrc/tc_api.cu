@@ -601,7 +601,6 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
 // systems and gmax only (a group holds about 0.7 gmax bodies), so a captured
 // step and a direct call sum alike.  A stack set below the default is kept as
 // the limit of whole walks.
-constexpr int kDefaultStack = 1024;
 constexpr double kPartTasks = 20.0;  // per SM
 int walk_parts(const tc_ctx* c)
 {

@@ -293,6 +293,7 @@ struct WalkArgs {
     int64_t band_cap;
     float4* grec;
 };
+constexpr int kDefaultStack = 1024;  // tc_config.stack of a new context
 constexpr int kBandChunk = 256;
 constexpr int kPartPlanes = 9;
 struct WalkConfig {

@@ -972,9 +972,12 @@ __host__ __forceinline__ WsShape ws_shape(const WalkConfig& c, int tile, bool ro
         return ws_team_bytes(tile, stack, w.nb, rows) * teams + (rows ? mlp_frag_bytes() : 0);
     };
     while (w.stack > 64 && bytes(w.stack) > kWsSmemMax) w.stack -= 16;
-    // the network and its rows take the room of a second block on the SM;
-    // a stack of more than 512 opened cells gives way
-    if (rows && bytes(512) <= kWsSmemMax / 2 - 1024)
+    // the network and its rows take the room of a second block on the SM; a
+    // stack no larger than the default gives way down to 512 opened cells,
+    // which hold more than that many nodes did (a step takes 8 of them where
+    // it took 32 nodes, and adds as many children to each).  A stack that was
+    // asked for is given, if need be with one block on the SM
+    if (rows && c.stack <= kDefaultStack && bytes(512) <= kWsSmemMax / 2 - 1024)
         while (w.stack > 512 && bytes(w.stack) > kWsSmemMax / 2 - 1024) w.stack -= 16;
     w.smem = bytes(w.stack);
     return w;
