@@ -166,8 +166,8 @@ int tc_ctx_forces(tc_ctx *ctx, float theta, float eps, float G);
 int tc_ctx_step(tc_ctx *ctx, float dt);
 
 /* Accelerations (n x 3) and, if pot != NULL and want_pot was set, the
- * potential (n) of the last force phase, original body order (unspecified
- * contents where the call reports a device error). */
+ * potential (n) of the last force phase, original body order (left as they
+ * are where the call reports a device error). */
 int tc_get_acc(tc_ctx *ctx, float *acc, float *pot);
 
 /* Current positions / velocities (n x 3 each; either may be NULL). */

@@ -418,6 +418,17 @@ int check_device(tc_ctx* c)
 
 bool finite(float x) { return std::isfinite(x); }
 
+// memory of the context's device
+bool on_device(const tc_ctx* c, const void* p)
+{
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == c->device;
+}
+
 // work enqueued on s goes into a graph (a step's, or one the caller captures)
 bool capturing(cudaStream_t s)
 {
@@ -1096,9 +1107,21 @@ int tc_get_acc(tc_ctx* c, float* acc, float* pot)
     if (!c) return fail(c, TC_EINVAL, "tc_get_acc: null context");
     if (!c->have_forces) return fail(c, TC_ESTATE, "tc_get_acc: no forces computed");
     if (pot && !c->forces_pot) return fail(c, TC_ESTATE, "tc_get_acc: potential not computed (want_pot = 0)");
+    // the caller's buffers stay as they are on an error: in this device's
+    // memory they are written by a kernel that looks at the error word, and
+    // one wait does for both; elsewhere the word comes first
+    if ((!acc || on_device(c, acc)) && (!pot || on_device(c, pot))) {
+        if (acc) launch_copy_good(acc, c->acc, 3 * c->n, c->info, c->stream);
+        if (pot) launch_copy_good(pot, c->pot, c->n, c->info, c->stream);
+        TC_CUDA(c, cudaGetLastError());
+        return check_device(c);
+    }
+    int r = check_device(c);
+    if (r) return r;
     if (acc) TC_CUDA(c, cudaMemcpyAsync(acc, c->acc, 3 * c->n * sizeof(float), cudaMemcpyDefault, c->stream));
     if (pot) TC_CUDA(c, cudaMemcpyAsync(pot, c->pot, c->n * sizeof(float), cudaMemcpyDefault, c->stream));
-    return check_device(c);  // waits for the copies too
+    TC_CUDA(c, cudaStreamSynchronize(c->stream));
+    return TC_OK;
 }
 
 int tc_get_state(tc_ctx* c, float* pos, float* vel)

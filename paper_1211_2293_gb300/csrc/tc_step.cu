@@ -70,6 +70,25 @@ __global__ void k_kick_drift(float* __restrict__ pos, float* __restrict__ vel, c
     }
 }
 
+// Results for the caller, who keeps what was there where the force phase
+// failed.  The kernel looks at the error word itself, so one wait serves the
+// copy and the word.
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_copy_good(float* __restrict__ dst, const float* __restrict__ src, int64_t n,
+                                                   const Info* info)
+{
+    if (warp_failed(info)) return;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int64_t done = 0;
+    if (VEC) {
+        const int64_t n4 = n >> 2;
+#pragma unroll 4
+        for (int64_t i = i0; i < n4; i += stride) reinterpret_cast<float4*>(dst)[i] = reinterpret_cast<const float4*>(src)[i];
+        done = n4 << 2;
+    }
+    for (int64_t i = done + i0; i < n; i += stride) dst[i] = src[i];
+}
+
 // KE, PE = 1/2 sum m pot, P, L in FP64; block sums, then FP64 atomics
 __global__ void k_diag(const float* __restrict__ pos, const float* __restrict__ vel, const float* __restrict__ mass,
                        const float* __restrict__ pot, int64_t n, double* __restrict__ out)
@@ -334,6 +353,16 @@ void launch_kick_drift(float* pos, float* vel, const float* acc, int64_t n, floa
                        cudaStream_t s)
 {
     launch_update<true>(pos, vel, acc, n, hkick, dt, info, s);
+}
+
+void launch_copy_good(float* dst, const float* src, int64_t n, const Info* info, cudaStream_t s)
+{
+    const bool vec = ((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15u) == 0;
+    int64_t g = nblk(vec ? (n + 3) / 4 : n, 256);
+    if (g > 8 * sm_count()) g = 8 * sm_count();
+    if (vec) k_copy_good<true><<<(unsigned)g, 256, 0, s>>>(dst, src, n, info);
+    else k_copy_good<false><<<(unsigned)g, 256, 0, s>>>(dst, src, n, info);
+    count_launches(1);
 }
 
 void launch_kick(float* vel, const float* acc, int64_t n, float hkick, const Info* info, cudaStream_t s)
