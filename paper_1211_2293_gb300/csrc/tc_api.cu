@@ -10,7 +10,9 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -115,7 +117,7 @@ struct tc_ctx {
     float* mlp_part = nullptr;    // per-warp partial gradients of a training step
     int64_t mlp_part_cap = 0;
     float* mlp_loss = nullptr;
-    float* mlp_sched = nullptr;   // learning rate and Adam bias corrections of every step
+    float* mlp_sched = nullptr;   // learning rate and Adam bias corrections of the next passes' steps
     int64_t mlp_sched_cap = 0;
     uint32_t* mlp_bar = nullptr;  // the training kernel's grid barrier
     unsigned long long* mlp_evals = nullptr;
@@ -1652,6 +1654,8 @@ int tc_mlp_loss_grad(tc_ctx* c, const float* X, const float* T, const float* W, 
     return check_device(c);
 }
 
+constexpr int64_t kSchedSteps = 2048;
+
 int tc_mlp_train(tc_ctx* c, const float* X, const float* T, const float* W, int32_t weight_mode, int64_t n,
                  int epochs, int batch, float lr, uint64_t seed, float band, float* losses)
 {
@@ -1665,6 +1669,22 @@ int tc_mlp_train(tc_ctx* c, const float* X, const float* T, const float* W, int3
     int r = mlp_alloc(c);
     if (r) return r;
     if ((r = mlp_scratch(c, n))) return r;
+    // every step's learning rate (cosine decay over all steps) and Adam bias
+    // corrections, those of a few passes on the device at a time: at least one
+    // pass's (12 bytes a step, a step has 16 rows of 140 bytes or more), up to
+    // kSchedSteps steps' where passes are shorter
+    const int64_t steps = (n + batch - 1) / batch, total_steps = epochs * steps;
+    const int64_t passes = std::max<int64_t>(1, std::min<int64_t>(epochs, kSchedSteps / steps));
+    const int blocks = mlp_train_blocks((int)std::min<int64_t>(batch, n), 2 * c->num_sms);
+    if ((r = mlp_part(c, blocks))) return r;
+    if (3 * passes * steps > c->mlp_sched_cap) {
+        c->mlp_sched_cap = 0;
+        TC_GROW(c, c->mlp_sched, 3 * passes * steps);
+        c->mlp_sched_cap = 3 * passes * steps;
+    }
+    if (!c->mlp_bar) TC_GROW(c, c->mlp_bar, 1);
+    const std::unique_ptr<float[]> sched(new (std::nothrow) float[3 * passes * steps]);
+    if (!sched) return fail(c, TC_ENOMEM, "tc_mlp_train: out of host memory");
     // the data as given, then (kernels) its sums, the model's maps (feature
     // means and scales, output RMS), fresh parameters, normalised rows and
     // scaled targets, loss weights
@@ -1697,34 +1717,24 @@ int tc_mlp_train(tc_ctx* c, const float* X, const float* T, const float* W, int3
     }
     TC_CUDA(c, cudaMemsetAsync(c->mlp_m, 0, kMlpNParamHost * sizeof(float), c->stream));
     TC_CUDA(c, cudaMemsetAsync(c->mlp_v, 0, kMlpNParamHost * sizeof(float), c->stream));
-    // every step's learning rate (cosine decay over all steps) and Adam bias
-    // corrections
-    const int64_t steps = (n + batch - 1) / batch, total_steps = epochs * steps;
-    const int blocks = mlp_train_blocks((int)std::min<int64_t>(batch, n), 2 * c->num_sms);
-    if ((r = mlp_part(c, blocks))) return r;
-    if (3 * total_steps > c->mlp_sched_cap) {
-        c->mlp_sched_cap = 0;
-        TC_GROW(c, c->mlp_sched, 3 * total_steps);
-        c->mlp_sched_cap = 3 * total_steps;
-    }
-    if (!c->mlp_bar) TC_GROW(c, c->mlp_bar, 1);
-    {
-        std::vector<float> sched(3 * total_steps);
-        for (int64_t k = 0; k < total_steps; k++) {
-            sched[3 * k] = (float)(0.5 * lr * (1.0 + std::cos(3.141592653589793 * (double)k / (double)total_steps)));
-            mlp_adam_corrections((int)(k + 1), &sched[3 * k + 1], &sched[3 * k + 2]);
-        }
-        TC_COPY(c, c->mlp_sched, sched.data(), sched.size() * sizeof(float));
-    }
     uint64_t key = seed;
     for (int ep = 0; ep < epochs; ep++) {
         // a fresh seeded permutation of the pairs each pass (on the device)
         key = key * 6364136223846793005ull + 1442695040888963407ull;
+        if (ep % passes == 0) {
+            const int64_t k0 = ep * steps, k1 = std::min(total_steps, k0 + passes * steps);
+            for (int64_t k = k0; k < k1; k++) {
+                float* at = &sched[3 * (k - k0)];
+                at[0] = (float)(0.5 * lr * (1.0 + std::cos(3.141592653589793 * (double)k / (double)total_steps)));
+                mlp_adam_corrections((int)(k + 1), at + 1, at + 2);
+            }
+            TC_COPY(c, c->mlp_sched, sched.get(), 3 * (k1 - k0) * sizeof(float));
+        }
         launch_mlp_shuffle(n, key, c->mlp_idx, c->stream);
         TC_CUDA(c, cudaMemsetAsync(c->mlp_loss, 0, sizeof(float), c->stream));
         cudaError_t e = launch_mlp_epoch(c->mlp_x, c->mlp_t, wdev, c->mlp_idx, (int)n, batch, blocks,
                                          c->mlp_dev, c->mlp_params, c->mlp_m, c->mlp_v,
-                                         c->mlp_sched + 3 * steps * ep, c->mlp_part, c->mlp_loss, c->mlp_bar,
+                                         c->mlp_sched + 3 * steps * (ep % passes), c->mlp_part, c->mlp_loss, c->mlp_bar,
                                          &c->info->err, c->stream);
         if (e != cudaSuccess) return fail(c, TC_ECUDA, "mlp training kernel: %s", cudaGetErrorString(e));
         if (losses) {

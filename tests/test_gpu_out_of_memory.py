@@ -139,3 +139,24 @@ def test_other_scratch_refused(monkeypatch, what):
         ctx.mlp_set(model, 0.5)
     assert np.array_equal(run(last), got)
     used.close()
+
+
+def test_training_memory_does_not_grow_with_the_passes(monkeypatch):
+    """Thousands of passes run in the memory that one takes (and 32 kB), and a
+    refused training leaves the model that was there."""
+    from paper_1211_2293_gb300 import tc
+
+    rng = np.random.default_rng(12)
+    X = rng.standard_normal((64, 13)).astype(np.float32)
+    T = (0.3 * X[:, :3]).astype(np.float32)
+    free = tc.Context()
+    want = free.mlp_train(X, T, epochs=8000, batch=16)
+    ctx = tc.Context()
+    k = _starved(tc, monkeypatch, lambda: ctx.mlp_train(X, T, epochs=1, batch=16), lambda: None, 4096)
+    model = ctx.mlp_get()[0]
+    monkeypatch.setenv("TC_ALLOC_CAP_BYTES", str(1 + k * 4096 + 32768))
+    with pytest.raises(tc.TcError) as e:
+        ctx.mlp_train(rng.standard_normal((5000, 13)).astype(np.float32), rng.standard_normal((5000, 3)).astype(np.float32))
+    assert e.value.code == tc.TC_ENOMEM and np.array_equal(ctx.mlp_get()[0], model)
+    assert np.array_equal(ctx.mlp_train(X, T, epochs=8000, batch=16), want)
+    assert np.array_equal(ctx.mlp_get()[0], free.mlp_get()[0])
