@@ -1433,14 +1433,17 @@ int tc_direct(tc_ctx* c, const int64_t* idx, int64_t ns, float eps, float G, dou
         TC_GROW(c, c->dir_out, 4 * ns);
         c->cap_idx = ns;
     }
-    const int64_t part = 4 * ns * direct_slices(c->n, ns);
-    if (part > c->cap_dir_part) {
+    // the slices' sums (30 MB at most on 152 SMs, none for a single slice); with
+    // less memory fewer slices, with none one
+    int slices = direct_slices(c->n, ns);
+    for (; slices > 1 && 4 * ns * slices > c->cap_dir_part; slices /= 2) {
         c->cap_dir_part = 0;
-        TC_GROW(c, c->dir_part, part);
-        c->cap_dir_part = part;
+        if (grow(c, &c->dir_part, 4 * ns * slices) != TC_OK) continue;
+        c->cap_dir_part = 4 * ns * slices;
+        break;
     }
     TC_CUDA(c, cudaMemcpyAsync(c->idx_dev, hidx.data(), ns * sizeof(int64_t), cudaMemcpyHostToDevice, c->stream));
-    launch_direct(c->pos, c->mass, c->sys_of, c->sysp, c->idx_dev, c->n, ns, eps * eps, G, c->dir_part, c->dir_out,
+    launch_direct(c->pos, c->mass, c->sys_of, c->sysp, c->idx_dev, ns, slices, eps * eps, G, c->dir_part, c->dir_out,
                   c->dir_out + 3 * ns, c->stream);
     TC_CUDA(c, cudaGetLastError());
     TC_CUDA(c, cudaMemcpyAsync(acc, c->dir_out, 3 * ns * sizeof(double), cudaMemcpyDefault, c->stream));

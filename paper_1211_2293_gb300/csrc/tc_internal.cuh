@@ -394,9 +394,11 @@ void launch_kick(float* vel, const float* acc, int64_t n, float hkick, const Inf
 void launch_copy_good(float* dst, const float* src, int64_t n, const Info* info, cudaStream_t s);
 void launch_diag(const float* pos, const float* vel, const float* mass, const float* pot,
                  int64_t n, Info* info, cudaStream_t s);
-int direct_slices(int64_t n, int64_t ns);  // slices of launch_direct's scratch (each 4 ns doubles)
+// source slices of a direct sum that fill the device; launch_direct's scratch
+// holds 4 ns doubles for each of two or more, one needs none
+int direct_slices(int64_t n, int64_t ns);
 void launch_direct(const float* pos, const float* mass, const uint32_t* sys_of, const SysParams* sysp,
-                   const int64_t* idx, int64_t n, int64_t ns, float eps2, float G, double* part, double* acc,
+                   const int64_t* idx, int64_t ns, int slices, float eps2, float G, double* part, double* acc,
                    double* pot, cudaStream_t s);
 
 // fast multipole method (tc_fmm.cu): the radii, then the walk of every cell.

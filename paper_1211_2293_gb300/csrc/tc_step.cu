@@ -129,7 +129,8 @@ __global__ void k_diag(const float* __restrict__ pos, const float* __restrict__ 
 //
 // Block (bx, s) takes the 256 targets from 256 bx on and slice s of the
 // source tiles of their systems (the union of the systems' ranges, tiles
-// counted from its start); k_direct_reduce adds the slices in order.  With
+// counted from its start); k_direct_reduce adds the slices in order (a single
+// one writes the results itself).  With
 // one block per 256 targets and no slices, the 4096 sampled targets of an
 // accuracy check kept 16 of 152 SMs busy: 44.6 ms over 2^20 bodies, 1.9 of
 // 80 TFLOP/s; sliced and packed 1.9 ms, 45 TFLOP/s.  A thread holds four
@@ -154,8 +155,8 @@ __device__ __forceinline__ float dir_rsqrt(float x)
 template <bool FTZ>
 __global__ void __launch_bounds__(kDirThreads, kDirBlocksPerSm)
     k_direct(const float* __restrict__ pos, const float* __restrict__ mass, const uint32_t* __restrict__ sys_of,
-             const SysParams* __restrict__ sysp, const int64_t* __restrict__ idx, int64_t ns, float eps2,
-             double* __restrict__ part)
+             const SysParams* __restrict__ sysp, const int64_t* __restrict__ idx, int64_t ns, float eps2, float G,
+             double* __restrict__ part, double* __restrict__ acc, double* __restrict__ pot)
 {
     __shared__ __align__(16) f2 tile[kDirTile * 4];  // {x, x}, {y, y}, {z, z}, {m, m} per source
     __shared__ long long lo_sh, hi_sh;
@@ -305,6 +306,13 @@ __global__ void __launch_bounds__(kDirThreads, kDirBlocksPerSm)
     for (int q = 0; q < NT; q++) {
         const int64_t t = t0 + q * kDirThreads + threadIdx.x;
         if (t >= ns) continue;
+        if (gridDim.y == 1) {
+            acc[3 * t] = (double)G * ax[q];
+            acc[3 * t + 1] = (double)G * ay[q];
+            acc[3 * t + 2] = (double)G * az[q];
+            if (pot) pot[t] = (double)G * (ph[q] + (double)(mass[idx[t]] * rsqrtf(eps2)));
+            continue;
+        }
         o[t] = ax[q];
         o[ns + t] = ay[q];
         o[2 * ns + t] = az[q];
@@ -444,17 +452,19 @@ int direct_slices(int64_t n, int64_t ns)
     return (int)(S < 1 ? 1 : S);
 }
 
-// part: direct_slices(n, ns) x 4 x ns doubles of scratch
+// part: slices x 4 x ns doubles of scratch, none for one slice
 void launch_direct(const float* pos, const float* mass, const uint32_t* sys_of, const SysParams* sysp,
-                   const int64_t* idx, int64_t n, int64_t ns, float eps2, float G, double* part, double* acc,
+                   const int64_t* idx, int64_t ns, int slices, float eps2, float G, double* part, double* acc,
                    double* pot, cudaStream_t s)
 {
-    const int S = direct_slices(n, ns);
-    const dim3 grid(nblk(ns, kDirTargets), (unsigned)S);
-    if (eps2 >= FLT_MIN) k_direct<true><<<grid, kDirThreads, 0, s>>>(pos, mass, sys_of, sysp, idx, ns, eps2, part);
-    else k_direct<false><<<grid, kDirThreads, 0, s>>>(pos, mass, sys_of, sysp, idx, ns, eps2, part);
-    k_direct_reduce<<<nblk(4 * ns, 256), 256, 0, s>>>(part, S, ns, mass, idx, eps2, G, acc, pot);
-    count_launches(2);
+    const dim3 grid(nblk(ns, kDirTargets), (unsigned)slices);
+    if (eps2 >= FLT_MIN)
+        k_direct<true><<<grid, kDirThreads, 0, s>>>(pos, mass, sys_of, sysp, idx, ns, eps2, G, part, acc, pot);
+    else k_direct<false><<<grid, kDirThreads, 0, s>>>(pos, mass, sys_of, sysp, idx, ns, eps2, G, part, acc, pot);
+    count_launches(1);
+    if (slices == 1) return;
+    k_direct_reduce<<<nblk(4 * ns, 256), 256, 0, s>>>(part, slices, ns, mass, idx, eps2, G, acc, pot);
+    count_launches(1);
 }
 
 }  // namespace tc

@@ -160,3 +160,35 @@ def test_training_memory_does_not_grow_with_the_passes(monkeypatch):
     assert e.value.code == tc.TC_ENOMEM and np.array_equal(ctx.mlp_get()[0], model)
     assert np.array_equal(ctx.mlp_train(X, T, epochs=8000, batch=16), want)
     assert np.array_equal(ctx.mlp_get()[0], free.mlp_get()[0])
+
+
+@pytest.mark.parametrize("systems", [1, 3])
+def test_direct_sum_without_its_scratch(monkeypatch, systems):
+    """Where the slices' sums find no memory fewer slices, or one, do: the same
+    tiles' sums, added in FP64 in another grouping."""
+    from paper_1211_2293_gb300 import tc
+
+    n = 20000
+    p, _, m = inputs.plummer(n, 13)
+    off = np.array([0, n]) if systems == 1 else np.array([0, 400, 9000, n])
+    idx = np.random.default_rng(14).permutation(n)[:300].astype(np.int64)
+    free = tc.Context()
+    free.build_batch(p, m, off, 8)
+    want = free.direct(idx, 0.01)
+
+    def build():
+        build.ctx = tc.Context()
+        build.ctx.build_batch(p, m, off, 8)
+
+    k = _starved(tc, monkeypatch, build, lambda: build.ctx.close(), 100000)
+    # room for the indices and results (14 kB) alone, for some slices, for all
+    for more in (32768, 200000, 400000, 1 << 20):
+        monkeypatch.setenv("TC_ALLOC_CAP_BYTES", str(1 + k * 100000 + more))
+        got = build.ctx.direct(idx, 0.01)
+        for a, b in zip(got, want):
+            # 80 tiles' sums: each addition rounds at 2^-53 of what is added so far
+            assert np.all(np.abs(a - b) <= 160 * 2.0**-53 * n * m[0] / 0.01**2)
+        acc = np.zeros((300, 3))
+        ctx = build.ctx
+        ctx._c(ctx._lib.tc_direct(ctx._h, idx.ctypes.data, 300, 0.01, 1.0, acc.ctypes.data, None))
+        assert np.array_equal(acc, got[0])
