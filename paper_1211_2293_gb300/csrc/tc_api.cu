@@ -551,7 +551,7 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
     c->scan = reinterpret_cast<unsigned long long*>(c->sb.tiles + 16);
     c->sb.status = c->scan + build_scan_words(n);
     launch_build_init(c->zero, (zero_words(n, status) + 1) / 2, c->sysp, c->nsys, c->info, synced, cs);
-    launch_bbox(c->pos, c->chunks, c->nchunks, c->sysp, &c->info->err, cs);
+    launch_bbox(c->pos, c->chunks, c->nchunks, c->sysp, c->nsys, &c->info->err, cs);
     // the keys go where the passes (and the completion) end in keys / perm
     const int moves = one_block ? 1 : plan.npass + (low_bit > 0 ? 1 : 0);
     uint64_t *ka = moves % 2 ? c->sb.keys_alt : c->keys, *kb = moves % 2 ? c->keys : c->sb.keys_alt;

@@ -188,8 +188,9 @@ __device__ void sys_cube(SysParams& P)
     P.uf = (float)(h * 0.5);
 }
 
-// one block per chunk (system, start, end, chunks of the system); the block
-// that completes a system's last chunk forms its root cube
+// one block per chunk (system, start, end, chunks of the system); CUBES: the
+// block that completes a system's last chunk forms its root cube
+template <bool CUBES>
 __global__ void __launch_bounds__(kBboxThreads) k_bbox(const float* pos, const int4* chunks,
                                                        SysParams* sysp, int32_t* err)
 {
@@ -224,6 +225,7 @@ __global__ void __launch_bounds__(kBboxThreads) k_bbox(const float* pos, const i
         for (int k = 0; k < kBboxThreads / 32; k++) r = a < 3 ? fminf(r, sm[a][k]) : fmaxf(r, sm[a][k]);
         if (a < 3) atomicMin(&sysp[ch.x].bb[a], f2o(r));
         else atomicMax(&sysp[ch.x].bb[a], f2o(r));
+        if (!CUBES) return;
         __threadfence();  // before this chunk counts as done
         __syncwarp(0x3fu);
         if (a == 0 && atomicAdd(&sysp[ch.x].done, 1) == ch.w - 1) {
@@ -231,6 +233,13 @@ __global__ void __launch_bounds__(kBboxThreads) k_bbox(const float* pos, const i
             sys_cube(sysp[ch.x]);
         }
     }
+}
+
+__global__ void k_cubes(SysParams* sysp, int nsys)
+{
+    pdl_begin();
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s < nsys) sys_cube(sysp[s]);
 }
 
 // ------------------------------------------------------------------ keys
@@ -1245,10 +1254,17 @@ void launch_build_init(uint4* zero, int64_t nzero, SysParams* sysp, int nsys, In
     count_launches(1);
 }
 
-void launch_bbox(const float* pos, const int4* chunks, int nchunks, SysParams* sysp, int32_t* err, ChainStream s)
+void launch_bbox(const float* pos, const int4* chunks, int nchunks, SysParams* sysp, int nsys, int32_t* err,
+                 ChainStream s)
 {
-    pdl_launch(k_bbox, nchunks, kBboxThreads, 0, s, pos, chunks, sysp, err);
-    count_launches(1);
+    if (nsys <= kCubeSystems) {
+        pdl_launch(k_bbox<true>, nchunks, kBboxThreads, 0, s, pos, chunks, sysp, err);
+        count_launches(1);
+        return;
+    }
+    pdl_launch(k_bbox<false>, nchunks, kBboxThreads, 0, s, pos, chunks, sysp, err);
+    pdl_launch(k_cubes, nblk(nsys, 128), 128, 0, s, sysp, nsys);
+    count_launches(2);
 }
 
 void launch_keys(const float* pos, const float* mass, int64_t n, const uint32_t* sys_of, const SysParams* sysp,

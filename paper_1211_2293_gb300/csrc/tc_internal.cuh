@@ -188,8 +188,15 @@ void launch_sys_ids(const int64_t* offsets, int nsys, int64_t n, uint32_t* sys_o
 void launch_build_init(uint4* zero, int64_t nzero, SysParams* sysp, int nsys, Info* info, bool reset_err,
                        ChainStream s);
 // bounding boxes, and each system's root cube once its last chunk is done;
-// chunks: (system, start, end, chunks of the system)
-void launch_bbox(const float* pos, const int4* chunks, int nchunks, SysParams* sysp, int32_t* err, ChainStream s);
+// chunks: (system, start, end, chunks of the system).  Batches of more than
+// kCubeSystems systems form the cubes in a launch of their own, a thread each:
+// by one thread of each block they are microseconds of FP64 latency that tens
+// of thousands of blocks queue for (builds of 512 x 1000 / 2048 x 16 / 8192 x
+// 16 / 65536 x 16 bodies: 258 / 124 / 189 / 643 us so, 260 / 113 / 159 / 455
+// with the launch)
+constexpr int kCubeSystems = 512;
+void launch_bbox(const float* pos, const int4* chunks, int nchunks, SysParams* sysp, int nsys, int32_t* err,
+                 ChainStream s);
 // Morton keys, indices and (ghist not null) the digit counts of the plan's passes
 void launch_keys(const float* pos, const float* mass, int64_t n, const uint32_t* sys_of, const SysParams* sysp,
                  uint64_t* keys, uint32_t* idx, const SortPlan& plan, uint32_t* ghist, int32_t* err, ChainStream s);
