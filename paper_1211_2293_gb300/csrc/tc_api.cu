@@ -593,8 +593,8 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
         c->depth_hint_n = n;
     }
     launch_emit_nodes(c->keys, c->delta, c->top, c->sys_of, n, c->lcnt, c->info, c->lstart, c->nt, cs);
-    launch_moments(c->body, c->delta, n, c->nsys, c->cap_m, depth, c->depth_hint, c->lstart, c->sysp, c->info, c->nt,
-                   c->cfg.quad != 0, cs);
+    launch_moments(c->body, c->keys, c->delta, n, c->nsys, c->cap_m, depth, c->depth_hint, c->lstart, c->sysp, c->info,
+                   c->nt, c->cfg.quad != 0, cs);
     launch_groups(c->cap_m, c->info, c->nt, c->cfg.gmax, n, c->gref_at, c->scan, c->gfirst, c->gref, c->part_done, cs);
     c->gorder_ready = false;
     TC_CUDA(c, cudaGetLastError());

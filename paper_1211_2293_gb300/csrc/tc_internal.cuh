@@ -224,8 +224,8 @@ void launch_emit_nodes(const uint64_t* keys, const int8_t* delta, const int8_t* 
 // get a launch each and any deeper ones one block, else all 21 levels get a
 // launch); each level reads its range on the device.  Also each system's mass.
 constexpr int64_t kClimbBodies = 1 << 19;  // (both ways timed: tc_build.cu, "moments")
-void launch_moments(const float4* body, const int8_t* delta, int64_t n, int nsys, int64_t cap_m, int depth,
-                    int depth_hint, const uint32_t* level_start, SysParams* sysp, const Info* info, NodeTables nt,
+void launch_moments(const float4* body, const uint64_t* keys, const int8_t* delta, int64_t n, int nsys,
+                    int64_t cap_m, int depth, int depth_hint, const uint32_t* level_start, SysParams* sysp, const Info* info, NodeTables nt,
                     bool quad, ChainStream s);
 // the body groups: gfirst[0..G], gref[0..G), info->G
 void launch_groups(int64_t cap_m, Info* info, const NodeTables nt, int gmax, int64_t n, int32_t* gref_at,
