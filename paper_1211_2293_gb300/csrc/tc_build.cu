@@ -15,7 +15,7 @@
 //   3. radix sort  stable sort by (system, key, index)    [tc_sort.cu]
 //   4. the bodies in Morton order as float4 (x, y, z, m): k_gather, or with
 //                  the sort's completion
-//   5. k_window / k_node_levels, k_scan_levels
+//   5. k_window, k_window_max, k_node_levels (or k_node_levels_tiled), k_scan_levels
 //                  which cubes of the recursive subdivision start at each
 //                  sorted body (a sliding-window test, below), how many of
 //                  each level per block of bodies, and their scan: the
@@ -408,11 +408,25 @@ __global__ void k_window(const uint64_t* keys, const uint32_t* sys_of, int64_t n
                : (int8_t)-1;
 }
 
-// leaf_max > kTileWindow: the window digits come from k_window
+// leaf_max > kTileWindow: the window digits come from k_window, a body's
+// deepest level into top[] by a thread each (four long windows one after
+// another in the threads of k_node_levels left few warps to wait for their
+// loads: 4096 bodies of leaf_max 4096 49 us with a thread each, 200 with four
+// bodies a thread)
+__global__ void __launch_bounds__(256) k_window_max(const int8_t* w, int64_t n, int leaf_max, int8_t* top)
+{
+    pdl_begin();
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= n) return;
+    int W = -1;
+    const int64_t j0 = s - leaf_max < 0 ? 0 : s - leaf_max;
+    for (int64_t j = j0; j <= s; j++) W = max(W, (int)w[j]);
+    top[s] = (int8_t)min(W + 1, kMaxLevel);
+}
+
 __global__ void __launch_bounds__(kNodeThreads) k_node_levels(const uint64_t* keys,
-                                                              const uint32_t* sys_of,
-                                                              const int8_t* w, int64_t n, int leaf_max,
-                                                              int8_t* delta, int8_t* top,
+                                                              const uint32_t* sys_of, int64_t n,
+                                                              int8_t* delta, const int8_t* top,
                                                               int32_t* gref_at, uint32_t* cnt,
                                                               int32_t* depth)
 {
@@ -425,12 +439,8 @@ __global__ void __launch_bounds__(kNodeThreads) k_node_levels(const uint64_t* ke
         d[r] = 0;
         if (s < n) {
             d[r] = (s == 0 || sys_of[s] != sys_of[s - 1]) ? -1 : common_digits(keys[s - 1], keys[s]);
-            int W = -1;
-            const int64_t j0 = s - leaf_max < 0 ? 0 : s - leaf_max;
-            for (int64_t j = j0; j <= s; j++) W = max(W, (int)w[j]);
-            t[r] = min(W + 1, kMaxLevel);
+            t[r] = top[s];
             delta[s] = (int8_t)d[r];
-            top[s] = (int8_t)t[r];
             gref_at[s] = 0;
         }
     }
@@ -1319,9 +1329,9 @@ void launch_node_levels(const uint64_t* keys, const uint32_t* sys_of, int64_t n,
         count_launches(1);
     } else {
         pdl_launch(k_window, nblk(n, 256), 256, 0, s, keys, sys_of, n, leaf_max, w);
-        pdl_launch(k_node_levels, nb, kNodeThreads, 0, s, keys, sys_of, w, n, leaf_max, delta, top, gref_at, cnt,
-                   &info->depth);
-        count_launches(2);
+        pdl_launch(k_window_max, nblk(n, 256), 256, 0, s, w, n, leaf_max, top);
+        pdl_launch(k_node_levels, nb, kNodeThreads, 0, s, keys, sys_of, n, delta, top, gref_at, cnt, &info->depth);
+        count_launches(3);
     }
     const int64_t nc = level_counts_size(n);
     uint32_t* counters = reinterpret_cast<uint32_t*>(scan + build_scan_words(n) - 1);
