@@ -560,7 +560,7 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
                 cs);
     const int64_t run_max = synced ? kSortRunMaxSynced : kSortRunMax;
     if (one_block) {
-        launch_sort_block(ka, va, kb, vb, n, plan, c->sys_of, c->pos, c->mass, c->body, run_max, &c->info->err, cs);
+        launch_sort_block(ka, va, kb, vb, n, plan, c->sys_of, c->pos, c->mass, c->body, cs);
     } else {
         launch_sort_passes(ka, va, kb, vb, n, plan, c->sys_of, c->sb, cs);
         if (low_bit > 0)

@@ -131,7 +131,7 @@ struct SortDigit {
 // bits of the system: as few digits as hold them together.
 struct SortPlan {
     int npass, low_bit, kb, sys_bits;
-    static SortPlan make(int nbits, int low_bit, int sys_bits)
+    __host__ __device__ static SortPlan make(int nbits, int low_bit, int sys_bits)
     {
         const int kb = nbits - low_bit;
         return SortPlan{(kb + sys_bits + 7) / 8, low_bit, kb, sys_bits};
@@ -171,7 +171,7 @@ void launch_sort_runs(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, 
 constexpr int64_t kBlockSortMax = 4096;
 void launch_sort_block(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout, int64_t n,
                        const SortPlan& plan, const uint32_t* sys_of, const float* pos, const float* mass, float4* body,
-                       int64_t run_max, int32_t* err, ChainStream s);
+                       ChainStream s);
 // A whole sort of (key, val) by bits [0, nbits) of key, in place.
 void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int nbits, SortBufs& b, cudaStream_t s);
 // self-test of the radix pass's bounded look-back (see tc_sort.cu)

@@ -434,10 +434,15 @@ __global__ void __launch_bounds__(256) k_sort_runs(const uint64_t* kin, const ui
 // or five passes of 4096 items took 10 us as a launch of its own (tile
 // counter, loads, look-back, stores); here all of them and the completion
 // take 26.  With 12 items a thread (10007 items) one block took 72 us, more
-// than the launches.
+// than the launches.  Runs of more than kBlockRun items (a tree far deeper
+// than the last one, or leaves of many bodies) are not ranked, in quadratic
+// time: the block goes on to sort every digit (builds of 4000 bodies in runs of
+// 64 / 100 / 200 / 400 / 1000: 158 / 196 / 272 / 448 / 933 us ranked, 153 / 157
+// / 163 / 193 / 254 so).
 namespace {
 
 constexpr int kBlockThreads = 1024, kBlockWarps = kBlockThreads / 32;
+constexpr int kBlockRun = 64;
 constexpr size_t block_sort_smem(int items)
 {
     return (size_t)kBlockThreads * items * (sizeof(uint64_t) + sizeof(uint32_t)) + kBlockWarps * 256 * sizeof(uint32_t);
@@ -447,8 +452,7 @@ template <int ITEMS>
 __global__ void __launch_bounds__(kBlockThreads, 1)
     k_sort_block(const uint64_t* kin, const uint32_t* vin, uint64_t* kout,
                  uint32_t* vout, int n, SortPlan plan, const uint32_t* sys_of,
-                 const float* pos, const float* mass, float4* body, int run_max,
-                 int32_t* err)
+                 const float* pos, const float* mass, float4* body)
 {
     pdl_begin();
     constexpr int WARP = 32 * ITEMS;
@@ -467,94 +471,108 @@ __global__ void __launch_bounds__(kBlockThreads, 1)
         key[r] = li < n ? kin[li] : 0ull;
         val[r] = li < n ? vin[li] : 0u;
     }
-    for (int p = 0; p < plan.npass; p++) {
-        const SortDigit dg = plan.digit(p);
-        for (int i = threadIdx.x; i < kBlockWarps * 256; i += kBlockThreads) wh[i] = 0u;
-        __syncthreads();
-        uint32_t rank[ITEMS];  // the digit above a 16-bit rank
-#pragma unroll
-        for (int r = 0; r < ITEMS; r++) {
-            const bool ok = w * WARP + r * 32 + lane < n;
-            const uint32_t dd = dg.of(key[r], dg.sys && ok ? sys_of[val[r]] : 0u);
-            unsigned peers = digit_peers(__ballot_sync(0xffffffffu, ok), dd);
-            if (!ok) peers = 0u;
-            uint32_t old = 0u;
-            if (peers && (peers & lt) == 0u) old = atomicAdd(&wh[w * 256 + dd], (uint32_t)__popc(peers));
-            __syncwarp();
-            rank[r] = (dd << 16) | (__shfl_sync(0xffffffffu, old, peers ? __ffs(peers) - 1 : lane) + __popc(peers & lt));
-        }
-        __syncthreads();
-        // where each (digit, warp) starts: thread (d, part) of four adds up
-        // eight warps of digit d, then the digits are scanned
-        {
-            const int d = threadIdx.x >> 2, part = threadIdx.x & 3;
-            uint32_t c[8], sum = 0;
-#pragma unroll
-            for (int k = 0; k < 8; k++) {
-                c[k] = wh[(part * 8 + k) * 256 + d];
-                sum += c[k];
-            }
-            uint32_t incl = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            if (lane == 31) wsum[w] = incl;
+    int st[ITEMS], en[ITEMS];  // the items' runs of equal top bits (and system)
+    for (;;) {
+        for (int p = 0; p < plan.npass; p++) {
+            const SortDigit dg = plan.digit(p);
+            for (int i = threadIdx.x; i < kBlockWarps * 256; i += kBlockThreads) wh[i] = 0u;
             __syncthreads();
-            uint32_t run = incl - sum;
-            for (int k = 0; k < w; k++) run += wsum[k];
+            uint32_t rank[ITEMS];  // the digit above a 16-bit rank
 #pragma unroll
-            for (int k = 0; k < 8; k++) {
-                wh[(part * 8 + k) * 256 + d] = run;
-                run += c[k];
+            for (int r = 0; r < ITEMS; r++) {
+                const bool ok = w * WARP + r * 32 + lane < n;
+                const uint32_t dd = dg.of(key[r], dg.sys && ok ? sys_of[val[r]] : 0u);
+                unsigned peers = digit_peers(__ballot_sync(0xffffffffu, ok), dd);
+                if (!ok) peers = 0u;
+                uint32_t old = 0u;
+                if (peers && (peers & lt) == 0u) old = atomicAdd(&wh[w * 256 + dd], (uint32_t)__popc(peers));
+                __syncwarp();
+                rank[r] = (dd << 16) | (__shfl_sync(0xffffffffu, old, peers ? __ffs(peers) - 1 : lane) + __popc(peers & lt));
+            }
+            __syncthreads();
+            // where each (digit, warp) starts: thread (d, part) of four adds up
+            // eight warps of digit d, then the digits are scanned
+            {
+                const int d = threadIdx.x >> 2, part = threadIdx.x & 3;
+                uint32_t c[8], sum = 0;
+#pragma unroll
+                for (int k = 0; k < 8; k++) {
+                    c[k] = wh[(part * 8 + k) * 256 + d];
+                    sum += c[k];
+                }
+                uint32_t incl = sum;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                if (lane == 31) wsum[w] = incl;
+                __syncthreads();
+                uint32_t run = incl - sum;
+                for (int k = 0; k < w; k++) run += wsum[k];
+#pragma unroll
+                for (int k = 0; k < 8; k++) {
+                    wh[(part * 8 + k) * 256 + d] = run;
+                    run += c[k];
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < ITEMS; r++) {
+                if (w * WARP + r * 32 + lane < n) {
+                    const uint32_t lp = wh[w * 256 + (rank[r] >> 16)] + (rank[r] & 0xffffu);
+                    skey[lp] = key[r];
+                    sval[lp] = val[r];
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < ITEMS; r++) {
+                const int li = w * WARP + r * 32 + lane;
+                if (li < n) {
+                    key[r] = skey[li];
+                    val[r] = sval[li];
+                }
             }
         }
-        __syncthreads();
+        if (plan.npass == 0) {
+#pragma unroll
+            for (int r = 0; r < ITEMS; r++) {
+                const int li = w * WARP + r * 32 + lane;
+                if (li < n) {
+                    skey[li] = key[r];
+                    sval[li] = val[r];
+                }
+            }
+            __syncthreads();
+        }
+        if (plan.low_bit == 0) break;
+        bool lng = false;
 #pragma unroll
         for (int r = 0; r < ITEMS; r++) {
-            if (w * WARP + r * 32 + lane < n) {
-                const uint32_t lp = wh[w * 256 + (rank[r] >> 16)] + (rank[r] & 0xffffu);
-                skey[lp] = key[r];
-                sval[lp] = val[r];
-            }
+            const int i = w * WARP + r * 32 + lane;
+            st[r] = i;
+            en[r] = i + 1;
+            if (i >= n) continue;
+            const uint32_t* so = plan.sys_bits > 0 ? sys_of : nullptr;
+            while (st[r] > 0 && i - st[r] < kBlockRun && same_run(skey, sval, so, plan.low_bit, st[r] - 1, i)) st[r]--;
+            while (en[r] < n && en[r] - i < kBlockRun && same_run(skey, sval, so, plan.low_bit, en[r], i)) en[r]++;
+            lng |= en[r] - st[r] > kBlockRun;
         }
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < ITEMS; r++) {
-            const int li = w * WARP + r * 32 + lane;
-            if (li < n) {
-                key[r] = skey[li];
-                val[r] = sval[li];
-            }
-        }
+        if (!__syncthreads_or(lng)) break;
+        // (the items lie in value order within equal keys, so do the passes leave them)
+        plan = SortPlan::make(plan.low_bit + plan.kb, 0, plan.sys_bits);
     }
-    if (plan.npass == 0) {
-#pragma unroll
-        for (int r = 0; r < ITEMS; r++) {
-            const int li = w * WARP + r * 32 + lane;
-            if (li < n) {
-                skey[li] = key[r];
-                sval[li] = val[r];
-            }
-        }
-        __syncthreads();
-    }
-    // the items' places: within its run of equal top bits (and system) each
-    // item goes to the rank of its (key, val)
+    // the items' places: within its run each item goes to the rank of its
+    // (key, val)
 #pragma unroll
     for (int r = 0; r < ITEMS; r++) {
         const int i = w * WARP + r * 32 + lane;
         if (i >= n) continue;
         int at = i;
         if (plan.low_bit > 0) {
-            const uint32_t* so = plan.sys_bits > 0 ? sys_of : nullptr;
-            int st = i, en = i + 1;
-            while (st > 0 && same_run(skey, sval, so, plan.low_bit, st - 1, i)) st--;
-            while (en < n && same_run(skey, sval, so, plan.low_bit, en, i)) en++;
-            if (en - st > run_max) atomicOr(err, kErrSortRun | kErrCapacity);
-            at = st;
-            for (int j = st; j < en; j++) at += before(skey[j], sval[j], key[r], val[r]) ? 1 : 0;
+            at = st[r];
+            for (int j = st[r]; j < en[r]; j++) at += before(skey[j], sval[j], key[r], val[r]) ? 1 : 0;
         }
         const int64_t v = val[r];
         kout[at] = key[r];
@@ -597,12 +615,11 @@ static_assert(kBlockSortMax == kBlockThreads * kBlockItems, "one block's items")
 
 void launch_sort_block(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout, int64_t n,
                        const SortPlan& plan, const uint32_t* sys_of, const float* pos, const float* mass, float4* body,
-                       int64_t run_max, int32_t* err, ChainStream s)
+                       ChainStream s)
 {
     sort_attributes();
-    const int rm = (int)(run_max < 1 || run_max > kSortRunMax ? kSortRunMax : run_max);
     pdl_launch(k_sort_block<kBlockItems>, 1, kBlockThreads, block_sort_smem(kBlockItems), s, kin, vin, kout, vout,
-               (int)n, plan, sys_of, pos, mass, body, rm, err);
+               (int)n, plan, sys_of, pos, mass, body);
     count_launches(1);
 }
 
