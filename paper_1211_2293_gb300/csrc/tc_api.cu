@@ -41,6 +41,7 @@ struct tc_ctx {
     int64_t n = 0, cap_n = 0;
     int nsys = 0, cap_sys = 0;
     std::vector<int64_t> off_h;  // system offsets (host)
+    double mean_sys = 0.0;       // bodies of the system that a body is in, on average
     int nchunks = 0, cap_chunks = 0;
     int64_t M = 0, cap_m = 0;  // nodes of the last synchronised build, node table capacity
     int leaf_max = 0;
@@ -495,6 +496,9 @@ int setup_systems(tc_ctx* c, const int64_t* off, int nsys)
     int r = ensure_systems(c, nsys, (int)ch.size());
     if (r) return r;
     c->off_h.assign(off, off + nsys + 1);
+    double squares = 0.0;
+    for (int s = 0; s < nsys; s++) squares += (double)(off[s + 1] - off[s]) * (double)(off[s + 1] - off[s]);
+    c->mean_sys = squares / (double)off[nsys];
     c->nsys = nsys;
     c->nchunks = (int)ch.size();
     TC_CUDA(c, cudaMemcpyAsync(c->off_dev, c->off_h.data(), (nsys + 1) * sizeof(int64_t), cudaMemcpyHostToDevice,
@@ -610,17 +614,26 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
 // / 26, 4096 86 / 55 / 40 / 38 / 45, 10000 185 / 113 / 73 / 55 / 69, 16000 357
 // / 203 / 122 / 101 / 101, 30000 140 / 88 / 96 / 113, 50000 149 / 128 / 144,
 // 70000 159 / 169 / 182, 10^6 1751 / 1868 / 2126: with many groups the cells
-// that all parts walk and the shorter tiles are lost time.  A rule on n, the
-// systems and gmax only (a group holds about 0.7 gmax bodies), so a captured
-// step and a direct call sum alike.  A stack set below the default is kept as
-// the limit of whole walks.
-constexpr double kPartTasks = 20.0;  // per SM
+// that all parts walk and the shorter tiles are lost time.  In a batch the
+// lists are no longer than a system, so a part stands for at least 64 bodies
+// of the system that a body is in on average, 512 where there are more tasks
+// than teams: batches of 300 x 7 / 1000 x 64 / 100 x 100 / 50 x 300 / 30 x 1000
+// / 10 x 2000 bodies take 11 / 16 / 19 / 28 / 52 / 69 us whole, 18 / 26 / 32 /
+// 41 / 60 / 52 by the rule of single systems, 11 / 16 / 19 / 25 / 51 / 50 so.
+// A rule on the systems' sizes and gmax only (a group holds about 0.7 gmax
+// bodies), so a captured step and a direct call sum alike; where the lists are
+// very short (bodies on a line, theta of 2) parts cost up to 20 us.  A stack
+// set below the default is kept as the limit of whole walks.
+constexpr double kPartTasks = 20.0, kTeams = 8.0;  // per SM
 int walk_parts(const tc_ctx* c)
 {
     if (c->cfg.stack < kDefaultStack) return 0;
     const double groups = std::max((double)c->n / (0.7 * c->cfg.gmax), (double)c->nsys);
     int log2 = 0;
     while (log2 < 3 && groups * (2 << log2) <= kPartTasks * c->num_sms) log2++;
+    while (c->nsys > 1 && log2 > 0 &&
+           c->mean_sys < (groups * (1 << log2) > kTeams * c->num_sms ? 512.0 : 64.0) * (1 << log2))
+        log2--;
     return log2;
 }
 // the sums of any parts of up to cap_n bodies in groups of up to 128 (10 MB at
