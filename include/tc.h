@@ -91,11 +91,14 @@ typedef struct tc_ctx tc_ctx;
  *             and 64 bodies whatever `tile` says), a consumer warp sums them
  *             (the default; in small systems several such pairs share a
  *             group's list); in the learned walk the producers run the
- *             network on the band cells they meet.  2: they record the band
- *             cells instead, and the network runs on all of them after the
- *             walk.  0: every warp
- *             walks and sums its own groups.  Same lists; the sums take the
- *             entries in another order (rounding-level differences). */
+ *             network on the band cells they meet.  Where that was the
+ *             slower one (batches of small systems, large quadrupole and
+ *             learned walks of short lists) split = 1 walks as 0 does.
+ *             2: the split walks always, the learned one's producers record
+ *             the band cells, and the network runs on all of them after the
+ *             walk.  0: every warp walks and sums its own groups.  Same
+ *             lists; the sums take the entries in another order
+ *             (rounding-level differences). */
 typedef struct {
     int32_t gmax;
     int32_t warps;

@@ -645,7 +645,51 @@ int64_t part_floats(const tc_ctx* c)
     return kPartPlanes * bodies;
 }
 
-int prepare_forces(tc_ctx* c)
+int walk_stack(const tc_ctx* c)
+{
+    int64_t st = c->cfg.stack;
+    if (c->cap_m < st) st = c->cap_m < 32 ? 32 : c->cap_m;  // a stack of M entries cannot overflow
+    return (int)((st + 3) & ~(int64_t)3);                   // keeps every warp's tiles 16-byte aligned
+}
+
+// Whether split = 1 takes the split walk, for a force phase at theta: it does
+// where it was the faster of the two.  Where it is not, the lists are short for
+// what a group costs its producer (hand-overs, the network), or too few teams
+// fit an SM; with few groups for an SM its parts always win.  Walks in us,
+// split / one warp:
+//   systems of a batch of 2 10^6 bodies in all of 33 / 100 / 300 / 512 / 1000
+//     bodies: 507/268 593/383 748/604 900/826 1175/1328, with 2 10^5 97/75
+//     57/54 81/84 110/117; of one leaf 187/237.  Quadrupole 450/344 661/515
+//     898/815 1134/1140 1608/1774.  Learned 592/306 804/461 1035/709 1245/948
+//     1679/1380, of 2000 / 4000 2064/1909 2371/2402; 10^5 bodies in 1000s
+//     125/114, 5 10^4 72/103
+//   learned, 2 10^6 bodies, theta 0.6 / 0.75 / 0.9: band 0.5 3208/3488 2448/2393
+//     2238/2056, band 0.1 6020/5464 3625/3202 2837/2494; 2 10^5 383/421 283/310
+//     264/279 and 613/655 388/399 320/330; a cube, band 0.5, 2183/2215
+//     1660/1489 1553/1322.  Groups of 32 (band 0.55) 10^5 207/211, 2 10^6
+//     3772/3355; of 128 220/454 and 3036/3204, in batches of 200 / 1000
+//     bodies 761/495 1727/1500
+//   quadrupole, 2 10^6 bodies, theta 0.55 / 0.7 / 0.9: 6885/7192 3605/3729
+//     2604/2649, in a cube 4086/4130 2025/2018 1553/1530, with the potential
+//     7612/7757 3985/4007 2878/2848 and 4502/4459 2238/2172 1716/1642
+//   fewer teams: quadrupole, 2 10^6 bodies, one warp a block 6630/3761, stack
+//     2048 4633/3940; learned (band 0.55), tile 256 3338/2858, warps 2 2962/2893
+bool takes_split(const tc_ctx* c, const WalkConfig& w, float theta)
+{
+    if (c->cfg.split != 1) return c->cfg.split == 2;
+    const double groups = std::max((double)c->n / (0.7 * w.gmax), (double)c->nsys) / c->num_sms;  // for an SM
+    const bool batch = c->nsys > 1 && c->mean_sys > c->leaf_max;
+    if (!w.quadw && !w.learned) return !(batch && c->mean_sys <= 300.0 && groups > 20.0);
+    if (groups <= 12.0) return true;
+    if (batch && c->mean_sys <= (w.quadw ? 600.0 : (w.gmax > 64 ? 1000.0 : 3000.0))) return false;
+    if (w.gmax > 64) return true;
+    if (w.warps == 1 || walk_ws_teams(w) < (int)kTeams) return false;
+    if (w.quadw) return groups <= 40.0 || theta <= (w.want_pot ? 0.62f : 0.8f);
+    if (w.gmax < 64) return groups <= 24.0;
+    return groups <= 40.0 || (theta <= 0.7f && c->mlp_band >= 0.8f * theta);
+}
+
+int prepare_forces(tc_ctx* c, float theta)
 {
     WalkConfig wc{};
     wc.gmax = c->cfg.gmax;
@@ -661,6 +705,8 @@ int prepare_forces(tc_ctx* c)
     // 64 bodies (tc_walk_ws.cuh measures both sides; four bodies a lane leave
     // it no registers); 2: the learned walk's network evaluated after the walk
     wc.split = c->cfg.split != 0 && !(wc.quadw && (wc.learned || c->cfg.gmax > 64));
+    wc.stack = walk_stack(c);
+    if (wc.split) wc.split = takes_split(c, wc, theta);
     wc.record = wc.learned && wc.split && c->cfg.split == 2;
     // one launch per size class: one warp per group only (the split walk
     // lays each group out over its lanes by its own size)
@@ -677,10 +723,6 @@ int prepare_forces(tc_ctx* c)
         // force phase, the groups are walked whole
         if (want > c->cap_part) wc.part_log2 = 0;
     }
-    int64_t st = c->cfg.stack;
-    if (c->cap_m < st) st = c->cap_m < 32 ? 32 : c->cap_m;  // a stack of M entries cannot overflow
-    st = (st + 3) & ~(int64_t)3;                            // keeps every warp's tiles 16-byte aligned
-    wc.stack = (int)st;
     if (wc.record) {
         // the band-cell record: 12 cells per body (the learned workloads
         // record 2 to 7) plus a chunk per producer warp of every size-class
@@ -835,7 +877,7 @@ int run_forces(tc_ctx* c, float theta, float eps, float G, cudaStream_t s, bool 
 int step_eager(tc_ctx* c, float dt)
 {
     cudaStream_t s = c->stream;
-    int r = prepare_forces(c);
+    int r = prepare_forces(c, c->theta);
     if (r) return r;
     cudaEvent_t t0 = phase_begin(c, s, 2);
     launch_kick_drift(c->pos, c->vel, c->acc, c->n, 0.5f * dt, dt, c->info, s);
@@ -873,7 +915,7 @@ int step_graph(tc_ctx* c, float dt)
     const bool timing = c->timing;
     // the walk of this configuration (list export, training pairs and another
     // configuration leave theirs); it may drop the graph
-    int r = prepare_forces(c);
+    int r = prepare_forces(c, c->theta);
     if (r) return r;
     const std::string key = graph_key(c, dt) + (timing ? "/timed" : "");
     // (a graph sorts the digits of the depth it was captured with: a deeper
@@ -1095,7 +1137,7 @@ int tc_ctx_forces(tc_ctx* c, float theta, float eps, float G)
     if (!finite(eps) || eps <= 0.f) return fail(c, TC_EINVAL, "tc_forces: eps must be finite and > 0");
     if (!finite(G)) return fail(c, TC_EINVAL, "tc_forces: G must be finite");
     if (c->cfg.learned && !c->have_mlp) return fail(c, TC_ESTATE, "tc_forces: learned = 1 but no model is set");
-    int r = prepare_forces(c);
+    int r = prepare_forces(c, theta);
     if (r) return r;
     return run_forces(c, theta, eps, G, c->stream, c->n <= kChainBodies);
 }
@@ -1801,7 +1843,7 @@ int tc_mlp_pairs(tc_ctx* c, float theta, float eps, float band, float prob, uint
     c->cfg.quadrupole = 0;
     c->cfg.split = 0;  // list export and pair emission live in k_walk
     c->walk_ready = false;
-    r = prepare_forces(c);
+    r = prepare_forces(c, theta);
     c->cfg = keep;
     if (r) return r;
     WalkArgs a{};
@@ -1910,7 +1952,7 @@ int tc_get_group_list(tc_ctx* c, int64_t group, float theta, int32_t* cells, int
     c->cfg.quadrupole = 0;
     c->cfg.split = 0;  // list export and pair emission live in k_walk
     c->walk_ready = false;
-    r = prepare_forces(c);
+    r = prepare_forces(c, theta);
     c->cfg = keep;
     if (r) return r;
     WalkArgs a{};
@@ -1999,7 +2041,7 @@ int tc_autotune(tc_ctx* c, float theta, float eps, float G, int reps, tc_config*
                     t.tile = tiles[ti];
                     t.warps = warps[wi];
                     rc = tc_set_config(c, &t);
-                    if (!rc) rc = prepare_forces(c);
+                    if (!rc) rc = prepare_forces(c, theta);
                     if (!rc) rc = run_forces(c, theta, eps, G, c->stream);  // warm-up
                     double tmin = 1e30;
                     for (int k = 0; k < reps && !rc; k++) {

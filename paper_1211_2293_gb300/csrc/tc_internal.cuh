@@ -322,6 +322,8 @@ struct WalkConfig {
 // host-side preparation of the walk kernel's launch (attributes, occupancy);
 // call before a stream capture
 cudaError_t prepare_walk(const WalkConfig& c, int num_sms, int* grid, size_t* smem);
+// teams of the split walk that fit an SM
+int walk_ws_teams(const WalkConfig& c);
 // reset_totals: zero the work-queue counters and (outside list export) the
 // interaction totals first -- the first launch of a force phase; the later
 // launches of a phase split over size classes count on counters of their own

@@ -2,6 +2,8 @@
 // tiles of TC_WALK_TILE entries, every mode.  The build compiles this file
 // once per tile in {64, 128, 256}, defining the macro, and once with 32, the
 // quadrupole walk.
+#include <algorithm>
+
 #include "tc_walk.cuh"
 #include "tc_walk_ws.cuh"
 
@@ -15,6 +17,15 @@
 namespace tc {
 
 #if TC_WALK_TILE == 32
+// by shared memory (and 1 KB a block of 228 on an SM) and by registers: 128 a
+// thread, the launch bounds' cap, so eight teams of two warps
+int walk_ws_teams(const WalkConfig& c)
+{
+    const WsShape w = ws_shape(c, c.quadw ? 32 : c.tile, c.learned && !c.record);
+    const int teams = w.threads / 64, by_smem = (int)(228 * 1024 / (w.smem + 1024));
+    return std::min(by_smem, 8 / teams) * teams;
+}
+
 cudaError_t prepare_walk_ws_t32(const WalkConfig& c, int num_sms, int* grid, size_t* smem)
 {
     if (!c.quadw || c.learned || !c.precise || c.gmax > 64) return cudaErrorInvalidValue;
