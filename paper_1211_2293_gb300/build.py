@@ -25,7 +25,7 @@ INCLUDE = os.path.join(ROOT, "include")
 # (object, source, defines): the walk kernels, one object per (bodies per
 # lane, tile), are the longest compiles and go first
 WALK_UNITS = [(f"tc_walk_b{b}_t{t}", "tc_walk_unit.cu", [f"-DTC_WALK_B={b}", f"-DTC_WALK_TILE={t}"])
-              for b in (4, 2, 1) for t in (128, 32, 64, 256)]
+              for b in (4, 2, 1) for t in (128, 64, 256)]
 WALK_WS_UNITS = [(f"tc_walk_ws_t{t}", "tc_walk_ws_unit.cu", [f"-DTC_WALK_TILE={t}"]) for t in (128, 32, 64, 256)]
 UNITS = WALK_WS_UNITS + WALK_UNITS + [(s[:-3], s, []) for s in ["tc_api.cu", "tc_walk.cu", "tc_sort.cu", "tc_build.cu", "tc_step.cu",
                                                "tc_noalloc.cu", "tc_mlp.cu", "tc_band.cu", "tc_fmm.cu",
