@@ -407,7 +407,7 @@ int check_device(tc_ctx* c)
         if (e & kErrStack) return fail(c, TC_EDEVICE, "walk stack overflow (raise tc_config.stack)");
         if (e & kErrWorkLoop) return fail(c, TC_EDEVICE, "a bounded device wait gave up");
         if (e & kErrFmmStack)
-            return fail(c, TC_EDEVICE, "the FMM's refinement stack (2048 sources per cell) overflowed; raise theta");
+            return fail(c, TC_EDEVICE, "the FMM's refinement stack (some 2500 sources per cell) overflowed; raise theta");
         if (e & (kErrFmmPool | kErrFmmSlab))
             return fail(c, TC_EDEVICE, "the FMM's unresolved-source lists still overflowed after regrowing");
         if (e & kErrBand)

@@ -586,8 +586,12 @@ __global__ void __launch_bounds__(kFmmWarps * 32, kFmmBlocksPerSm) k_fmm_walk(Fm
             const int4 pb = __ldg(a.fnode + 3 * (int64_t)P + 2);
             nch = pb.w >> 8;
             pz = pb.z;
-            // the parent's records (its ticket is an earlier one, so the warp
-            // that holds it has started)
+            // the parent's records.  Its ticket is an earlier one, though it
+            // may still be untaken among the eight that another block holds.
+            // The wait ends: of the unfinished cells the first waits for
+            // nobody, and if it is untaken, the warps of the block that holds
+            // it are at cells of earlier tickets (a block takes its cells in
+            // order), which are finished, so one of them takes it
             if (lane == 0) {
                 volatile const int32_t* done = &a.near_cnt[P];
                 const long long t0 = clock64();

@@ -623,9 +623,11 @@ __global__ void __launch_bounds__(kTrainWarps * 32) k_mlp_epoch(const float* __r
 // the parameters: it adds the eight blocks' sums (distributed shared memory),
 // updates, and stores the parameter in all eight blocks, which turn them into
 // the BF16 copies the next step reads.  Same operations, same order, same
-// network.  Bound by mma.sync, which takes some 27 cycles a scheduler
-// here: 7.3 of a step's 17 thousand cycles are forward and backward, two tiles
-// a scheduler, 2.6 the gradient's products, 2.2 the two cluster barriers.  The
+// network.  Bound by latency at two warps a scheduler: of six cycles an
+// instruction waits, 1.9 are for shared memory, 1.4 fixed latencies, 0.7 loads
+// and 0.7 barriers, while the tensor unit is busy 11 % (8 cycles a mma.sync).
+// 7.3 of a step's 17 thousand cycles are forward and backward, two tiles a
+// scheduler, 2.6 the gradient's products, 2.2 the two cluster barriers.  The
 // sums' and parameters' exchange was 3.9 when each of a thread's three
 // elements was read, updated and stored in turn, and the row indices of the
 // next tile cost their latency when they were not loaded a tile ahead.

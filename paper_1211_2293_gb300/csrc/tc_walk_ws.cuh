@@ -425,9 +425,11 @@ __device__ __forceinline__ unsigned ws_incl_scan(unsigned x)
 // the correction's network.  1: the producer records them, and the group's
 // record (box centre and frame), for k_band_eval after the walk; 2: the
 // producer runs the network on 32 of them at a time, as k_walk does, and hands
-// the group's correction over with its last tile.  The mma.sync of a call take
-// a scheduler's tensor unit 2.4 thousand cycles, six calls a group: the
-// producers are then as long at a group as the consumers.  Plummer spheres at
+// the group's correction over with its last tile.  What that costs is
+// instructions and their fetch, not the tensor unit (2^20 bodies at theta
+// 0.667, band 0.55: 1.31 ms against 1.00 without a band cell; 13 % more
+// instructions, fetch stalls 0.47 -> 0.79 per issue, issue 60 -> 55 %, the
+// tensor unit busy 6 % of the cycles, 8 a mma.sync).  Plummer spheres at
 // theta 0.67, band 0.55, us, one-warp walk / recorded / in the producers: 5000
 // bodies 154 / 79 / 48, 20000 182 / 100 / 77, 300000 446 / 424 / 414, 2^22
 // 5326 / 5273 / 5205.
