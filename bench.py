@@ -1289,8 +1289,9 @@ def run_learned(args, rank, world, local_rank):
 def run_profile_case(args):
     """One small case of a kernel family, for an ncu capture, then exit:
     build: a uniform cube built twice (eager builds; capture the second);
-    learned: one learned walk (seeded random network, band 0.5, theta 0.9)
-    on a 2^20-body Plummer sphere; quadrupole: one quadrupole walk (theta
+    learned: one learned walk (seeded random network) on a 2^20-body Plummer
+    sphere at the opening angle and band of the default line's learned path
+    (0.667, 0.55); quadrupole: one quadrupole walk (theta
     0.7) on the same sphere; fmm: two FMM passes (theta 0.55) on a Plummer
     sphere of --n bodies (default 2^20); band: two learned force phases with
     the network after the walk (split 2: k_band_eval, the same random network,
@@ -1401,9 +1402,9 @@ def run_profile_case(args):
         rng = np.random.default_rng(0)
         params = (rng.standard_normal(tc.MLP_NPARAM) * 0.1).astype(np.float32)
         model = np.concatenate([params, np.zeros(13), np.ones(13), np.full(3, 1e-3)]).astype(np.float32)
-        ctx.mlp_set(model, 0.5)
+        ctx.mlp_set(model, 0.55)
         ctx.set_config(learned=1)
-        ctx.forces(0.9, 1e-3)
+        ctx.forces(0.667, 1e-3)
         ctx.sync()
         print(f"learned walk: Plummer N={n}, evals {ctx.mlp_evals()}")
     else:
