@@ -72,21 +72,23 @@ __global__ void k_kick_drift(float* __restrict__ pos, float* __restrict__ vel, c
 
 // Results for the caller, who keeps what was there where the force phase
 // failed.  The kernel looks at the error word itself, so one wait serves the
-// copy and the word.
-template <bool VEC>
-__global__ void __launch_bounds__(256) k_copy_good(float* __restrict__ dst, const float* __restrict__ src, int64_t n,
+// copy and the word.  A thread copies kCopy elements, all loads first; the
+// first block the `rest` floats behind them.
+constexpr int kCopy = 4;
+template <typename T>
+__global__ void __launch_bounds__(256) k_copy_good(T* __restrict__ dst, const T* __restrict__ src, int64_t n, int rest,
                                                    const Info* info)
 {
+    const int64_t i0 = (int64_t)blockIdx.x * (256 * kCopy) + threadIdx.x;
+    T x[kCopy];
+#pragma unroll
+    for (int k = 0; k < kCopy; k++)
+        if (i0 + k * 256 < n) x[k] = src[i0 + k * 256];
     if (warp_failed(info)) return;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t done = 0;
-    if (VEC) {
-        const int64_t n4 = n >> 2;
-#pragma unroll 4
-        for (int64_t i = i0; i < n4; i += stride) reinterpret_cast<float4*>(dst)[i] = reinterpret_cast<const float4*>(src)[i];
-        done = n4 << 2;
-    }
-    for (int64_t i = done + i0; i < n; i += stride) dst[i] = src[i];
+#pragma unroll
+    for (int k = 0; k < kCopy; k++)
+        if (i0 + k * 256 < n) dst[i0 + k * 256] = x[k];
+    if (i0 < rest) reinterpret_cast<float*>(dst + n)[i0] = reinterpret_cast<const float*>(src + n)[i0];
 }
 
 // KE, PE = 1/2 sum m pot, P, L in FP64; block sums, then FP64 atomics
@@ -366,10 +368,11 @@ void launch_kick_drift(float* pos, float* vel, const float* acc, int64_t n, floa
 void launch_copy_good(float* dst, const float* src, int64_t n, const Info* info, cudaStream_t s)
 {
     const bool vec = ((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15u) == 0;
-    int64_t g = nblk(vec ? (n + 3) / 4 : n, 256);
-    if (g > 8 * sm_count()) g = 8 * sm_count();
-    if (vec) k_copy_good<true><<<(unsigned)g, 256, 0, s>>>(dst, src, n, info);
-    else k_copy_good<false><<<(unsigned)g, 256, 0, s>>>(dst, src, n, info);
+    const auto go = [&](auto* to, const auto* from, int64_t k, int rest) {
+        k_copy_good<<<nblk(k + (rest > 0), 256 * kCopy), 256, 0, s>>>(to, from, k, rest, info);
+    };
+    if (vec) go(reinterpret_cast<float4*>(dst), reinterpret_cast<const float4*>(src), n >> 2, (int)(n & 3));
+    else go(dst, src, n, 0);
     count_launches(1);
 }
 
