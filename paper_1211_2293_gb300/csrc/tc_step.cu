@@ -154,7 +154,9 @@ __device__ __forceinline__ float dir_rsqrt(float x)
     return FTZ ? rsqrt_sfu(x) : rsqrtf(x);
 }
 
-template <bool FTZ>
+// ONE: a single slice, which writes the results (a branch instead cost the
+// sliced sums 1.3 %)
+template <bool FTZ, bool ONE>
 __global__ void __launch_bounds__(kDirThreads, kDirBlocksPerSm)
     k_direct(const float* __restrict__ pos, const float* __restrict__ mass, const uint32_t* __restrict__ sys_of,
              const SysParams* __restrict__ sysp, const int64_t* __restrict__ idx, int64_t ns, float eps2, float G,
@@ -308,7 +310,7 @@ __global__ void __launch_bounds__(kDirThreads, kDirBlocksPerSm)
     for (int q = 0; q < NT; q++) {
         const int64_t t = t0 + q * kDirThreads + threadIdx.x;
         if (t >= ns) continue;
-        if (gridDim.y == 1) {
+        if (ONE) {
             acc[3 * t] = (double)G * ax[q];
             acc[3 * t + 1] = (double)G * ay[q];
             acc[3 * t + 2] = (double)G * az[q];
@@ -461,10 +463,12 @@ void launch_direct(const float* pos, const float* mass, const uint32_t* sys_of, 
                    double* pot, cudaStream_t s)
 {
     const dim3 grid(nblk(ns, kDirTargets), (unsigned)slices);
-    if (eps2 >= FLT_MIN)
-        k_direct<true><<<grid, kDirThreads, 0, s>>>(pos, mass, sys_of, sysp, idx, ns, eps2, G, part, acc, pot);
-    else k_direct<false><<<grid, kDirThreads, 0, s>>>(pos, mass, sys_of, sysp, idx, ns, eps2, G, part, acc, pot);
-    count_launches(1);
+    const auto go = [&](auto* kernel) {
+        kernel<<<grid, kDirThreads, 0, s>>>(pos, mass, sys_of, sysp, idx, ns, eps2, G, part, acc, pot);
+        count_launches(1);
+    };
+    if (slices == 1) eps2 >= FLT_MIN ? go(k_direct<true, true>) : go(k_direct<false, true>);
+    else eps2 >= FLT_MIN ? go(k_direct<true, false>) : go(k_direct<false, false>);
     if (slices == 1) return;
     k_direct_reduce<<<nblk(4 * ns, 256), 256, 0, s>>>(part, slices, ns, mass, idx, eps2, G, acc, pot);
     count_launches(1);
