@@ -1168,8 +1168,7 @@ int tc_get_acc(tc_ctx* c, float* acc, float* pot)
     // memory they are written by a kernel that looks at the error word, and
     // one wait does for both; elsewhere the word comes first
     if ((!acc || on_device(c, acc)) && (!pot || on_device(c, pot))) {
-        if (acc) launch_copy_good(acc, c->acc, 3 * c->n, c->info, c->stream);
-        if (pot) launch_copy_good(pot, c->pot, c->n, c->info, c->stream);
+        launch_copy_good(acc, c->acc, pot, c->pot, c->n, c->info, c->stream);
         TC_CUDA(c, cudaGetLastError());
         return check_device(c);
     }

@@ -506,8 +506,8 @@ __global__ void __launch_bounds__(kNodeThreads) k_node_levels_tiled(const uint64
 }
 
 // Exclusive scan of the counts in place, one pass; the total is the number of
-// nodes (info->M follows with the records).  A look-back that gave up raises kErrCapacity too, so nothing is
-// placed by offsets that are not known.
+// nodes (info->M follows with the records).  A look-back that gave up raises
+// kErrCapacity too, so nothing is placed by offsets that are not known.
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 16;
 constexpr int kScanTile = kScanThreads * kScanItems;
@@ -1348,8 +1348,8 @@ void launch_emit_nodes(const uint64_t* keys, const int8_t* delta, const int8_t* 
 }
 
 void launch_moments(const float4* body, const uint64_t* keys, const int8_t* delta, int64_t n, int nsys,
-                    int64_t cap_m, int depth, int depth_hint, const uint32_t* level_start, SysParams* sysp, const Info* info, NodeTables nt,
-                    bool quad, ChainStream s)
+                    int64_t cap_m, int depth, int depth_hint, const uint32_t* level_start, SysParams* sysp,
+                    const Info* info, NodeTables nt, bool quad, ChainStream s)
 {
     const unsigned g = gsgrid(cap_m, 128);
     const bool climb = n <= kClimbBodies;

@@ -399,8 +399,10 @@ void launch_fp32_probe(bool paired, int blocks, int iters, float* out, cudaStrea
 void launch_kick_drift(float* pos, float* vel, const float* acc, int64_t n, float hkick, float dt,
                        const Info* info, cudaStream_t s);
 void launch_kick(float* vel, const float* acc, int64_t n, float hkick, const Info* info, cudaStream_t s);
-// n floats to dst, memory of this device, unless the error word is set
-void launch_copy_good(float* dst, const float* src, int64_t n, const Info* info, cudaStream_t s);
+// n bodies' accelerations and potentials (either may be null) to memory of this
+// device, unless the error word is set
+void launch_copy_good(float* acc, const float* from_acc, float* pot, const float* from_pot, int64_t n,
+                      const Info* info, cudaStream_t s);
 void launch_diag(const float* pos, const float* vel, const float* mass, const float* pot,
                  int64_t n, Info* info, cudaStream_t s);
 // source slices of a direct sum that fill the device; launch_direct's scratch

@@ -72,23 +72,35 @@ __global__ void k_kick_drift(float* __restrict__ pos, float* __restrict__ vel, c
 
 // Results for the caller, who keeps what was there where the force phase
 // failed.  The kernel looks at the error word itself, so one wait serves the
-// copy and the word.  A thread copies kCopy elements, all loads first; the
-// first block the `rest` floats behind them.
+// copy and the word, and takes both arrays in one launch (a call with the
+// potential over 2079 bodies 31 us, its wait included, 34 as two copies): the
+// first `blocks` blocks the accelerations.  A thread copies kCopy elements, all loads first; an array's
+// first block the up to three floats behind them.
 constexpr int kCopy = 4;
 template <typename T>
-__global__ void __launch_bounds__(256) k_copy_good(T* __restrict__ dst, const T* __restrict__ src, int64_t n, int rest,
-                                                   const Info* info)
+struct CopyJob {
+    T* dst;
+    const T* src;
+    int64_t n;
+    int rest;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_copy_good(CopyJob<T> acc, CopyJob<T> pot, unsigned blocks, const Info* info)
 {
-    const int64_t i0 = (int64_t)blockIdx.x * (256 * kCopy) + threadIdx.x;
+    const bool first = blockIdx.x < blocks;
+    const CopyJob<T> j = first ? acc : pot;
+    const int64_t i0 = (int64_t)(first ? blockIdx.x : blockIdx.x - blocks) * (256 * kCopy) + threadIdx.x;
     T x[kCopy];
 #pragma unroll
     for (int k = 0; k < kCopy; k++)
-        if (i0 + k * 256 < n) x[k] = src[i0 + k * 256];
+        if (i0 + k * 256 < j.n) x[k] = j.src[i0 + k * 256];
     if (warp_failed(info)) return;
 #pragma unroll
     for (int k = 0; k < kCopy; k++)
-        if (i0 + k * 256 < n) dst[i0 + k * 256] = x[k];
-    if (i0 < rest) reinterpret_cast<float*>(dst + n)[i0] = reinterpret_cast<const float*>(src + n)[i0];
+        if (i0 + k * 256 < j.n) j.dst[i0 + k * 256] = x[k];
+    if (i0 < j.rest)
+        reinterpret_cast<float*>(j.dst + j.n)[i0] = reinterpret_cast<const float*>(j.src + j.n)[i0];
 }
 
 // KE, PE = 1/2 sum m pot, P, L in FP64; block sums, then FP64 atomics
@@ -367,15 +379,28 @@ void launch_kick_drift(float* pos, float* vel, const float* acc, int64_t n, floa
     launch_update<true>(pos, vel, acc, n, hkick, dt, info, s);
 }
 
-void launch_copy_good(float* dst, const float* src, int64_t n, const Info* info, cudaStream_t s)
+// acc or pot may be null
+void launch_copy_good(float* acc, const float* from_acc, float* pot, const float* from_pot, int64_t n,
+                      const Info* info, cudaStream_t s)
 {
-    const bool vec = ((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15u) == 0;
-    const auto go = [&](auto* to, const auto* from, int64_t k, int rest) {
-        k_copy_good<<<nblk(k + (rest > 0), 256 * kCopy), 256, 0, s>>>(to, from, k, rest, info);
+    const auto go = [&](auto zero) {
+        using T = decltype(zero);
+        constexpr int64_t w = sizeof(T) / sizeof(float);
+        const auto job = [&](float* to, const float* from, int64_t k) {
+            if (!to) k = 0;
+            return CopyJob<T>{reinterpret_cast<T*>(to), reinterpret_cast<const T*>(from), k / w, (int)(k % w)};
+        };
+        const auto blocks = [&](const CopyJob<T>& j) { return nblk(j.n + (j.rest > 0), 256 * kCopy); };
+        const CopyJob<T> a = job(acc, from_acc, 3 * n), p = job(pot, from_pot, n);
+        const unsigned ga = blocks(a), gp = blocks(p);
+        if (ga + gp == 0) return;
+        k_copy_good<T><<<ga + gp, 256, 0, s>>>(a, p, ga, info);
+        count_launches(1);
     };
-    if (vec) go(reinterpret_cast<float4*>(dst), reinterpret_cast<const float4*>(src), n >> 2, (int)(n & 3));
-    else go(dst, src, n, 0);
-    count_launches(1);
+    const uintptr_t all = reinterpret_cast<uintptr_t>(acc) | reinterpret_cast<uintptr_t>(from_acc) |
+                          reinterpret_cast<uintptr_t>(pot) | reinterpret_cast<uintptr_t>(from_pot);
+    if ((all & 15u) == 0) go(float4{});
+    else go(0.f);
 }
 
 void launch_kick(float* vel, const float* acc, int64_t n, float hkick, const Info* info, cudaStream_t s)
