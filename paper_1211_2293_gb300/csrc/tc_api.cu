@@ -536,7 +536,9 @@ int build_tree(tc_ctx* c, bool synced, cudaStream_t s, bool all_digits = false)
     // deeper tree gives longer runs, which the completion still orders: up
     // to kSortRunMax bodies a run inside a step; in a synchronised build up
     // to kSortRunMaxSynced, past which the build is redone sorting every
-    // digit).  With no earlier depth every digit is sorted.
+    // digit; the one-block sort of small n has no such limit, it sorts every
+    // digit itself where a run is long).  With no earlier depth every digit is
+    // sorted.
     int low_bit = 0;
     if (!all_digits && c->depth_hint >= 0 && (!synced || n == c->depth_hint_n)) {
         const int levels = std::min(kMaxLevel, c->depth_hint + kSortMarginLevels);
